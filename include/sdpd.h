@@ -305,8 +305,8 @@ sdpd_status sdpd_graph_kernels(sdpd_ctx *ctx, long long *n_kernels);
  * box); on wall axes positions outside the box are used as given.  A
  * particle whose position is not finite gets d = p = NaN and is nobody's
  * neighbour; the other particles are unaffected.
- * Scratch: one file-scope __device__ array of about 2 MB (cell keys, slots,
- * counts, starts, permutation) held by every GPU that loads the library until
+ * Scratch: one file-scope __device__ array of about 4 MB (cell keys, slots,
+ * counts, starts, records) held by every GPU that loads the library until
  * the process exits.  At most SDPD_NOALLOC_MAX_PARTICLES particles and
  * SDPD_NOALLOC_MAX_CELLS cells of width >= r_c (periodic axes: floor(box/r_c)
  * cells, >= 3; wall axes: the box plus 2 r_c on each side); larger inputs are
