@@ -15,6 +15,7 @@
 // (16 g + c) * 128 of a 32 KB tile; descriptor leading-dimension offset 128 B
 // (next K chunk), stride-dimension offset 2048 B (next 8-row group).  Every
 // address an MMA can touch lies inside its 32 KB tile.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -37,6 +38,9 @@ __host__ __device__ constexpr int off_W(int l) { return OFF_B0 + WID + (l - 1) *
 __host__ __device__ constexpr int off_b(int l) { return off_W(l) + WID * WID; }
 constexpr int OFF_W4 = OFF_B0 + WID + 3 * (WID * WID + WID), OFF_B4 = OFF_W4 + WID;
 static_assert(OFF_B4 + 1 == NPARAM, "parameter layout");
+// one tile's gradient share: padded so that every share starts on 16 bytes
+constexpr int GSTRIDE = (NPARAM + 3) / 4 * 4;
+static_assert(off_W(1) % 4 == 0 && (WID * WID + WID) % 4 == 0, "weight gradients are stored as float4");
 
 // instruction descriptor of kind::f16: D FP32 (bits 4-5 = 1), A BF16 (bits
 // 7-9 = 1), B BF16 (bits 10-12 = 1), both K-major, N >> 3 at bits 17-22,
@@ -191,83 +195,18 @@ __device__ __forceinline__ void put8(uint8_t *tile, int r, int k0, const float *
     *reinterpret_cast<uint4 *>(tile + core_off(r, k0)) = *reinterpret_cast<uint4 *>(h);
 }
 
-__device__ __forceinline__ void put1(uint8_t *tile, int r, int k, float v)
-{
-    *reinterpret_cast<__nv_bfloat16 *>(tile + core_off(r, k)) = __float2bfloat16_rn(v);
-}
-
-// D(128 x 128, TMEM) (+)= A(tile) . B(tile)^T over K = 128 in eight K = 16
-// steps, issued by thread 0; every thread waits for completion.  Returns
-// false if the wait timed out (error recorded).
-__device__ bool gemm_128(uint8_t *A, uint8_t *B, uint32_t dtmem, bool accumulate, uint64_t *mbar,
-                         uint32_t &parity, int *err)
-{
-    proxy_fence();
-    tc_fence_before();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        tc_fence_after();
-        const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
-#pragma unroll
-        for (int s = 0; s < 8; ++s)
-            mma_bf16(dtmem, make_desc(a0 + s * 256), make_desc(b0 + s * 256), (accumulate || s > 0) ? 1 : 0);
-        mma_commit(mbar);
-    }
-    const bool ok = mbar_wait(mbar, parity);
-    if (!ok) {
-        // record the failure, then give the MMAs in flight one more bounded
-        // wait before the caller frees tensor memory
-        if (threadIdx.x == 0) atomicOr(err, ERR_MMA_TIMEOUT);
-        (void)mbar_wait(mbar, parity);
-    }
-    parity ^= 1u;
-    tc_fence_after();
-    return __syncthreads_and(ok ? 1 : 0) != 0;
-}
-
-// Row t (= this thread) of the accumulator, column chunk c (16 values).
-__device__ __forceinline__ void acc_row16(uint32_t taddr, int c, float v[16])
-{
-    const uint32_t lane_base = (uint32_t)((threadIdx.x >> 5) * 32) << 16;
-    tc_ld16(taddr + lane_base + (uint32_t)(c * 16), v);
-}
-
 struct Net {
     float *P;            // FP32 master parameters [NPARAM]
     float *G;            // gradients [NPARAM]
     float *M, *V;        // Adam moments
     __nv_bfloat16 *Wb;   // BF16 copies of W1..W3 [3][128][128]
-    float *Z, *H0, *D;   // training scratch: Z [4][Bmax][128], first-layer input copy, dz buffers
-    float *Gp, *Lp;      // per-tile gradient shares [Bmax/128][NPARAM] and squared-error sums
-    float *Y, *DY, *loss;
+    float *Gp, *Lp;      // per-tile gradient shares [tiles][GSTRIDE] and squared-error sums
+    float *loss;
     int *err;
     int bmax;
     long long step;
     cudaStream_t own;
 };
-
-// Stage the BF16 weights of layer l (as B operand: rows = out, K = in) or
-// its transpose (rows = in, K = out).
-__device__ void stage_weights(uint8_t *tile, const __nv_bfloat16 *W, bool transpose)
-{
-    const int t = threadIdx.x;
-    if (!transpose) {
-        float v[8];
-        for (int c = 0; c < 16; ++c) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = __bfloat162float(W[t * WID + 8 * c + i]);
-            put8(tile, t, 8 * c, v);
-        }
-    } else {
-        // row i = t of W^T: column t of W
-        float v[8];
-        for (int c = 0; c < 16; ++c) {
-#pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = __bfloat162float(W[(8 * c + i) * WID + t]);
-            put8(tile, t, 8 * c, v);
-        }
-    }
-}
 
 // ------------------------------------------------------------- inference
 // Persistent over 128-row tiles with NWG warpgroups per CTA: each warpgroup
@@ -405,195 +344,362 @@ __global__ void __launch_bounds__(128 * NWG, 1) k_mlp_forward(const float *__res
 }
 
 // ------------------------------------------------------------- training
-// One CTA per 128-row tile of the batch: forward (pre-activations kept in Z),
-// backward through every layer for the tile's rows, the tile's share of each
-// gradient into its row of Gp [ntile][NPARAM] and its squared-error sum into
-// Lp[tile]; k_mlp_reduce adds the tiles in a fixed order.  The output
-// gradient dy = 2 (y - t) / B needs no sum across tiles, so the tiles are
-// independent.  Thread t owns batch row tile * 128 + t (TMEM lane t) in the
-// row-wise steps and output unit t in the column-wise sums.
-__global__ void __launch_bounds__(128, 1) k_mlp_grad(Net net, const float *__restrict__ X,
-                                                     const float *__restrict__ T, int B)
+// One CTA of 16 warps per tile of ROWS batch rows: forward, backward, the
+// tile's share of each gradient into its row of Gp [ntile][GSTRIDE] and its
+// squared-error sum into Lp[tile]; k_mlp_reduce adds the tiles in a fixed
+// order.  The output gradient dy = 2 (y - t) / B needs no sum across tiles, so
+// the tiles are independent.
+//
+// The step is a chain of small layers, so its latency is the bound, not a
+// rate: a tile is 16 or 32 rows (not the 128 an MMA would take as M), which
+// spreads a batch of 256 over 16 CTAs, and every layer is computed
+// transposed.  Features are the M dimension (TMEM lanes), batch rows the N
+// dimension (columns), so all 16 warps share the element-wise work of a
+// layer: thread (warp w, lane) owns feature o = 32 (w & 3) + lane of rows
+// RPT (w >> 2) .. + RPT - 1, and its pre-activations of all layers stay in
+// registers.  What a 128-row CTA of four warps took 345 us for (its
+// pre-activations in global memory, each thread striding over its row, and
+// operands transposed through 2-byte stores) takes 23 us for a batch of 256
+// and 28 us for 4,096 (cold caches).
+//
+// One physical form of an operand serves every GEMM that reads it, as K-major
+// or, transposed, as MN-major (instruction descriptor bits 15 and 16):
+//   forward  z^T  = W a^T    A = W   (M = out, K = in)  B = a  (N = row, K = in)
+//   input    dh^T = W^T dz^T A = W^T (M = in,  K = out) B = dz (N = row, K = out)
+//   weights  gW   = dz^T a   A = dz^T (M = out, K = row) B = a^T (N = in, K = row)
+// Tiles hold 8-row x 16-byte core matrices without swizzle: row group g and
+// 16-byte chunk c at TG g + TC c, with the chunks 144 bytes apart so that the
+// 2-byte stores of a warp (32 features of one row) fall on different banks.
+// K-major: leading offset TC (next chunk along K), stride offset TG (next 8
+// rows); MN-major: stride offset TC (next 8 along M or N), leading offset TG
+// (next 8 along K).
+constexpr uint32_t TC = 144, TG = 16 * TC;
+constexpr uint32_t W_BYTES = 16 * TG;                      // 128 rows
+constexpr uint32_t ID_BASE = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(WID >> 4) << 24);
+__host__ __device__ constexpr uint32_t idesc_n(int n, int ta, int tb)
 {
+    return ID_BASE | ((uint32_t)ta << 15) | ((uint32_t)tb << 16) | ((uint32_t)(n >> 3) << 17);
+}
+
+__device__ __forceinline__ uint64_t desc_of(uint32_t saddr, uint32_t lead, uint32_t stride)
+{
+    return (uint64_t)((saddr >> 4) & 0x3FFFu) | ((uint64_t)(lead >> 4) << 16) | ((uint64_t)(stride >> 4) << 32) |
+           ((uint64_t)1 << 46);
+}
+
+__device__ __forceinline__ void mma_any(uint32_t dtmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc, int accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(dtmem),
+        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate));
+}
+
+template <int N>
+__device__ __forceinline__ void tc_ld_cols(uint32_t taddr, float *v)
+{
+    uint32_t r[N];
+    if constexpr (N == 4) {
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                     : "r"(taddr));
+    } else {
+        static_assert(N == 8, "4 or 8 columns");
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                     : "r"(taddr));
+    }
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < N; ++i) v[i] = __uint_as_float(r[i]);
+}
+
+__device__ __forceinline__ void cp_async16(uint32_t saddr, const void *g)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(saddr), "l"(g) : "memory");
+}
+
+constexpr int GRAD_THREADS = 512;
+template <int ROWS> struct GradSmem {
+    static constexpr uint32_t A_BYTES = (ROWS / 8) * TG;   // one activation tile
+    static constexpr uint32_t OFF_A = 3 * W_BYTES;         // a0, a1, a2 (inputs of the hidden layers)
+    static constexpr uint32_t OFF_DZ = OFF_A + 3 * A_BYTES;
+    static constexpr uint32_t OFF_H = OFF_DZ + A_BYTES;    // FP32 [128][ROWS + 1]: last hidden layer
+    static constexpr uint32_t OFF_SUM = OFF_H + 128 * (ROWS + 1) * 4;   // FP32 [4][128][4]: partial sums
+    static constexpr uint32_t OFF_X = OFF_SUM + 4 * 128 * 4 * 4;        // FP32 [ROWS][4]: inputs, dy
+    static constexpr uint32_t OFF_BAR = OFF_X + ROWS * 16; // 7 mbarriers, TMEM slot, flag
+    static constexpr uint32_t BYTES = OFF_BAR + 128;
+};
+
+template <int ROWS>
+__global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(Net net, const float *__restrict__ X,
+                                                              const float *__restrict__ T, int B)
+{
+    using S = GradSmem<ROWS>;
+    constexpr int RPT = ROWS / 4;             // rows of a thread
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t *sA = smem;                       // A operand
-    uint8_t *sB = smem + TILE_BYTES;          // B operand
-    uint8_t *sC = smem + 2 * TILE_BYTES;      // second A (weight-gradient GEMM)
-    uint8_t *sD = smem + 3 * TILE_BYTES;      // second B
-    uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + 4 * TILE_BYTES);
-    uint32_t *slot = reinterpret_cast<uint32_t *>(smem + 4 * TILE_BYTES + 16);
-    float *red = reinterpret_cast<float *>(smem + 4 * TILE_BYTES + 32);   // 4 floats
-    const int t = threadIdx.x;
-    const int tile = blockIdx.x;
-    const int r0 = tile * WID;                // first batch row of the tile
-    const int nrow = min(WID, B - r0);        // rows of this tile
-    const int row = r0 + t;
-    const bool valid = t < nrow;
-    const int bm = net.bmax;
-    float *Z = net.Z;                         // [4][bmax][128]
-    float *Dc = net.D, *Dn = net.D + (size_t)bm * WID;   // dz of the current / next layer
-    float *Gp = net.Gp + (size_t)tile * NPARAM;
-    const float *P = net.P;
-    if (t == 0) mbar_init(mbar);
-    if (t < 32) tc_alloc(slot, 256);
+    const uint32_t sbase = smem_u32(smem);
+    float *hbuf = reinterpret_cast<float *>(smem + S::OFF_H);
+    float *sums = reinterpret_cast<float *>(smem + S::OFF_SUM);
+    float4 *xs = reinterpret_cast<float4 *>(smem + S::OFF_X);
+    uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + S::OFF_BAR);
+    uint32_t *slot = reinterpret_cast<uint32_t *>(smem + S::OFF_BAR + 64);
+    volatile int *flag = reinterpret_cast<int *>(smem + S::OFF_BAR + 72);
+    const int t = threadIdx.x, w = t >> 5, cg = w >> 2;
+    const int o = (w & 3) * 32 + (t & 31);    // this thread's feature
+    const int r0 = blockIdx.x * ROWS;         // first batch row of the tile
+    const float *__restrict__ P = net.P;
+    float *__restrict__ Gp = net.Gp + (size_t)blockIdx.x * GSTRIDE;
+    // the weight tiles, one copy group per layer
+    for (int l = 0; l < 3; ++l) {
+        for (int q = t; q < WID * 16; q += GRAD_THREADS) {
+            const int r = q >> 4, c = q & 15;
+            cp_async16(sbase + l * W_BYTES + (r >> 3) * TG + c * TC + (r & 7) * 16,
+                       net.Wb + (l * WID + r) * WID + 8 * c);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    if (t < 7) mbar_init(mbar + t);
+    if (t == 0) *flag = 0;
+    if (w == 0) tc_alloc(slot, 512);
+    if (t < ROWS) {
+        const int row = r0 + t;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row < B) { x.x = X[3 * row]; x.y = X[3 * row + 1]; x.z = X[3 * row + 2]; }
+        xs[t] = x;
+    }
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t taddr = *slot;             // columns [0,128): activations; [128,256): weight gradients
-    uint32_t parity = 0;
-    bool ok = true;
-    float v[16];
-    // ---------------- forward, keeping the pre-activations
-    const float x0 = valid ? X[3 * row] : 0.f, x1 = valid ? X[3 * row + 1] : 0.f, x2 = valid ? X[3 * row + 2] : 0.f;
-    for (int c = 0; c < 16; ++c) {
-        float h[8];
+    const uint32_t tm = *slot;
+    const uint32_t lanes = (uint32_t)((w & 3) * 32) << 16;
+    // TMEM: z_l / dh columns [0, 32), [32, 64), [64, 96); gW_l at 128 l (l = 1..3)
+    const uint32_t zcol[3] = { tm, tm + 32u, tm + 64u };
+    // one bf16 per row of this thread into a tile [row][feature]
+    auto put = [&](uint32_t off, const float *v) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int o = 8 * c + i;
-            const float z = P[OFF_W0 + 3 * o] * x0 + P[OFF_W0 + 3 * o + 1] * x1 + P[OFF_W0 + 3 * o + 2] * x2 +
-                            P[OFF_B0 + o];
-            Z[(0 * bm + row) * WID + o] = valid ? z : 0.f;
-            h[i] = valid ? gelu(z) : 0.f;
+        for (int i = 0; i < RPT; ++i) {
+            const int r = cg * RPT + i;
+            *reinterpret_cast<__nv_bfloat16 *>(smem + off + (r >> 3) * TG + (o >> 3) * TC + (r & 7) * 16 + (o & 7) * 2) =
+                __float2bfloat16_rn(v[i]);
         }
-        put8(sA, t, 8 * c, h);
-    }
-    float y = 0.f;
-    for (int l = 1; l <= 3 && ok; ++l) {
-        stage_weights(sB, net.Wb + (l - 1) * WID * WID, false);
-        ok = gemm_128(sA, sB, taddr, false, mbar, parity, net.err);
-        if (!ok) break;
-        for (int c = 0; c < 8; ++c) {
-            acc_row16(taddr, c, v);
+    };
+    // every thread waits for MMA group k; a timeout in any thread is seen by
+    // all at the next barrier
+    auto wait = [&](int k) {
+        if (!mbar_wait(mbar + k, 0)) {
+            *flag = 1;
+            atomicOr(net.err, ERR_MMA_TIMEOUT);
+            (void)mbar_wait(mbar + k, 0);
+        }
+        tc_fence_after();
+    };
+    float z[4][RPT];
+    // ---------------- forward, the pre-activations kept
+    {
+        const float w0 = P[OFF_W0 + 3 * o], w1 = P[OFF_W0 + 3 * o + 1], w2 = P[OFF_W0 + 3 * o + 2], b0 = P[OFF_B0 + o];
+        float h[RPT];
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int o = 16 * c + i;
-                const float z = v[i] + P[off_b(l) + o];
-                Z[(l * bm + row) * WID + o] = valid ? z : 0.f;
-                const float h = valid ? gelu(z) : 0.f;
-                if (l < 3) v[i] = h;
-                else y += h * P[OFF_W4 + o];
-            }
-            if (l < 3) {
-                put8(sA, t, 16 * c, v);
-                put8(sA, t, 16 * c + 8, v + 8);
-            }
+        for (int i = 0; i < RPT; ++i) {
+            const float4 x = xs[cg * RPT + i];
+            z[0][i] = w0 * x.x + w1 * x.y + w2 * x.z + b0;
+            h[i] = gelu(z[0][i]);
+        }
+        put(S::OFF_A, h);
+    }
+#pragma unroll
+    for (int l = 1; l <= 3; ++l) {
+        if (l == 1) asm volatile("cp.async.wait_group 2;\n" ::: "memory");
+        else if (l == 2) asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        proxy_fence();
+        __syncthreads();
+        if (t == 0) {
+            tc_fence_after();
+            const uint32_t a0 = sbase + (l - 1) * W_BYTES, b0 = sbase + S::OFF_A + (l - 1) * S::A_BYTES;
+#pragma unroll
+            for (int s = 0; s < 8; ++s)
+                mma_any(zcol[l - 1], desc_of(a0 + s * 2 * TC, TC, TG), desc_of(b0 + s * 2 * TC, TC, TG),
+                        idesc_n(ROWS, 0, 0), s > 0);
+            mma_commit(mbar + l - 1);
+        }
+        const float bias = P[off_b(l) + o];
+        wait(l - 1);
+        float v[RPT], h[RPT];
+        tc_ld_cols<RPT>(zcol[l - 1] + lanes + (uint32_t)(cg * RPT), v);
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            z[l][i] = v[i] + bias;
+            h[i] = gelu(z[l][i]);
+        }
+        if (l < 3) {
+            put(S::OFF_A + l * S::A_BYTES, h);
+        } else {
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) hbuf[o * (ROWS + 1) + cg * RPT + i] = h[i];
         }
         tc_fence_before();
-        __syncthreads();
     }
-    if (!ok) goto done;
-    {
-        float dy = 0.f, sq = 0.f;
-        if (valid) {
+    __syncthreads();
+    // output layer: the row's sum over the features in order, one thread per row
+    if (w == 0) {
+        float y = 0.f, dy = 0.f, sq = 0.f;
+        const int row = r0 + t;
+        if (t < ROWS && row < B) {
+#pragma unroll 8
+            for (int k = 0; k < WID; ++k) y += hbuf[k * (ROWS + 1) + t] * P[OFF_W4 + k];
             y += P[OFF_B4];
-            net.Y[row] = y;
             dy = 2.0f * (y - T[row]) / (float)B;
             sq = (y - T[row]) * (y - T[row]);
         }
-        net.DY[row] = dy;   // 0 on the rows past B (the scratch holds whole tiles)
-        // the tile's squared-error sum, fixed order: warps, then warps 0..3
+        if (t < ROWS) xs[t].w = dy;   // 0 on the rows past B
+        float gb = dy;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-        if ((t & 31) == 0) red[t >> 5] = sq;
-        __syncthreads();
-        if (t == 0) net.Lp[tile] = (red[0] + red[1]) + (red[2] + red[3]);
-        // output layer (thread t = unit o): gW4 = sum_rows dy gelu(z3), gb4 = sum_rows dy
-        float gw = 0.f, gb = 0.f;
-        for (int r = 0; r < nrow; ++r) {
-            const float d = net.DY[r0 + r];
-            gw += d * gelu(Z[(3 * bm + r0 + r) * WID + t]);
-            gb += d;
+        for (int k = 16; k > 0; k >>= 1) {
+            sq += __shfl_xor_sync(0xffffffffu, sq, k);
+            gb += __shfl_xor_sync(0xffffffffu, gb, k);
         }
-        Gp[OFF_W4 + t] = gw;
-        if (t == 0) Gp[OFF_B4] = gb;
-        // dz of the last hidden layer for this thread's row
-        for (int o = 0; o < WID; ++o)
-            Dc[row * WID + o] = valid ? dy * P[OFF_W4 + o] * gelu_prime(Z[(3 * bm + row) * WID + o]) : 0.f;
+        if (t == 0) {
+            net.Lp[blockIdx.x] = sq;
+            Gp[OFF_B4] = gb;
+        }
     }
     __syncthreads();
-    // ---------------- hidden layers l = 3, 2, 1 (z_l = W_l a_{l-1} + b_l)
-    for (int l = 3; l >= 1 && ok; --l) {
-        // weight gradient over the tile: A = dz^T (rows = unit o, K = row), B = a^T (rows = input i, K = row)
-        for (int o = 0; o < WID; ++o) {
-            put1(sC, o, t, Dc[row * WID + o]);
-            put1(sD, o, t, valid ? gelu(Z[((l - 1) * bm + row) * WID + o]) : 0.f);
-        }
-        ok = gemm_128(sC, sD, taddr + 128, false, mbar, parity, net.err);
-        if (!ok) break;
-        for (int c = 0; c < 8; ++c) {
-            acc_row16(taddr + 128, c, v);
+    // sums over a thread's rows of up to 4 values, then over the 4 row groups
+    // in order: this thread's value `q` of feature o lands in sums[..]
+    auto store_sum = [&](float4 v) { reinterpret_cast<float4 *>(sums)[cg * 128 + o] = v; };
+    auto load_sum = [&]() {
+        const float4 *q = reinterpret_cast<const float4 *>(sums);
+        const float4 a = q[o], b = q[128 + o], c = q[256 + o], d = q[384 + o];
+        return make_float4(((a.x + b.x) + c.x) + d.x, ((a.y + b.y) + c.y) + d.y, ((a.z + b.z) + c.z) + d.z,
+                           ((a.w + b.w) + c.w) + d.w);
+    };
+    float dz[RPT];
+    {
+        const float w4 = P[OFF_W4 + o];
+        float gw = 0.f, gb = 0.f;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) Gp[off_W(l) + t * WID + 16 * c + i] = v[i];
+        for (int i = 0; i < RPT; ++i) {
+            const float dy = xs[cg * RPT + i].w;
+            dz[i] = dy * w4 * gelu_prime(z[3][i]);
+            gw += dy * gelu(z[3][i]);
+            gb += dz[i];
         }
-        {
-            float gb = 0.f;
-            for (int r = 0; r < nrow; ++r) gb += Dc[(r0 + r) * WID + t];
-            Gp[off_b(l) + t] = gb;
-        }
+        store_sum(make_float4(gw, gb, 0.f, 0.f));
+    }
+    // ---------------- hidden layers l = 3, 2, 1 (z_l = W_l a_{l-1} + b_l)
+#pragma unroll
+    for (int l = 3; l >= 1; --l) {
+        put(S::OFF_DZ, dz);
+        proxy_fence();
         tc_fence_before();
         __syncthreads();
-        // input gradient: dh = dz W_l (A = dz rows, B = W_l^T), dz_{l-1} = dh gelu'(z_{l-1})
-        stage_weights(sB, net.Wb + (l - 1) * WID * WID, true);
-        for (int c = 0; c < 16; ++c) put8(sA, t, 8 * c, Dc + row * WID + 8 * c);
-        ok = gemm_128(sA, sB, taddr, false, mbar, parity, net.err);
-        if (!ok) break;
-        for (int c = 0; c < 8; ++c) {
-            acc_row16(taddr, c, v);
+        if (t == 0) {
+            tc_fence_after();
+            // input gradient first: the chain waits for it
+            const uint32_t a0 = sbase + (l - 1) * W_BYTES, d0 = sbase + S::OFF_DZ;
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int o = 16 * c + i;
-                Dn[row * WID + o] = valid ? v[i] * gelu_prime(Z[((l - 1) * bm + row) * WID + o]) : 0.f;
+            for (int s = 0; s < 8; ++s)
+                mma_any(zcol[l - 1], desc_of(a0 + s * 2 * TG, TG, TC), desc_of(d0 + s * 2 * TC, TC, TG),
+                        idesc_n(ROWS, 1, 0), s > 0);
+            mma_commit(mbar + 6 - l);
+            // the weight gradient: read from tensor memory at the end
+            const uint32_t p0 = sbase + S::OFF_A + (l - 1) * S::A_BYTES;
+#pragma unroll
+            for (int s = 0; s < ROWS / 16; ++s)
+                mma_any(tm + 128u * (uint32_t)l, desc_of(d0 + s * 2 * TG, TG, TC), desc_of(p0 + s * 2 * TG, TG, TC),
+                        idesc_n(WID, 1, 1), s > 0);
+            mma_commit(mbar + 6);
+        }
+        if (cg == 0) {
+            const float4 v = load_sum();
+            if (l == 3) {
+                Gp[OFF_W4 + o] = v.x;
+                Gp[off_b(3) + o] = v.y;
+            } else {
+                Gp[off_b(l) + o] = v.x;
             }
         }
-        tc_fence_before();
-        __syncthreads();
-        float *tmp = Dc;
-        Dc = Dn;
-        Dn = tmp;
-    }
-    if (ok) {
-        // input layer (thread t = unit o): gW0 = dz_0^T x, gb0 = sum dz_0
+        wait(6 - l);
+        float v[RPT];
+        tc_ld_cols<RPT>(zcol[l - 1] + lanes + (uint32_t)(cg * RPT), v);
         float g0 = 0.f, g1 = 0.f, g2 = 0.f, gb = 0.f;
-        for (int r = 0; r < nrow; ++r) {
-            const float d = Dc[(r0 + r) * WID + t];
-            g0 += d * X[3 * (r0 + r)];
-            g1 += d * X[3 * (r0 + r) + 1];
-            g2 += d * X[3 * (r0 + r) + 2];
-            gb += d;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) {
+            dz[i] = v[i] * gelu_prime(z[l - 1][i]);
+            gb += dz[i];
+            if (l == 1) {
+                const float4 x = xs[cg * RPT + i];
+                g0 += dz[i] * x.x;
+                g1 += dz[i] * x.y;
+                g2 += dz[i] * x.z;
+            }
         }
-        Gp[OFF_W0 + 3 * t] = g0;
-        Gp[OFF_W0 + 3 * t + 1] = g1;
-        Gp[OFF_W0 + 3 * t + 2] = g2;
-        Gp[OFF_B0 + t] = gb;
+        // the weight-gradient MMAs still read the dz tile: wait for them before
+        // the next layer's dz overwrites it
+        if (!mbar_wait(mbar + 6, (uint32_t)(3 - l) & 1u)) {
+            *flag = 1;
+            atomicOr(net.err, ERR_MMA_TIMEOUT);
+            (void)mbar_wait(mbar + 6, (uint32_t)(3 - l) & 1u);
+        }
+        __syncthreads();   // the sums above have been read
+        store_sum(l == 1 ? make_float4(gb, g0, g1, g2) : make_float4(gb, 0.f, 0.f, 0.f));
     }
-done:
+    tc_fence_after();
+    __syncthreads();
+    if (cg == 0) {
+        // input layer
+        const float4 v = load_sum();
+        Gp[OFF_B0 + o] = v.x;
+        Gp[OFF_W0 + 3 * o] = v.y;
+        Gp[OFF_W0 + 3 * o + 1] = v.z;
+        Gp[OFF_W0 + 3 * o + 2] = v.w;
+    }
+    if (*flag == 0) {
+        // the weight gradients: lane = output unit, columns = inputs
+#pragma unroll
+        for (int l = 1; l <= 3; ++l) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                float v[8];
+                tc_ld_cols<8>(tm + 128u * (uint32_t)l + lanes + (uint32_t)(cg * 32 + c * 8), v);
+                float4 *dst = reinterpret_cast<float4 *>(Gp + off_W(l) + o * WID + cg * 32 + c * 8);
+                dst[0] = make_float4(v[0], v[1], v[2], v[3]);
+                dst[1] = make_float4(v[4], v[5], v[6], v[7]);
+            }
+        }
+    }
     tc_fence_before();
     __syncthreads();
-    if (t < 32) tc_dealloc(taddr, 256);
+    if (w == 0) tc_dealloc(tm, 512);
 }
 
 // Gradient and loss of the batch: the tiles' shares added in tile order.
+__device__ __forceinline__ float tile_sum(const float *__restrict__ q, size_t stride, int ntile)
+{
+    float g = 0.f;
+#pragma unroll 8
+    for (int i = 0; i < ntile; ++i) g += q[(size_t)i * stride];
+    return g;
+}
+__device__ __forceinline__ void loss_of(const Net &net, int ntile, int B) { *net.loss = tile_sum(net.Lp, 1, ntile) / (float)B; }
+
 __global__ void k_mlp_reduce(Net net, int ntile, int B)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k < NPARAM) {
-        float g = 0.f;
-        for (int i = 0; i < ntile; ++i) g += net.Gp[(size_t)i * NPARAM + k];
-        net.G[k] = g;
-    }
-    if (k == 0) {
-        float l = 0.f;
-        for (int i = 0; i < ntile; ++i) l += net.Lp[i];
-        *net.loss = l / (float)B;
-    }
+    if (k < NPARAM) net.G[k] = tile_sum(net.Gp + k, GSTRIDE, ntile);
+    if (k == 0) loss_of(net, ntile, B);
 }
 
-// Adam (Kingma & Ba) on the FP32 masters; refreshes the BF16 copies.
-__global__ void k_mlp_adam(Net net, float lr, float b1, float b2, float eps, float c1, float c2)
+// The same sums followed by Adam (Kingma & Ba) on the FP32 masters; refreshes
+// the BF16 copies.
+__global__ void k_mlp_reduce_adam(Net net, int ntile, int B, float lr, float b1, float b2, float eps, float c1, float c2)
 {
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
+    if (k == 0) loss_of(net, ntile, B);
     if (k >= NPARAM) return;
-    const float g = net.G[k];
+    const float g = tile_sum(net.Gp + k, GSTRIDE, ntile);
+    net.G[k] = g;
     const float m = b1 * net.M[k] + (1.f - b1) * g;
     const float v = b2 * net.V[k] + (1.f - b2) * g * g;
     net.M[k] = m;
@@ -623,7 +729,11 @@ struct sdpd_mlp {
 };
 
 namespace {
-constexpr size_t SMEM_BYTES = 4 * TILE_BYTES + 64;
+// Batch rows per CTA of the gradient kernel: 16 up to 512 rows (more CTAs and
+// a shorter chain each), 32 beyond (half the gradient shares to add).
+constexpr int SMALL_ROWS = 512;
+int grad_tiles(int batch) { return batch <= SMALL_ROWS ? (batch + 15) / 16 : (batch + 31) / 32; }
+int grad_tiles_max(int bmax) { return std::max(grad_tiles(std::min(bmax, SMALL_ROWS)), grad_tiles(bmax)); }
 
 sdpd_status mlp_fail(sdpd_status s, const std::string &m)
 {
@@ -638,6 +748,24 @@ sdpd_status mlp_err(sdpd_mlp *h)
         return mlp_fail(SDPD_E_CUDA, "mlp: reading the error word");
     if (e) return mlp_fail(SDPD_E_TIMEOUT, "mlp: tensor-core completion wait timed out");
     return SDPD_OK;
+}
+sdpd_status launch_grad(sdpd_mlp *h, const float *X, const float *T, int batch, cudaStream_t st)
+{
+    (void)cudaGetLastError();
+    const int ntile = grad_tiles(batch);
+    if (batch <= SMALL_ROWS)
+        k_mlp_grad<16><<<ntile, GRAD_THREADS, GradSmem<16>::BYTES, st>>>(h->net, X, T, batch);
+    else
+        k_mlp_grad<32><<<ntile, GRAD_THREADS, GradSmem<32>::BYTES, st>>>(h->net, X, T, batch);
+    return cudaGetLastError() == cudaSuccess ? SDPD_OK : mlp_fail(SDPD_E_CUDA, "mlp_gradients: launch");
+}
+
+sdpd_status read_loss(sdpd_mlp *h, float *loss, cudaStream_t st, const char *what)
+{
+    if (cudaMemcpyAsync(loss, h->net.loss, 4, cudaMemcpyDefault, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+        return mlp_fail(SDPD_E_CUDA, what);
+    return mlp_err(h);
 }
 }  // namespace
 
@@ -657,10 +785,8 @@ sdpd_status mlp_init(int in, int width, int depth, unsigned long long seed, int 
     auto A = [&](void **p, size_t bytes) { return cudaMalloc(p, bytes) == cudaSuccess; };
     bool ok = A((void **)&n.P, NPARAM * 4) && A((void **)&n.G, NPARAM * 4) && A((void **)&n.M, NPARAM * 4) &&
               A((void **)&n.V, NPARAM * 4) && A((void **)&n.Wb, 3 * WID * WID * 2) &&
-              A((void **)&n.Z, (size_t)4 * n.bmax * WID * 4) && A((void **)&n.D, (size_t)2 * n.bmax * WID * 4) &&
-              A((void **)&n.Gp, (size_t)(n.bmax / WID) * NPARAM * 4) && A((void **)&n.Lp, (size_t)(n.bmax / WID) * 4) &&
-              A((void **)&n.Y, (size_t)n.bmax * 4) && A((void **)&n.DY, (size_t)n.bmax * 4) &&
-              A((void **)&n.loss, 4) && A((void **)&n.err, 4);
+              A((void **)&n.Gp, (size_t)grad_tiles_max(n.bmax) * GSTRIDE * 4) &&
+              A((void **)&n.Lp, (size_t)grad_tiles_max(n.bmax) * 4) && A((void **)&n.loss, 4) && A((void **)&n.err, 4);
     if (!ok) {
         delete h;
         return mlp_fail(SDPD_E_OOM, "mlp_init: cudaMalloc failed");
@@ -691,7 +817,8 @@ sdpd_status mlp_init(int in, int width, int depth, unsigned long long seed, int 
     n.step = 0;
     k_mlp_refresh<<<(3 * WID * WID + 255) / 256, 256>>>(n);
     cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FWD_SMEM);
-    cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BYTES);
+    cudaFuncSetAttribute(k_mlp_grad<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GradSmem<16>::BYTES);
+    cudaFuncSetAttribute(k_mlp_grad<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GradSmem<32>::BYTES);
     if (cudaDeviceSynchronize() != cudaSuccess) {
         mlp_destroy(h);
         return mlp_fail(SDPD_E_CUDA, "mlp_init: initialisation failed");
@@ -705,7 +832,7 @@ void mlp_destroy(sdpd_mlp *h)
     if (!h) return;
     cudaDeviceSynchronize();
     Net &n = h->net;
-    void *ps[] = { n.P, n.G, n.M, n.V, n.Wb, n.Z, n.D, n.Gp, n.Lp, n.Y, n.DY, n.loss, n.err };
+    void *ps[] = { n.P, n.G, n.M, n.V, n.Wb, n.Gp, n.Lp, n.loss, n.err };
     for (void *p : ps) cudaFree(p);
     delete h;
 }
@@ -740,39 +867,29 @@ sdpd_status mlp_gradients(sdpd_mlp *h, const float *X, const float *T, int batch
     if (!h || !X || !T) return mlp_fail(SDPD_E_INVALID, "mlp_gradients: NULL argument");
     if (batch < 1 || batch > h->net.bmax) return mlp_fail(SDPD_E_INVALID, "mlp_gradients: batch out of range");
     cudaStream_t st = (cudaStream_t)stream;
-    (void)cudaGetLastError();
-    const int ntile = (batch + WID - 1) / WID;
-    k_mlp_grad<<<ntile, 128, SMEM_BYTES, st>>>(h->net, X, T, batch);
-    k_mlp_reduce<<<(NPARAM + 255) / 256, 256, 0, st>>>(h->net, ntile, batch);
+    const sdpd_status s = launch_grad(h, X, T, batch, st);
+    if (s != SDPD_OK) return s;
+    k_mlp_reduce<<<(NPARAM + 255) / 256, 256, 0, st>>>(h->net, grad_tiles(batch), batch);
     if (cudaGetLastError() != cudaSuccess) return mlp_fail(SDPD_E_CUDA, "mlp_gradients: launch");
-    if (loss) {
-        if (cudaMemcpyAsync(loss, h->net.loss, 4, cudaMemcpyDefault, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return mlp_fail(SDPD_E_CUDA, "mlp_gradients: loss");
-        return mlp_err(h);
-    }
-    return SDPD_OK;
+    return loss ? read_loss(h, loss, st, "mlp_gradients: loss") : SDPD_OK;
 }
 
 sdpd_status mlp_train_step(sdpd_mlp *h, const float *X, const float *T, int batch, float lr, float *loss,
                            void *stream)
 {
-    sdpd_status s = mlp_gradients(h, X, T, batch, nullptr, stream);
-    if (s != SDPD_OK) return s;
+    if (!h || !X || !T) return mlp_fail(SDPD_E_INVALID, "mlp_gradients: NULL argument");
+    if (batch < 1 || batch > h->net.bmax) return mlp_fail(SDPD_E_INVALID, "mlp_gradients: batch out of range");
     cudaStream_t st = (cudaStream_t)stream;
+    const sdpd_status s = launch_grad(h, X, T, batch, st);
+    if (s != SDPD_OK) return s;
     h->net.step += 1;
     const double b1 = 0.9, b2 = 0.999;
     const float c1 = (float)(1.0 - std::pow(b1, (double)h->net.step));
     const float c2 = (float)(1.0 - std::pow(b2, (double)h->net.step));
-    k_mlp_adam<<<(NPARAM + 255) / 256, 256, 0, st>>>(h->net, lr, (float)b1, (float)b2, 1e-8f, c1, c2);
+    k_mlp_reduce_adam<<<(NPARAM + 255) / 256, 256, 0, st>>>(h->net, grad_tiles(batch), batch, lr, (float)b1, (float)b2,
+                                                           1e-8f, c1, c2);
     if (cudaGetLastError() != cudaSuccess) return mlp_fail(SDPD_E_CUDA, "mlp_train_step: launch");
-    if (loss) {
-        if (cudaMemcpyAsync(loss, h->net.loss, 4, cudaMemcpyDefault, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return mlp_fail(SDPD_E_CUDA, "mlp_train_step: loss");
-        return mlp_err(h);
-    }
-    return SDPD_OK;
+    return loss ? read_loss(h, loss, st, "mlp_train_step: loss") : SDPD_OK;
 }
 
 sdpd_status mlp_infer(sdpd_mlp *h, const float *X, float *Y, long long n, void *stream)
