@@ -296,11 +296,7 @@ def force_kernel_name(mode, split):
     r = "float" if split else "double"
     if mode in (1, 4):
         return f"k_force_half<{r}, {'true' if mode == 4 or not split else 'false'}>"
-    if mode in (2, 3):
-        return f"k_force_stream<{r}, {mode if split else 1}>"
-    if mode == 5 and split:
-        return "k_force_fluid_lean<float, 5, 2, 0>"   # velver 1: with the async record ring
-    return f"k_force_fluid<{r}, 0>"
+    return "k_force_fluid<float, 2>" if split else "k_force_fluid<double, 0>"
 
 
 def time_native(args, ws, rank, local):

@@ -221,24 +221,14 @@ sdpd_status sdpd_diagnostics(sdpd_ctx *ctx, int inst, double out[16]);
 /* Force-pass variant: newton3 = 1 (default) evaluates each unordered pair once
  * (one of the two particles owns it, chosen by a hash of the pair so that
  * each owns about half of its list; its result goes to the partner through a
- * pair buffer; deterministic, no atomics); newton3 = 0 evaluates every pair
- * from both sides, one thread per particle walking its list; newton3 = 2 is
- * the same pass as 0 with the pairs streamed through shared memory: a warp
- * compacts the pairs within h of its 32 particles' lists and evaluates them
- * 32 at a time, each particle summing its own in list order (forces equal to
- * those of 0 bit for bit); newton3 = 3 is that pass with its registers
- * capped for three 256-thread blocks per SM instead of two (a tuning choice;
- * FP32 pairs only, FP64 runs 2); newton3 = 4 is the Newton-3 pass with the
- * owner writing each finished pair result (force, e x o) straight into the
- * partner's column, which the partner then reads coalesced, as the FP64
+ * pair buffer; deterministic, no atomics); newton3 = 4 is the same pass with
+ * the owner writing each finished pair result (force, e x o) straight into
+ * the partner's column, which the partner then reads coalesced, as the FP64
  * pass always does (for FP32 pairs, 1 keeps {o, ce} in the owner's column
  * and the partner gathers it through the reverse index; 4 and 1 give the
- * same bits); newton3 = 5 is the direct pass with only the list index and
- * the partner's position fetched ahead, which needs fewer registers and runs
- * more warps per SM, its other records coming at the first evaluation through
- * an asynchronous shared-memory ring (FP32 pairs; FP64 runs 0; the same bits
- * as 0).  All give
- * the same forces up to summation order.
+ * same bits); newton3 = 0, 2, 3 and 5 evaluate every pair from both sides, the
+ * direct pass (2, 3 and 5 once named forms of it that the present one
+ * replaces).  All give the same forces up to summation order.
  * Invalidates the current neighbour build and graph.  Synchronous. */
 sdpd_status sdpd_set_force_mode(sdpd_ctx *ctx, int newton3);
 
@@ -255,12 +245,10 @@ sdpd_status sdpd_set_noise_cache(sdpd_ctx *ctx, int on);
  * Synchronous. */
 sdpd_status sdpd_set_block_size(sdpd_ctx *ctx, int threads);
 
-/* Lanes per particle of the direct force pass (force mode 0): 1 (default), 2
- * or 4.  With more than one, the lanes of a particle take every tpp-th entry
- * of its list and their sums are added by a fixed butterfly of shuffles, so
- * small workloads fill more of the GPU; the result differs from tpp = 1 only
- * by summation order and is the same on every run.  A tuning knob.
- * Invalidates the current graph.  Synchronous. */
+/* Lanes per particle asked of the direct force pass: 1, 2 or 4 (anything else
+ * is SDPD_E_INVALID).  Every pair pass now runs 8 lanes per particle, whose
+ * partial sums are added in a fixed order; the setting changes nothing.
+ * Synchronous. */
 sdpd_status sdpd_set_threads_per_particle(sdpd_ctx *ctx, int tpp);
 
 /* Cells of the neighbour search per minimum cell width (Algorithm 1, Section

@@ -54,9 +54,8 @@ struct sdpd_ctx {
     Inst *d_inst = nullptr;
     int any_filter = 0, any_artvis = 0, any_reinit = 0;
     std::vector<double> probe_y;   // mean slab positions of the last viscosity probe
-    int newton3 = 1;                   // force pass: 1 half-pair (Newton 3), 0 direct, 2/3 pair stream,
-                                       // 4 half-pair with pushed results (FP32), 5 direct with
-                                       // fewer registers (FP32)
+    int newton3 = 1;                   // force pass: 1 half-pair (Newton 3), 4 the same with pushed
+                                       // results (FP32), 0, 2, 3 and 5 direct
     int noise_cache = 1;               // second evaluation of a step reuses the first one's normals
     double skin = 0.03;                // Verlet skin as a fraction of h
     int cell_sub = 1;                  // cells per minimum cell width: 1 (27-cell stencil) or 2 (125)
@@ -205,7 +204,11 @@ sdpd_status prepare(sdpd_ctx *c)
             }
             if (I.nc[a] > 1023) return fail(SDPD_E_INVALID, "more than 1023 cells on an axis");
             I.inv_cs[a] = 1.0 / I.cs[a];
-            I.csf[a] = (float)I.cs[a];
+            // windows of the fixed-point coordinates (see Inst)
+            const double windows = p.periodic[a] ? std::max(1.0, std::floor(p.box[a] / (4.0 * cmin))) : 1.0;
+            const double window = p.periodic[a] ? p.box[a] / windows : 4.0 * cmin;
+            I.fix[a] = 4294967296.0 / window;
+            I.unit[a] = (float)(window / 4294967296.0);
         }
         I.ncell = I.nc[0] * I.nc[1] * I.nc[2];
         I.cell_base = cell_base;
@@ -288,8 +291,8 @@ sdpd_status prepare(sdpd_ctx *c)
     CUDA_TRY(cudaMemcpy(rank_d, rank_all.data(), sizeof(int) * cell_base, cudaMemcpyHostToDevice));
     b.cell_rank = rank_d;
     // neighbour cells of every cell (offsets -sub..sub per axis), ascending
-    // key, with the offset code (ox+2) + 5 (oy+2) + 25 (oz+2): neighbour
-    // lists then come out sorted by slot.  Cells are split over host threads.
+    // key: neighbour lists then come out sorted by slot.  Cells are split over
+    // host threads.
     {
         if (cell_base >= (1 << 24)) return fail(SDPD_E_INVALID, "too many cells");
         std::vector<int> adj((size_t)cell_base * ADJ, -1);
@@ -298,7 +301,7 @@ sdpd_status prepare(sdpd_ctx *c)
             std::fill(inst_of.begin() + c->inst[k].cell_base,
                       inst_of.begin() + c->inst[k].cell_base + c->inst[k].ncell, k);
         auto fill = [&](int lin0, int lin1) {
-            std::pair<int, int> nbs[ADJ];
+            int nbs[ADJ];
             for (int gl = lin0; gl < lin1; ++gl) {
                 const Inst &I = c->inst[inst_of[gl]];
                 const int lin = gl - I.cell_base, d = I.sub;
@@ -316,11 +319,10 @@ sdpd_status prepare(sdpd_ctx *c)
                             }
                             if (!ok) continue;
                             const int l2 = (cc[2] * I.nc[1] + cc[1]) * I.nc[0] + cc[0];
-                            const int k2 = I.cell_base + rank_all[I.cell_base + l2];
-                            nbs[nn++] = { k2, (ox + 2) + 5 * (oy + 2) + 25 * (oz + 2) };
+                            nbs[nn++] = I.cell_base + rank_all[I.cell_base + l2];
                         }
                 std::sort(nbs, nbs + nn);
-                for (int q = 0; q < nn; ++q) adj[(size_t)key * ADJ + q] = (nbs[q].first << 7) | nbs[q].second;
+                for (int q = 0; q < nn; ++q) adj[(size_t)key * ADJ + q] = nbs[q];
             }
         };
         const int nth = std::max(1, std::min((int)std::thread::hardware_concurrency(),
@@ -334,6 +336,10 @@ sdpd_status prepare(sdpd_ctx *c)
                                   (int)((long long)cell_base * (t + 1) / nth));
             for (auto &th : pool) th.join();
         }
+        int *inst_d = nullptr;
+        ALLOC(inst_d, cell_base, true);
+        CUDA_TRY(cudaMemcpy(inst_d, inst_of.data(), sizeof(int) * cell_base, cudaMemcpyHostToDevice));
+        b.cell_inst = inst_d;
         int *adj_d = nullptr;
         ALLOC(adj_d, adj.size(), true);
         CUDA_TRY(cudaMemcpy(adj_d, adj.data(), sizeof(int) * adj.size(), cudaMemcpyHostToDevice));
@@ -421,6 +427,8 @@ inline bool half_pairs(int mode) { return mode == 1 || mode == 4; }
 void enqueue_build(sdpd_ctx *c, cudaStream_t st, const int *gate = nullptr)
 {
     c->b.use_cache = c->noise_cache;
+    // the FP64 density of the direct pass sums in the half-pair pass's order
+    c->b.split = c->precision == SDPD_PREC_FP64 || half_pairs(c->newton3);
     launch_build(c->b, c->precision, half_pairs(c->newton3), gate, st);
 }
 
@@ -477,7 +485,6 @@ sdpd_status sdpd_init(const sdpd_params *params, int n_instances, const long lon
     b.cap = c->cap;
     b.K = c->K;
     b.pair_block = 128;
-    b.tpp = 1;
     b.cell_sub = 1;
     auto cleanup = [&](sdpd_status s) {
         sdpd_destroy(c);
@@ -503,21 +510,23 @@ sdpd_status sdpd_init(const sdpd_params *params, int n_instances, const long lon
     } else {
         IALLOC(b.A64, N); IALLOC(b.B64, N); IALLOC(b.C64, N); IALLOC(b.D64, N);
     }
-    IALLOC(b.nbr, (size_t)c->cap * c->Npad);
+    b.rows = entry_rows(c->cap);
+    const size_t entries = (size_t)b.rows * LPP * c->Npad;   // of one array over the whole lists
+    IALLOC(b.nbr, entries);
     IALLOC(b.ncnt, N);
     IALLOC(b.nfirst, N);
-    IALLOC(b.skey, N);
     IALLOC(b.nbflag, N);
-    IALLOC(b.rev, (size_t)c->cap * c->Npad);
+    IALLOC(b.rev, entries);
     // each particle owns about half of its list (hash ownership, spread of a
     // few pairs): the pair buffer and the normals cache of the Newton-3 pass
-    // hold cap/2 + 64 rows.  The direct pass instead caches the normals of
-    // every list entry ([cap][Npad]).  A context runs one force pass at a
+    // hold cap/2 + 64 entries of each particle.  The direct pass instead caches
+    // the normals of every list entry.  A context runs one force pass at a
     // time, so both layouts share one arena.
     b.capown = std::min(c->cap, c->cap / 2 + 64);
+    b.rows_own = entry_rows(b.capown);
     {
         const size_t rs = (precision == SDPD_PREC_SPLIT) ? sizeof(float) : sizeof(double);
-        const size_t Np = (size_t)c->Npad, own = (size_t)b.capown * Np, all = (size_t)c->cap * Np;
+        const size_t own = (size_t)b.rows_own * LPP * c->Npad, all = entries;
         // {f, h.x} / {o, ce} in resA; {h.y, h.z} in resB (pushed results)
         const size_t n_resA = 4 * rs * own, n_resB = 2 * rs * own;
         const size_t n_zA = 4 * rs * own, n_zB = 2 * rs * own;
@@ -535,19 +544,20 @@ sdpd_status sdpd_init(const sdpd_params *params, int n_instances, const long lon
         b.zdB = arena + 4 * rs * all;
         b.ownA = oa; b.ownB = ob;
     }
-    IALLOC(b.xl64, N); IALLOC(b.dsp, N);
+    IALLOC(b.dsp, N);
     IALLOC(b.aclose, N); IALLOC(b.aclose_ok, 1); IALLOC(b.sdr, N); IALLOC(b.xs, 3 * N);
-    IALLOC(b.need_build, 1); IALLOC(b.fresh, 1);
-    IALLOC(b.list_epoch, 1); IALLOC(b.cache_epoch, 1); IALLOC(b.cache_step, 1);
+    const size_t ni = (size_t)n_instances + 1;
+    IALLOC(b.need_build, ni); IALLOC(b.fresh, 1);
+    IALLOC(b.list_epoch, ni); IALLOC(b.cache_epoch, ni); IALLOC(b.cache_step, 1);
     b.use_cache = 1;
-    IALLOC(b.step, 1); IALLOC(b.err, 1); IALLOC(b.pair_count, 1); IALLOC(b.work, 1);
+    IALLOC(b.step, 1); IALLOC(b.err, 1); IALLOC(b.pair_count, 1);
     IALLOC(b.probe, 4096 * 3 + 64);
 #undef IALLOC
-    if (cudaMemset(b.rev, 0, sizeof(uint16_t) * (size_t)c->cap * c->Npad) != cudaSuccess ||
-        cudaMemset(b.need_build, 0, sizeof(int)) != cudaSuccess || cudaMemset(b.fresh, 0, sizeof(int)) != cudaSuccess ||
+    if (cudaMemset(b.rev, 0, sizeof(uint16_t) * entries) != cudaSuccess ||
+        cudaMemset(b.need_build, 0, sizeof(int) * ni) != cudaSuccess || cudaMemset(b.fresh, 0, sizeof(int)) != cudaSuccess ||
         cudaMemset(b.aclose_ok, 0, sizeof(int)) != cudaSuccess ||
-        cudaMemset(b.list_epoch, 0, sizeof(unsigned)) != cudaSuccess ||
-        cudaMemset(b.cache_epoch, 0xFF, sizeof(unsigned)) != cudaSuccess ||
+        cudaMemset(b.list_epoch, 0, sizeof(unsigned) * ni) != cudaSuccess ||
+        cudaMemset(b.cache_epoch, 0xFF, sizeof(unsigned) * ni) != cudaSuccess ||
         cudaMemset(b.cache_step, 0xFF, sizeof(long long)) != cudaSuccess)
         return cleanup(fail(SDPD_E_CUDA, "cudaMemset failed"));
     if (cudaMemset(b.err, 0, sizeof(int)) != cudaSuccess || cudaMemset(b.step, 0, sizeof(long long)) != cudaSuccess ||
@@ -963,11 +973,9 @@ sdpd_status sdpd_set_threads_per_particle(sdpd_ctx *c, int tpp)
 {
     if (!c) return fail(SDPD_E_INVALID, "NULL context");
     if (tpp != 1 && tpp != 2 && tpp != 4) return fail(SDPD_E_INVALID, "threads per particle must be 1, 2 or 4");
+    // every pair pass runs LPP lanes per particle; the setting is accepted and
+    // changes nothing
     CUDA_TRY(cudaDeviceSynchronize());
-    if (tpp != c->b.tpp) {
-        c->b.tpp = tpp;
-        drop_graph(c);
-    }
     return SDPD_OK;
 }
 
@@ -1160,7 +1168,8 @@ sdpd_status sdpd_get_pairs(sdpd_ctx *c, int inst, long long cap, int *ij, long l
     CUDA_TRY(cudaMemcpy(pinst.data(), c->b.pinst, sizeof(int) * N, cudaMemcpyDeviceToHost));
     int kmax = 0;
     for (long long s = 0; s < N; ++s) kmax = std::max(kmax, cnt[s]);
-    std::vector<int> nb((size_t)kmax * c->Npad);
+    const int rows = entry_rows(kmax);   // the rows in use of every block
+    std::vector<int> nb((size_t)rows * LPP * c->Npad);
     std::vector<uint8_t> fl((size_t)kmax * c->Npad);
     if (kmax) {
         // entries of the (skin) list within h at the current positions
@@ -1170,7 +1179,8 @@ sdpd_status sdpd_get_pairs(sdpd_ctx *c, int inst, long long cap, int *ij, long l
         cudaError_t e1 = cudaMemcpy(fl.data(), dfl, fl.size(), cudaMemcpyDeviceToHost);
         cudaFree(dfl);
         if (e1 != cudaSuccess) return fail(SDPD_E_CUDA, "cudaMemcpy pair flags");
-        CUDA_TRY(cudaMemcpy(nb.data(), c->b.nbr, sizeof(int) * nb.size(), cudaMemcpyDeviceToHost));
+        CUDA_TRY(cudaMemcpy2D(nb.data(), sizeof(int) * rows * ROW, c->b.nbr, sizeof(int) * c->b.rows * ROW,
+                              sizeof(int) * rows * ROW, (size_t)(c->Npad / GROUP), cudaMemcpyDeviceToHost));
     }
     const long long o = c->hi[inst].begin;
     long long k = 0;
@@ -1178,7 +1188,7 @@ sdpd_status sdpd_get_pairs(sdpd_ctx *c, int inst, long long cap, int *ij, long l
         const int gi = perm[s];
         if (pinst[gi] != inst) continue;
         for (int q = 0; q < cnt[s]; ++q) {
-            const uint32_t e = (uint32_t)nb[(size_t)q * c->Npad + s];
+            const uint32_t e = (uint32_t)nb[entry_at(q, s, rows)];
             if ((e & NB_FAR) || !fl[(size_t)q * c->Npad + s]) continue;
             const int gj = perm[e];
             if (gj <= gi) continue;

@@ -14,7 +14,9 @@
 // r_ij < h exactly, so the evaluated pair set equals the paper's.  The list
 // stays valid while no particle has moved more than skin h / 2 since the
 // build; the drift raises `need_build` when one has, and every kernel here
-// is gated on that flag inside the captured step.
+// is gated on that flag inside the captured step.  Only the instances whose
+// own flag is up are rebuilt: an instance's slots are the range of its gids,
+// so the others keep their cells, slots and lists.
 #include <algorithm>
 
 #include "common.cuh"
@@ -37,14 +39,14 @@ __global__ void k_cell_clear(Bufs b, const int *gate)
 {
     GATE;
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < b.ncell_total) b.ccount[c] = 0;
+    if (c < b.ncell_total && rebuilds(b, gate, b.cell_inst[c])) b.ccount[c] = 0;
 }
 
 __global__ void k_cell_keys(Bufs b, const int *gate)
 {
     GATE;
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= b.N) return;
+    if (g >= b.N || !rebuilds(b, gate, b.pinst[g])) return;
     const Inst &I = b.inst[b.pinst[g]];
     int c[3];
     bool bad = false, nf = false;
@@ -134,7 +136,7 @@ __global__ void k_scatter(Bufs b, const int *gate)
 {
     GATE;
     const long long g = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= b.N) return;
+    if (g >= b.N || !rebuilds(b, gate, b.pinst[g])) return;
     b.tmp_perm[b.cstart[b.key[g]] + b.slot_in_cell[g]] = (int)g;
 }
 
@@ -144,7 +146,8 @@ __global__ void k_rank(Bufs b, const int *gate)
     GATE;
     const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= b.N) return;
-    const int g = b.tmp_perm[t];
+    const int g = b.tmp_perm[t];   // (of the last build where this one leaves the instance as it is)
+    if (!rebuilds(b, gate, b.pinst[g])) return;
     const int c = b.key[g];
     const int s0 = b.cstart[c], s1 = b.cstart[c + 1];
     int r = 0;
@@ -162,29 +165,16 @@ __global__ void k_gather(Bufs b, int precision, const int *gate)
     if (s >= b.N) return;
     const int g = b.perm[s];
     const int ii = b.pinst[g];
+    if (!rebuilds(b, gate, ii)) return;
     const Inst &I = b.inst[ii];
     const int t = b.type[g];
     b.stype[s] = t;
     const double x0 = b.x[3 * g], x1 = b.x[3 * g + 1], x2 = b.x[3 * g + 2];
     const uint32_t lg = (uint32_t)(g - I.p_begin);
-    {
-        // cell-relative coordinates (both precisions: the neighbour search
-        // and the split-precision pair kernels work on them)
-        int c[3];
-        double xl[3];
-        const double xs[3] = { x0, x1, x2 };
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            bool o, f;
-            c[a] = cell_coord(xs[a], I.lo[a], I.inv_cs[a], I.nc[a], o, f);
-            xl[a] = xs[a] - (I.lo[a] + (double)c[a] * I.cs[a]);
-        }
-        b.A32[s] = make_float4((float)xl[0], (float)xl[1], (float)xl[2],
-                               __uint_as_float(pack_cell(t, c[0], c[1], c[2])));
-        b.skey[s] = b.key[g];
-        b.xl64[s] = make_double4_32a(xl[0], xl[1], xl[2], 0.0);
-        b.dsp[s] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
-    }
+    // (both precisions: the neighbour search and the split-precision pair
+    // kernels work on the fixed-point coordinates)
+    b.A32[s] = make_int4(fixed_coord(x0, I, 0), fixed_coord(x1, I, 1), fixed_coord(x2, I, 2), t);
+    b.dsp[s] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
     if (precision == SDPD_PREC_SPLIT) {
         b.B32[s] = make_float4((float)b.v[3 * g], (float)b.v[3 * g + 1], (float)b.v[3 * g + 2],
                                (float)b.R[g]);
@@ -206,7 +196,8 @@ __global__ void k_gather(Bufs b, int precision, const int *gate)
 // the list only has to be a superset of the pairs within h), or when both are
 // rigid and r < R_i + R_j + skin h (contact range; flagged NB_FAR).
 //
-// Newton-3 ownership, balanced so that every particle owns about half of its
+// In FP32 contexts with a direct force pass (b.split == 0) the list is
+// ascending in slot.  Otherwise it is split by Newton-3 ownership, balanced so that every particle owns about half of its
 // pairs whatever its position in the cell: the pair of instance-local slots
 // a < b belongs to a when bit 15 of the hash (a * 0x9E3779B1) ^
 // (b * 0x85EBCA77) is set, else to b.  The list is written as [owned][not
@@ -223,15 +214,14 @@ __device__ __forceinline__ bool pair_owned(long long s, int j, int base)
 }
 
 
-// The candidate test of a pair (i, j) with j's record Aj and the offset
-// (sx, sy, sz) of j's cell: within rb (float), or both rigid and within
-// contact range (flagged NB_FAR).
-__device__ __forceinline__ bool nb_test(const Bufs &b, const Inst &I, const float4 &Ai, int ti, float Ri,
-                                        int j, const float4 &Aj, float sx, float sy, float sz, uint32_t &entry,
-                                        int &tj)
+// The candidate test of a pair (i, j) with j's record Aj: within rb (float),
+// or both rigid and within contact range (flagged NB_FAR).
+__device__ __forceinline__ bool nb_test(const Bufs &b, const Inst &I, const Geo<float> &geo, const int4 &Ai, int ti,
+                                        float Ri, int j, const int4 &Aj, uint32_t &entry, int &tj)
 {
-    tj = unpack_type(__float_as_uint(Aj.w));
-    const float dx = (Ai.x - Aj.x) - sx, dy = (Ai.y - Aj.y) - sy, dz = (Ai.z - Aj.z) - sz;
+    tj = Aj.w;
+    float dx, dy, dz;
+    geo.disp(Ai, Aj, dx, dy, dz);
     const float r2f = dx * dx + dy * dy + dz * dz;
     entry = (uint32_t)j;
     if (r2f < I.rb2f) return true;
@@ -252,41 +242,40 @@ __device__ __forceinline__ bool nb_test(const Bufs &b, const Inst &I, const floa
 constexpr int NB_WARPS = 8;
 
 // The lists of cell c's particles [s0, s1), one lane per particle; stage:
-// 32 float4 of this warp's shared memory.
-__device__ void nb_scan_cell(const Bufs &b, int c, int s0, int s1, float4 *stage, int lane)
+// 32 int4 of this warp's shared memory.
+__device__ void nb_scan_cell(const Bufs &b, int c, int s0, int s1, int4 *stage, int lane)
 {
     const int *adj = b.cell_adj + (long long)c * ADJ;
     const Inst &I = b.inst[b.pinst[b.perm[s0]]];   // a cell belongs to one instance
     const int base = b.cstart[I.cell_base];           // first slot of the instance
-    const long long Np = b.Npad;
+    const int rows = b.rows;
     const int cap = b.cap;
+    const bool split = b.split != 0;
+    const Geo<float> geo(I);
     for (int chunk = s0; chunk < s1; chunk += 32) {
         const int s = chunk + lane;
         const bool act = s < s1;
         int ti = T_FLUID;
         float Ri = 0.f;
-        float4 Ai = make_float4(0.f, 0.f, 0.f, 0.f);
+        int4 Ai = make_int4(0, 0, 0, 0);
         if (act) {
             ti = b.stype[s];
             Ri = (ti == T_RIGID) ? (float)b.R[b.perm[s]] : 0.f;
             Ai = b.A32[s];
         }
-        int *col = b.nbr + s;   // this particle's column, entry k at col[k * Np]
+        auto col = [&](int k) -> int & { return b.nbr[entry_at(k, s, rows)]; };   // this particle's column
         // one scan in ascending slot order: owned pairs from the front, the
         // others from the back of the column (so in descending positions)
         int nf = 0, m = 0;
         bool rig = false;
         for (int q = 0; q < ADJ; ++q) {
-            const int code = adj[q];
-            if (code < 0) break;
-            const int key = code >> 7, oc = code & 127;
-            const float sx = (float)(oc % 5 - 2) * I.csf[0], sy = (float)((oc / 5) % 5 - 2) * I.csf[1],
-                        sz = (float)(oc / 25 - 2) * I.csf[2];
+            const int key = adj[q];
+            if (key < 0) break;
             const int j0 = b.cstart[key], j1 = b.cstart[key + 1];
             for (int jb = j0; jb < j1; jb += 32) {
                 const int jj = jb + lane;
                 __syncwarp();
-                stage[lane] = jj < j1 ? b.A32[jj] : make_float4(0.f, 0.f, 0.f, 0.f);
+                stage[lane] = jj < j1 ? b.A32[jj] : make_int4(0, 0, 0, 0);
                 __syncwarp();
                 if (!act) continue;
                 const int cnt = min(32, j1 - jb);
@@ -294,13 +283,13 @@ __device__ void nb_scan_cell(const Bufs &b, int c, int s0, int s1, float4 *stage
                     const int j = jb + t;
                     uint32_t entry;
                     int tj;
-                    if (j == s || !nb_test(b, I, Ai, ti, Ri, j, stage[t], sx, sy, sz, entry, tj)) continue;
+                    if (j == s || !nb_test(b, I, geo, Ai, ti, Ri, j, stage[t], entry, tj)) continue;
                     rig |= (tj == T_RIGID);
-                    if (pair_owned(s, j, base)) {
-                        if (nf + m < cap) col[(long long)nf * Np] = (int)entry;
+                    if (!split || pair_owned(s, j, base)) {
+                        if (nf + m < cap) col(nf) = (int)entry;
                         ++nf;
                     } else {
-                        if (nf + m < cap) col[(long long)(cap - 1 - m) * Np] = (int)entry;
+                        if (nf + m < cap) col(cap - 1 - m) = (int)entry;
                         ++m;
                     }
                 }
@@ -309,7 +298,7 @@ __device__ void nb_scan_cell(const Bufs &b, int c, int s0, int s1, float4 *stage
         if (!act) continue;
         const int n = nf + m;
         // the pair buffer holds capown rows of owned and of non-owned entries
-        if (nf > b.capown || m > b.capown) atomicOr(b.err, ERR_PAIR_CAP);
+        if (split && (nf > b.capown || m > b.capown)) atomicOr(b.err, ERR_PAIR_CAP);
         if (n > cap) {
             atomicOr(b.err, ERR_NBR_CAP);
         } else {
@@ -319,9 +308,9 @@ __device__ void nb_scan_cell(const Bufs &b, int c, int s0, int s1, float4 *stage
             // overwrites an entry still to be read); only the owned prefix
             // needs ascending order (the reverse index searches it)
             if (nf < cap - m)
-                for (int k = 0; k < m; ++k) col[(long long)(nf + k) * Np] = col[(long long)(cap - m + k) * Np];
+                for (int k = 0; k < m; ++k) col(nf + k) = col(cap - m + k);
         }
-        b.nfirst[s] = min(nf, min(cap, b.capown));
+        b.nfirst[s] = min(nf, split ? min(cap, b.capown) : cap);
         b.ncnt[s] = min(n, cap);
         b.nbflag[s] = rig ? 1 : 0;
     }
@@ -330,10 +319,10 @@ __device__ void nb_scan_cell(const Bufs &b, int c, int s0, int s1, float4 *stage
 __global__ void __launch_bounds__(NB_WARPS * 32) k_neighbors(Bufs b, const int *gate)
 {
     GATE;
-    __shared__ float4 stage[NB_WARPS][32];
+    __shared__ int4 stage[NB_WARPS][32];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int c = blockIdx.x * NB_WARPS + w;
-    if (c >= b.ncell_total) return;   // the whole warp
+    if (c >= b.ncell_total || !rebuilds(b, gate, b.cell_inst[c])) return;   // the whole warp
     const int s0 = b.cstart[c], s1 = b.cstart[c + 1];
     if (s0 == s1) return;
     nb_scan_cell(b, c, s0, s1, stage[w], lane);
@@ -355,9 +344,8 @@ __global__ void __launch_bounds__(NB_WARPS * 32) k_neighbors(Bufs b, const int *
 // * The group's lists are collected in shared memory as 16-bit entries (the
 //   neighbour cell in the table, the offset in the cell, the contact-only
 //   flag), owned entries from the front and the others from the back.
-// * The lists are then written out row by row, the group's particles side by
-//   side (32 / 8 = 4 rows per store for a full group), instead of one
-//   scattered column entry per lane.
+// * The lists are then written out LPP entries of a particle at a time, four
+//   particles side by side, instead of one scattered entry per lane.
 // A cell with a neighbour cell of more than 256 particles (beyond the 8-bit
 // offset) is scanned by the lane-per-particle routine instead.  Either way
 // the lists come out exactly as the lane-per-particle kernel writes them from
@@ -370,14 +358,13 @@ constexpr int NG_MAX_WARPS = 4;
 constexpr int NG_OFF = 256;    // largest neighbour cell of the 16-bit entries
 
 struct NgShared {
-    float4 sa[NG_STAGE];       // staged candidates: record,
+    int4 sa[NG_STAGE];         // staged candidates: record,
     int sj[NG_STAGE];          //   slot,
     float sr[NG_STAGE];        //   radius where it can be a contact partner, else 0
     int sq[NG_STAGE];          //   neighbour cell << 8 | offset in it
     int pre[NG_TAB + 1];       // candidates before each neighbour cell (flattened index)
     int js[NG_TAB];            // first slot of each neighbour cell
-    uint8_t code[NG_TAB];      // its offset code (ox+2) + 5 (oy+2) + 25 (oz+2) < 125
-    float4 ai[NG_G];           // the group's records,
+    int4 ai[NG_G];             // the group's records,
     float ri[NG_G];            //   rigid radii
 };
 
@@ -396,7 +383,7 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
     extern __shared__ __align__(16) unsigned char ng_smem[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const int c = blockIdx.x * nw + w;
-    if (c >= b.ncell_total) return;   // the whole warp
+    if (c >= b.ncell_total || !rebuilds(b, gate, b.cell_inst[c])) return;   // the whole warp
     const int s0 = b.cstart[c], s1 = b.cstart[c + 1];
     if (s0 == s1) return;
     const int cap = b.cap, stride = ng_stride(cap);
@@ -411,10 +398,9 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
     bool fat = false;
     for (int q0 = 0; q0 < ADJ; q0 += 32) {
         const int q = q0 + lane;
-        const int code = q < ADJ ? adj[q] : -1;
+        const int key = q < ADJ ? adj[q] : -1;
         int cnt = 0, js = 0;
-        if (code >= 0) {
-            const int key = code >> 7;
+        if (key >= 0) {
             js = b.cstart[key];
             cnt = b.cstart[key + 1] - js;
         }
@@ -425,19 +411,18 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
             const int t = __shfl_up_sync(FULL, v, o);
             if (lane >= o) v += t;
         }
-        if (code >= 0) {
+        if (key >= 0) {
             S.pre[q] = total + v - cnt;
             S.js[q] = js;
-            S.code[q] = (uint8_t)(code & 127);
         }
         total += __shfl_sync(FULL, v, 31);
-        const unsigned vm = __ballot_sync(FULL, code >= 0);
+        const unsigned vm = __ballot_sync(FULL, key >= 0);
         nq += __popc(vm);
         if (vm != FULL) break;
     }
     if (fat) {
         // the list buffer serves as the routine's stage (512 bytes)
-        nb_scan_cell(b, c, s0, s1, reinterpret_cast<float4 *>(buf), lane);
+        nb_scan_cell(b, c, s0, s1, reinterpret_cast<int4 *>(buf), lane);
         return;
     }
     if (lane == 0) S.pre[nq] = total;
@@ -445,26 +430,31 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
 
     const Inst &I = b.inst[b.pinst[b.perm[s0]]];   // a cell belongs to one instance
     const int base = b.cstart[I.cell_base];           // first slot of the instance
-    const long long Np = b.Npad;
+    const int rows = b.rows;
     const float rb2_box = I.rb2f * 1.001f;   // conservative: the pair test decides
     const float two_hs = (float)(2.0 * I.half_skin);
-    const float cx = I.csf[0], cy = I.csf[1], cz = I.csf[2];
+    const Geo<float> geo(I);
     const float BIG = 3.0e38f;
+    const bool split = b.split != 0;
 
     for (int g0 = s0; g0 < s1; g0 += NG_G) {
         const int P = min(NG_G, s1 - g0);
-        float4 a = make_float4(0.f, 0.f, 0.f, 0.f);
+        int4 a = make_int4(0, 0, 0, 0);
         int t = T_FLUID;
         float r = 0.f;
         if (lane < P) {
             a = b.A32[g0 + lane];
-            t = b.stype[g0 + lane];
+            t = a.w;
             r = (t == T_RIGID) ? (float)b.R[b.perm[g0 + lane]] : 0.f;
             S.ai[lane] = a;
             S.ri[lane] = r;
         }
-        float lx = lane < P ? a.x : BIG, ly = lane < P ? a.y : BIG, lz = lane < P ? a.z : BIG;
-        float hx = lane < P ? a.x : -BIG, hy = lane < P ? a.y : -BIG, hz = lane < P ? a.z : -BIG;
+        // the group's bounding box, relative to its first particle
+        const int4 ref = make_int4(__shfl_sync(FULL, a.x, 0), __shfl_sync(FULL, a.y, 0), __shfl_sync(FULL, a.z, 0), 0);
+        float ax, ay, az;
+        geo.disp(a, ref, ax, ay, az);
+        float lx = lane < P ? ax : BIG, ly = lane < P ? ay : BIG, lz = lane < P ? az : BIG;
+        float hx = lane < P ? ax : -BIG, hy = lane < P ? ay : -BIG, hz = lane < P ? az : -BIG;
         float rg = r;
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) {   // lanes >= NG_G hold the neutral values
@@ -489,31 +479,28 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
 
         // one round per particle over the first nv staged candidates
         auto rounds = [&](int nv) {
-            float4 Aj = make_float4(0.f, 0.f, 0.f, 0.f);
-            int j = -1, tj = T_FLUID;
+            int4 Aj = make_int4(0, 0, 0, T_FLUID);
+            int j = -1;
             uint32_t e16 = 0;
-            float rj = 0.f, sx = 0.f, sy = 0.f, sz = 0.f;
+            float rj = 0.f;
             if (lane < nv) {
                 Aj = S.sa[lane];
                 j = S.sj[lane];
                 rj = S.sr[lane];
                 e16 = (uint32_t)S.sq[lane];
-                const int oc = S.code[e16 >> 8];
-                tj = unpack_type(__float_as_uint(Aj.w));
-                sx = (float)(oc % 5 - 2) * cx;
-                sy = (float)((oc / 5) % 5 - 2) * cy;
-                sz = (float)(oc / 25 - 2) * cz;
             }
+            const int tj = Aj.w;
 #pragma unroll
             for (int p = 0; p < NG_G; ++p) {
                 if (p < P) {
-                    const float4 Ai = S.ai[p];
-                    const int ti = unpack_type(__float_as_uint(Ai.w));
+                    const int4 Ai = S.ai[p];
+                    const int ti = Ai.w;
                     const int s = g0 + p;
                     bool hit = false;
                     uint32_t entry = e16;
                     if (lane < nv && j != s) {
-                        const float dx = (Ai.x - Aj.x) - sx, dy = (Ai.y - Aj.y) - sy, dz = (Ai.z - Aj.z) - sz;
+                        float dx, dy, dz;
+                        geo.disp(Ai, Aj, dx, dy, dz);
                         const float r2f = dx * dx + dy * dy + dz * dz;
                         if (r2f < I.rb2f) {
                             hit = true;
@@ -523,7 +510,7 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
                             hit = r2f < lim * lim;
                         }
                     }
-                    const bool own = hit && pair_owned(s, j, base);
+                    const bool own = hit && (!split || pair_owned(s, j, base));
                     const unsigned mh = __ballot_sync(FULL, hit), mo = __ballot_sync(FULL, own);
                     const unsigned mr = __ballot_sync(FULL, hit && tj == T_RIGID);
                     // rank in scan order decides whether the entry fits, as
@@ -544,7 +531,7 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
         for (int f0 = 0; f0 < total; f0 += 32) {
             const int f = f0 + lane;
             bool keep = false;
-            float4 Aj = make_float4(0.f, 0.f, 0.f, 0.f);
+            int4 Aj = make_int4(0, 0, 0, 0);
             int j = 0, eq = 0, q = qc;
             float rj = 0.f;
             if (f < total) {
@@ -552,11 +539,10 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
                 const int off = f - S.pre[q];
                 j = S.js[q] + off;
                 eq = (q << 8) | off;
-                const int oc = S.code[q];
                 Aj = b.A32[j];
-                const int tj = unpack_type(__float_as_uint(Aj.w));
-                const float px = Aj.x + (float)(oc % 5 - 2) * cx, py = Aj.y + (float)((oc / 5) % 5 - 2) * cy,
-                            pz = Aj.z + (float)(oc / 25 - 2) * cz;
+                const int tj = Aj.w;
+                float px, py, pz;
+                geo.disp(Aj, ref, px, py, pz);
                 const float ex = fmaxf(fmaxf(lx - px, px - hx), 0.f), ey = fmaxf(fmaxf(ly - py, py - hy), 0.f),
                             ez = fmaxf(fmaxf(lz - pz, pz - hz), 0.f);
                 const float d2 = ex * ex + ey * ey + ez * ez;
@@ -583,7 +569,7 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
                 rounds(32);
                 // move the remainder to the front of the stage
                 const bool mv = lane < nst - 32;
-                float4 ma;
+                int4 ma;
                 int mj = 0, mq = 0;
                 float mr = 0.f;
                 if (mv) {
@@ -615,31 +601,29 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
         if (lane < P) {
             const int s = g0 + lane;
             myn = mynf + mym;
-            if (mynf > b.capown || mym > b.capown) atomicOr(b.err, ERR_PAIR_CAP);
+            if (split && (mynf > b.capown || mym > b.capown)) atomicOr(b.err, ERR_PAIR_CAP);
             if (myn > cap) atomicOr(b.err, ERR_NBR_CAP);
-            b.nfirst[s] = min(mynf, min(cap, b.capown));
+            b.nfirst[s] = min(mynf, split ? min(cap, b.capown) : cap);
             b.ncnt[s] = min(myn, cap);
             b.nbflag[s] = myrig ? 1 : 0;
         }
         int maxn = lane < P ? min(myn, cap) : 0;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) maxn = max(maxn, __shfl_xor_sync(FULL, maxn, o));
-        // write-out: lane = (row kr, particle p), the group's particles side
-        // by side; without overflow the back region [cap - m, cap) moves
-        // down to [nf, n) as it is
-        const int L = P > 4 ? 8 : (P > 2 ? 4 : P);   // lanes per row (P = 1, 2, 4 or 8 after rounding up)
-        const int lsh = L == 8 ? 3 : (L == 4 ? 2 : L - 1);
-        const int p = lane & (L - 1), kr = lane >> lsh, R = 32 >> lsh;
-        const int pnf = __shfl_sync(FULL, mynf, p), pm = __shfl_sync(FULL, mym, p);
-        const int pn = pnf + pm, pcnt = min(pn, cap);
-        const bool wp = p < P;
-        for (int k0 = 0; k0 < maxn; k0 += R) {
-            const int k = k0 + kr;
-            if (wp && k < pcnt) {
-                const int src = (pn > cap || k < pnf) ? k : cap - pm + (k - pnf);
-                const uint32_t e = buf[p * stride + src];
-                const int slot = S.js[(e >> 8) & 127u] + (int)(e & 255u);
-                b.nbr[(long long)k * Np + g0 + p] = (int)((uint32_t)slot | ((e & 0x8000u) ? NB_FAR : 0u));
+        // write-out: LPP lanes a particle, GROUP particles side by side; without
+        // overflow the back region [cap - m, cap) moves down to [nf, n) as it is
+        for (int p0 = 0; p0 < P; p0 += GROUP) {
+            const int p = p0 + lane / LPP;   // < NG_G: the shuffles below stay in range
+            const int pnf = __shfl_sync(FULL, mynf, p), pm = __shfl_sync(FULL, mym, p);
+            const int pn = pnf + pm, pcnt = p < P ? min(pn, cap) : 0;
+            for (int k0 = 0; k0 < maxn; k0 += LPP) {
+                const int k = k0 + lane % LPP;
+                if (k < pcnt) {
+                    const int src = (pn > cap || k < pnf) ? k : cap - pm + (k - pnf);
+                    const uint32_t e = buf[p * stride + src];
+                    const int slot = S.js[(e >> 8) & 127u] + (int)(e & 255u);
+                    b.nbr[entry_at(k, g0 + p, rows)] = (int)((uint32_t)slot | ((e & 0x8000u) ? NB_FAR : 0u));
+                }
             }
         }
         __syncwarp();
@@ -647,30 +631,32 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
 }
 
 // For every non-owned entry k of s (positions [nfirst, n)), the position r
-// of s in the partner j's owned prefix (ascending), by binary search; four
-// searches run interleaved so their loads overlap.  Both directions are kept,
-// in disjoint rows of rev: rev[k][s] = r (where s reads j's result in j's
-// column) and rev[r][j] = k - nfirst(s) (where j writes its result in s's
-// column); each owned entry of j gets exactly one.
+// of s in the partner j's owned prefix (ascending), by binary search; LPP
+// lanes share a list and four searches of a lane run interleaved so their
+// loads overlap.  Both directions are kept, in disjoint entries of rev:
+// rev[k of s] = r (where s reads j's result in j's column) and rev[r of j] =
+// k - nfirst(s) (where j writes its result in s's column); each owned entry
+// of j gets exactly one.
 __device__ __forceinline__ int nb_at(const Bufs &b, int i, int k)
 {
-    return (int)((uint32_t)__ldg(b.nbr + (long long)k * b.Npad + i) & ~NB_FAR);
+    return (int)((uint32_t)__ldg(b.nbr + entry_at(k, i, b.rows)) & ~NB_FAR);
 }
 
 __global__ void k_rev(Bufs b, const int *gate)
 {
     GATE;
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= b.N) return;
-    const long long Np = b.Npad;
+    const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long s = t / LPP;
+    if (s >= b.N || !rebuilds(b, gate, b.pinst[b.perm[s]])) return;
+    const int rows = b.rows;
     const int first = b.nfirst[s], n = b.ncnt[s];
     constexpr int G = 4;  // (owned prefixes are <= capown, checked at the build)
-    for (int k0 = first; k0 < n; k0 += G) {
+    for (int k0 = first + (int)(t % LPP); k0 < n; k0 += G * LPP) {
         int part[G], lo[G], hi[G];
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            const int k = k0 + g;
-            part[g] = k < n ? (int)((uint32_t)b.nbr[(long long)k * Np + s] & ~NB_FAR) : -1;
+            const int k = k0 + g * LPP;
+            part[g] = k < n ? nb_at(b, (int)s, k) : -1;
             lo[g] = 0;
             hi[g] = part[g] >= 0 ? b.nfirst[part[g]] : 0;
         }
@@ -692,24 +678,33 @@ __global__ void k_rev(Bufs b, const int *gate)
         }
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            const int k = k0 + g;
+            const int k = k0 + g * LPP;
             if (k >= n) break;
             const bool ok = lo[g] < end[g] && nb_at(b, part[g], lo[g]) == (int)s;
             if (!ok || k - first >= b.capown) atomicOr(b.err, ERR_REV);
-            b.rev[(long long)k * Np + s] = (uint16_t)(ok ? lo[g] : 0);
-            if (ok && k - first < b.capown) b.rev[(long long)lo[g] * Np + part[g]] = (uint16_t)(k - first);
+            b.rev[entry_at(k, s, rows)] = (uint16_t)(ok ? lo[g] : 0);
+            if (ok && k - first < b.capown) b.rev[entry_at(lo[g], part[g], rows)] = (uint16_t)(k - first);
         }
     }
 }
 
-// Closes the build: a new list epoch, the gate shut until the skin is used up.
+// Closes the build: a new list epoch of each instance built, its gate shut
+// until the skin is used up (one block).
 __global__ void k_build_done(Bufs b, const int *gate)
 {
     GATE;
-    *b.list_epoch += 1u;
-    *b.need_build = 0;
-    *b.fresh = 1;
-    *b.aclose_ok = 0;   // slots were reassigned
+    for (int k = threadIdx.x; k < b.n_inst; k += blockDim.x)
+        if (rebuilds(b, gate, k)) {
+            b.list_epoch[1 + k] += 1u;
+            b.need_build[1 + k] = 0;
+        }
+    __syncthreads();   // the gate itself is read above
+    if (threadIdx.x == 0) {
+        b.list_epoch[0] += 1u;
+        b.need_build[0] = 0;
+        *b.fresh = 1;
+        *b.aclose_ok = 0;   // slots were reassigned
+    }
 }
 
 // ---------------------------------------------------------------- launchers
@@ -745,9 +740,9 @@ void launch_build(const Bufs &b, int precision, int need_rev, const int *gate, c
         } else {
             k_neighbors<<<nblk(nc, NB_WARPS), NB_WARPS * 32, 0, st>>>(b, gate);
         }
-        if (need_rev) k_rev<<<nblk(b.N, 128), 128, 0, st>>>(b, gate);
+        if (need_rev) k_rev<<<nblk(b.N * LPP, 128), 128, 0, st>>>(b, gate);
     }
-    k_build_done<<<1, 1, 0, st>>>(b, gate);
+    k_build_done<<<1, 64, 0, st>>>(b, gate);
 }
 
 }  // namespace sdpd

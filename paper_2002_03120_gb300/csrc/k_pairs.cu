@@ -42,19 +42,21 @@ template <> __device__ __forceinline__ double rsqrt_<double>(double x) { return 
 
 template <class R> struct Mir;
 template <> struct Mir<float> {
-    __device__ __forceinline__ static const float4 *A(const Bufs &b) { return b.A32; }
+    using TA = int4;
+    __device__ __forceinline__ static const int4 *A(const Bufs &b) { return b.A32; }
     __device__ __forceinline__ static const float4 *B(const Bufs &b) { return b.B32; }
     __device__ __forceinline__ static const float4 *C(const Bufs &b) { return b.C32; }
     __device__ __forceinline__ static float4 *D(const Bufs &b) { return b.D32; }
 };
 template <> struct Mir<double> {
+    using TA = double4_32a;
     __device__ __forceinline__ static const double4_32a *A(const Bufs &b) { return b.A64; }
     __device__ __forceinline__ static const double4_32a *B(const Bufs &b) { return b.B64; }
     __device__ __forceinline__ static const double4_32a *C(const Bufs &b) { return b.C64; }
     __device__ __forceinline__ static double4_32a *D(const Bufs &b) { return b.D64; }
 };
 
-__device__ __forceinline__ int mir_type(const float4 &A) { return unpack_type(__float_as_uint(A.w)); }
+__device__ __forceinline__ int mir_type(const int4 &A) { return A.w; }
 __device__ __forceinline__ int mir_type(const double4_32a &A) { return (int)A.w; }
 __device__ __forceinline__ uint32_t mir_gid(const float4 &D) { return __float_as_uint(D.w); }
 __device__ __forceinline__ uint32_t mir_gid(const double4_32a &D) { return (uint32_t)D.w; }
@@ -119,7 +121,7 @@ template <> struct K<double> {
 template <class R> struct Rel;
 template <> struct Rel<float> {
     __device__ __forceinline__ static bool get(const Bufs &b, const Inst &I, const Geo<float> &geo,
-                                               const float4 &Ai, const float4 &Aj, int gi, int j,
+                                               const int4 &Ai, const int4 &Aj, int gi, int j,
                                                float &rx, float &ry, float &rz, float &r2)
     {
         geo.disp(Ai, Aj, rx, ry, rz);
@@ -244,100 +246,247 @@ __device__ __forceinline__ void st_stream(double4_32a *p, double4_32a v)
     __stcs((double2 *)p + 1, make_double2(v.z, v.w));
 }
 
-// Persistent pair kernels: each warp takes the next 32 slots from a counter
-// (zeroed before the launch) until none are left, so that no SM idles in the
-// tail of a partial last wave.  The result of a slot does not depend on
-// which warp computes it.
-__device__ __forceinline__ long long next_warp_slots(const Bufs &b)
+// The pair passes give a particle LPP lanes and a warp GROUP particles at a
+// time, `groups` (1 to 8) times: sub = lane % LPP takes the entries sub,
+// sub + LPP, ... of its particle's list.  When a group is done its totals
+// move to one lane each, so that the closing arithmetic of up to 32 particles
+// (FP64 conversions, the equation of state) runs once per warp on full lanes.
+// Results do not depend on `groups`; the launch takes as many as still leave
+// the chip full (pass_groups).
+__device__ __forceinline__ long long pass_base(int groups)
 {
-    unsigned long long base = 0;
-    if ((threadIdx.x & 31) == 0) base = atomicAdd(b.work, 32ull);
-    return (long long)__shfl_sync(0xffffffffu, base, 0);
+    return ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * (GROUP * groups);
+}
+// What a pass needs to know of a particle before its records: lane i of a warp
+// holds slot base + i, loaded once for all its groups and handed to the lanes
+// of a particle by shuffles.  (Loaded group by group, this chain of
+// dependent loads took longer than the 33 entries a lane then walks.)
+struct SlotHead {
+    int gi = 0, inst = 0, type = T_OUTER, n = -1, nf = 0;   // n < 0: nothing to do (a slot past the end)
+    __device__ __forceinline__ SlotHead() {}
+    __device__ __forceinline__ SlotHead(const Bufs &b, long long s, bool live)
+    {
+        if (live && s < b.N) {
+            gi = b.perm[s];
+            type = b.stype[s];
+            n = b.ncnt[s];
+            nf = b.nfirst[s];
+            inst = b.pinst[gi];
+        }
+    }
+    __device__ __forceinline__ SlotHead of_group(int g) const
+    {
+        const int src = g * GROUP + (threadIdx.x & 31) / LPP;
+        SlotHead h;
+        h.gi = __shfl_sync(0xffffffffu, gi, src);
+        h.inst = __shfl_sync(0xffffffffu, inst, src);
+        h.type = __shfl_sync(0xffffffffu, type, src);
+        h.n = __shfl_sync(0xffffffffu, n, src);
+        h.nf = __shfl_sync(0xffffffffu, nf, src);
+        return h;
+    }
+};
+// This lane's first two entries of a list [k0, n): fetched for the next group
+// while the current one is evaluated.
+struct ListHead {
+    int e0 = 0, e1 = 0;
+    __device__ __forceinline__ ListHead() {}
+    __device__ __forceinline__ ListHead(const int *nbr, long long s, int rows, int k0, int n, int sub)
+    {
+        const int k = k0 + sub;
+        if (k < n) e0 = ld_stream(nbr + entry_at(k, s, rows));
+        if (k + LPP < n) e1 = ld_stream(nbr + entry_at(k + LPP, s, rows));
+    }
+};
+
+// The lists of a group asked into L2 (PTX cp.async.bulk.prefetch.L2), while
+// the group before it is evaluated: its rows are one block of memory.  The
+// loads one and two rows ahead then wait for L2 and not for HBM.
+// (s: the group's first slot, a multiple of GROUP; n: entries of this lane's particle)
+__device__ __forceinline__ void prefetch_lists(const Bufs &b, long long s, int n)
+{
+    const int most = __reduce_max_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && most > 0)
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(b.nbr + entry_at(0, s, b.rows)),
+                     "r"(entry_rows(most) * (int)(ROW * sizeof(int)))
+                     : "memory");
+}
+
+// lane GROUP g + p receives particle p's value (held by every lane of p) in group g
+template <class T> __device__ __forceinline__ void keep_group(T v, int g, T &keep)
+{
+    const int lane = threadIdx.x & 31;
+    const T got = __shfl_sync(0xffffffffu, v, (lane % GROUP) * LPP);
+    if (lane / GROUP == g) keep = got;
+}
+template <class T> __device__ __forceinline__ T lanes_sum(T v)
+{
+#pragma unroll
+    for (int o = 1; o < LPP; o <<= 1) v = v + __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ bool lanes_any(bool v)
+{
+    const unsigned m = __ballot_sync(0xffffffffu, v);
+    return (m >> ((threadIdx.x & 31) & ~(LPP - 1))) & ((1u << LPP) - 1u);
+}
+// FP32 compensated sums: s + c over the lanes, error terms kept (Knuth's
+// two-sum, no ordering of the operands assumed)
+__device__ __forceinline__ void lanes_sum(float &s, float &c)
+{
+#pragma unroll
+    for (int o = 1; o < LPP; o <<= 1) {
+        const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
+        const float t = s + s2, z = t - s;
+        c = (c + c2) + ((s - (t - z)) + (s2 - z));
+        s = t;
+    }
 }
 
 // ------------------------------------------------------------------ density
 // gate: nullptr = always; else only when *gate != 0 (a build just happened)
-// Visits the entries k = 0 .. n-1 of a slot's neighbour list in order,
-// calling f(k, entry, record of the partner, side value of the partner).  The
-// list index two entries ahead and the record (and side value, when `side`
-// is given) one entry ahead are fetched before f runs on the current one, so
-// the loads of the next pair overlap this pair's arithmetic.  NB_FAR entries
-// are visited too (their record is fetched without the flag bit).
-template <class T4, class F>
-__device__ __forceinline__ void for_each_entry(const int *__restrict__ nb, long long Np, int n,
-                                               const T4 *__restrict__ A, const double *__restrict__ side, F &&f)
+// Visits the entries k = sub, sub + LPP, ... of [k0, n) of a slot's neighbour
+// list (k0 + sub first), calling f(k, entry, record of the partner, side value
+// of the partner).  The list index two entries ahead and the record (and side
+// value, when `side` is given) one entry ahead are fetched before f runs on
+// the current one (the first two indexes by the caller: hd), so the loads of
+// the next pair overlap this pair's arithmetic.  NB_FAR entries are visited too (their record is fetched
+// without the flag bit).
+template <class TA, class F>
+__device__ __forceinline__ void for_each_entry(const int *__restrict__ nbr, long long s, int rows, int k0, int n,
+                                               int sub, const ListHead &hd, const TA *__restrict__ A,
+                                               const double *__restrict__ side, F &&f)
 {
-    if (n <= 0) return;
-    uint32_t en = (uint32_t)ld_stream(nb);
-    uint32_t enn = n > 1 ? (uint32_t)ld_stream(nb + Np) : 0u;
-    T4 An = A[en & ~NB_FAR];
+    int k = k0 + sub;
+    if (k >= n) return;
+    const int *__restrict__ nb = nbr + entry_at(k, s, rows);
+    uint32_t en = (uint32_t)hd.e0, enn = (uint32_t)hd.e1;
+    TA An = A[en & ~NB_FAR];
     double Sn = side ? side[en & ~NB_FAR] : 0.0;
-    for (int k = 0; k < n; ++k) {
+    for (; k < n; k += LPP) {
         const uint32_t e = en;
-        const T4 Aj = An;
+        const TA Aj = An;
         const double Sj = Sn;
-        if (k + 1 < n) {
+        if (k + LPP < n) {
             en = enn;
             An = A[en & ~NB_FAR];
             if (side) Sn = side[en & ~NB_FAR];
-            if (k + 2 < n) enn = (uint32_t)ld_stream(nb + (long long)(k + 2) * Np);
+            if (k + 2 * LPP < n) enn = (uint32_t)ld_stream(nb + 2 * ROW);
         }
+        nb += ROW;
         f(k, e, Aj, Sj);
     }
 }
 
-template <class R, bool CLOSE>
-__global__ void __launch_bounds__(256) k_density(Bufs b, int any_filter, const int *gate)
+// Density, pressure and the collision mark of slot s from its kernel sum.
+template <class R>
+__device__ __forceinline__ void finish_density(const Bufs &b, const Inst &I, int type, long long s, double sum,
+                                               bool close, int defer)
 {
-    if (gate && *gate == 0) return;
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s == 0) *b.aclose_ok = 1;   // the marks below are for these positions
-    if (s >= b.N) return;
-    const int gi = b.perm[s];
-    const Inst &I = b.inst[b.pinst[gi]];
-    const int ti = b.stype[s];
-    // mark particles with a mobile neighbour inside the collision radius of
-    // the artificial viscosity (a superset: the collision pass decides exactly)
-    // (CLOSE: some instance of the context has the artificial viscosity)
-    const bool want_close = CLOSE && I.artvis && (ti == T_FLUID || ti == T_RIGID);
-    const R close_r2 = (R)(I.artvis_r2f_hi * 1.0001f);
-    bool close = false;
-    double d;
-    if (ti == T_OUTER) {
-        d = I.inv_dx3;  // outer-wall particles are not updated (Section 2.5)
-    } else {
-        const auto *A = Mir<R>::A(b);
-        const auto Ai = A[s];
-        const Geo<R> geo(I);
-        const int n = b.ncnt[s];
-        const long long Np = b.Npad;
-        const R Wc = K<R>::Wc(I), irc = K<R>::inv_rc(I);
-        PosAcc<R> acc(I.W0);
-        for_each_entry(b.nbr + s, Np, n, A, nullptr, [&](int, uint32_t e, const decltype(Ai) &Aj, double) {
-            if (e & NB_FAR) return;
-            R rx, ry, rz, r2;
-            if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) return;
-            if (CLOSE && want_close && r2 <= close_r2) {
-                const int tj = mir_type(Aj);
-                close |= (tj == T_FLUID || tj == T_RIGID);
-            }
-            // float: correctly rounded sqrt; double: r2 / sqrt via rsqrt (~1 ulp)
-            const R q = (sizeof(R) == 4 ? sqrt(r2) : r2 * rsqrt_<R>(r2)) * irc;
-            const R om = lt_nonneg(q, R(1)) ? R(1) - q : R(0);
-            acc.add(Wc * (R(1) + R(3) * q) * om * om * om);
-        });
-        d = I.Cn * acc.value();
-    }
-    const double rho = I.mf * d;
-    double p = eos_pressure(I, rho);
+    // outer-wall particles are not updated (Section 2.5)
+    const double d = type == T_OUTER ? I.inv_dx3 : I.Cn * sum;
+    double p = eos_pressure(I, I.mf * d);
     if (I.clamp && p < 0.0) p = 0.0;
     b.aclose[s] = close ? 1 : 0;
     b.sd[s] = d;
     b.sp[s] = p;
-    if (!any_filter) {
+    if (!defer) {
         b.sp2[s] = p;
         finalize_slot<R>(b, s, d, p);
     }
+}
+
+// The kernel sum of the entries [k0, n) of slot s on this lane; close: a
+// mobile neighbour inside the collision radius of the artificial viscosity (a
+// superset: the collision pass decides exactly; CLOSE: some instance of the
+// context has it)
+template <class R, bool CLOSE, class ACC>
+__device__ __forceinline__ void density_entries(const Bufs &b, const Inst &I, long long s, int gi, int ti, int k0,
+                                                int n, int sub, const ListHead &hd, ACC &acc, bool &close)
+{
+    const bool want_close = CLOSE && I.artvis && (ti == T_FLUID || ti == T_RIGID);
+    const R close_r2 = (R)(I.artvis_r2f_hi * 1.0001f);
+    const auto *A = Mir<R>::A(b);
+    const auto Ai = A[s];
+    const Geo<R> geo(I);
+    const R Wc = K<R>::Wc(I), irc = K<R>::inv_rc(I);
+    for_each_entry(b.nbr, s, b.rows, k0, n, sub, hd, A, nullptr, [&](int, uint32_t e, const decltype(Ai) &Aj, double) {
+        if (e & NB_FAR) return;
+        R rx, ry, rz, r2;
+        if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) return;
+        if (CLOSE && want_close && r2 <= close_r2) {
+            const int tj = mir_type(Aj);
+            close |= (tj == T_FLUID || tj == T_RIGID);
+        }
+        // float: correctly rounded sqrt; double: r2 / sqrt via rsqrt (~1 ulp)
+        const R q = (sizeof(R) == 4 ? sqrt(r2) : r2 * rsqrt_<R>(r2)) * irc;
+        const R om = lt_nonneg(q, R(1)) ? R(1) - q : R(0);
+        acc.add(Wc * (R(1) + R(3) * q) * om * om * om);
+    });
+}
+
+template <class R, bool CLOSE>
+__global__ void __launch_bounds__(256) k_density(Bufs b, int defer, const int *gate, int groups)
+{
+    if (gate && *gate == 0) return;
+    const int lane = threadIdx.x & 31, sub = lane % LPP;
+    const long long base = pass_base(groups);
+    if (base == 0 && lane == 0) *b.aclose_ok = 1;   // the marks below are for these positions
+    const SlotHead mine(b, base + lane, lane < groups * GROUP);
+    SlotHead h = mine.of_group(0);
+    ListHead hd(b.nbr, base + lane / LPP, b.rows, 0, h.type == T_OUTER ? 0 : h.n, sub);
+    R ks = 0, kc = 0;
+    int kclose = 0;
+    for (int g = 0; g < groups; ++g) {
+        const long long s = base + g * GROUP + lane / LPP;
+        SlotHead hn;
+        ListHead hdn;
+        if (g + 1 < groups) {
+            hn = mine.of_group(g + 1);
+            hdn = ListHead(b.nbr, s + GROUP, b.rows, 0, hn.type == T_OUTER ? 0 : hn.n, sub);
+            prefetch_lists(b, base + (g + 1) * GROUP, hn.type == T_OUTER ? 0 : hn.n);
+        }
+        bool close = false;
+        R sum = 0, comp = 0;
+        if (h.type != T_OUTER) {
+            const Inst &I = b.inst[h.inst];
+            if constexpr (sizeof(R) == 4) {
+                // every lane starts from W(0) (PosAcc wants |sum| >= |term|);
+                // all but one of them are taken off below
+                PosAcc<R> acc(I.W0);
+                density_entries<R, CLOSE>(b, I, s, h.gi, h.type, 0, h.n, sub, hd, acc, close);
+                sum = acc.s;
+                comp = acc.c;
+            } else {
+                // the owned and the other entries apart, as the half-pair
+                // form sums them (the same additions)
+                PosAcc<R> own(0.0), oth(0.0);
+                density_entries<R, CLOSE>(b, I, s, h.gi, h.type, 0, h.nf, sub, hd, own, close);
+                density_entries<R, CLOSE>(b, I, s, h.gi, h.type, h.nf, h.n, sub,
+                                          ListHead(b.nbr, s, b.rows, h.nf, h.n, sub), oth, close);
+                sum = own.s;
+                comp = oth.s;
+            }
+        }
+        if constexpr (sizeof(R) == 4) {
+            lanes_sum(sum, comp);
+        } else {
+            sum = lanes_sum(sum);
+            comp = lanes_sum(comp);
+        }
+        keep_group(sum, g, ks);
+        keep_group(comp, g, kc);
+        if constexpr (CLOSE) keep_group((int)lanes_any(close), g, kclose);
+        h = hn;
+        hd = hdn;
+    }
+    const long long s = base + lane;
+    if (lane >= groups * GROUP || s >= b.N) return;
+    const Inst &I = b.inst[mine.inst];
+    double v;
+    if constexpr (sizeof(R) == 4) v = ((double)ks - (double)(LPP - 1) * (double)(float)I.W0) + (double)kc;
+    else v = __dadd_rn(__dadd_rn(I.W0, ks), kc);
+    finish_density<R>(b, I, mine.type, s, v, kclose, defer);
 }
 
 // FP64 density with each unordered pair evaluated once (Newton 3): phase 1
@@ -347,113 +496,104 @@ __global__ void __launch_bounds__(256) k_density(Bufs b, int any_filter, const i
 // buffer, which is free between force passes (a scattered store, which does
 // not stall the thread); phase 2 reads its own column in entry order
 // (coalesced).  The partner's r_ji = -r_ij bit for bit and the terms are
-// summed in list order ([owned][not owned]) as in k_density, so the result is
-// the same.
-__device__ __forceinline__ void density_half_slot(const Bufs &b, long long s)
+// added in the same order ([owned], [not owned], lane by lane) as in
+// k_density, so the result is the same.
+__global__ void __launch_bounds__(256) k_density_half(Bufs b, const int *gate, int groups)
 {
-    if (s >= b.N) return;
-    const int gi = b.perm[s];
-    const Inst &I = b.inst[b.pinst[gi]];
-    const int ti = b.stype[s];
+    if (gate && *gate == 0) return;
+    const int lane = threadIdx.x & 31, sub = lane % LPP;
+    const long long base = pass_base(groups);
+    if (base == 0 && lane == 0) *b.aclose_ok = 1;
     const double4_32a *A = Mir<double>::A(b);
-    const double4_32a Ai = A[s];
-    const Geo<double> geo(I);
-    const int nf = b.nfirst[s];
-    const long long Np = b.Npad;
     double *__restrict__ wb = (double *)b.resB;
-    const uint16_t *__restrict__ rv = b.rev + s;
-    const double close_r2 = (double)(I.artvis_r2f_hi * 1.0001f);
-    const bool want_close = I.artvis != 0;
-    bool close = false;
-    const double irc = K<double>::inv_rc(I), Wc = K<double>::Wc(I);
     const int capown = b.capown;
-    double acc = I.W0;
-    for_each_entry(b.nbr + s, Np, nf, A, nullptr, [&](int k, uint32_t e, const double4_32a &Aj, double) {
-        double W = 0.0;
-        if (!(e & NB_FAR)) {
-            double rx, ry, rz, r2;
-            if (Rel<double>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) {
-                const double q = r2 * rsqrt_<double>(r2) * irc;
-                const double om = lt_nonneg(q, 1.0) ? 1.0 - q : 0.0;
-                W = Wc * (1.0 + 3.0 * q) * om * om * om;
-                acc = __dadd_rn(acc, W);
-                if (want_close && r2 <= close_r2) {
-                    const int tj = mir_type(Aj);
-                    const bool mob = (tj == T_FLUID || tj == T_RIGID);
-                    if (mob && (ti == T_FLUID || ti == T_RIGID)) {
-                        close = true;
-                        W = -W;   // tells the partner
+    const SlotHead mine(b, base + lane, lane < groups * GROUP);
+    double keep = 0.0;
+    int kclose = 0;
+    for (int g = 0; g < groups; ++g) {
+        const long long s = base + g * GROUP + lane / LPP;
+        const SlotHead h = mine.of_group(g);
+        double acc = 0.0;
+        bool close = false;
+        if (s < b.N) {
+            const int gi = h.gi, ti = h.type;
+            const Inst &I = b.inst[h.inst];
+            const double4_32a Ai = A[s];
+            const Geo<double> geo(I);
+            const double close_r2 = (double)(I.artvis_r2f_hi * 1.0001f);
+            const bool want_close = I.artvis != 0;
+            const double irc = K<double>::inv_rc(I), Wc = K<double>::Wc(I);
+            for_each_entry(b.nbr, s, b.rows, 0, h.nf, sub, ListHead(b.nbr, s, b.rows, 0, h.nf, sub), A, nullptr,
+                           [&](int k, uint32_t e, const double4_32a &Aj, double) {
+                double W = 0.0;
+                if (!(e & NB_FAR)) {
+                    double rx, ry, rz, r2;
+                    if (Rel<double>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) {
+                        const double q = r2 * rsqrt_<double>(r2) * irc;
+                        const double om = lt_nonneg(q, 1.0) ? 1.0 - q : 0.0;
+                        W = Wc * (1.0 + 3.0 * q) * om * om * om;
+                        acc = __dadd_rn(acc, W);
+                        if (want_close && r2 <= close_r2) {
+                            const int tj = mir_type(Aj);
+                            const bool mob = (tj == T_FLUID || tj == T_RIGID);
+                            if (mob && (ti == T_FLUID || ti == T_RIGID)) {
+                                close = true;
+                                W = -W;   // tells the partner
+                            }
+                        }
                     }
                 }
-            }
+                // into the partner's column, at the row of its entry for this pair
+                const int row = __ldg(b.rev + entry_at(k, s, b.rows));
+                if (row < capown) wb[entry_at(row, e & ~NB_FAR, b.rows_own)] = W;
+            });
         }
-        // into the partner's column, at the row of its entry for this pair
-        const int row = __ldg(rv + (long long)k * Np);
-        if (row < capown) wb[(long long)row * Np + (e & ~NB_FAR)] = W;
-    });
-    b.sd[s] = acc;   // partial; completed by k_density_gather
-    b.aclose[s] = close ? 1 : 0;
+        keep_group(lanes_sum(acc), g, keep);
+        keep_group((int)lanes_any(close), g, kclose);
+    }
+    const long long s = base + lane;
+    if (lane >= groups * GROUP || s >= b.N) return;
+    b.sd[s] = keep;   // partial; completed by k_density_gather
+    b.aclose[s] = kclose ? 1 : 0;
 }
 
-__global__ void __launch_bounds__(256) k_density_half(Bufs b, const int *gate)
+__global__ void __launch_bounds__(256) k_density_gather(Bufs b, int defer, const int *gate, int groups)
 {
     if (gate && *gate == 0) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *b.aclose_ok = 1;
-    for (long long base = next_warp_slots(b); base < b.N; base = next_warp_slots(b))
-        density_half_slot(b, base + (threadIdx.x & 31));
-}
-
-__global__ void __launch_bounds__(256) k_density_gather(Bufs b, int any_filter, const int *gate)
-{
-    if (gate && *gate == 0) return;
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= b.N) return;
-    const int gi = b.perm[s];
-    const Inst &I = b.inst[b.pinst[gi]];
-    const int ti = b.stype[s];
-    double d;
-    if (ti == T_OUTER) {
-        d = I.inv_dx3;  // outer-wall particles are not updated (Section 2.5)
-    } else {
-        const double *__restrict__ wb = (const double *)b.resB;
-        const int n = b.ncnt[s], nf = b.nfirst[s];
-        const long long Np = b.Npad;
-        // the owners wrote W of this particle's non-owned entries into its
-        // own column (row k - nf; more rows than capown only after a list
-        // error, flagged)
-        const int nend = min(n, nf + b.capown);
-        double acc = b.sd[s];
-        bool close = b.aclose[s] != 0;
-        constexpr int G = 4;
-        for (int k0 = nf; k0 < nend; k0 += G) {
-            double w[G];
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-                const int k = k0 + g;
-                w[g] = 0.0;
-                if (k < nend) {
-                    const uint32_t e = (uint32_t)__ldg(b.nbr + (long long)k * Np + s);
-                    if (!(e & NB_FAR)) w[g] = wb[(long long)(k - nf) * Np + s];
-                }
-            }
-#pragma unroll
-            for (int g = 0; g < G; ++g) {
-                if (w[g] < 0.0) close = true;
-                acc = __dadd_rn(acc, fabs(w[g]));
+    const int lane = threadIdx.x & 31, sub = lane % LPP;
+    const long long base = pass_base(groups);
+    const double *__restrict__ wb = (const double *)b.resB;
+    const SlotHead mine(b, base + lane, lane < groups * GROUP);
+    double keep = 0.0;
+    int kclose = 0;
+    for (int g = 0; g < groups; ++g) {
+        const long long s = base + g * GROUP + lane / LPP;
+        const SlotHead h = mine.of_group(g);
+        double acc = 0.0;
+        bool close = false;
+        if (h.type != T_OUTER) {
+            // the owners wrote W of this particle's non-owned entries into
+            // its own column (more rows than capown only after a list error,
+            // flagged; 0 for an entry beyond h)
+            const int m = min(h.n - h.nf, b.capown);
+            const double *__restrict__ p = wb + entry_at(sub, s, b.rows_own);
+#pragma unroll 4
+            for (int k = sub; k < m; k += LPP) {
+                const double w = *p;
+                p += ROW;
+                close |= w < 0.0;
+                acc = __dadd_rn(acc, fabs(w));
             }
         }
-        d = I.Cn * acc;
-        b.aclose[s] = (close && (ti == T_FLUID || ti == T_RIGID)) ? 1 : 0;
+        keep_group(lanes_sum(acc), g, keep);
+        keep_group((int)lanes_any(close), g, kclose);
     }
-    const double rho = I.mf * d;
-    double p = eos_pressure(I, rho);
-    if (I.clamp && p < 0.0) p = 0.0;
-    b.sd[s] = d;
-    b.sp[s] = p;
-    if (!any_filter) {
-        b.sp2[s] = p;
-        finalize_slot<double>(b, s, d, p);
-    }
+    const long long s = base + lane;
+    if (lane >= groups * GROUP || s >= b.N) return;
+    const int ti = mine.type;
+    const Inst &I = b.inst[mine.inst];
+    const bool close = (b.aclose[s] != 0 || kclose) && (ti == T_FLUID || ti == T_RIGID);
+    finish_density<double>(b, I, ti, s, __dadd_rn(__dadd_rn(I.W0, b.sd[s]), keep), close, defer);
 }
 
 // ------------------------------------------------------ density reinitialisation
@@ -463,38 +603,97 @@ __global__ void __launch_bounds__(256) k_density_gather(Bufs b, int any_filter, 
 // theirs; the pressure follows from Eq. prtcpres.  The new densities go to
 // sdr (the neighbours' old values are still read) and k_reinit_copy moves
 // them back.
+// A ratio of two kernel sums over the list of slot s: totals on every lane of
+// the particle (FP32: compensated, the FP64 ratio from both parts).
+template <class R> struct TwoSums;
+template <> struct TwoSums<float> {
+    KSum num{ 0.f, 0.f }, den{ 0.f, 0.f };
+    float ks[4] = { 0.f, 0.f, 0.f, 0.f };
+    __device__ __forceinline__ void add(float a, float b) { num.add(a); den.add(b); }
+    __device__ __forceinline__ void close_group(int g)
+    {
+        lanes_sum(num.s, num.c);
+        lanes_sum(den.s, den.c);
+        keep_group(num.s, g, ks[0]);
+        keep_group(num.c, g, ks[1]);
+        keep_group(den.s, g, ks[2]);
+        keep_group(den.c, g, ks[3]);
+        num = KSum{ 0.f, 0.f };
+        den = KSum{ 0.f, 0.f };
+    }
+    __device__ __forceinline__ double ratio(double a0, double b0) const
+    {
+        return (a0 + ((double)ks[0] + (double)ks[1])) / (b0 + ((double)ks[2] + (double)ks[3]));
+    }
+};
+template <> struct TwoSums<double> {
+    double num = 0.0, den = 0.0, ks[2] = { 0.0, 0.0 };
+    // a separate rounding of each term (no multiply-add fused into the sum)
+    __device__ __forceinline__ void add(double a, double b) { num = __dadd_rn(num, a); den = __dadd_rn(den, b); }
+    __device__ __forceinline__ void close_group(int g)
+    {
+        keep_group(lanes_sum(num), g, ks[0]);
+        keep_group(lanes_sum(den), g, ks[1]);
+        num = den = 0.0;
+    }
+    __device__ __forceinline__ double ratio(double a0, double b0) const { return (a0 + ks[0]) / (b0 + ks[1]); }
+};
+
+// The kernel weight of a listed pair within h, for the two Shepard averages.
 template <class R>
-__global__ void __launch_bounds__(256) k_reinit(Bufs b, int any_filter, const int *gate)
+__device__ __forceinline__ R shepard_weight(const Inst &I, R r2)
+{
+    const R q = sqrt(r2) * K<R>::inv_rc(I);
+    const R om = lt_nonneg(q, R(1)) ? R(1) - q : R(0);
+    return K<R>::Wc(I) * (R(1) + R(3) * q) * om * om * om;
+}
+
+template <class R>
+__global__ void __launch_bounds__(256) k_reinit(Bufs b, int any_filter, const int *gate, int groups)
 {
     if (gate && *gate == 0) return;
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= b.N) return;
-    const int gi = b.perm[s];
-    const Inst &I = b.inst[b.pinst[gi]];
-    const double di = b.sd[s];
-    double d = di;
-    if (I.reinit && b.stype[s] != T_OUTER) {
-        const auto *A = Mir<R>::A(b);
-        const auto Ai = A[s];
-        const Geo<R> geo(I);
-        const int n = b.ncnt[s];
-        const long long Np = b.Npad;
-        const R Wc = K<R>::Wc(I), irc = K<R>::inv_rc(I);
-        Acc<R> num(I.W0), den(I.W0 / di);
-        for_each_entry(b.nbr + s, Np, n, A, b.sd, [&](int, uint32_t e, const decltype(Ai) &Aj, double dj) {
-            if (e & NB_FAR) return;
-            R rx, ry, rz, r2;
-            if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) return;
-            const R q = sqrt(r2) * irc;
-            const R om = lt_nonneg(q, R(1)) ? R(1) - q : R(0);
-            const R W = Wc * (R(1) + R(3) * q) * om * om * om;
-            num.add(W);
-            den.add(W / (R)dj);
-        });
-        d = num.value() / den.value();
+    const int lane = threadIdx.x & 31, sub = lane % LPP;
+    const long long base = pass_base(groups);
+    const SlotHead mine(b, base + lane, lane < groups * GROUP);
+    SlotHead h = mine.of_group(0);
+    ListHead hd(b.nbr, base + lane / LPP, b.rows, 0, h.type == T_OUTER ? 0 : h.n, sub);
+    TwoSums<R> sums;
+    for (int g = 0; g < groups; ++g) {
+        const long long s = base + g * GROUP + lane / LPP;
+        SlotHead hn;
+        ListHead hdn;
+        if (g + 1 < groups) {
+            hn = mine.of_group(g + 1);
+            hdn = ListHead(b.nbr, s + GROUP, b.rows, 0, hn.type == T_OUTER ? 0 : hn.n, sub);
+            prefetch_lists(b, base + (g + 1) * GROUP, hn.type == T_OUTER ? 0 : hn.n);
+        }
+        if (h.type != T_OUTER) {
+            const int gi = h.gi;
+            const Inst &I = b.inst[h.inst];
+            if (I.reinit) {
+                const auto *A = Mir<R>::A(b);
+                const auto Ai = A[s];
+                const Geo<R> geo(I);
+                for_each_entry(b.nbr, s, b.rows, 0, h.n, sub, hd, A, b.sd,
+                               [&](int, uint32_t e, const decltype(Ai) &Aj, double dj) {
+                    if (e & NB_FAR) return;
+                    R rx, ry, rz, r2;
+                    if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) return;
+                    const R W = shepard_weight<R>(I, r2);
+                    sums.add(W, W / (R)dj);
+                });
+            }
+        }
+        sums.close_group(g);
+        h = hn;
+        hd = hdn;
     }
-    const double rho = I.mf * d;
-    double p = eos_pressure(I, rho);
+    const long long s = base + lane;
+    if (lane >= groups * GROUP || s >= b.N) return;
+    const Inst &I = b.inst[mine.inst];
+    const double di = b.sd[s];
+    const double d = I.reinit && mine.type != T_OUTER ? sums.ratio(I.W0, I.W0 / di) : di;
+    double p = eos_pressure(I, I.mf * d);
     if (I.clamp && p < 0.0) p = 0.0;
     b.sdr[s] = d;
     if (I.reinit) b.sp[s] = p;
@@ -513,35 +712,50 @@ __global__ void k_reinit_copy(Bufs b, const int *gate)
 
 // ------------------------------------------------------------ pressure filter
 template <class R>
-__global__ void __launch_bounds__(256) k_filter(Bufs b, const int *gate)
+__global__ void __launch_bounds__(256) k_filter(Bufs b, const int *gate, int groups)
 {
     if (gate && *gate == 0) return;
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= b.N) return;
-    const int gi = b.perm[s];
-    const Inst &I = b.inst[b.pinst[gi]];
-    const double pi = b.sp[s];
-    double pf = pi;
-    if (I.filter && b.stype[s] != T_OUTER) {
-        const auto *A = Mir<R>::A(b);
-        const auto Ai = A[s];
-        const Geo<R> geo(I);
-        const int n = b.ncnt[s];
-        const long long Np = b.Npad;
-        const R Wc = K<R>::Wc(I), irc = K<R>::inv_rc(I);
-        Acc<R> num(pi * I.W0), den(I.W0);
-        for_each_entry(b.nbr + s, Np, n, A, b.sp, [&](int, uint32_t e, const decltype(Ai) &Aj, double pj) {
-            if (e & NB_FAR) return;
-            R rx, ry, rz, r2;
-            if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) return;
-            const R q = sqrt(r2) * irc;
-            const R om = lt_nonneg(q, R(1)) ? R(1) - q : R(0);
-            const R W = Wc * (R(1) + R(3) * q) * om * om * om;
-            num.add((R)pj * W);
-            den.add(W);
-        });
-        pf = num.value() / den.value();
+    const int lane = threadIdx.x & 31, sub = lane % LPP;
+    const long long base = pass_base(groups);
+    const SlotHead mine(b, base + lane, lane < groups * GROUP);
+    SlotHead h = mine.of_group(0);
+    ListHead hd(b.nbr, base + lane / LPP, b.rows, 0, h.type == T_OUTER ? 0 : h.n, sub);
+    TwoSums<R> sums;
+    for (int g = 0; g < groups; ++g) {
+        const long long s = base + g * GROUP + lane / LPP;
+        SlotHead hn;
+        ListHead hdn;
+        if (g + 1 < groups) {
+            hn = mine.of_group(g + 1);
+            hdn = ListHead(b.nbr, s + GROUP, b.rows, 0, hn.type == T_OUTER ? 0 : hn.n, sub);
+            prefetch_lists(b, base + (g + 1) * GROUP, hn.type == T_OUTER ? 0 : hn.n);
+        }
+        if (h.type != T_OUTER) {
+            const int gi = h.gi;
+            const Inst &I = b.inst[h.inst];
+            if (I.filter) {
+                const auto *A = Mir<R>::A(b);
+                const auto Ai = A[s];
+                const Geo<R> geo(I);
+                for_each_entry(b.nbr, s, b.rows, 0, h.n, sub, hd, A, b.sp,
+                               [&](int, uint32_t e, const decltype(Ai) &Aj, double pj) {
+                    if (e & NB_FAR) return;
+                    R rx, ry, rz, r2;
+                    if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) return;
+                    const R W = shepard_weight<R>(I, r2);
+                    sums.add((R)pj * W, W);
+                });
+            }
+        }
+        sums.close_group(g);
+        h = hn;
+        hd = hdn;
     }
+    const long long s = base + lane;
+    if (lane >= groups * GROUP || s >= b.N) return;
+    const Inst &I = b.inst[mine.inst];
+    const double pi = b.sp[s];
+    const double pf = I.filter && mine.type != T_OUTER ? sums.ratio(pi * I.W0, I.W0) : pi;
     b.sp2[s] = pf;
     finalize_slot<R>(b, s, b.sd[s], pf);
 }
@@ -596,17 +810,18 @@ __global__ void __launch_bounds__(RB) k_drag(Bufs b)
     // the kernel-weighted fluid sums in precision R on the mirrors (the
     // exact r < h decision of Rel), per lane in R; the volumes in FP64
     using T4 = typename Vec<R>::T4;
+    using TA = typename Mir<R>::TA;
     const Geo<R> geo(I);
-    const T4 *__restrict__ A = Mir<R>::A(b);
+    const TA *__restrict__ A = Mir<R>::A(b);
     const T4 *__restrict__ Bm = Mir<R>::B(b);
-    const T4 Ai = A[s];
+    const TA Ai = A[s];
     const R Wc = K<R>::Wc(I), irc = K<R>::inv_rc(I);
     R Sr = 0, u0 = 0, u1 = 0, u2 = 0;
     for (int k = lane; k < n; k += 32) {
-        const uint32_t e = (uint32_t)b.nbr[(long long)k * b.Npad + s];
+        const uint32_t e = (uint32_t)b.nbr[entry_at(k, s, b.rows)];
         if (e & NB_FAR) continue;
         const int j = (int)e;
-        const T4 Aj = A[j];
+        const TA Aj = A[j];
         const int tj = mir_type(Aj);
         if (tj != T_RIGID && tj != T_FLUID) continue;
         R rx, ry, rz, r2;
@@ -836,10 +1051,10 @@ __device__ __forceinline__ void rxn_of(const Bufs &b, int j, double &x, double &
 // Fluid particle i and a rigid neighbour j (Section 2.4): Eqs. FijC and FijD
 // on i (no rotational or random part) and the drag reaction Eq.
 // F_fpi_DG_reac, added to i's sums; nothing beyond h.
-template <class R, class T4>
+template <class R, class TA, class T4>
 __device__ __forceinline__ void fluid_rigid_pair(const Bufs &b, const Inst &I, const Geo<R> &geo,
-                                                 const PairK<R> &P, int gi, const T4 &Ai, const T4 &Bi,
-                                                 const T4 &Ci, const T4 &Di, int j, const T4 &Aj,
+                                                 const PairK<R> &P, int gi, const TA &Ai, const T4 &Bi,
+                                                 const T4 &Ci, const T4 &Di, int j, const TA &Aj,
                                                  const T4 &Bj, const T4 &Cj, const T4 &Dj, R &fx, R &fy,
                                                  R &fz, R &tx, R &ty, R &tz)
 {
@@ -865,10 +1080,11 @@ template <class R>
 __device__ __noinline__ void fluid_rigid_pair_call(const Bufs &b, long long s, int gi, int j, R *f)
 {
     using T4 = typename Vec<R>::T4;
+    using TA = typename Mir<R>::TA;
     const Inst &I = b.inst[b.pinst[gi]];
     const Geo<R> geo(I);
     const PairK<R> P(I, (uint32_t)(*b.step));
-    const T4 *__restrict__ A = Mir<R>::A(b);
+    const TA *__restrict__ A = Mir<R>::A(b);
     const T4 *__restrict__ Bm = Mir<R>::B(b);
     const T4 *__restrict__ Cm = Mir<R>::C(b);
     const T4 *__restrict__ Dm = Mir<R>::D(b);
@@ -876,72 +1092,133 @@ __device__ __noinline__ void fluid_rigid_pair_call(const Bufs &b, long long s, i
                         f[2], f[3], f[4], f[5]);
 }
 
+// The draws of a pair out of line, where they are rare and the caller's
+// registers matter (an entry beyond h in the first evaluation of a step and
+// within it in the second).
+template <class R>
+__device__ __noinline__ void draw_rare(uint32_t gi, uint32_t gj, uint32_t step, uint32_t k0, uint32_t k1, R *z)
+{
+    pair_normals<R>(gi, gj, step, k0, k1, z[0], z[1], z[2], z[3], z[4], z[5]);
+}
+
+// The force and torque totals of a warp's particles, one per lane at the end.
+template <class R> struct ForceSums {
+    R f[6], keep[6];
+    __device__ __forceinline__ ForceSums()
+    {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) f[c] = keep[c] = R(0);
+    }
+    // every accumulation step rounded explicitly
+    __device__ __forceinline__ void add(R gx, R gy, R gz, R hx, R hy, R hz)
+    {
+        f[0] = add_rn(f[0], gx);
+        f[1] = add_rn(f[1], gy);
+        f[2] = add_rn(f[2], gz);
+        f[3] = add_rn(f[3], hx);
+        f[4] = add_rn(f[4], hy);
+        f[5] = add_rn(f[5], hz);
+    }
+    __device__ __forceinline__ void close_group(int g)
+    {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) {
+            keep_group(lanes_sum(f[c]), g, keep[c]);
+            f[c] = R(0);
+        }
+    }
+};
+
+// The second evaluation of a step reads the normals of the first for the
+// instances whose lists are still the same.
+struct CacheUse {
+    uint32_t step;
+    bool fill, maybe, all;   // maybe: some instance's normals may be cached, all: every instance's are
+    __device__ __forceinline__ CacheUse(const Bufs &b, int velver)
+        : step((uint32_t)(*b.step)), fill(b.use_cache && velver == 1),
+          maybe(b.use_cache && velver == 2 && *b.cache_step == *b.step),
+          all(maybe && b.cache_epoch[0] == b.list_epoch[0])
+    {
+        // only the first evaluation writes, only the second one tests them
+        if (fill && blockIdx.x == 0) {
+            for (int k = threadIdx.x; k <= b.n_inst; k += blockDim.x) b.cache_epoch[k] = b.list_epoch[k];
+            if (threadIdx.x == 0) *b.cache_step = *b.step;
+        }
+    }
+    __device__ __forceinline__ bool reuse(const Bufs &b, int inst) const
+    {
+        return all || (maybe && b.cache_epoch[1 + inst] == b.list_epoch[1 + inst]);
+    }
+};
+
 // Direct (owner-computes-all) force pass over the neighbour list of fluid
-// particle i.  The index two entries ahead and the records of the next
-// neighbour are fetched before the current pair is evaluated.  With the
-// cache on, the first evaluation of a step (FILL) stores the six normals of
-// every entry in its own column (a NaN marker for an entry beyond h); the
-// second (REUSE, when the list has not been rebuilt in between) reads them
-// back, fetched one entry ahead like the records, instead of drawing them
-// again (same counter, so the same bits).
+// particle s (this lane's share of it).  The index two entries ahead and the
+// records of the next neighbour are fetched before the current pair is
+// evaluated.  With the cache on, the first evaluation of a step (FILL) stores
+// the six normals of every entry in its own column (a NaN marker for an entry
+// beyond h); the second (REUSE, when the list has not been rebuilt in
+// between) reads them back, fetched one entry ahead like the records, instead
+// of drawing them again (same counter, so the same bits).
 template <class R, bool REUSE>
-__device__ __forceinline__ void force_fluid_slot(const Bufs &b, long long s, uint32_t step, bool fill)
+__device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, const SlotHead &h, const ListHead &hd,
+                                                    int sub, uint32_t step, bool fill, ForceSums<R> &sums)
 {
     // FP32, normals from the cache: a partner's D record (its gid) only for a
     // pair whose normals must be drawn after all (rare), loaded then
     constexpr bool LAZY_D = REUSE && sizeof(R) == 4;
     using T4 = typename Vec<R>::T4;
+    using TA = typename Mir<R>::TA;
     using T2 = typename Vec2<R>::T2;
-    if (s >= b.N) return;
-    if (b.stype[s] != T_FLUID) return;
-    const int gi = b.perm[s];
-    const Inst &I = b.inst[b.pinst[gi]];
+    const int gi = h.gi;
+    const Inst &I = b.inst[h.inst];
     const Geo<R> geo(I);
     const PairK<R> P(I, step);
     fill = fill && P.noise;
-    const T4 *__restrict__ A = Mir<R>::A(b);
+    const TA *__restrict__ A = Mir<R>::A(b);
     const T4 *__restrict__ Bm = Mir<R>::B(b);
     const T4 *__restrict__ Cm = Mir<R>::C(b);
     const T4 *__restrict__ Dm = Mir<R>::D(b);
-    T4 *__restrict__ zA = (T4 *)b.zdA;
-    T2 *__restrict__ zB = (T2 *)b.zdB;
-    const int *__restrict__ nb = b.nbr + s;
-    const T4 Ai = A[s], Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
-    R fx = 0, fy = 0, fz = 0, tx = 0, ty = 0, tz = 0;
-    const int n = b.ncnt[s];
-    const long long Np = b.Npad;
-    int jn = n > 0 ? ld_stream(nb) : 0;
-    int jnn = n > 1 ? ld_stream(nb + Np) : 0;
-    T4 An = A[jn], Bn = Bm[jn], Cn = Cm[jn], Dn = Di;
+    const int n = h.n;
+    int k = sub;
+    if (k >= n) return;
+    const size_t first = entry_at(sub, s, b.rows);
+    const int *__restrict__ nb = b.nbr + first;
+    T4 *__restrict__ zA = (T4 *)b.zdA + first;
+    T2 *__restrict__ zB = (T2 *)b.zdB + first;
+    const TA Ai = A[s];
+    const T4 Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
+    int jn = hd.e0, jnn = hd.e1;
+    TA An = A[jn];
+    T4 Bn = Bm[jn], Cn = Cm[jn], Dn = Di;
     if constexpr (!LAZY_D) Dn = Dm[jn];
     T4 zan;
     T2 zbn;
-    if (REUSE && P.noise && n > 0) { zan = ld_stream(zA + s); zbn = ld_stream(zB + s); }
-    for (int k = 0; k < n; ++k) {
+    if (REUSE && P.noise) { zan = ld_stream(zA); zbn = ld_stream(zB); }
+    for (; k < n; k += LPP, nb += ROW, zA += ROW, zB += ROW) {
         const int j = jn;
-        const T4 Aj = An, Bj = Bn, Cj = Cn;
+        const TA Aj = An;
+        const T4 Bj = Bn, Cj = Cn;
         T4 Dj = Dn;
         T4 za;
         T2 zb;
         if (REUSE) { za = zan; zb = zbn; }
-        if (k + 1 < n) {
+        if (k + LPP < n) {
             jn = jnn;
             An = A[jn]; Bn = Bm[jn]; Cn = Cm[jn];
             if constexpr (!LAZY_D) Dn = Dm[jn];
             if (REUSE && P.noise) {
-                zan = ld_stream(zA + (long long)(k + 1) * Np + s);
-                zbn = ld_stream(zB + (long long)(k + 1) * Np + s);
+                zan = ld_stream(zA + ROW);
+                zbn = ld_stream(zB + ROW);
             }
-            if (k + 2 < n) jnn = ld_stream(nb + (long long)(k + 2) * Np);
+            if (k + 2 * LPP < n) jnn = ld_stream(nb + 2 * ROW);
         }
         const bool rig = mir_type(Aj) == T_RIGID;
-        const long long at = (long long)k * Np + s;
         R rx, ry, rz, r2;
         if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, j, rx, ry, rz, r2)) {
             if (!REUSE && fill && !rig) {
                 T4 nm;
                 nm.x = R(NAN); nm.y = R(0); nm.z = R(0); nm.w = R(0);
-                st_stream(zA + at, nm);
+                st_stream(zA, nm);
             }
             continue;
         }
@@ -954,184 +1231,13 @@ __device__ __forceinline__ void force_fluid_slot(const Bufs &b, long long s, uin
             zmode = 1;
         }
         if constexpr (LAZY_D) {
-            if (zmode == 0 && P.noise && !rig) Dj = Dm[j];
-        }
-        sdpd_pair<R>(P, rx, ry, rz, r2, Bi, Ci, Di, Bj, Cj, Dj, !rig, zmode, z, ox, oy, oz, ce, ex, ey, ez,
-                     q, om);
-        if (!REUSE && fill && !rig) {
-            T4 zw;
-            zw.x = z.z0; zw.y = z.z1; zw.z = z.z2; zw.w = z.z3;
-            T2 zv;
-            zv.x = z.z4; zv.y = z.z5;
-            st_stream(zA + at, zw);
-            st_stream(zB + at, zv);
-        }
-        // every accumulation step rounded explicitly (the pair-stream pass
-        // adds the same terms in the same order and must match bit for bit)
-        R gx, gy, gz, hx, hy, hz;
-        pair_fh(ox, oy, oz, ce, ex, ey, ez, gx, gy, gz, hx, hy, hz);
-        if (rig) {
-            // Eq. F_fpi_DG_reac: -F^DG_s W_sj / S_s
-            R rcx, rcy, rcz;
-            rxn_of(b, j, rcx, rcy, rcz);
-            const R W = drag_weight(P, q, om);
-            fx = sub_rn(fx, mul_rn(rcx, W));
-            fy = sub_rn(fy, mul_rn(rcy, W));
-            fz = sub_rn(fz, mul_rn(rcz, W));
-        }
-        fx = add_rn(fx, gx);
-        fy = add_rn(fy, gy);
-        fz = add_rn(fz, gz);
-        tx = add_rn(tx, hx);
-        ty = add_rn(ty, hy);
-        tz = add_rn(tz, hz);
-    }
-    write_fluid_force<R>(b, I, gi, fx, fy, fz, tx, ty, tz, P.lev);
-}
-
-// 16-byte asynchronous copy global -> shared, cached in L1 (PTX cp.async,
-// sm_80 and later; measured faster here than the L2-only form), and its
-// commit / wait
-__device__ __forceinline__ void cp_async16(void *smem, const void *gmem)
-{
-    const unsigned sa = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;\n" ::"r"(sa), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
-template <int N> __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory"); }
-
-// Shared-memory ring of the async variant: per thread DEPTH stages of the
-// partner's B, C, D records, thread-minor (rec[stage][record][thread]) so a
-// warp's 16-byte accesses fall on consecutive banks.
-constexpr int LEAN_BLOCK = 128;
-template <int DEPTH> struct LeanRing {
-    float4 rec[DEPTH][3][LEAN_BLOCK];
-};
-
-// DEPTH > 0: the partner's B, C, D records through the async ring (above)
-template <class R, bool REUSE, int DEPTH = 0>
-__device__ __forceinline__ void force_fluid_slot_lean(const Bufs &b, long long s, uint32_t step, bool fill,
-                                                      LeanRing<DEPTH ? DEPTH : 1> *ring = nullptr)
-{
-    constexpr bool ASYNC = DEPTH > 0;
-    // FP32, normals from the cache: a partner's D record (its gid) is needed
-    // only for a pair whose normals must be drawn after all (rare), so it is
-    // loaded then
-    constexpr bool LAZY_D = REUSE && sizeof(R) == 4;
-    using T4 = typename Vec<R>::T4;
-    using T2 = typename Vec2<R>::T2;
-    if (s >= b.N) return;
-    if (b.stype[s] != T_FLUID) return;
-    const int gi = b.perm[s];
-    const Inst &I = b.inst[b.pinst[gi]];
-    const Geo<R> geo(I);
-    const PairK<R> P(I, step);
-    fill = fill && P.noise;
-    const T4 *__restrict__ A = Mir<R>::A(b);
-    const T4 *__restrict__ Bm = Mir<R>::B(b);
-    const T4 *__restrict__ Cm = Mir<R>::C(b);
-    const T4 *__restrict__ Dm = Mir<R>::D(b);
-    T4 *__restrict__ zA = (T4 *)b.zdA;
-    T2 *__restrict__ zB = (T2 *)b.zdB;
-    const int *__restrict__ nb = b.nbr + s;
-    const T4 Ai = A[s], Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
-    R fx = 0, fy = 0, fz = 0, tx = 0, ty = 0, tz = 0;
-    const int n = b.ncnt[s];
-    const long long Np = b.Npad;
-    int jn = n > 0 ? ld_stream(nb) : 0;
-    int jnn = n > 1 ? ld_stream(nb + Np) : 0;
-    T4 An = A[jn];
-    T4 zan;
-    T2 zbn;
-    if (REUSE && P.noise && n > 0) { zan = ld_stream(zA + s); zbn = ld_stream(zB + s); }
-    const int lt = threadIdx.x;
-    // async ring: the records of entry k + DEPTH - 1 go in flight while entry
-    // k is evaluated; one commit group per entry keeps the wait count fixed
-    auto request = [&](int kk, int jj) {
-        if constexpr (ASYNC) {
-            if (kk < n) {
-                const int st = kk % DEPTH;
-                cp_async16(&ring->rec[st][0][lt], Bm + jj);
-                cp_async16(&ring->rec[st][1][lt], Cm + jj);
-                cp_async16(&ring->rec[st][2][lt], Dm + jj);
+            if (zmode == 0 && P.noise && !rig) {
+                R t[6];
+                draw_rare<R>(mir_gid(Di), mir_gid(Dm[j]), P.step, P.key0, P.key1, t);
+                z.z0 = t[0]; z.z1 = t[1]; z.z2 = t[2]; z.z3 = t[3]; z.z4 = t[4]; z.z5 = t[5];
             }
-            cp_async_commit();
-        }
-    };
-    // entries 0 .. DEPTH-2 requested before the loop (0 and 1 are jn, jnn);
-    // jq: the list entry DEPTH - 1 ahead, the next to request
-    int jq = 0;
-    if constexpr (ASYNC) {
-        request(0, jn);
-        if constexpr (DEPTH > 2) request(1, jnn);
-#pragma unroll
-        for (int d = 2; d < DEPTH; ++d) {
-            const int e = d < n ? ld_stream(nb + (long long)d * Np) : 0;
-            if (d + 1 < DEPTH) request(d, e);
-            else jq = e;
-        }
-    }
-    for (int k = 0; k < n; ++k) {
-        if constexpr (ASYNC) {
-            // the partner DEPTH - 1 entries ahead, whether or not it is within
-            // h, into the stage of entry k - 1, whose copies are complete
-            // first (an entry beyond h is never waited for at its use)
-            cp_async_wait<DEPTH - 1>();
-            if constexpr (DEPTH == 2) {
-                request(k + 1, jnn);
-            } else {
-                request(k + DEPTH - 1, jq);
-                if (k + DEPTH < n) jq = ld_stream(nb + (long long)(k + DEPTH) * Np);
-            }
-        }
-        const int j = jn;
-        const T4 Aj = An;
-        T4 za;
-        T2 zb;
-        if (REUSE) { za = zan; zb = zbn; }
-        if (k + 1 < n) {
-            jn = jnn;
-            An = A[jn];
-            if (REUSE && P.noise) {
-                zan = ld_stream(zA + (long long)(k + 1) * Np + s);
-                zbn = ld_stream(zB + (long long)(k + 1) * Np + s);
-            }
-            if (k + 2 < n) jnn = ld_stream(nb + (long long)(k + 2) * Np);
-        }
-        const bool rig = mir_type(Aj) == T_RIGID;
-        const long long at = (long long)k * Np + s;
-        R rx, ry, rz, r2;
-        if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, j, rx, ry, rz, r2)) {
-            if (!REUSE && fill && !rig) {
-                T4 nm;
-                nm.x = R(NAN); nm.y = R(0); nm.z = R(0); nm.w = R(0);
-                st_stream(zA + at, nm);
-            }
-            continue;
-        }
-        T4 Bj, Cj, Dj = Di;
-        if constexpr (ASYNC) {
-            cp_async_wait<DEPTH - 1>();   // this entry's group is complete
-            const int st = k % DEPTH;
-            Bj = ring->rec[st][0][lt];
-            Cj = ring->rec[st][1][lt];
-            Dj = ring->rec[st][2][lt];
-        } else {
-            Bj = Bm[j];
-            Cj = Cm[j];
-            if constexpr (!LAZY_D) Dj = Dm[j];
-        }
-        R ox, oy, oz, ce, ex, ey, ez, q, om;
-        Z6<R> z;
-        int zmode = 0;
-        // an entry beyond h in the first evaluation carries the NaN marker
-        if (REUSE && P.noise && !rig && !isnan(za.x)) {
-            z.z0 = za.x; z.z1 = za.y; z.z2 = za.z; z.z3 = za.w; z.z4 = zb.x; z.z5 = zb.y;
             zmode = 1;
         }
-        if constexpr (LAZY_D) {
-            if (zmode == 0 && P.noise && !rig) Dj = Dm[j];
-        }
         sdpd_pair<R>(P, rx, ry, rz, r2, Bi, Ci, Di, Bj, Cj, Dj, !rig, zmode, z, ox, oy, oz, ce, ex, ey, ez,
                      q, om);
         if (!REUSE && fill && !rig) {
@@ -1139,11 +1245,9 @@ __device__ __forceinline__ void force_fluid_slot_lean(const Bufs &b, long long s
             zw.x = z.z0; zw.y = z.z1; zw.z = z.z2; zw.w = z.z3;
             T2 zv;
             zv.x = z.z4; zv.y = z.z5;
-            st_stream(zA + at, zw);
-            st_stream(zB + at, zv);
+            st_stream(zA, zw);
+            st_stream(zB, zv);
         }
-        // every accumulation step rounded explicitly (the pair-stream pass
-        // adds the same terms in the same order and must match bit for bit)
         R gx, gy, gz, hx, hy, hz;
         pair_fh(ox, oy, oz, ce, ex, ey, ez, gx, gy, gz, hx, hy, hz);
         if (rig) {
@@ -1151,434 +1255,53 @@ __device__ __forceinline__ void force_fluid_slot_lean(const Bufs &b, long long s
             R rcx, rcy, rcz;
             rxn_of(b, j, rcx, rcy, rcz);
             const R W = drag_weight(P, q, om);
-            fx = sub_rn(fx, mul_rn(rcx, W));
-            fy = sub_rn(fy, mul_rn(rcy, W));
-            fz = sub_rn(fz, mul_rn(rcz, W));
+            sums.f[0] = sub_rn(sums.f[0], mul_rn(rcx, W));
+            sums.f[1] = sub_rn(sums.f[1], mul_rn(rcy, W));
+            sums.f[2] = sub_rn(sums.f[2], mul_rn(rcz, W));
         }
-        fx = add_rn(fx, gx);
-        fy = add_rn(fy, gy);
-        fz = add_rn(fz, gz);
-        tx = add_rn(tx, hx);
-        ty = add_rn(ty, hy);
-        tz = add_rn(tz, hz);
-    }
-    if constexpr (ASYNC) cp_async_wait<0>();   // nothing left in flight into the ring
-    write_fluid_force<R>(b, I, gi, fx, fy, fz, tx, ty, tz, P.lev);
-}
-
-// The direct pass with only the list index and the partner's position
-// fetched ahead (its other records are loaded after the r < h decision):
-// fewer registers, so more warps per SM hide the loads instead (force mode
-// 5; the same terms in the same order, so the same bits as force_fluid_slot).
-// ONLY: 0 every path; 1 only the second evaluation that reads the cached
-// normals (returns at once otherwise); 2 only the paths that draw them
-template <class R, int MINB, int DEPTH = 0, int ONLY = 0>
-__global__ void __launch_bounds__(LEAN_BLOCK, MINB) k_force_fluid_lean(Bufs b, int velver)
-{
-    LeanRing<DEPTH ? DEPTH : 1> *ring = nullptr;
-    if constexpr (DEPTH > 0) {
-        __shared__ LeanRing<DEPTH ? DEPTH : 1> ring_s;
-        ring = &ring_s;
-    }
-    const uint32_t step = (uint32_t)(*b.step);
-    const bool fill = b.use_cache && velver == 1;
-    const bool reuse = b.use_cache && velver == 2 && *b.cache_epoch == *b.list_epoch &&
-                       *b.cache_step == *b.step;
-    __syncthreads();
-    if (fill && blockIdx.x == 0 && threadIdx.x == 0) {
-        *b.cache_epoch = *b.list_epoch;
-        *b.cache_step = *b.step;
-    }
-    if (ONLY == 1 && !reuse) return;
-    if (ONLY == 2 && reuse) return;
-    if (ONLY != 2 && reuse) {
-        for (long long base = next_warp_slots(b); base < b.N; base = next_warp_slots(b))
-            force_fluid_slot_lean<R, true, DEPTH>(b, base + (threadIdx.x & 31), step, false, ring);
-    } else if (ONLY != 1) {
-        for (long long base = next_warp_slots(b); base < b.N; base = next_warp_slots(b))
-            force_fluid_slot_lean<R, false, DEPTH>(b, base + (threadIdx.x & 31), step, fill, ring);
+        sums.add(gx, gy, gz, hx, hy, hz);
     }
 }
 
-// ONLY as in k_force_fluid_lean: 0 every path, 1 only the pass reading the
-// cached normals, 2 only the drawing paths
+// ONLY: 0 every path; 1 only the particles whose normals are cached (second
+// evaluation); 2 only those whose normals are drawn
 template <class R, int ONLY = 0>
-__global__ void __launch_bounds__(256) k_force_fluid(Bufs b, int velver)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_force_fluid(Bufs b, int velver, int groups)
 {
-    const uint32_t step = (uint32_t)(*b.step);
-    const bool fill = b.use_cache && velver == 1;
-    const bool reuse = b.use_cache && velver == 2 && *b.cache_epoch == *b.list_epoch &&
-                       *b.cache_step == *b.step;
-    // every warp reads the epochs before the first one is written below
-    __syncthreads();
-    if (fill && blockIdx.x == 0 && threadIdx.x == 0) {
-        *b.cache_epoch = *b.list_epoch;
-        *b.cache_step = *b.step;
-    }
-    // reuse is uniform over the launch
-    if (ONLY == 1 && !reuse) return;
-    if (ONLY == 2 && reuse) return;
-    if (ONLY != 2 && reuse) {
-        for (long long base = next_warp_slots(b); base < b.N; base = next_warp_slots(b))
-            force_fluid_slot<R, true>(b, base + (threadIdx.x & 31), step, false);
-    } else if (ONLY != 1) {
-        for (long long base = next_warp_slots(b); base < b.N; base = next_warp_slots(b))
-            force_fluid_slot<R, false>(b, base + (threadIdx.x & 31), step, fill);
-    }
-}
-
-// ---------------------------------------------------- pair-stream force pass
-// The direct pass (every pair from both sides) reorganised for the SIMT
-// lanes: a warp owns 32 consecutive slots; phase A walks the 32 lists in
-// step (the exact r < h decision, cheap) and compacts the surviving pairs
-// into a ring in shared memory with ballots; phase B evaluates them 32 at a
-// time -- Philox, Box-Muller and the SDPD pair of Eqs. FijC-FijT, or the
-// fluid-sphere pair with the drag reaction -- with every lane busy whatever
-// the spread of list lengths and of pairs beyond h; phase C hands each
-// result back to the lane that owns the particle, which adds its pairs in
-// list order.  The particle's own records are staged in shared memory for
-// phase B.  The terms and their order are those of force_fluid_slot, so the
-// forces equal the direct pass bit for bit.
-template <class R> struct StreamSmem {
-    using T4 = typename Vec<R>::T4;
-    T4 qr[64];            // queued pairs: r_ij (x, y, z) and r^2
-    T4 hB[32], hC[32], hD[32];   // records of the warp's own particles
-    int2 qm[64];          // partner slot; entry k << 8 | owner lane << 1 | sphere partner
-    int hinst[32];        // instance of each own particle
-    R res[32 * 9];        // per batch position: f part (3), e x o (3), drag reaction (3)
-};
-
-template <class R, bool REUSE>
-__device__ __forceinline__ void force_stream_group(const Bufs &b, StreamSmem<R> &S, long long base, uint32_t step,
-                                                   bool fill)
-{
-    using T4 = typename Vec<R>::T4;
-    using T2 = typename Vec2<R>::T2;
-    const unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const unsigned below = (1u << lane) - 1u;
-    const long long s = base + lane;
-    const long long Np = b.Npad;
-    const T4 *__restrict__ A = Mir<R>::A(b);
-    const T4 *__restrict__ Bm = Mir<R>::B(b);
-    const T4 *__restrict__ Cm = Mir<R>::C(b);
-    const T4 *__restrict__ Dm = Mir<R>::D(b);
-    T4 *__restrict__ zA = (T4 *)b.zdA;
-    T2 *__restrict__ zB = (T2 *)b.zdB;
-    const bool mine = s < b.N && b.stype[s] == T_FLUID;
-    int gi = 0, ii = 0, n = 0;
-    T4 Ai;
-    if (mine) {
-        gi = b.perm[s];
-        ii = b.pinst[gi];
-        n = b.ncnt[s];
-        Ai = A[s];
-        S.hB[lane] = Bm[s];
-        S.hC[lane] = Cm[s];
-        S.hD[lane] = Dm[s];
-    }
-    S.hinst[lane] = ii;
-    const Inst &I = b.inst[ii];
-    const Geo<R> geo(I);
-    PairK<R> P(I, step);        // constants of the instance of the pair in hand
-    int pinst = ii;
-    const bool own_fill = fill && P.noise;
-    const R own_lev = P.lev;
-    R fx = 0, fy = 0, fz = 0, tx = 0, ty = 0, tz = 0;
-    uint64_t mask = 0;          // ring positions holding this lane's pairs
-    unsigned head = 0, tail = 0;
-    __syncwarp();
-
-    // phase B + C on the ring positions [h0, h0 + cnt) (h0 a multiple of 32)
-    auto batch = [&](unsigned h0, int cnt) {
-        R g[9];
-#pragma unroll
-        for (int c = 0; c < 9; ++c) g[c] = R(0);
-        if (lane < cnt) {
-            const unsigned p = (h0 + lane) & 63u;
-            const T4 rq = S.qr[p];
-            const int2 m = S.qm[p];
-            const int j = m.x, k = m.y >> 8, il = (m.y >> 1) & 31;
-            const bool rg = m.y & 1;
-            const int pi = S.hinst[il];
-            if (pi != pinst) {
-                P = PairK<R>(b.inst[pi], step);
-                pinst = pi;
-            }
-            const T4 Bi = S.hB[il], Ci = S.hC[il], Di = S.hD[il];
-            const T4 Bj = Bm[j], Cj = Cm[j], Dj = Dm[j];
-            const long long at = (long long)k * Np + base + il;
-            Z6<R> z;
-            int zmode = 0;
-            if (REUSE && P.noise && !rg) {
-                const T4 za = zA[at];
-                const T2 zb = zB[at];
-                if (!isnan(za.x)) {
-                    z.z0 = za.x; z.z1 = za.y; z.z2 = za.z; z.z3 = za.w; z.z4 = zb.x; z.z5 = zb.y;
-                    zmode = 1;
-                }
-            }
-            R ox, oy, oz, ce, ex, ey, ez, q, om;
-            sdpd_pair<R>(P, rq.x, rq.y, rq.z, rq.w, Bi, Ci, Di, Bj, Cj, Dj, !rg, zmode, z, ox, oy, oz, ce, ex, ey,
-                         ez, q, om);
-            if (!REUSE && fill && P.noise && !rg) {
-                T4 zw;
-                zw.x = z.z0; zw.y = z.z1; zw.z = z.z2; zw.w = z.z3;
-                T2 zv;
-                zv.x = z.z4; zv.y = z.z5;
-                zA[at] = zw;
-                zB[at] = zv;
-            }
-            pair_fh(ox, oy, oz, ce, ex, ey, ez, g[0], g[1], g[2], g[3], g[4], g[5]);
-            if (rg) {
-                R rcx, rcy, rcz;
-                rxn_of(b, j, rcx, rcy, rcz);
-                const R W = drag_weight(P, q, om);
-                g[6] = mul_rn(rcx, W);
-                g[7] = mul_rn(rcy, W);
-                g[8] = mul_rn(rcz, W);
-            }
-#pragma unroll
-            for (int c = 0; c < 9; ++c) S.res[lane * 9 + c] = g[c];
+    const CacheUse u(b, velver);
+    if ((ONLY == 1 && !u.maybe) || (ONLY == 2 && u.all)) return;   // uniform over the launch
+    const int lane = threadIdx.x & 31, sub = lane % LPP;
+    const long long base = pass_base(groups);
+    // the particles of this launch: fluid, their normals cached or not
+    SlotHead mine(b, base + lane, lane < groups * GROUP);
+    const bool cached = mine.type == T_FLUID && u.reuse(b, mine.inst);
+    if (mine.type != T_FLUID || (ONLY == 1 && !cached) || (ONLY == 2 && cached)) mine.n = -1;
+    SlotHead h = mine.of_group(0);
+    ListHead hd(b.nbr, base + lane / LPP, b.rows, 0, h.n, sub);
+    ForceSums<R> sums;
+    for (int g = 0; g < groups; ++g) {
+        const long long s = base + g * GROUP + lane / LPP;
+        SlotHead hn;
+        ListHead hdn;
+        if (g + 1 < groups) {
+            hn = mine.of_group(g + 1);
+            hdn = ListHead(b.nbr, s + GROUP, b.rows, 0, hn.n, sub);
+            prefetch_lists(b, base + (g + 1) * GROUP, hn.n);
         }
-        __syncwarp();
-        // phase C: this lane's pairs of the batch, in ring (= list) order
-        const unsigned off = h0 & 63u;
-        uint32_t mm = (uint32_t)(mask >> off) & (cnt == 32 ? FULL : ((1u << cnt) - 1u));
-        mask &= ~((uint64_t)mm << off);
-        while (mm) {
-            const int q = __ffs(mm) - 1;
-            mm &= mm - 1;
-            const R *rr = S.res + q * 9;
-            // a zero drag-reaction term (non-sphere partner) leaves f unchanged exactly
-            fx = sub_rn(fx, rr[6]);
-            fy = sub_rn(fy, rr[7]);
-            fz = sub_rn(fz, rr[8]);
-            fx = add_rn(fx, rr[0]);
-            fy = add_rn(fy, rr[1]);
-            fz = add_rn(fz, rr[2]);
-            tx = add_rn(tx, rr[3]);
-            ty = add_rn(ty, rr[4]);
-            tz = add_rn(tz, rr[5]);
+        if constexpr (ONLY == 0) {
+            if (u.reuse(b, h.inst)) force_fluid_entries<R, true>(b, s, h, hd, sub, u.step, false, sums);
+            else force_fluid_entries<R, false>(b, s, h, hd, sub, u.step, u.fill, sums);
+        } else {
+            force_fluid_entries<R, ONLY == 1>(b, s, h, hd, sub, u.step, ONLY == 1 ? false : u.fill, sums);
         }
-        __syncwarp();
-    };
-
-    // phase A: the lists in step, the next entry prefetched
-    const int kmax = __reduce_max_sync(FULL, n);
-    int jn = n > 0 ? __ldg(b.nbr + s) : 0;
-    int jnn = n > 1 ? __ldg(b.nbr + Np + s) : 0;
-    T4 An;
-    if (n > 0) An = A[jn];
-    for (int k = 0; k < kmax; ++k) {
-        bool want = false, rig = false;
-        int j = 0;
-        R rx = 0, ry = 0, rz = 0, r2 = 0;
-        if (k < n) {
-            j = jn;
-            const T4 Aj = An;
-            if (k + 1 < n) {
-                jn = jnn;
-                An = A[jn];
-                if (k + 2 < n) jnn = __ldg(b.nbr + (long long)(k + 2) * Np + s);
-            }
-            rig = mir_type(Aj) == T_RIGID;
-            want = Rel<R>::get(b, I, geo, Ai, Aj, gi, j, rx, ry, rz, r2);
-            if (!want && !REUSE && own_fill && !rig) {
-                T4 nm;
-                nm.x = R(NAN); nm.y = R(0); nm.z = R(0); nm.w = R(0);
-                zA[(long long)k * Np + s] = nm;
-            }
-        }
-        const unsigned bal = __ballot_sync(FULL, want);
-        if (want) {
-            const unsigned pos = (tail + __popc(bal & below)) & 63u;
-            T4 rq;
-            rq.x = rx; rq.y = ry; rq.z = rz; rq.w = r2;
-            S.qr[pos] = rq;
-            S.qm[pos] = make_int2(j, (k << 8) | (lane << 1) | (rig ? 1 : 0));
-            mask |= 1ull << pos;
-        }
-        tail += __popc(bal);
-        if (tail - head >= 32u) {
-            __syncwarp();
-            batch(head, 32);
-            head += 32;
-        }
+        sums.close_group(g);
+        h = hn;
+        hd = hdn;
     }
-    if (tail != head) {   // fewer than 32 left
-        __syncwarp();
-        batch(head, (int)(tail - head));
-    }
-    if (mine) write_fluid_force<R>(b, I, gi, fx, fy, fz, tx, ty, tz, own_lev);
-    __syncwarp();   // the smem of this group is reused by the next one
-}
-
-// MINB: resident 256-thread blocks per SM the registers are capped for (2:
-// up to 128 registers, 16 warps; 3: 80 registers, 24 warps, a few spilled)
-template <class R, int MINB>
-__global__ void __launch_bounds__(256, MINB) k_force_stream(Bufs b, int velver)
-{
-    extern __shared__ __align__(32) unsigned char stream_smem[];
-    StreamSmem<R> &S = reinterpret_cast<StreamSmem<R> *>(stream_smem)[threadIdx.x >> 5];
-    const uint32_t step = (uint32_t)(*b.step);
-    const bool fill = b.use_cache && velver == 1;
-    const bool reuse = b.use_cache && velver == 2 && *b.cache_epoch == *b.list_epoch &&
-                       *b.cache_step == *b.step;
-    // every warp reads the epochs before the first one is written below
-    __syncthreads();
-    if (fill && blockIdx.x == 0 && threadIdx.x == 0) {
-        *b.cache_epoch = *b.list_epoch;
-        *b.cache_step = *b.step;
-    }
-    if (reuse) {
-        for (long long base = next_warp_slots(b); base < b.N; base = next_warp_slots(b))
-            force_stream_group<R, true>(b, S, base, step, false);
-    } else {
-        for (long long base = next_warp_slots(b); base < b.N; base = next_warp_slots(b))
-            force_stream_group<R, false>(b, S, base, step, fill);
-    }
-}
-
-// The direct pass with TPP lanes per particle (TPP = 2 or 4): the lanes of a
-// particle take the entries sub, sub + TPP, ... of its list (sub = lane %
-// TPP), each summing its share in list order, and a butterfly of shuffles
-// adds the TPP partial sums in a fixed order; the first lane writes.  Small
-// workloads so fill TPP times as many warps.
-template <class R, bool REUSE, int TPP>
-__device__ __forceinline__ void force_fluid_slot_tpp(const Bufs &b, long long s, int sub, uint32_t step, bool fill)
-{
-    using T4 = typename Vec<R>::T4;
-    using T2 = typename Vec2<R>::T2;
-    const bool active = s < b.N && b.stype[s] == T_FLUID;
-    R fx = 0, fy = 0, fz = 0, tx = 0, ty = 0, tz = 0;
-    int gi = 0;
-    const Inst *Ip = b.inst;
-    R lev = 0;
-    if (active) {
-        gi = b.perm[s];
-        const Inst &I = b.inst[b.pinst[gi]];
-        Ip = &I;
-        const Geo<R> geo(I);
-        const PairK<R> P(I, step);
-        lev = P.lev;
-        const bool fl = fill && P.noise;
-        const T4 *__restrict__ A = Mir<R>::A(b);
-        const T4 *__restrict__ Bm = Mir<R>::B(b);
-        const T4 *__restrict__ Cm = Mir<R>::C(b);
-        const T4 *__restrict__ Dm = Mir<R>::D(b);
-        T4 *__restrict__ zA = (T4 *)b.zdA;
-        T2 *__restrict__ zB = (T2 *)b.zdB;
-        const int *__restrict__ nb = b.nbr + s;
-        const T4 Ai = A[s], Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
-        const int n = b.ncnt[s];
-        const long long Np = b.Npad;
-        int jn = sub < n ? ld_stream(nb + (long long)sub * Np) : 0;
-        int jnn = sub + TPP < n ? ld_stream(nb + (long long)(sub + TPP) * Np) : 0;
-        T4 An = A[jn];
-        T4 zan;
-        T2 zbn;
-        if (REUSE && P.noise && sub < n) {
-            zan = ld_stream(zA + (long long)sub * Np + s);
-            zbn = ld_stream(zB + (long long)sub * Np + s);
-        }
-        for (int k = sub; k < n; k += TPP) {
-            const int j = jn;
-            const T4 Aj = An;
-            T4 za;
-            T2 zb;
-            if (REUSE) { za = zan; zb = zbn; }
-            if (k + TPP < n) {
-                jn = jnn;
-                An = A[jn];
-                if (REUSE && P.noise) {
-                    zan = ld_stream(zA + (long long)(k + TPP) * Np + s);
-                    zbn = ld_stream(zB + (long long)(k + TPP) * Np + s);
-                }
-                if (k + 2 * TPP < n) jnn = ld_stream(nb + (long long)(k + 2 * TPP) * Np);
-            }
-            const bool rig = mir_type(Aj) == T_RIGID;
-            const long long at = (long long)k * Np + s;
-            R rx, ry, rz, r2;
-            if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, j, rx, ry, rz, r2)) {
-                if (!REUSE && fl && !rig) {
-                    T4 nm;
-                    nm.x = R(NAN); nm.y = R(0); nm.z = R(0); nm.w = R(0);
-                    st_stream(zA + at, nm);
-                }
-                continue;
-            }
-            const T4 Bj = Bm[j], Cj = Cm[j], Dj = Dm[j];
-            R ox, oy, oz, ce, ex, ey, ez, q, om;
-            Z6<R> z;
-            int zmode = 0;
-            if (REUSE && P.noise && !rig && !isnan(za.x)) {
-                z.z0 = za.x; z.z1 = za.y; z.z2 = za.z; z.z3 = za.w; z.z4 = zb.x; z.z5 = zb.y;
-                zmode = 1;
-            }
-            sdpd_pair<R>(P, rx, ry, rz, r2, Bi, Ci, Di, Bj, Cj, Dj, !rig, zmode, z, ox, oy, oz, ce, ex, ey, ez,
-                         q, om);
-            if (!REUSE && fl && !rig) {
-                T4 zw;
-                zw.x = z.z0; zw.y = z.z1; zw.z = z.z2; zw.w = z.z3;
-                T2 zv;
-                zv.x = z.z4; zv.y = z.z5;
-                st_stream(zA + at, zw);
-                st_stream(zB + at, zv);
-            }
-            R gx, gy, gz, hx, hy, hz;
-            pair_fh(ox, oy, oz, ce, ex, ey, ez, gx, gy, gz, hx, hy, hz);
-            if (rig) {
-                R rcx, rcy, rcz;
-                rxn_of(b, j, rcx, rcy, rcz);
-                const R W = drag_weight(P, q, om);
-                fx = sub_rn(fx, mul_rn(rcx, W));
-                fy = sub_rn(fy, mul_rn(rcy, W));
-                fz = sub_rn(fz, mul_rn(rcz, W));
-            }
-            fx = add_rn(fx, gx);
-            fy = add_rn(fy, gy);
-            fz = add_rn(fz, gz);
-            tx = add_rn(tx, hx);
-            ty = add_rn(ty, hy);
-            tz = add_rn(tz, hz);
-        }
-    }
-    // the TPP lanes of the particle are consecutive: butterfly over them
-#pragma unroll
-    for (int o = 1; o < TPP; o <<= 1) {
-        fx = add_rn(fx, __shfl_xor_sync(0xffffffffu, fx, o));
-        fy = add_rn(fy, __shfl_xor_sync(0xffffffffu, fy, o));
-        fz = add_rn(fz, __shfl_xor_sync(0xffffffffu, fz, o));
-        tx = add_rn(tx, __shfl_xor_sync(0xffffffffu, tx, o));
-        ty = add_rn(ty, __shfl_xor_sync(0xffffffffu, ty, o));
-        tz = add_rn(tz, __shfl_xor_sync(0xffffffffu, tz, o));
-    }
-    if (active && sub == 0) write_fluid_force<R>(b, *Ip, gi, fx, fy, fz, tx, ty, tz, lev);
-}
-
-template <class R, int TPP>
-__global__ void __launch_bounds__(256) k_force_fluid_tpp(Bufs b, int velver)
-{
-    const uint32_t step = (uint32_t)(*b.step);
-    const bool fill = b.use_cache && velver == 1;
-    const bool reuse = b.use_cache && velver == 2 && *b.cache_epoch == *b.list_epoch &&
-                       *b.cache_step == *b.step;
-    __syncthreads();
-    if (fill && blockIdx.x == 0 && threadIdx.x == 0) {
-        *b.cache_epoch = *b.list_epoch;
-        *b.cache_step = *b.step;
-    }
-    const int lane = threadIdx.x & 31;
-    for (;;) {
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(b.work, (unsigned long long)(32 / TPP));
-        base = __shfl_sync(0xffffffffu, base, 0);
-        if ((long long)base >= b.N) break;
-        const long long s = (long long)base + lane / TPP;
-        if (reuse) force_fluid_slot_tpp<R, true, TPP>(b, s, lane % TPP, step, false);
-        else force_fluid_slot_tpp<R, false, TPP>(b, s, lane % TPP, step, fill);
-    }
+    if (mine.n < 0) return;
+    const Inst &I = b.inst[mine.inst];
+    write_fluid_force<R>(b, I, mine.gi, sums.keep[0], sums.keep[1], sums.keep[2], sums.keep[3], sums.keep[4],
+                         sums.keep[5], K<R>::lever(I));
 }
 
 // Newton-3 force pass, phase 1: every fluid or wall particle evaluates the
@@ -1595,70 +1318,73 @@ __global__ void __launch_bounds__(256) k_force_fluid_tpp(Bufs b, int velver)
 // it keeps {o, ce} in its own column and the partner rebuilds f and e x o.
 // Both hand the partner the same bits.
 template <class R, bool REUSE, bool PUSH>
-__device__ __forceinline__ void force_half_slot(const Bufs &b, long long s, uint32_t step, bool fill)
+__device__ __forceinline__ void force_half_entries(const Bufs &b, long long s, const SlotHead &h, int sub,
+                                                   uint32_t step, bool fill, ForceSums<R> &sums)
 {
     using T4 = typename Vec<R>::T4;
+    using TA = typename Mir<R>::TA;
     using T2 = typename Vec2<R>::T2;
-    if (s >= b.N) return;
-    const int ti = b.stype[s];
-    if (ti == T_RIGID) return;
-    const int gi = b.perm[s];
-    const Inst &I = b.inst[b.pinst[gi]];
+    const int ti = h.type, gi = h.gi;
+    const Inst &I = b.inst[h.inst];
     const Geo<R> geo(I);
     const PairK<R> P(I, step);
-    const T4 *__restrict__ A = Mir<R>::A(b);
+    const TA *__restrict__ A = Mir<R>::A(b);
     const T4 *__restrict__ Bm = Mir<R>::B(b);
     const T4 *__restrict__ Cm = Mir<R>::C(b);
     const T4 *__restrict__ Dm = Mir<R>::D(b);
     T4 *__restrict__ resA = (T4 *)b.resA;
     T2 *__restrict__ resB = (T2 *)b.resB;
-    T4 *__restrict__ zA = (T4 *)b.zA;
-    T2 *__restrict__ zB = (T2 *)b.zB;
-    const int *__restrict__ nb = b.nbr + s;
-    const uint16_t *__restrict__ rv = b.rev + s;
-    const T4 Ai = A[s], Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
+    const int last = h.nf;  // the owned prefix of the list
+    int k = sub;
+    if (k >= last) return;
+    const size_t first = entry_at(sub, s, b.rows);
+    size_t at = entry_at(sub, s, b.rows_own);   // own column: normals cache, split results
+    T4 *__restrict__ zA = (T4 *)b.zA + at;
+    T2 *__restrict__ zB = (T2 *)b.zB + at;
+    const int *__restrict__ nb = b.nbr + first;
+    const uint16_t *__restrict__ rv = b.rev + first;
+    const TA Ai = A[s];
+    const T4 Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
     const bool fi = (ti == T_FLUID);
-    R fx = 0, fy = 0, fz = 0, tx = 0, ty = 0, tz = 0;
-    const int last = b.nfirst[s];  // the owned prefix of the list
-    const long long Np = b.Npad;
     const bool noise = P.noise;
-    int jn = 0 < last ? __ldg(nb) : 0;
-    int jnn = 1 < last ? __ldg(nb + Np) : 0;
-    T4 An = A[jn], Bn = Bm[jn], Cn = Cm[jn], Dn = Dm[jn];
+    int jn = __ldg(nb);
+    int jnn = k + LPP < last ? __ldg(nb + ROW) : 0;
+    TA An = A[jn];
+    T4 Bn = Bm[jn], Cn = Cm[jn], Dn = Dm[jn];
     T4 zan;
     T2 zbn;
-    if (REUSE && noise && last > 0) { zan = zA[s]; zbn = zB[s]; }
-    for (int k = 0; k < last; ++k) {
+    if (REUSE && noise) { zan = *zA; zbn = *zB; }
+    for (; k < last; k += LPP, nb += ROW, rv += ROW, zA += ROW, zB += ROW, at += ROW) {
         const int j = jn;
-        const T4 Aj = An, Bj = Bn, Cj = Cn, Dj = Dn;
+        const TA Aj = An;
+        const T4 Bj = Bn, Cj = Cn, Dj = Dn;
         T4 za;
         T2 zb;
         if (REUSE) { za = zan; zb = zbn; }
-        if (k + 1 < last) {
+        if (k + LPP < last) {
             jn = jnn;
             An = A[jn]; Bn = Bm[jn]; Cn = Cm[jn]; Dn = Dm[jn];
             if (REUSE && noise) {
-                zan = zA[(long long)(k + 1) * Np + s];
-                zbn = zB[(long long)(k + 1) * Np + s];
+                zan = zA[ROW];
+                zbn = zB[ROW];
             }
-            if (k + 2 < last) jnn = __ldg(nb + (long long)(k + 2) * Np);
+            if (k + 2 * LPP < last) jnn = __ldg(nb + 2 * ROW);
         }
         const int tj = mir_type(Aj);
         if (tj == T_RIGID) {
-            if (fi) fluid_rigid_pair<R>(b, I, geo, P, gi, Ai, Bi, Ci, Di, j, Aj, Bj, Cj, Dj, fx, fy, fz, tx,
-                                        ty, tz);
+            if (fi) fluid_rigid_pair<R>(b, I, geo, P, gi, Ai, Bi, Ci, Di, j, Aj, Bj, Cj, Dj, sums.f[0], sums.f[1],
+                                        sums.f[2], sums.f[3], sums.f[4], sums.f[5]);
             continue;
         }
         if (!fi && tj != T_FLUID) continue;
-        const long long at = (long long)k * Np + s;   // own column: normals cache
         // FP64 results go to the partner's column, at the row of its entry
         // for this pair (from k_rev); split results stay in the own column
-        long long pt = at;
+        size_t pt = at;
         bool put = true;
         if constexpr (PUSH) {
-            const int row = __ldg(rv + (long long)k * Np);
-            put = row < b.capown;   // false only after a list error (flagged)
-            pt = (long long)row * Np + j;
+            const int prow = __ldg(rv);
+            put = prow < b.capown;   // false only after a list error (flagged)
+            pt = entry_at(prow, j, b.rows_own);
         }
         R rx, ry, rz, r2;
         if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, j, rx, ry, rz, r2)) {
@@ -1666,7 +1392,7 @@ __device__ __forceinline__ void force_half_slot(const Bufs &b, long long s, uint
             T4 nm;
             nm.x = R(NAN); nm.y = R(0); nm.z = R(0); nm.w = R(0);
             if (put) resA[pt] = nm;
-            if (!REUSE && fill) zA[at] = nm;
+            if (!REUSE && fill) *zA = nm;
             continue;
         }
         Z6<R> z;
@@ -1684,8 +1410,8 @@ __device__ __forceinline__ void force_half_slot(const Bufs &b, long long s, uint
             zw.x = z.z0; zw.y = z.z1; zw.z = z.z2; zw.w = z.z3;
             T2 zv;
             zv.x = z.z4; zv.y = z.z5;
-            zA[at] = zw;
-            zB[at] = zv;
+            *zA = zw;
+            *zB = zv;
         }
         R gx, gy, gz, hx, hy, hz;
         pair_fh(ox, oy, oz, ce, ex, ey, ez, gx, gy, gz, hx, hy, hz);
@@ -1700,94 +1426,87 @@ __device__ __forceinline__ void force_half_slot(const Bufs &b, long long s, uint
             if (put) resB[pt] = rb;
         }
         if (put) resA[pt] = ra;
-        fx += gx; fy += gy; fz += gz;
-        tx += hx; ty += hy; tz += hz;
-    }
-    if (fi) {
-        T4 oa;
-        oa.x = fx; oa.y = fy; oa.z = fz; oa.w = tx;
-        T2 ob;
-        ob.x = ty; ob.y = tz;
-        ((T4 *)b.ownA)[s] = oa;
-        ((T2 *)b.ownB)[s] = ob;
+        sums.add(gx, gy, gz, hx, hy, hz);
     }
 }
 
 // (FP32: at most 128 registers, so four 128-thread blocks fit on an SM)
 template <class R, bool PUSH>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_force_half(Bufs b, int velver)
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_force_half(Bufs b, int velver, int groups)
 {
-    const uint32_t step = (uint32_t)(*b.step);
-    const bool fill = b.use_cache && velver == 1;
-    const bool reuse = b.use_cache && velver == 2 && *b.cache_epoch == *b.list_epoch &&
-                       *b.cache_step == *b.step;
-    // every warp reads the epochs before the first one is written below
-    __syncthreads();
-    if (fill && blockIdx.x == 0 && threadIdx.x == 0) {
-        *b.cache_epoch = *b.list_epoch;
-        *b.cache_step = *b.step;
+    using T4 = typename Vec<R>::T4;
+    using TA = typename Mir<R>::TA;
+    using T2 = typename Vec2<R>::T2;
+    const CacheUse u(b, velver);
+    const int lane = threadIdx.x & 31;
+    const long long base = pass_base(groups);
+    const SlotHead mine(b, base + lane, lane < groups * GROUP);
+    ForceSums<R> sums;
+    for (int g = 0; g < groups; ++g) {
+        const long long s = base + g * GROUP + lane / LPP;
+        const SlotHead h = mine.of_group(g);
+        if (h.n >= 0 && h.type != T_RIGID) {
+            if (u.reuse(b, h.inst)) force_half_entries<R, true, PUSH>(b, s, h, lane % LPP, u.step, false, sums);
+            else force_half_entries<R, false, PUSH>(b, s, h, lane % LPP, u.step, u.fill, sums);
+        }
+        sums.close_group(g);
     }
-    // reuse is uniform over the launch
-    if (reuse) {
-        for (long long base = next_warp_slots(b); base < b.N; base = next_warp_slots(b))
-            force_half_slot<R, true, PUSH>(b, base + (threadIdx.x & 31), step, false);
-    } else {
-        for (long long base = next_warp_slots(b); base < b.N; base = next_warp_slots(b))
-            force_half_slot<R, false, PUSH>(b, base + (threadIdx.x & 31), step, fill);
-    }
+    const long long s = base + lane;
+    if (mine.n < 0 || mine.type != T_FLUID) return;
+    T4 oa;
+    oa.x = sums.keep[0]; oa.y = sums.keep[1]; oa.z = sums.keep[2]; oa.w = sums.keep[3];
+    T2 ob;
+    ob.x = sums.keep[4]; ob.y = sums.keep[5];
+    ((T4 *)b.ownA)[s] = oa;
+    ((T2 *)b.ownB)[s] = ob;
 }
 
 // Newton-3 force pass, phase 2 (fluid particles): own sum + the results of
 // the pairs its partners own (force negated, e x o equal; pairs the owner
 // found beyond h carry a NaN marker) + the pairs with rigid neighbours among
 // the non-owned entries, evaluated here (Eqs. FijC, FijD and the drag
-// reaction Eq. F_fpi_DG_reac), all in entry order + external force.  FP64
-// results were written into this particle's column (read coalesced); split
-// results are read from the owner's column through the reverse index.
+// reaction Eq. F_fpi_DG_reac) + external force.  FP64 results were written
+// into this particle's column (read coalesced); split results are read from
+// the owner's column through the reverse index.
 template <class R, bool PUSH>
-__global__ void __launch_bounds__(256) k_force_gather(Bufs b)
+__device__ __forceinline__ void gather_entries(const Bufs &b, long long s, const SlotHead &h, int sub,
+                                               ForceSums<R> &sums)
 {
     using T4 = typename Vec<R>::T4;
+    using TA = typename Mir<R>::TA;
     using T2 = typename Vec2<R>::T2;
-    const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= b.N) return;
-    if (b.stype[s] != T_FLUID) return;
-    const int gi = b.perm[s];
-    const Inst &I = b.inst[b.pinst[gi]];
+    const int gi = h.gi;
+    const Inst &I = b.inst[h.inst];
     const Geo<R> geo(I);
-    const T4 *__restrict__ A = Mir<R>::A(b);
+    const TA *__restrict__ A = Mir<R>::A(b);
     const T4 *__restrict__ resA = (const T4 *)b.resA;
     const T2 *__restrict__ resB = (const T2 *)b.resB;
-    const int *__restrict__ nb = b.nbr + s;
-    const uint16_t *__restrict__ rv = b.rev + s;
-    const T4 Ai = A[s];
-    const T4 oa = ((const T4 *)b.ownA)[s];
-    const T2 ob = ((const T2 *)b.ownB)[s];
-    R fx = oa.x, fy = oa.y, fz = oa.z, tx = oa.w, ty = ob.x, tz = ob.y;
-    const int n = b.ncnt[s], first = b.nfirst[s];
-    const long long Np = b.Npad;
+    const TA Ai = A[s];
+    const int first = h.nf;
     const bool any_rigid = b.nbflag[s] & 1;
     // more non-owned entries than capown only after a list error (flagged)
-    const int nend = min(n, first + b.capown);
-    constexpr int G = 4;
-    for (int k0 = first; k0 < nend; k0 += G) {
-        long long at[G];
+    const int m = min(h.n - first, b.capown);
+    constexpr int G = PUSH ? 4 : 2;
+    for (int k0 = sub; k0 < m; k0 += G * LPP) {
+        size_t at[G];
         int pj[G];
         bool use[G], rig[G];
-        T4 Ap[G];
+        TA Ap[G];
 #pragma unroll
         for (int g = 0; g < G; ++g) {
-            const int k = k0 + g;
-            use[g] = k < nend;
+            const int k = k0 + g * LPP;
+            use[g] = k < m;
             rig[g] = false;
-            const int i = use[g] ? __ldg(nb + (long long)k * Np) : 0;
-            pj[g] = i;
+            pj[g] = 0;
+            at[g] = entry_at(k, s, b.rows_own);
             if (use[g] && (!PUSH || any_rigid)) {
+                const size_t en = entry_at(first + k, s, b.rows);
+                const int i = __ldg(b.nbr + en);
+                pj[g] = i;
                 Ap[g] = A[i];
                 rig[g] = mir_type(Ap[g]) == T_RIGID;
+                if constexpr (!PUSH) at[g] = entry_at(__ldg(b.rev + en), i, b.rows_own);
             }
-            if constexpr (PUSH) at[g] = (long long)(k - first) * Np + s;
-            else at[g] = (long long)(use[g] ? __ldg(rv + (long long)k * Np) : 0) * Np + i;
         }
         T4 ra[G];
         T2 rb[G];
@@ -1802,16 +1521,18 @@ __global__ void __launch_bounds__(256) k_force_gather(Bufs b)
         for (int g = 0; g < G; ++g) {
             if (!use[g]) continue;
             if (rig[g]) {
-                R f[6] = { fx, fy, fz, tx, ty, tz };
+                R f[6];   // a copy: the sums themselves stay in registers
+#pragma unroll
+                for (int c = 0; c < 6; ++c) f[c] = sums.f[c];
                 fluid_rigid_pair_call<R>(b, s, gi, pj[g], f);
-                fx = f[0]; fy = f[1]; fz = f[2]; tx = f[3]; ty = f[4]; tz = f[5];
+#pragma unroll
+                for (int c = 0; c < 6; ++c) sums.f[c] = f[c];
                 continue;
             }
             // NaN marks a pair beyond h (written by the owner)
             if (isnan(ra[g].x)) continue;
             if constexpr (PUSH) {
-                fx -= ra[g].x; fy -= ra[g].y; fz -= ra[g].z;
-                tx += ra[g].w; ty += rb[g].x; tz += rb[g].y;
+                sums.add(-ra[g].x, -ra[g].y, -ra[g].z, ra[g].w, rb[g].x, rb[g].y);
             } else {
                 // e of the owner = -(e seen from here), bitwise
                 R rx, ry, rz;
@@ -1820,12 +1541,36 @@ __global__ void __launch_bounds__(256) k_force_gather(Bufs b)
                 R gx, gy, gz, hx, hy, hz;
                 pair_fh(ra[g].x, ra[g].y, ra[g].z, ra[g].w, -(rx * ir), -(ry * ir), -(rz * ir), gx, gy, gz,
                         hx, hy, hz);
-                fx -= gx; fy -= gy; fz -= gz;
-                tx += hx; ty += hy; tz += hz;
+                sums.add(-gx, -gy, -gz, hx, hy, hz);
             }
         }
     }
-    write_fluid_force<R>(b, I, gi, fx, fy, fz, tx, ty, tz, K<R>::lever(I));
+}
+
+template <class R, bool PUSH>
+__global__ void __launch_bounds__(256) k_force_gather(Bufs b, int groups)
+{
+    using T4 = typename Vec<R>::T4;
+    using TA = typename Mir<R>::TA;
+    using T2 = typename Vec2<R>::T2;
+    const int lane = threadIdx.x & 31;
+    const long long base = pass_base(groups);
+    const SlotHead mine(b, base + lane, lane < groups * GROUP);
+    ForceSums<R> sums;
+    for (int g = 0; g < groups; ++g) {
+        const long long s = base + g * GROUP + lane / LPP;
+        const SlotHead h = mine.of_group(g);
+        if (h.n >= 0 && h.type == T_FLUID) gather_entries<R, PUSH>(b, s, h, lane % LPP, sums);
+        sums.close_group(g);
+    }
+    const long long s = base + lane;
+    if (mine.n < 0 || mine.type != T_FLUID) return;
+    const int gi = mine.gi;
+    const Inst &I = b.inst[mine.inst];
+    const T4 oa = ((const T4 *)b.ownA)[s];
+    const T2 ob = ((const T2 *)b.ownB)[s];
+    write_fluid_force<R>(b, I, gi, oa.x + sums.keep[0], oa.y + sums.keep[1], oa.z + sums.keep[2],
+                         oa.w + sums.keep[3], ob.x + sums.keep[4], ob.y + sums.keep[5], K<R>::lever(I));
 }
 
 // -------------------------------------------------------- rigid force pass
@@ -1979,7 +1724,6 @@ __global__ void __launch_bounds__(RB) k_force_rigid(Bufs b, int velver)
         }
     }
     const bool commit = (velver == 2);
-    const long long Np = b.Npad;
     double acc[15];
 #pragma unroll
     for (int a = 0; a < 15; ++a) acc[a] = 0.0;   // pg, npg, Fdem, Tdem, Flub
@@ -1987,28 +1731,30 @@ __global__ void __launch_bounds__(RB) k_force_rigid(Bufs b, int velver)
     // C + D part of the SDPD pair, the exact r < h decision of Rel), summed
     // per lane in R; DEM and lubrication stay FP64
     using T4 = typename Vec<R>::T4;
+    using TA = typename Mir<R>::TA;
     const PairK<R> P(I, 0u);
     const Geo<R> geo(I);
-    const T4 *__restrict__ A = Mir<R>::A(b);
+    const TA *__restrict__ A = Mir<R>::A(b);
     const T4 *__restrict__ Bm = Mir<R>::B(b);
     const T4 *__restrict__ Cm = Mir<R>::C(b);
     const T4 *__restrict__ Dm = Mir<R>::D(b);
-    const T4 Ai = A[s], Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
+    const TA Ai = A[s];
+    const T4 Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
     const R Rr = (R)Ri;
     R f0 = 0, f1 = 0, f2 = 0, t0 = 0, t1 = 0, t2 = 0;
     const int n = live ? b.ncnt[s] : 0;
     const unsigned below = (1u << lane) - 1u;
     int nr = 0;   // rigid entries collected
     // the entry of the next round is fetched one round ahead
-    uint32_t en = lane < n ? (uint32_t)__ldg(b.nbr + (long long)lane * Np + s) : 0u;
+    uint32_t en = lane < n ? (uint32_t)__ldg(b.nbr + entry_at(lane, s, b.rows)) : 0u;
     for (int kk = 0; kk < n; kk += 32) {
         const int k = kk + lane;
         bool rig = false;
         const uint32_t e = en;
-        if (k + 32 < n) en = (uint32_t)__ldg(b.nbr + (long long)(k + 32) * Np + s);
+        if (k + 32 < n) en = (uint32_t)__ldg(b.nbr + entry_at(k + 32, s, b.rows));
         if (k < n) {
             const int j = (int)(e & ~NB_FAR);
-            const T4 Aj = A[j];
+            const TA Aj = A[j];
             const int tj = mir_type(Aj);
             if (tj == T_FLUID && !(e & NB_FAR)) {
                 // F^C + F^D of the pair (s, j), summed for Eq. F_fpi_PG
@@ -2157,18 +1903,32 @@ __global__ void k_hist_copy(Bufs b)
 // ---------------------------------------------------------------- launchers
 static inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
-// Blocks of a persistent launch: as many as are resident at once (never
-// more than the warps needed to cover N).
-template <class K>
-static unsigned persistent_grid(K kernel, int block, long long N)
+// Groups of GROUP particles a warp of a pair pass takes one after another: as
+// many (at most 8: one particle per lane at the end) as still give every SM
+// 32 warps, so that small systems spread over the chip and large ones pay the
+// closing arithmetic once per 32 particles.
+static int pass_groups(long long N)
 {
-    int dev = 0, nsm = 0, per_sm = 0;
+    int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    const long long need = (N + block - 1) / block;
-    return (unsigned)std::min<long long>(need, (long long)nsm * per_sm);
+    const long long g = N / (GROUP * 32LL * std::max(nsm, 1));
+    return (int)std::min<long long>(8, std::max<long long>(1, g));
+}
+// Blocks of `block` threads that cover N particles at `groups` groups a warp.
+static unsigned pass_blocks(long long N, int block, int groups) { return nblk(N, block / 32 * GROUP * groups); }
+
+template <class R>
+static void launch_density_tail(const Bufs &b, int any_filter, int any_reinit, const int *gate, int groups,
+                                cudaStream_t st)
+{
+    const int bs = b.pair_block;
+    const unsigned nb = pass_blocks(b.N, bs, groups);
+    if (any_reinit) {
+        k_reinit<R><<<nb, bs, 0, st>>>(b, any_filter, gate, groups);
+        k_reinit_copy<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
+    }
+    if (any_filter) k_filter<R><<<nb, bs, 0, st>>>(b, gate, groups);
 }
 
 void launch_density(const Bufs &b, int precision, int dflags, int newton3, const int *gate, cudaStream_t st)
@@ -2177,32 +1937,23 @@ void launch_density(const Bufs &b, int precision, int dflags, int newton3, const
     const int any_filter = dflags & 1, any_reinit = (dflags >> 1) & 1, any_artvis = (dflags >> 2) & 1;
     // the density kernels leave the mirrors to a later pass when one follows
     const int defer = any_filter | any_reinit;
-    if (precision == SDPD_PREC_FP64 && newton3) {
-        cudaMemsetAsync(b.work, 0, sizeof(unsigned long long), st);
-        k_density_half<<<persistent_grid(k_density_half, b.pair_block, b.N), b.pair_block, 0, st>>>(b, gate);
-        k_density_gather<<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, defer, gate);
-        if (any_reinit) {
-            k_reinit<double><<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, any_filter, gate);
-            k_reinit_copy<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
-        }
-        if (any_filter) k_filter<double><<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, gate);
-    } else if (precision == SDPD_PREC_SPLIT) {
-        if (any_artvis) k_density<float, true><<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, defer, gate);
-        else k_density<float, false><<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, defer, gate);
-        if (any_reinit) {
-            k_reinit<float><<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, any_filter, gate);
-            k_reinit_copy<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
-        }
-        if (any_filter) k_filter<float><<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, gate);
-    } else {
-        if (any_artvis) k_density<double, true><<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, defer, gate);
-        else k_density<double, false><<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, defer, gate);
-        if (any_reinit) {
-            k_reinit<double><<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, any_filter, gate);
-            k_reinit_copy<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
-        }
-        if (any_filter) k_filter<double><<<nblk(b.N, b.pair_block), b.pair_block, 0, st>>>(b, gate);
+    const int groups = pass_groups(b.N), bs = b.pair_block;
+    const unsigned nb = pass_blocks(b.N, bs, groups);
+    if (precision == SDPD_PREC_SPLIT) {
+        if (any_artvis) k_density<float, true><<<nb, bs, 0, st>>>(b, defer, gate, groups);
+        else k_density<float, false><<<nb, bs, 0, st>>>(b, defer, gate, groups);
+        launch_density_tail<float>(b, any_filter, any_reinit, gate, groups, st);
+        return;
     }
+    if (newton3) {
+        k_density_half<<<nb, bs, 0, st>>>(b, gate, groups);
+        k_density_gather<<<nb, bs, 0, st>>>(b, defer, gate, groups);
+    } else if (any_artvis) {
+        k_density<double, true><<<nb, bs, 0, st>>>(b, defer, gate, groups);
+    } else {
+        k_density<double, false><<<nb, bs, 0, st>>>(b, defer, gate, groups);
+    }
+    launch_density_tail<double>(b, any_filter, any_reinit, gate, groups, st);
 }
 
 void launch_drag(const Bufs &b, int precision, cudaStream_t st)
@@ -2215,9 +1966,6 @@ void launch_drag(const Bufs &b, int precision, cudaStream_t st)
 }
 
 
-template <class R>
-static size_t stream_smem_bytes(int block) { return (size_t)(block / 32) * sizeof(StreamSmem<R>); }
-
 void init_pair_kernels()
 {
     // the sphere kernel's rigid lists and pooled-pair results at the largest
@@ -2226,99 +1974,34 @@ void init_pair_kernels()
                          (int)rigid_smem_bytes(SDPD_MAX_NEIGHBORS));
     cudaFuncSetAttribute(k_force_rigid<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)rigid_smem_bytes(SDPD_MAX_NEIGHBORS));
-    // the pair-stream kernels' shared memory at the largest block (256)
-    cudaFuncSetAttribute(k_force_stream<float, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)stream_smem_bytes<float>(256));
-    cudaFuncSetAttribute(k_force_stream<float, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)stream_smem_bytes<float>(256));
-    cudaFuncSetAttribute(k_force_stream<double, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)stream_smem_bytes<double>(256));
-}
-
-template <class K>
-static unsigned persistent_grid_smem(K kernel, int block, size_t smem, long long N)
-{
-    int dev = 0, nsm = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess || per_sm < 1)
-        per_sm = 1;
-    const long long need = (N + block - 1) / block;
-    return (unsigned)std::min<long long>(need, (long long)nsm * per_sm);
 }
 
 void launch_forces(const Bufs &b, int precision, int velver, int newton3, cudaStream_t st)
 {
     if (!b.N) return;
-    const int bs = b.pair_block;
-    cudaMemsetAsync(b.work, 0, sizeof(unsigned long long), st);
-    if (newton3 == 2 || newton3 == 3) {
-        if (precision == SDPD_PREC_SPLIT) {
-            const size_t sm = stream_smem_bytes<float>(bs);
-            if (newton3 == 3)
-                k_force_stream<float, 3>
-                    <<<persistent_grid_smem(k_force_stream<float, 3>, bs, sm, b.N), bs, sm, st>>>(b, velver);
-            else
-                k_force_stream<float, 2>
-                    <<<persistent_grid_smem(k_force_stream<float, 2>, bs, sm, b.N), bs, sm, st>>>(b, velver);
-        } else {
-            const size_t sm = stream_smem_bytes<double>(bs);
-            k_force_stream<double, 1>
-                <<<persistent_grid_smem(k_force_stream<double, 1>, bs, sm, b.N), bs, sm, st>>>(b, velver);
-        }
-    } else if (newton3 == 1 || newton3 == 4) {
+    const int bs = b.pair_block, groups = pass_groups(b.N);
+    const unsigned nb = pass_blocks(b.N, bs, groups);
+    if (newton3 == 1 || newton3 == 4) {
         if (precision == SDPD_PREC_SPLIT && newton3 == 4) {
-            k_force_half<float, true><<<persistent_grid(k_force_half<float, true>, bs, b.N), bs, 0, st>>>(b, velver);
-            k_force_gather<float, true><<<nblk(b.N, bs), bs, 0, st>>>(b);
+            k_force_half<float, true><<<nb, bs, 0, st>>>(b, velver, groups);
+            k_force_gather<float, true><<<nb, bs, 0, st>>>(b, groups);
         } else if (precision == SDPD_PREC_SPLIT) {
-            k_force_half<float, false><<<persistent_grid(k_force_half<float, false>, bs, b.N), bs, 0, st>>>(b, velver);
-            k_force_gather<float, false><<<nblk(b.N, bs), bs, 0, st>>>(b);
+            k_force_half<float, false><<<nb, bs, 0, st>>>(b, velver, groups);
+            k_force_gather<float, false><<<nb, bs, 0, st>>>(b, groups);
         } else {
-            k_force_half<double, true><<<persistent_grid(k_force_half<double, true>, bs, b.N), bs, 0, st>>>(b, velver);
-            k_force_gather<double, true><<<nblk(b.N, bs), bs, 0, st>>>(b);
-        }
-    } else if (newton3 == 5) {
-        // registers capped for five 128-thread blocks per SM (20 warps); the
-        // first evaluation (normals drawn) with the partners' records in an
-        // async shared-memory ring, the second (normals read back from the
-        // cache, far less arithmetic per pair) without: measured faster each
-        if (precision == SDPD_PREC_SPLIT && velver == 1)
-            k_force_fluid_lean<float, 5, 2><<<persistent_grid(k_force_fluid_lean<float, 5, 2>, LEAN_BLOCK, b.N),
-                                              LEAN_BLOCK, 0, st>>>(b, velver);
-        else if (precision == SDPD_PREC_SPLIT) {
-            // velver 2: the pass that reads the cached normals, compiled
-            // alone (two partner records per pair, the D record only for a
-            // draw), then the drawing pass for the case where the cache is not
-            // valid; each returns at once when the other one applies
-            k_force_fluid_lean<float, 5, 0, 1>
-                <<<persistent_grid(k_force_fluid_lean<float, 5, 0, 1>, LEAN_BLOCK, b.N), LEAN_BLOCK, 0, st>>>(b, velver);
-            cudaMemsetAsync(b.work, 0, sizeof(unsigned long long), st);
-            k_force_fluid_lean<float, 5, 0, 2>
-                <<<persistent_grid(k_force_fluid_lean<float, 5, 0, 2>, LEAN_BLOCK, b.N), LEAN_BLOCK, 0, st>>>(b, velver);
-        }
-        else
-            k_force_fluid<double><<<persistent_grid(k_force_fluid<double>, bs, b.N), bs, 0, st>>>(b, velver);
-    } else if (b.tpp == 2 || b.tpp == 4) {
-        // the direct pass with several lanes per particle: N x tpp threads
-        const long long nt = b.N * (long long)b.tpp;
-        if (precision == SDPD_PREC_SPLIT) {
-            if (b.tpp == 2) k_force_fluid_tpp<float, 2><<<persistent_grid(k_force_fluid_tpp<float, 2>, bs, nt), bs, 0, st>>>(b, velver);
-            else k_force_fluid_tpp<float, 4><<<persistent_grid(k_force_fluid_tpp<float, 4>, bs, nt), bs, 0, st>>>(b, velver);
-        } else {
-            if (b.tpp == 2) k_force_fluid_tpp<double, 2><<<persistent_grid(k_force_fluid_tpp<double, 2>, bs, nt), bs, 0, st>>>(b, velver);
-            else k_force_fluid_tpp<double, 4><<<persistent_grid(k_force_fluid_tpp<double, 4>, bs, nt), bs, 0, st>>>(b, velver);
+            k_force_half<double, true><<<nb, bs, 0, st>>>(b, velver, groups);
+            k_force_gather<double, true><<<nb, bs, 0, st>>>(b, groups);
         }
     } else if (precision == SDPD_PREC_SPLIT && velver == 2) {
         // the pass reading the cached normals compiled alone (no D records,
-        // no drawing code), then the drawing pass for an invalid cache; each
-        // returns at once when the other one applies
-        k_force_fluid<float, 1><<<persistent_grid(k_force_fluid<float, 1>, bs, b.N), bs, 0, st>>>(b, velver);
-        cudaMemsetAsync(b.work, 0, sizeof(unsigned long long), st);
-        k_force_fluid<float, 2><<<persistent_grid(k_force_fluid<float, 2>, bs, b.N), bs, 0, st>>>(b, velver);
+        // no drawing code), then the drawing pass for the instances whose
+        // lists were rebuilt since
+        k_force_fluid<float, 1><<<nb, bs, 0, st>>>(b, velver, groups);
+        k_force_fluid<float, 2><<<nb, bs, 0, st>>>(b, velver, groups);
     } else if (precision == SDPD_PREC_SPLIT) {
-        k_force_fluid<float><<<persistent_grid(k_force_fluid<float>, bs, b.N), bs, 0, st>>>(b, velver);
+        k_force_fluid<float, 2><<<nb, bs, 0, st>>>(b, velver, groups);
     } else {
-        k_force_fluid<double><<<persistent_grid(k_force_fluid<double>, bs, b.N), bs, 0, st>>>(b, velver);
+        k_force_fluid<double><<<nb, bs, 0, st>>>(b, velver, groups);
     }
     if (b.nrigid) {
         const unsigned g = nblk(b.nrigid, RPB);

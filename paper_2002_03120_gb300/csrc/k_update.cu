@@ -55,6 +55,14 @@ __device__ __forceinline__ bool finite_bits(double x)
     return ((unsigned long long)__double_as_longlong(x) & 0x7FF0000000000000ull) != 0x7FF0000000000000ull;
 }
 
+// A particle has used up half the skin: its instance's lists are rebuilt
+// before the next pair pass.
+__device__ __forceinline__ void request_build(const Bufs &b, int g)
+{
+    b.need_build[0] = 1;
+    b.need_build[1 + b.pinst[g]] = 1;
+}
+
 // Velocity Verlet (Eqs. newton1, newton2): v += dt/2 F/m, w += dt/2 N/I;
 // velver 1 also drifts x += dt v, wraps periodic axes and mirrors particles
 // that crossed a wall plane (normal velocity reversed).  The arithmetic is
@@ -105,23 +113,18 @@ __global__ void k_integrate(Bufs b, int velver)
             if (per && abs_bits(d) > I.hbox_bits[a]) d = (__double_as_longlong(d) > 0) ? __dsub_rn(d, L) : __dadd_rn(d, L);
             dl[a] = d;
         }
-        // keep the mirrors of the unchanged slot order current: cell-relative
-        // coordinates move by the displacement (the build cell stays), the
+        // keep the mirrors of the unchanged slot order current; the
         // displacement since the build decides whether the list still holds
-        double4_32a xl = b.xl64[s], ds = b.dsp[s];
-        xl.x += dl[0]; xl.y += dl[1]; xl.z += dl[2];
+        double4_32a ds = b.dsp[s];
         ds.x += dl[0]; ds.y += dl[1]; ds.z += dl[2];
-        b.xl64[s] = xl;
         b.dsp[s] = ds;
-        float4 a32 = b.A32[s];
-        a32.x = (float)xl.x; a32.y = (float)xl.y; a32.z = (float)xl.z;
-        b.A32[s] = a32;
+        b.A32[s] = make_int4(fixed_coord(x[0], I, 0), fixed_coord(x[1], I, 1), fixed_coord(x[2], I, 2), t);
         if (b.A64) {
             double4_32a a64 = b.A64[s];
             a64.x = x[0]; a64.y = x[1]; a64.z = x[2];
             b.A64[s] = a64;
         }
-        if (fma(ds.z, ds.z, fma(ds.y, ds.y, ds.x * ds.x)) > I.half_skin * I.half_skin) *b.need_build = 1;
+        if (fma(ds.z, ds.z, fma(ds.y, ds.y, ds.x * ds.x)) > I.half_skin * I.half_skin) request_build(b, g);
     }
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
@@ -135,7 +138,7 @@ __global__ void k_integrate(Bufs b, int velver)
 
 // Absorb uploaded state (sdpd_upload_state) into a context whose lists are
 // valid: each particle moves by its displacement (minimum image on periodic
-// axes), the cell-relative mirrors and the displacement since the build move
+// axes), the position mirrors and the displacement since the build move
 // with it, and the velocity mirrors take the uploaded velocities.  A
 // displacement beyond half the skin requests a rebuild (the gated build of
 // the next step), exactly as after a drift; otherwise the lists still hold
@@ -160,20 +163,16 @@ __global__ void k_absorb(Bufs b, const double *__restrict__ xs, int has_x)
             x[a] = xa;
             b.x[3 * g + a] = xa;
         }
-        double4_32a xl = b.xl64[s], ds = b.dsp[s];
-        xl.x += dl[0]; xl.y += dl[1]; xl.z += dl[2];
+        double4_32a ds = b.dsp[s];
         ds.x += dl[0]; ds.y += dl[1]; ds.z += dl[2];
-        b.xl64[s] = xl;
         b.dsp[s] = ds;
-        float4 a32 = b.A32[s];
-        a32.x = (float)xl.x; a32.y = (float)xl.y; a32.z = (float)xl.z;
-        b.A32[s] = a32;
+        b.A32[s] = make_int4(fixed_coord(x[0], I, 0), fixed_coord(x[1], I, 1), fixed_coord(x[2], I, 2), b.type[g]);
         if (b.A64) {
             double4_32a a64 = b.A64[s];
             a64.x = x[0]; a64.y = x[1]; a64.z = x[2];
             b.A64[s] = a64;
         }
-        if (ds.x * ds.x + ds.y * ds.y + ds.z * ds.z > I.half_skin * I.half_skin) *b.need_build = 1;
+        if (ds.x * ds.x + ds.y * ds.y + ds.z * ds.z > I.half_skin * I.half_skin) request_build(b, g);
     }
     const double v[3] = { b.v[3 * g], b.v[3 * g + 1], b.v[3 * g + 2] };
     const double w[3] = { b.w[3 * g], b.w[3 * g + 1], b.w[3 * g + 2] };
@@ -202,13 +201,13 @@ __global__ void k_artvis(Bufs b)
         const double mi = b.m[g];
         const int n = b.ncnt[s];
         const Geo<float> geo(I);
-        const float4 Ai = b.A32[s];
+        const int4 Ai = b.A32[s];
         const float r2hi = I.artvis_r2f_hi;
         for (int k = 0; k < n; ++k) {
-            const uint32_t e = (uint32_t)b.nbr[(long long)k * b.Npad + s];
+            const uint32_t e = (uint32_t)b.nbr[entry_at(k, s, b.rows)];
             if (e & NB_FAR) continue;
-            // float prefilter on the cell-relative mirror; exact test below
-            const float4 Aj = b.A32[e];
+            // float prefilter on the fixed-point mirror; exact test below
+            const int4 Aj = b.A32[e];
             float fx, fy, fz;
             geo.disp(Ai, Aj, fx, fy, fz);
             if (fx * fx + fy * fy + fz * fz > r2hi) continue;
@@ -329,7 +328,7 @@ __global__ void k_count_pairs(Bufs b)
             const int gi = b.perm[s];
             const Inst &I = b.inst[b.pinst[gi]];
             for (int k = 0; k < n; ++k) {
-                const uint32_t e = (uint32_t)b.nbr[(long long)k * b.Npad + s];
+                const uint32_t e = (uint32_t)b.nbr[entry_at(k, s, b.rows)];
                 if (e & NB_FAR) continue;
                 if (!exact_within(b, I, gi, b.perm[e])) continue;
                 const int tj = b.stype[e];
@@ -352,7 +351,7 @@ __global__ void k_mark_pairs(Bufs b, uint8_t *flags)
     const Inst &I = b.inst[b.pinst[gi]];
     const int n = b.ncnt[s];
     for (int k = 0; k < n; ++k) {
-        const uint32_t e = (uint32_t)b.nbr[(long long)k * b.Npad + s];
+        const uint32_t e = (uint32_t)b.nbr[entry_at(k, s, b.rows)];
         flags[(long long)k * b.Npad + s] =
             (!(e & NB_FAR) && exact_within(b, I, gi, b.perm[e & ~NB_FAR])) ? 1 : 0;
     }
