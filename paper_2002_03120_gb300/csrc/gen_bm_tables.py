@@ -2,9 +2,10 @@
 Box-Muller transform of the GPU pair kernels (correctly rounded doubles,
 computed with mpmath at 60 digits).
 
-  LOG_TAB[j]  = { ln(1 + j/128), 1 / (1 + j/128) }             j = 0..127
-  LOG_E[e]    = (e - 24) ln 2                                   e = 0..31
-  SC_TAB[h]   = { sin(pi/2 h/256), cos(pi/2 h/256) }            h = 0..255
+  LOG_TAB[j]  = { -2 ln(1 + j/2048), 1 / (1 + j/2048) }           j = 0..2047
+  LOG_E[e]    = -2 (e - 24) ln 2                                  e = 0..31
+  SC_HI[h]    = { sin(pi/2 h/1024), cos(pi/2 h/1024) }             h = 0..1023
+  SC_LO[l]    = { sin, cos of pi/2 (2 l + 1) / 2^22 }              l = 0..2047
 
 Run:  python gen_bm_tables.py  (in this directory)
 """
@@ -23,20 +24,19 @@ def main():
     lines = ["// Generated by gen_bm_tables.py; do not edit.",
              "// Tables of the table-driven FP64 Box-Muller transform (correctly rounded).",
              "#pragma once", ""]
-    lines.append("static __device__ const double2 BM_LOG_TAB[128] = {")
-    for j in range(128):
-        c = 1 + mpmath.mpf(j) / 128
-        lines.append(f"    {{{d(mpmath.log(c))}, {d(1 / c)}}},")
-    lines.append("};")
-    lines.append("static __device__ const double BM_LOG_E[32] = {")
-    for e in range(32):
-        lines.append(f"    {d((e - 24) * mpmath.log(2))},")
-    lines.append("};")
-    lines.append("static __device__ const double2 BM_SC_TAB[256] = {")
-    for h in range(256):
-        a = mpmath.pi / 2 * h / 256
-        lines.append(f"    {{{d(mpmath.sin(a))}, {d(mpmath.cos(a))}}},")
-    lines.append("};")
+
+    def table(decl, rows):
+        lines.append(decl + " = {")
+        lines.extend("    " + r + "," for r in rows)
+        lines.append("};")
+
+    c = [1 + mpmath.mpf(j) / 2048 for j in range(2048)]
+    table("static __device__ const double2 BM_LOG_TAB[2048]", [f"{{{d(-2 * mpmath.log(x))}, {d(1 / x)}}}" for x in c])
+    table("static __device__ const double BM_LOG_E[32]", [d(-2 * (e - 24) * mpmath.log(2)) for e in range(32)])
+    hi = [mpmath.pi / 2 * h / 1024 for h in range(1024)]
+    lo = [mpmath.pi / 2 * (2 * k + 1) / 2 ** 22 for k in range(2048)]
+    table("static __device__ const double2 BM_SC_HI[1024]", [f"{{{d(mpmath.sin(x))}, {d(mpmath.cos(x))}}}" for x in hi])
+    table("static __device__ const double2 BM_SC_LO[2048]", [f"{{{d(mpmath.sin(x))}, {d(mpmath.cos(x))}}}" for x in lo])
     out = os.path.join(os.path.dirname(os.path.abspath(__file__)), "bm_tables.cuh")
     with open(out, "w") as f:
         f.write("\n".join(lines) + "\n")

@@ -182,10 +182,10 @@ __global__ void k_gather(Bufs b, int precision, const int *gate)
                                (float)b.m[g]);
         b.D32[s].w = __uint_as_float(lg);
     } else {
-        b.A64[s] = make_double4_32a(x0, x1, x2, (double)t);
+        b.A64[s] = make_double4_32a(x0, x1, x2, __longlong_as_double(t));
         b.B64[s] = make_double4_32a(b.v[3 * g], b.v[3 * g + 1], b.v[3 * g + 2], b.R[g]);
         b.C64[s] = make_double4_32a(b.w[3 * g], b.w[3 * g + 1], b.w[3 * g + 2], b.m[g]);
-        b.D64[s].w = (double)lg;
+        b.D64[s].w = __longlong_as_double((long long)lg);
     }
 }
 

@@ -20,6 +20,7 @@
 // from the counter (min gid, max gid, step) or, in the second evaluation of a
 // step, read back from the first one's cache (same counter, same bits).
 #include <algorithm>
+#define BM_TABLES
 #include "common.cuh"
 
 namespace sdpd {
@@ -31,14 +32,14 @@ template <class R> struct Vec2;
 template <> struct Vec2<float> { using T2 = float2; };
 template <> struct Vec2<double> { using T2 = double2; };
 
-// a < b for a, b >= 0: the value compare in FP32, the bit-pattern compare
-// (same result, integer pipe) in FP64
-__device__ __forceinline__ bool lt_nonneg(float a, float b) { return a < b; }
-__device__ __forceinline__ bool lt_nonneg(double a, double b) { return abs_bits(a) < abs_bits(b); }
-
-template <class R> __device__ __forceinline__ R rsqrt_(R x);
-template <> __device__ __forceinline__ float rsqrt_<float>(float x) { return rsqrtf(x); }
-template <> __device__ __forceinline__ double rsqrt_<double>(double x) { return rsqrt(x); }
+// 1 - q of q = r / h, not below 0 (q of a pair within h exceeds 1 by rounding
+// at most; FP64: the sign tested on the high word)
+__device__ __forceinline__ float one_minus(float q) { return q < 1.0f ? 1.0f - q : 0.0f; }
+__device__ __forceinline__ double one_minus(double q)
+{
+    const double om = 1.0 - q;
+    return __double2hiint(om) < 0 ? 0.0 : om;
+}
 
 template <class R> struct Mir;
 template <> struct Mir<float> {
@@ -57,9 +58,9 @@ template <> struct Mir<double> {
 };
 
 __device__ __forceinline__ int mir_type(const int4 &A) { return A.w; }
-__device__ __forceinline__ int mir_type(const double4_32a &A) { return (int)A.w; }
+__device__ __forceinline__ int mir_type(const double4_32a &A) { return __double2loint(A.w); }
 __device__ __forceinline__ uint32_t mir_gid(const float4 &D) { return __float_as_uint(D.w); }
-__device__ __forceinline__ uint32_t mir_gid(const double4_32a &D) { return (uint32_t)D.w; }
+__device__ __forceinline__ uint32_t mir_gid(const double4_32a &D) { return (uint32_t)__double2loint(D.w); }
 // The density terms of a particle for the pair routine.  FP32 records keep
 // p/d^2 in B.w and 1/d in C.w, next to the velocity and the spin, so that a
 // pass reading no gid (the second evaluation, normals from the cache) needs
@@ -69,18 +70,10 @@ __device__ __forceinline__ float mir_pd2(const float4 &B, const float4 &) { retu
 __device__ __forceinline__ double mir_pd2(const double4_32a &, const double4_32a &D) { return D.x; }
 __device__ __forceinline__ float mir_invd(const float4 &C, const float4 &) { return C.w; }
 __device__ __forceinline__ double mir_invd(const double4_32a &, const double4_32a &D) { return D.y; }
-// om / sqrt(d_i d_j); FP32: x rsqrt(x) of x = 1/d_i 1/d_j > 0 (the hardware
-// reciprocal square root, about 2 ulp, the same in every pass)
-__device__ __forceinline__ float mir_rs(float om, const float4 &Ci, const float4 &, const float4 &Cj, const float4 &)
-{
-    const float x = Ci.w * Cj.w;
-    return om * (x * rsqrtf(x));
-}
-__device__ __forceinline__ double mir_rs(double om, const double4_32a &, const double4_32a &Di, const double4_32a &,
-                                         const double4_32a &Dj)
-{
-    return om * Di.z * Dj.z;
-}
+// 1 / sqrt(d); FP32: x rsqrt(x) of x = 1/d > 0 (the hardware reciprocal square
+// root, about 2 ulp, the same in every pass)
+__device__ __forceinline__ float mir_rsd(const float4 &C, const float4 &) { return C.w * rsqrt_ftz(C.w); }
+__device__ __forceinline__ double mir_rsd(const double4_32a &, const double4_32a &D) { return D.z; }
 
 template <class R> struct K;  // kernel constants in precision R
 template <> struct K<float> {
@@ -138,7 +131,7 @@ template <> struct Rel<double> {
     {
         geo.disp(Ai, Aj, rx, ry, rz);
         r2 = __dadd_rn(__dadd_rn(__dmul_rn(rx, rx), __dmul_rn(ry, ry)), __dmul_rn(rz, rz));
-        return abs_bits(r2) < abs_bits(geo.rc2);   // r2 >= 0: the bit order is the value order
+        return lt_pos(r2, geo.rc2);
     }
 };
 
@@ -418,9 +411,11 @@ __device__ __forceinline__ void density_entries(const Bufs &b, const Inst &I, lo
             const int tj = mir_type(Aj);
             close |= (tj == T_FLUID || tj == T_RIGID);
         }
-        // float: correctly rounded sqrt; double: r2 / sqrt via rsqrt (~1 ulp)
-        const R q = (sizeof(R) == 4 ? sqrt(r2) : r2 * rsqrt_<R>(r2)) * irc;
-        const R om = lt_nonneg(q, R(1)) ? R(1) - q : R(0);
+        // float: correctly rounded sqrt
+        R r = 0, ir;
+        if constexpr (sizeof(R) == 4) r = sqrtf(r2);
+        else root_and_inverse(r2, r, ir);
+        const R q = r * irc, om = one_minus(q);
         acc.add(Wc * (R(1) + R(3) * q) * om * om * om);
     });
 }
@@ -529,8 +524,9 @@ __global__ void __launch_bounds__(256) k_density_half(Bufs b, const int *gate, i
                 if (!(e & NB_FAR)) {
                     double rx, ry, rz, r2;
                     if (Rel<double>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) {
-                        const double q = r2 * rsqrt_<double>(r2) * irc;
-                        const double om = lt_nonneg(q, 1.0) ? 1.0 - q : 0.0;
+                        double r, ir;
+                        root_and_inverse(r2, r, ir);
+                        const double q = r * irc, om = one_minus(q);
                         W = Wc * (1.0 + 3.0 * q) * om * om * om;
                         acc = __dadd_rn(acc, W);
                         if (want_close && r2 <= close_r2) {
@@ -538,7 +534,7 @@ __global__ void __launch_bounds__(256) k_density_half(Bufs b, const int *gate, i
                             const bool mob = (tj == T_FLUID || tj == T_RIGID);
                             if (mob && (ti == T_FLUID || ti == T_RIGID)) {
                                 close = true;
-                                W = -W;   // tells the partner
+                                W = flip_sign(W, 0x80000000u);   // tells the partner
                             }
                         }
                     }
@@ -581,8 +577,8 @@ __global__ void __launch_bounds__(256) k_density_gather(Bufs b, int defer, const
             for (int k = sub; k < m; k += LPP) {
                 const double w = *p;
                 p += ROW;
-                close |= w < 0.0;
-                acc = __dadd_rn(acc, fabs(w));
+                close |= __double2hiint(w) < 0;
+                acc = __dadd_rn(acc, __hiloint2double(hi_abs(w), __double2loint(w)));
             }
         }
         keep_group(lanes_sum(acc), g, keep);
@@ -643,8 +639,10 @@ template <> struct TwoSums<double> {
 template <class R>
 __device__ __forceinline__ R shepard_weight(const Inst &I, R r2)
 {
-    const R q = sqrt(r2) * K<R>::inv_rc(I);
-    const R om = lt_nonneg(q, R(1)) ? R(1) - q : R(0);
+    R r = 0, ir;
+    if constexpr (sizeof(R) == 4) r = sqrtf(r2);
+    else root_and_inverse(r2, r, ir);
+    const R q = r * K<R>::inv_rc(I), om = one_minus(q);
     return K<R>::Wc(I) * (R(1) + R(3) * q) * om * om * om;
 }
 
@@ -830,7 +828,9 @@ __global__ void __launch_bounds__(RB) k_drag(Bufs b)
             const double Rj = b.R[b.perm[j]];
             Vsum += 4.0 / 3.0 * PI * Rj * Rj * Rj;
         } else {
-            const R q = sqrt(r2) * irc, om = R(1) - q;
+            R r, ir;
+            root_and_inverse(r2, r, ir);
+            const R q = r * irc, om = R(1) - q;
             const R W = Wc * (R(1) + R(3) * q) * om * om * om;
             const T4 Bj = Bm[j];
             Sr += W;
@@ -903,23 +903,30 @@ __device__ __forceinline__ void ext_accel(const Inst &I, const double *x, double
 }
 
 // -------------------------------------------------------- fluid force pass
-// Constants of the SDPD pair force in precision R, held in registers.
-// Products of instance constants are folded once per thread:
-//   A1 = -cd Ca, A2 = cd (Ca + 2 Cb) / 3, A3 = -cr Ca / 2 (Eqs. FijD, FijR with
-//   gamma_a = Ca F/(d_i d_j), gamma_b = Cb F/(d_i d_j)); T1 = ct Ka / sqrt(dt),
-//   T3 = ct (Kb - Ka) / (3 sqrt(dt)) (Eq. FijT with sigma = K sqrt(F)/sqrt(d_i d_j)).
+// Constants of the SDPD pair force on one particle i in precision R, held in
+// registers.  With om = 1 - q and g = om^2 / d_j the coefficients of Eqs. FijC,
+// FijD, FijR and FijT are products of g or om and constants of i:
+//   PC = cc Fc, A1 = -cd Ca Fc/d_i, A2 = cd (Ca + 2 Cb) Fc/(3 d_i),
+//   A3 = -cr Ca Fc/(2 d_i) (gamma_a = Ca F/(d_i d_j), gamma_b = Cb F/(d_i d_j)),
+//   T1 = ct Ka/sqrt(dt d_i), T3 = ct (Kb - Ka)/(3 sqrt(dt d_i)) (sigma = K
+//   sqrt(F)/sqrt(d_i d_j)).
 template <class R> struct PairK {
-    R irc, Fc, Wc, cc, A1, A2, A3, T1, T3, lev;
+    R irc, Wc, PC, A1, A2, A3, T1, T3;
     bool noise;
     uint32_t step, key0, key1;
-    __device__ __forceinline__ PairK(const Inst &I, uint32_t st)
-        : irc(K<R>::inv_rc(I)), Fc(K<R>::Fc(I)), Wc(K<R>::Wc(I)), cc(K<R>::cc(I)),
-          A1(-K<R>::cd(I) * K<R>::Ca(I)),
-          A2(K<R>::cd(I) * (K<R>::Ca(I) + R(2) * K<R>::Cb(I)) * R(1.0 / 3.0)),
-          A3(R(-0.5) * K<R>::cr(I) * K<R>::Ca(I)),
-          T1(K<R>::ct(I) * K<R>::isdt(I) * K<R>::Ka(I)),
-          T3(K<R>::ct(I) * K<R>::isdt(I) * (K<R>::Kb(I) - K<R>::Ka(I)) * R(1.0 / 3.0)),
-          lev(K<R>::lever(I)), noise(I.noise != 0), step(st), key0(I.key0), key1(I.key1) {}
+    template <class T4>
+    __device__ __forceinline__ PairK(const Inst &I, uint32_t st, const T4 &Ci, const T4 &Di)
+        : irc(K<R>::inv_rc(I)), Wc(K<R>::Wc(I)), PC(K<R>::cc(I) * K<R>::Fc(I)), noise(I.noise != 0), step(st),
+          key0(I.key0), key1(I.key1)
+    {
+        const R fd = K<R>::Fc(I) * mir_invd(Ci, Di);
+        A1 = -K<R>::cd(I) * K<R>::Ca(I) * fd;
+        A2 = K<R>::cd(I) * (K<R>::Ca(I) + R(2) * K<R>::Cb(I)) * R(1.0 / 3.0) * fd;
+        A3 = R(-0.5) * K<R>::cr(I) * K<R>::Ca(I) * fd;
+        const R t = K<R>::ct(I) * K<R>::isdt(I) * mir_rsd(Ci, Di);
+        T1 = t * K<R>::Ka(I);
+        T3 = t * (K<R>::Kb(I) - K<R>::Ka(I)) * R(1.0 / 3.0);
+    }
 };
 
 
@@ -983,40 +990,44 @@ __device__ __forceinline__ void sdpd_pair(const PairK<R> &P, R rx, R ry, R rz, R
                                           R &oy, R &oz, R &ce, R &ex, R &ey, R &ez, R &q, R &om)
 {
     const R is2 = R(0.70710678118654752440);
-    const R ir = rsqrt_<R>(r2);
-    q = r2 * ir * P.irc;
-    om = lt_nonneg(q, R(1)) ? R(1) - q : R(0);
-    const R Fk = P.Fc * om * om;
+    R r, ir;
+    root_and_inverse(r2, r, ir);
+    q = r * P.irc;
+    om = one_minus(q);
+    const R om2 = om * om, g = om2 * mir_invd(Cj, Dj);
     ex = rx * ir; ey = ry * ir; ez = rz * ir;
     const R vx = Bi.x - Bj.x, vy = Bi.y - Bj.y, vz = Bi.z - Bj.z;
     const R ev = ex * vx + ey * vy + ez * vz;
-    const R gf = Fk * mir_invd(Ci, Di) * mir_invd(Cj, Dj);
-    const R c1 = P.A1 * gf;
+    const R c1 = P.A1 * g;
     // Eq. FijC (central) + the central part of Eq. FijD
-    ce = P.cc * (mir_pd2(Bi, Di) + mir_pd2(Bj, Dj)) * Fk * (r2 * ir) - P.A2 * gf * ev;
+    ce = P.PC * (mir_pd2(Bi, Di) + mir_pd2(Bj, Dj)) * (om2 * r) - P.A2 * g * ev;
     ox = c1 * vx; oy = c1 * vy; oz = c1 * vz;
     if (!with_rt) return;
     // Eq. FijR
     const R wx = Ci.x + Cj.x, wy = Ci.y + Cj.y, wz = Ci.z + Cj.z;
-    const R c3 = P.A3 * gf;
+    const R c3 = P.A3 * g;
     ox += c3 * (ry * wz - rz * wy);
     oy += c3 * (rz * wx - rx * wz);
     oz += c3 * (rx * wy - ry * wx);
-    // Eq. FijT: (sa S + (sb - sa) tr(S)/3 1) . e / sqrt(dt).  Every operation
-    // on the normals is spelled out (no contraction left to the compiler), so
-    // normals drawn here and normals read back from the cache give the same
-    // force bits.
+    // Eq. FijT: (sa S + (sb - sa) tr(S)/3 1) . e / sqrt(dt); z holds the three
+    // diagonal normals and the three others times 1/sqrt(2), the entries of S.
+    // Every operation on them is spelled out (no contraction left to the
+    // compiler), so normals drawn here and normals read back from the cache
+    // give the same force bits.
     if (P.noise) {
-        if (zmode == 0)
+        if (zmode == 0) {
             pair_normals<R>(mir_gid(Di), mir_gid(Dj), P.step, P.key0, P.key1, z.z0, z.z1, z.z2, z.z3,
                             z.z4, z.z5);
-        const R rs = mir_rs(om, Ci, Di, Cj, Dj);
+            z.z3 = mul_rn(z.z3, is2);
+            z.z4 = mul_rn(z.z4, is2);
+            z.z5 = mul_rn(z.z5, is2);
+        }
+        const R rs = om * mir_rsd(Cj, Dj);
         const R sa = P.T1 * rs;
-        const R sxy = mul_rn(z.z3, is2), sxz = mul_rn(z.z4, is2), syz = mul_rn(z.z5, is2);
         ce = fma_rn(P.T3 * rs, add_rn(add_rn(z.z0, z.z1), z.z2), ce);
-        ox = fma_rn(sa, fma_rn(sxz, ez, fma_rn(sxy, ey, mul_rn(z.z0, ex))), ox);
-        oy = fma_rn(sa, fma_rn(syz, ez, fma_rn(z.z1, ey, mul_rn(sxy, ex))), oy);
-        oz = fma_rn(sa, fma_rn(z.z2, ez, fma_rn(syz, ey, mul_rn(sxz, ex))), oz);
+        ox = fma_rn(sa, fma_rn(z.z4, ez, fma_rn(z.z3, ey, mul_rn(z.z0, ex))), ox);
+        oy = fma_rn(sa, fma_rn(z.z5, ez, fma_rn(z.z1, ey, mul_rn(z.z3, ex))), oy);
+        oz = fma_rn(sa, fma_rn(z.z2, ez, fma_rn(z.z5, ey, mul_rn(z.z4, ex))), oz);
     }
 }
 
@@ -1083,11 +1094,11 @@ __device__ __noinline__ void fluid_rigid_pair_call(const Bufs &b, long long s, i
     using TA = typename Mir<R>::TA;
     const Inst &I = b.inst[b.pinst[gi]];
     const Geo<R> geo(I);
-    const PairK<R> P(I, (uint32_t)(*b.step));
     const TA *__restrict__ A = Mir<R>::A(b);
     const T4 *__restrict__ Bm = Mir<R>::B(b);
     const T4 *__restrict__ Cm = Mir<R>::C(b);
     const T4 *__restrict__ Dm = Mir<R>::D(b);
+    const PairK<R> P(I, (uint32_t)(*b.step), Cm[s], Dm[s]);
     fluid_rigid_pair<R>(b, I, geo, P, gi, A[s], Bm[s], Cm[s], Dm[s], j, A[j], Bm[j], Cm[j], Dm[j], f[0], f[1],
                         f[2], f[3], f[4], f[5]);
 }
@@ -1099,6 +1110,7 @@ template <class R>
 __device__ __noinline__ void draw_rare(uint32_t gi, uint32_t gj, uint32_t step, uint32_t k0, uint32_t k1, R *z)
 {
     pair_normals<R>(gi, gj, step, k0, k1, z[0], z[1], z[2], z[3], z[4], z[5]);
+    for (int c = 3; c < 6; ++c) z[c] = mul_rn(z[c], R(0.70710678118654752440));
 }
 
 // The force and torque totals of a warp's particles, one per lane at the end.
@@ -1172,8 +1184,6 @@ __device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, 
     const int gi = h.gi;
     const Inst &I = b.inst[h.inst];
     const Geo<R> geo(I);
-    const PairK<R> P(I, step);
-    fill = fill && P.noise;
     const TA *__restrict__ A = Mir<R>::A(b);
     const T4 *__restrict__ Bm = Mir<R>::B(b);
     const T4 *__restrict__ Cm = Mir<R>::C(b);
@@ -1187,6 +1197,8 @@ __device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, 
     T2 *__restrict__ zB = (T2 *)b.zdB + first;
     const TA Ai = A[s];
     const T4 Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
+    const PairK<R> P(I, step, Ci, Di);
+    fill = fill && P.noise;
     int jn = hd.e0, jnn = hd.e1;
     TA An = A[jn];
     T4 Bn = Bm[jn], Cn = Cm[jn], Dn = Di;
@@ -1226,7 +1238,7 @@ __device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, 
         Z6<R> z;
         int zmode = 0;
         // an entry beyond h in the first evaluation carries the NaN marker
-        if (REUSE && P.noise && !rig && !isnan(za.x)) {
+        if (REUSE && P.noise && !rig && !is_nan(za.x)) {
             z.z0 = za.x; z.z1 = za.y; z.z2 = za.z; z.z3 = za.w; z.z4 = zb.x; z.z5 = zb.y;
             zmode = 1;
         }
@@ -1327,7 +1339,6 @@ __device__ __forceinline__ void force_half_entries(const Bufs &b, long long s, c
     const int ti = h.type, gi = h.gi;
     const Inst &I = b.inst[h.inst];
     const Geo<R> geo(I);
-    const PairK<R> P(I, step);
     const TA *__restrict__ A = Mir<R>::A(b);
     const T4 *__restrict__ Bm = Mir<R>::B(b);
     const T4 *__restrict__ Cm = Mir<R>::C(b);
@@ -1345,6 +1356,7 @@ __device__ __forceinline__ void force_half_entries(const Bufs &b, long long s, c
     const uint16_t *__restrict__ rv = b.rev + first;
     const TA Ai = A[s];
     const T4 Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
+    const PairK<R> P(I, step, Ci, Di);
     const bool fi = (ti == T_FLUID);
     const bool noise = P.noise;
     int jn = __ldg(nb);
@@ -1398,7 +1410,7 @@ __device__ __forceinline__ void force_half_entries(const Bufs &b, long long s, c
         Z6<R> z;
         int zmode = 0;
         // an entry beyond h in the first evaluation carries the NaN marker
-        if (REUSE && noise && !isnan(za.x)) {
+        if (REUSE && noise && !is_nan(za.x)) {
             z.z0 = za.x; z.z1 = za.y; z.z2 = za.z; z.z3 = za.w; z.z4 = zb.x; z.z5 = zb.y;
             zmode = 1;
         }
@@ -1530,14 +1542,15 @@ __device__ __forceinline__ void gather_entries(const Bufs &b, long long s, const
                 continue;
             }
             // NaN marks a pair beyond h (written by the owner)
-            if (isnan(ra[g].x)) continue;
+            if (is_nan(ra[g].x)) continue;
             if constexpr (PUSH) {
                 sums.add(-ra[g].x, -ra[g].y, -ra[g].z, ra[g].w, rb[g].x, rb[g].y);
             } else {
                 // e of the owner = -(e seen from here), bitwise
                 R rx, ry, rz;
                 geo.disp(Ai, Ap[g], rx, ry, rz);
-                const R ir = rsqrt_<R>(rx * rx + ry * ry + rz * rz);
+                R rr, ir;
+                root_and_inverse(rx * rx + ry * ry + rz * rz, rr, ir);
                 R gx, gy, gz, hx, hy, hz;
                 pair_fh(ra[g].x, ra[g].y, ra[g].z, ra[g].w, -(rx * ir), -(ry * ir), -(rz * ir), gx, gy, gz,
                         hx, hy, hz);
@@ -1732,7 +1745,6 @@ __global__ void __launch_bounds__(RB) k_force_rigid(Bufs b, int velver)
     // per lane in R; DEM and lubrication stay FP64
     using T4 = typename Vec<R>::T4;
     using TA = typename Mir<R>::TA;
-    const PairK<R> P(I, 0u);
     const Geo<R> geo(I);
     const TA *__restrict__ A = Mir<R>::A(b);
     const T4 *__restrict__ Bm = Mir<R>::B(b);
@@ -1740,6 +1752,7 @@ __global__ void __launch_bounds__(RB) k_force_rigid(Bufs b, int velver)
     const T4 *__restrict__ Dm = Mir<R>::D(b);
     const TA Ai = A[s];
     const T4 Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
+    const PairK<R> P(I, 0u, Ci, Di);
     const R Rr = (R)Ri;
     R f0 = 0, f1 = 0, f2 = 0, t0 = 0, t1 = 0, t2 = 0;
     const int n = live ? b.ncnt[s] : 0;

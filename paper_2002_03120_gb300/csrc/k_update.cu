@@ -1,6 +1,7 @@
 // k_update.cu -- update(velver) of Algorithm 1 (velocity Verlet, boundary
 // treatment, collision-method artificial viscosity) and the reductions of the
 // viscometer read-out and the diagnostics.
+#define BM_TABLES
 #include "common.cuh"
 
 namespace sdpd {
