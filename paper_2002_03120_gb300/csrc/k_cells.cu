@@ -233,14 +233,9 @@ __device__ __forceinline__ bool nb_test(const Bufs &b, const Inst &I, const Geo<
     return false;
 }
 
-// One warp per cell, its particles 32 at a time: all lanes share the cell's
-// neighbour cells (27, or 125 with half-size cells), so the candidates' records are read once per warp --
-// 32 consecutive records, coalesced, into shared memory -- and every lane
-// tests them from there (broadcast reads) instead of each lane loading every
-// candidate from global memory.  Cells and candidates are visited in
-// ascending order, as a per-particle scan would.
-constexpr int NB_WARPS = 8;
-
+// The fallback for cells with a crowded neighbour (below): one lane per
+// particle, 32 at a time, every lane testing the same candidates, which are
+// staged 32 at a time in shared memory and visited in ascending order.
 // The lists of cell c's particles [s0, s1), one lane per particle; stage:
 // 32 int4 of this warp's shared memory.
 __device__ void nb_scan_cell(const Bufs &b, int c, int s0, int s1, int4 *stage, int lane)
@@ -316,54 +311,48 @@ __device__ void nb_scan_cell(const Bufs &b, int c, int s0, int s1, int4 *stage, 
     }
 }
 
-__global__ void __launch_bounds__(NB_WARPS * 32) k_neighbors(Bufs b, const int *gate)
-{
-    GATE;
-    __shared__ int4 stage[NB_WARPS][32];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int c = blockIdx.x * NB_WARPS + w;
-    if (c >= b.ncell_total || !rebuilds(b, gate, b.cell_inst[c])) return;   // the whole warp
-    const int s0 = b.cstart[c], s1 = b.cstart[c + 1];
-    if (s0 == s1) return;
-    nb_scan_cell(b, c, s0, s1, stage[w], lane);
-}
-
-// Half-size cells hold about 11 particles, too few for one lane per particle.
-// This form gives the lanes candidates instead.
-//
-// A warp takes one cell. It flattens the candidates of the cell's
-// neighbour cells (ascending key, then slot), and takes the cell's particles
-// in groups of NG_G. For each group:
+// The lists: lanes are candidates.  `parts` warps share a cell, each taking
+// every parts-th group of NG_G of its particles.  A warp flattens the
+// candidates of the cell's neighbour cells (ascending key, then slot; cells
+// whose slots follow one another are one run).  For each group:
 // * Every batch of 32 candidates is tested against the group's bounding box,
-//   widened to the list radius. About half of the 125-cell stencil survives
-//   for a half cell, against 27 cells' worth of candidates for a full cell.
+//   widened to the list radius: about 40 % of the 27-cell stencil of full
+//   cells survives, about half of the 125-cell stencil of half cells.
 // * The survivors are compacted in order into a staging area.
 // * Each full stage of 32 runs one round per particle of the group: every
 //   lane tests its candidate against that particle. Ballots place the hits in
 //   scan order.
 // * The group's lists are collected in shared memory as 16-bit entries (the
-//   neighbour cell in the table, the offset in the cell, the contact-only
-//   flag), owned entries from the front and the others from the back.
+//   run, the offset in it, the contact-only flag): in FP32 direct contexts in
+//   order, else owned entries from the front and the others from the back.
 // * The lists are then written out LPP entries of a particle at a time, four
 //   particles side by side, instead of one scattered entry per lane.
-// A cell with a neighbour cell of more than 256 particles (beyond the 8-bit
-// offset) is scanned by the lane-per-particle routine instead.  Either way
-// the lists come out exactly as the lane-per-particle kernel writes them from
-// the same cells: the same entries in the same order, the same counts and
-// flags.
+// A cell with a crowded neighbour cell (beyond the offsets of the entries) is
+// scanned by the lane-per-particle routine above instead, which writes the
+// same lists: the same entries in the same order, the same counts and flags.
+// Full cells were once scanned by that routine alone, one warp for a cell of
+// some 70 particles: 2.9 ms for 8,192 particles (128 warps on the chip), 0.1
+// ms by this one.
 constexpr int NG_G = 8;        // particles per group
-constexpr int NG_TAB = 128;    // neighbour-cell table entries (>= ADJ)
+constexpr int NG_TAB = 128;    // runs (>= ADJ)
 constexpr int NG_STAGE = 64;   // staged candidates (one batch on top of a partial stage)
 constexpr int NG_MAX_WARPS = 4;
-constexpr int NG_OFF = 256;    // largest neighbour cell of the 16-bit entries
+
+// 16-bit entries: offset bits, and the largest neighbour cell; a run never
+// exceeds twice that (it is cut where the flattened index passes a multiple).
+// Full cells: up to 27 runs of 1,024; half cells: up to 125 runs of 256.
+template <int SUB> struct NgEntry {
+    static constexpr int BITS = SUB == 1 ? 10 : 8;
+    static constexpr int CELL = 1 << (BITS - 1);
+};
 
 struct NgShared {
     int4 sa[NG_STAGE];         // staged candidates: record,
     int sj[NG_STAGE];          //   slot,
     float sr[NG_STAGE];        //   radius where it can be a contact partner, else 0
-    int sq[NG_STAGE];          //   neighbour cell << 8 | offset in it
-    int pre[NG_TAB + 1];       // candidates before each neighbour cell (flattened index)
-    int js[NG_TAB];            // first slot of each neighbour cell
+    int sq[NG_STAGE];          //   16-bit entry
+    int pre[NG_TAB + 1];       // candidates before each run (flattened index)
+    int js[NG_TAB];            // first slot of each run
     int4 ai[NG_G];             // the group's records,
     float ri[NG_G];            //   rigid radii
 };
@@ -377,67 +366,85 @@ __host__ __device__ constexpr size_t ng_warp_bytes(int cap)
     return ng_head() + (size_t)NG_G * ng_stride(cap) * sizeof(uint16_t);
 }
 
-__global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, const int *gate)
+template <int SUB, bool SPLIT>
+__global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors(Bufs b, int parts, const int *gate)
 {
     GATE;
+    constexpr int BITS = NgEntry<SUB>::BITS, CELL = NgEntry<SUB>::CELL;
+    constexpr int NADJ = (2 * SUB + 1) * (2 * SUB + 1) * (2 * SUB + 1);
     extern __shared__ __align__(16) unsigned char ng_smem[];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const int c = blockIdx.x * nw + w;
+    const long long wg = (long long)blockIdx.x * nw + w;
+    const int c = (int)(wg / parts), part = (int)(wg % parts);
     if (c >= b.ncell_total || !rebuilds(b, gate, b.cell_inst[c])) return;   // the whole warp
     const int s0 = b.cstart[c], s1 = b.cstart[c + 1];
-    if (s0 == s1) return;
+    if (s0 + part * NG_G >= s1) return;
     const int cap = b.cap, stride = ng_stride(cap);
     unsigned char *mine = ng_smem + (size_t)w * ng_warp_bytes(cap);
     NgShared &S = *reinterpret_cast<NgShared *>(mine);
     uint16_t *buf = reinterpret_cast<uint16_t *>(mine + ng_head());
     const unsigned FULL = 0xffffffffu, lt = (1u << lane) - 1u;
 
-    // neighbour-cell table (valid codes are a prefix of the row)
+    // the runs of the neighbour cells (valid keys are a prefix of the row)
     const int *adj = b.cell_adj + (long long)c * ADJ;
-    int total = 0, nq = 0;
+    int total = 0, nq = 0, last_end = -1, last_bucket = 0;
     bool fat = false;
-    for (int q0 = 0; q0 < ADJ; q0 += 32) {
+    for (int q0 = 0; q0 < NADJ; q0 += 32) {
         const int q = q0 + lane;
-        const int key = q < ADJ ? adj[q] : -1;
+        const int key = q < NADJ ? adj[q] : -1;
         int cnt = 0, js = 0;
         if (key >= 0) {
             js = b.cstart[key];
             cnt = b.cstart[key + 1] - js;
         }
-        fat = fat || __any_sync(FULL, cnt > NG_OFF);
+        fat = fat || __any_sync(FULL, cnt > CELL);
         int v = cnt;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int t = __shfl_up_sync(FULL, v, o);
             if (lane >= o) v += t;
         }
-        if (key >= 0) {
-            S.pre[q] = total + v - cnt;
-            S.js[q] = js;
+        const int first = total + v - cnt, bucket = first / CELL;
+        // the filled cell before this one: where it ended
+        const unsigned filled = __ballot_sync(FULL, cnt > 0), before = filled & lt;
+        const int src = before ? 31 - __clz(before) : 0;
+        int pe = __shfl_sync(FULL, js + cnt, src), pb = __shfl_sync(FULL, bucket, src);
+        if (!before) {
+            pe = last_end;
+            pb = last_bucket;
         }
+        const unsigned starts = __ballot_sync(FULL, cnt > 0 && (js != pe || bucket != pb));
+        if ((starts >> lane) & 1u) {
+            const int r = nq + __popc(starts & lt);
+            S.pre[r] = first;
+            S.js[r] = js;
+        }
+        nq += __popc(starts);
         total += __shfl_sync(FULL, v, 31);
-        const unsigned vm = __ballot_sync(FULL, key >= 0);
-        nq += __popc(vm);
-        if (vm != FULL) break;
+        if (filled) {
+            const int l = 31 - __clz(filled);
+            last_end = __shfl_sync(FULL, js + cnt, l);
+            last_bucket = __shfl_sync(FULL, bucket, l);
+        }
+        if (__ballot_sync(FULL, key >= 0) != FULL) break;
     }
     if (fat) {
         // the list buffer serves as the routine's stage (512 bytes)
-        nb_scan_cell(b, c, s0, s1, reinterpret_cast<int4 *>(buf), lane);
+        if (part == 0) nb_scan_cell(b, c, s0, s1, reinterpret_cast<int4 *>(buf), lane);
         return;
     }
     if (lane == 0) S.pre[nq] = total;
     __syncwarp();
 
-    const Inst &I = b.inst[b.pinst[b.perm[s0]]];   // a cell belongs to one instance
-    const int base = b.cstart[I.cell_base];           // first slot of the instance
+    const Inst &I = b.inst[b.cell_inst[c]];   // a cell belongs to one instance
+    const int base = b.cstart[I.cell_base];   // first slot of the instance
     const int rows = b.rows;
-    const float rb2_box = I.rb2f * 1.001f;   // conservative: the pair test decides
+    const float rb2 = I.rb2f, rb2_box = rb2 * 1.001f;   // conservative: the pair test decides
     const float two_hs = (float)(2.0 * I.half_skin);
     const Geo<float> geo(I);
     const float BIG = 3.0e38f;
-    const bool split = b.split != 0;
 
-    for (int g0 = s0; g0 < s1; g0 += NG_G) {
+    for (int g0 = s0 + part * NG_G; g0 < s1; g0 += parts * NG_G) {
         const int P = min(NG_G, s1 - g0);
         int4 a = make_int4(0, 0, 0, 0);
         int t = T_FLUID;
@@ -449,7 +456,7 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
             S.ai[lane] = a;
             S.ri[lane] = r;
         }
-        // the group's bounding box, relative to its first particle
+        // the group's bounding box, relative to its first particle (all in one cell)
         const int4 ref = make_int4(__shfl_sync(FULL, a.x, 0), __shfl_sync(FULL, a.y, 0), __shfl_sync(FULL, a.z, 0), 0);
         float ax, ay, az;
         geo.disp(a, ref, ax, ay, az);
@@ -469,13 +476,21 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
         lx = __shfl_sync(FULL, lx, 0); ly = __shfl_sync(FULL, ly, 0); lz = __shfl_sync(FULL, lz, 0);
         hx = __shfl_sync(FULL, hx, 0); hy = __shfl_sync(FULL, hy, 0); hz = __shfl_sync(FULL, hz, 0);
         rg = __shfl_sync(FULL, rg, 0);
+        // its centre and half widths: the wrapping difference to the centre is
+        // the image of a candidate nearest to the box, also where a periodic
+        // axis holds only three cells
+        const float bx = 0.5f * (hx - lx), by = 0.5f * (hy - ly), bz = 0.5f * (hz - lz);
+        const int4 mid = make_int4((int)((unsigned)ref.x + (unsigned)__float2int_rn(0.5f * (lx + hx) / geo.u0)),
+                                   (int)((unsigned)ref.y + (unsigned)__float2int_rn(0.5f * (ly + hy) / geo.u1)),
+                                   (int)((unsigned)ref.z + (unsigned)__float2int_rn(0.5f * (lz + hz) / geo.u2)), 0);
         const bool grp_rigid = __any_sync(FULL, lane < P && t == T_RIGID);
         __syncwarp();
 
+        // nf: entries (SPLIT: owned ones), m: not owned ones, rig: any sphere
         int nf[NG_G], m[NG_G];
-        bool rig[NG_G];
+        unsigned rig = 0;
 #pragma unroll
-        for (int p = 0; p < NG_G; ++p) { nf[p] = 0; m[p] = 0; rig[p] = false; }
+        for (int p = 0; p < NG_G; ++p) { nf[p] = 0; m[p] = 0; }
 
         // one round per particle over the first nv staged candidates
         auto rounds = [&](int nv) {
@@ -489,72 +504,78 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
                 rj = S.sr[lane];
                 e16 = (uint32_t)S.sq[lane];
             }
-            const int tj = Aj.w;
+            const unsigned valid = nv >= 32 ? FULL : (1u << nv) - 1u;
+            const bool rigid_j = Aj.w == T_RIGID;
+            const unsigned mrig = __ballot_sync(FULL, rigid_j);
 #pragma unroll
             for (int p = 0; p < NG_G; ++p) {
                 if (p < P) {
                     const int4 Ai = S.ai[p];
-                    const int ti = Ai.w;
                     const int s = g0 + p;
-                    bool hit = false;
                     uint32_t entry = e16;
-                    if (lane < nv && j != s) {
-                        float dx, dy, dz;
-                        geo.disp(Ai, Aj, dx, dy, dz);
-                        const float r2f = dx * dx + dy * dy + dz * dz;
-                        if (r2f < I.rb2f) {
-                            hit = true;
-                        } else if (ti == T_RIGID && tj == T_RIGID) {
-                            const float lim = (S.ri[p] + rj + two_hs) * 1.0001f;
-                            entry |= 0x8000u;   // contact range only
-                            hit = r2f < lim * lim;
+                    float dx, dy, dz;
+                    geo.disp(Ai, Aj, dx, dy, dz);
+                    const float r2f = dx * dx + dy * dy + dz * dz;
+                    bool hit = r2f < rb2 && j != s;
+                    if (grp_rigid && Ai.w == T_RIGID && rigid_j && !hit && j != s) {
+                        const float lim = (S.ri[p] + rj + two_hs) * 1.0001f;
+                        entry |= 0x8000u;   // contact range only
+                        hit = r2f < lim * lim;
+                    }
+                    const unsigned mh = __ballot_sync(FULL, hit) & valid;
+                    if (!SPLIT) {
+                        const int pos = nf[p] + __popc(mh & lt);
+                        if (((mh >> lane) & 1u) && pos < cap) buf[p * stride + pos] = (uint16_t)entry;
+                        nf[p] += __popc(mh);
+                    } else {
+                        const unsigned mo = __ballot_sync(FULL, pair_owned(s, j, base)) & mh;
+                        // rank in scan order decides whether the entry fits, as
+                        // the per-particle scan writes while nf + m < cap
+                        if (((mh >> lane) & 1u) && nf[p] + m[p] + __popc(mh & lt) < cap) {
+                            const int pos = ((mo >> lane) & 1u) ? nf[p] + __popc(mo & lt)
+                                                               : cap - 1 - (m[p] + __popc(mh & ~mo & lt));
+                            buf[p * stride + pos] = (uint16_t)entry;
                         }
+                        nf[p] += __popc(mo);
+                        m[p] += __popc(mh & ~mo);
                     }
-                    const bool own = hit && (!split || pair_owned(s, j, base));
-                    const unsigned mh = __ballot_sync(FULL, hit), mo = __ballot_sync(FULL, own);
-                    const unsigned mr = __ballot_sync(FULL, hit && tj == T_RIGID);
-                    // rank in scan order decides whether the entry fits, as
-                    // the per-particle scan writes while nf + m < cap
-                    if (hit && nf[p] + m[p] + __popc(mh & lt) < cap) {
-                        const int pos = own ? nf[p] + __popc(mo & lt) : cap - 1 - (m[p] + __popc(mh & ~mo & lt));
-                        buf[p * stride + pos] = (uint16_t)entry;
-                    }
-                    nf[p] += __popc(mo);
-                    m[p] += __popc(mh & ~mo);
-                    rig[p] = rig[p] || (mr != 0u);
+                    if (mh & mrig) rig |= 1u << p;
                 }
             }
             __syncwarp();
         };
 
-        int nst = 0, qc = 0;
+        int nst = 0, qc = 0;   // staged candidates; the run of the batch's first candidate
         for (int f0 = 0; f0 < total; f0 += 32) {
             const int f = f0 + lane;
+            // the runs that begin inside this batch, as bits at their first
+            // candidate (runs are not empty: at most one begins at a place)
+            int nx = qc + 1 + lane < nq ? S.pre[qc + 1 + lane] - f0 : 32;
+            const unsigned begin = __reduce_or_sync(FULL, nx < 32 ? 1u << nx : 0u);
+            const int q = qc + __popc(begin & (lt | (1u << lane)));
             bool keep = false;
             int4 Aj = make_int4(0, 0, 0, 0);
-            int j = 0, eq = 0, q = qc;
+            int j = 0, eq = 0;
             float rj = 0.f;
             if (f < total) {
-                while (S.pre[q + 1] <= f) ++q;
                 const int off = f - S.pre[q];
                 j = S.js[q] + off;
-                eq = (q << 8) | off;
+                eq = (q << BITS) | off;
                 Aj = b.A32[j];
-                const int tj = Aj.w;
                 float px, py, pz;
-                geo.disp(Aj, ref, px, py, pz);
-                const float ex = fmaxf(fmaxf(lx - px, px - hx), 0.f), ey = fmaxf(fmaxf(ly - py, py - hy), 0.f),
-                            ez = fmaxf(fmaxf(lz - pz, pz - hz), 0.f);
+                geo.disp(Aj, mid, px, py, pz);
+                const float ex = fmaxf(fabsf(px) - bx, 0.f), ey = fmaxf(fabsf(py) - by, 0.f),
+                            ez = fmaxf(fabsf(pz) - bz, 0.f);
                 const float d2 = ex * ex + ey * ey + ez * ez;
                 float lim2 = rb2_box;
-                if (grp_rigid && tj == T_RIGID) {
+                if (grp_rigid && Aj.w == T_RIGID) {
                     rj = (float)b.R[b.perm[j]];
                     const float L = (rg + rj + two_hs) * (1.0001f * 1.0005f);
                     lim2 = fmaxf(lim2, L * L);
                 }
                 keep = d2 < lim2;
             }
-            qc = __shfl_sync(FULL, q, 31);   // the cell of this batch's last candidate
+            qc += __popc(begin);
             const unsigned km = __ballot_sync(FULL, keep);
             if (keep) {
                 const int pos = nst + __popc(km & lt);
@@ -593,36 +614,33 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors_grp(Bufs b, con
 
         // counts and flags of the group's particles
         int mynf = 0, mym = 0;
-        bool myrig = false;
 #pragma unroll
         for (int p = 0; p < NG_G; ++p)
-            if (lane == p) { mynf = nf[p]; mym = m[p]; myrig = rig[p]; }
+            if (lane == p) { mynf = nf[p]; mym = m[p]; }
         int myn = 0;
         if (lane < P) {
             const int s = g0 + lane;
             myn = mynf + mym;
-            if (split && (mynf > b.capown || mym > b.capown)) atomicOr(b.err, ERR_PAIR_CAP);
+            if (SPLIT && (mynf > b.capown || mym > b.capown)) atomicOr(b.err, ERR_PAIR_CAP);
             if (myn > cap) atomicOr(b.err, ERR_NBR_CAP);
-            b.nfirst[s] = min(mynf, split ? min(cap, b.capown) : cap);
+            b.nfirst[s] = min(mynf, SPLIT ? min(cap, b.capown) : cap);
             b.ncnt[s] = min(myn, cap);
-            b.nbflag[s] = myrig ? 1 : 0;
+            b.nbflag[s] = (rig >> lane) & 1u;
         }
-        int maxn = lane < P ? min(myn, cap) : 0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) maxn = max(maxn, __shfl_xor_sync(FULL, maxn, o));
+        const int maxn = __reduce_max_sync(FULL, lane < P ? min(myn, cap) : 0);
         // write-out: LPP lanes a particle, GROUP particles side by side; without
         // overflow the back region [cap - m, cap) moves down to [nf, n) as it is
         for (int p0 = 0; p0 < P; p0 += GROUP) {
             const int p = p0 + lane / LPP;   // < NG_G: the shuffles below stay in range
             const int pnf = __shfl_sync(FULL, mynf, p), pm = __shfl_sync(FULL, mym, p);
             const int pn = pnf + pm, pcnt = p < P ? min(pn, cap) : 0;
-            for (int k0 = 0; k0 < maxn; k0 += LPP) {
-                const int k = k0 + lane % LPP;
+            int *out = b.nbr + entry_at(lane % LPP, g0 + p, rows);
+            for (int k = lane % LPP; k < maxn; k += LPP, out += ROW) {
                 if (k < pcnt) {
-                    const int src = (pn > cap || k < pnf) ? k : cap - pm + (k - pnf);
+                    const int src = (!SPLIT || pn > cap || k < pnf) ? k : cap - pm + (k - pnf);
                     const uint32_t e = buf[p * stride + src];
-                    const int slot = S.js[(e >> 8) & 127u] + (int)(e & 255u);
-                    b.nbr[entry_at(k, g0 + p, rows)] = (int)((uint32_t)slot | ((e & 0x8000u) ? NB_FAR : 0u));
+                    const int slot = S.js[(e & 0x7FFFu) >> BITS] + (int)(e & ((1u << BITS) - 1u));
+                    *out = (int)((uint32_t)slot | ((e & 0x8000u) ? NB_FAR : 0u));
                 }
             }
         }
@@ -717,7 +735,23 @@ static_assert(ng_warp_bytes(SDPD_MAX_NEIGHBORS) <= NG_SMEM_MAX, "list buffers of
 
 void init_cell_kernels()
 {
-    cudaFuncSetAttribute(k_neighbors_grp, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NG_SMEM_MAX);
+    cudaFuncSetAttribute(k_neighbors<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NG_SMEM_MAX);
+    cudaFuncSetAttribute(k_neighbors<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NG_SMEM_MAX);
+    cudaFuncSetAttribute(k_neighbors<2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NG_SMEM_MAX);
+    cudaFuncSetAttribute(k_neighbors<2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)NG_SMEM_MAX);
+}
+
+template <int SUB>
+static void launch_lists(const Bufs &b, const int *gate, cudaStream_t st)
+{
+    // warps per cell: a full cell holds about eight groups, a half cell one or
+    // two (more than one warp for them only where cells alone leave SMs idle)
+    const int parts = SUB == 1 ? 8 : (b.ncell_total < 4096 ? 2 : 1);
+    const size_t wb = ng_warp_bytes(b.cap);
+    const int ngw = (int)std::min<size_t>(NG_MAX_WARPS, NG_SMEM_MAX / wb);
+    const unsigned nb = nblk((long long)b.ncell_total * parts, ngw);
+    if (b.split) k_neighbors<SUB, true><<<nb, ngw * 32, ngw * wb, st>>>(b, parts, gate);
+    else k_neighbors<SUB, false><<<nb, ngw * 32, ngw * wb, st>>>(b, parts, gate);
 }
 
 void launch_build(const Bufs &b, int precision, int need_rev, const int *gate, cudaStream_t st)
@@ -733,13 +767,8 @@ void launch_build(const Bufs &b, int precision, int need_rev, const int *gate, c
         k_scatter<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
         k_rank<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
         k_gather<<<nblk(b.N, 256), 256, 0, st>>>(b, precision, gate);
-        if (b.cell_sub == 2) {
-            const size_t wb = ng_warp_bytes(b.cap);
-            const int ngw = (int)std::min<size_t>(NG_MAX_WARPS, NG_SMEM_MAX / wb);
-            k_neighbors_grp<<<nblk(nc, ngw), ngw * 32, ngw * wb, st>>>(b, gate);
-        } else {
-            k_neighbors<<<nblk(nc, NB_WARPS), NB_WARPS * 32, 0, st>>>(b, gate);
-        }
+        if (b.cell_sub == 2) launch_lists<2>(b, gate, st);
+        else launch_lists<1>(b, gate, st);
         if (need_rev) k_rev<<<nblk(b.N * LPP, 128), 128, 0, st>>>(b, gate);
     }
     k_build_done<<<1, 64, 0, st>>>(b, gate);
