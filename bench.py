@@ -296,7 +296,7 @@ def force_kernel_name(mode, split):
     r = "float" if split else "double"
     if mode in (1, 4):
         return f"k_force_half<{r}, {'true' if mode == 4 or not split else 'false'}>"
-    return "k_force_fluid<float, 2>" if split else "k_force_fluid<double, 0>"
+    return "k_force_draw" if split else "k_force_fluid"
 
 
 def time_native(args, ws, rank, local):

@@ -411,6 +411,7 @@ sdpd_status check_err(sdpd_ctx *c)
     if (e & ERR_REV) return fail(SDPD_E_STATE, "neighbour lists not symmetric");
     if (e & ERR_NONFINITE) return fail(SDPD_E_NONFINITE, "non-finite position, velocity or spin");
     if (e & ERR_DOMAIN) return fail(SDPD_E_DOMAIN, "particle outside the grid (crossed a wall axis, or moved more than a box length in one step)");
+    if (e & ERR_TIMEOUT) return fail(SDPD_E_TIMEOUT, "a copy into shared memory did not complete");
     return fail(SDPD_E_CUDA, "unknown device error");
 }
 
@@ -540,8 +541,7 @@ sdpd_status sdpd_init(const sdpd_params *params, int n_instances, const long lon
         b.resB = n_resB ? arena + n_resA : dummy;
         b.zA = arena + n_resA + n_resB;
         b.zB = arena + n_resA + n_resB + n_zA;
-        b.zdA = arena;
-        b.zdB = arena + 4 * rs * all;
+        b.zd = arena;
         b.ownA = oa; b.ownB = ob;
     }
     IALLOC(b.dsp, N);

@@ -1163,21 +1163,25 @@ struct CacheUse {
     }
 };
 
-// Direct (owner-computes-all) force pass over the neighbour list of fluid
-// particle s (this lane's share of it).  The index two entries ahead and the
+// The direct (owner-computes-all) force pass in FP64 over the neighbour list of
+// fluid particle s (this lane's share of it).  The index two entries ahead and the
 // records of the next neighbour are fetched before the current pair is
 // evaluated.  With the cache on, the first evaluation of a step (FILL) stores
 // the six normals of every entry in its own column (a NaN marker for an entry
 // beyond h); the second (REUSE, when the list has not been rebuilt in
-// between) reads them back, fetched one entry ahead like the records, instead
-// of drawing them again (same counter, so the same bits).
+// between) reads them back instead of drawing them again (same counter, so
+// the same bits).
+template <class R> struct NormalRow {   // a row of 32 entries of the cache
+    using T4 = typename Vec<R>::T4;
+    using T2 = typename Vec2<R>::T2;
+    T4 a[ROW];
+    T2 b[ROW];
+};
+
 template <class R, bool REUSE>
 __device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, const SlotHead &h, const ListHead &hd,
                                                     int sub, uint32_t step, bool fill, ForceSums<R> &sums)
 {
-    // FP32, normals from the cache: a partner's D record (its gid) only for a
-    // pair whose normals must be drawn after all (rare), loaded then
-    constexpr bool LAZY_D = REUSE && sizeof(R) == 4;
     using T4 = typename Vec<R>::T4;
     using TA = typename Mir<R>::TA;
     using T2 = typename Vec2<R>::T2;
@@ -1188,39 +1192,34 @@ __device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, 
     const T4 *__restrict__ Bm = Mir<R>::B(b);
     const T4 *__restrict__ Cm = Mir<R>::C(b);
     const T4 *__restrict__ Dm = Mir<R>::D(b);
-    const int n = h.n;
+    const int n = h.n, lane = threadIdx.x & 31;   // lane: also the entry's place in its row
     int k = sub;
     if (k >= n) return;
-    const size_t first = entry_at(sub, s, b.rows);
-    const int *__restrict__ nb = b.nbr + first;
-    T4 *__restrict__ zA = (T4 *)b.zdA + first;
-    T2 *__restrict__ zB = (T2 *)b.zdB + first;
+    const int *__restrict__ nb = b.nbr + entry_at(sub, s, b.rows);
+    NormalRow<R> *__restrict__ zr = (NormalRow<R> *)b.zd + (size_t)(s / GROUP) * b.rows;
     const TA Ai = A[s];
     const T4 Bi = Bm[s], Ci = Cm[s], Di = Dm[s];
     const PairK<R> P(I, step, Ci, Di);
     fill = fill && P.noise;
     int jn = hd.e0, jnn = hd.e1;
     TA An = A[jn];
-    T4 Bn = Bm[jn], Cn = Cm[jn], Dn = Di;
-    if constexpr (!LAZY_D) Dn = Dm[jn];
+    T4 Bn = Bm[jn], Cn = Cm[jn], Dn = Dm[jn];
     T4 zan;
     T2 zbn;
-    if (REUSE && P.noise) { zan = ld_stream(zA); zbn = ld_stream(zB); }
-    for (; k < n; k += LPP, nb += ROW, zA += ROW, zB += ROW) {
+    if (REUSE && P.noise) { zan = ld_stream(zr->a + lane); zbn = ld_stream(zr->b + lane); }
+    for (; k < n; k += LPP, nb += ROW, ++zr) {
         const int j = jn;
         const TA Aj = An;
-        const T4 Bj = Bn, Cj = Cn;
-        T4 Dj = Dn;
+        const T4 Bj = Bn, Cj = Cn, Dj = Dn;
         T4 za;
         T2 zb;
         if (REUSE) { za = zan; zb = zbn; }
         if (k + LPP < n) {
             jn = jnn;
-            An = A[jn]; Bn = Bm[jn]; Cn = Cm[jn];
-            if constexpr (!LAZY_D) Dn = Dm[jn];
+            An = A[jn]; Bn = Bm[jn]; Cn = Cm[jn]; Dn = Dm[jn];
             if (REUSE && P.noise) {
-                zan = ld_stream(zA + ROW);
-                zbn = ld_stream(zB + ROW);
+                zan = ld_stream(zr[1].a + lane);
+                zbn = ld_stream(zr[1].b + lane);
             }
             if (k + 2 * LPP < n) jnn = ld_stream(nb + 2 * ROW);
         }
@@ -1230,7 +1229,7 @@ __device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, 
             if (!REUSE && fill && !rig) {
                 T4 nm;
                 nm.x = R(NAN); nm.y = R(0); nm.z = R(0); nm.w = R(0);
-                st_stream(zA, nm);
+                st_stream(zr->a + lane, nm);
             }
             continue;
         }
@@ -1242,14 +1241,6 @@ __device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, 
             z.z0 = za.x; z.z1 = za.y; z.z2 = za.z; z.z3 = za.w; z.z4 = zb.x; z.z5 = zb.y;
             zmode = 1;
         }
-        if constexpr (LAZY_D) {
-            if (zmode == 0 && P.noise && !rig) {
-                R t[6];
-                draw_rare<R>(mir_gid(Di), mir_gid(Dm[j]), P.step, P.key0, P.key1, t);
-                z.z0 = t[0]; z.z1 = t[1]; z.z2 = t[2]; z.z3 = t[3]; z.z4 = t[4]; z.z5 = t[5];
-            }
-            zmode = 1;
-        }
         sdpd_pair<R>(P, rx, ry, rz, r2, Bi, Ci, Di, Bj, Cj, Dj, !rig, zmode, z, ox, oy, oz, ce, ex, ey, ez,
                      q, om);
         if (!REUSE && fill && !rig) {
@@ -1257,8 +1248,8 @@ __device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, 
             zw.x = z.z0; zw.y = z.z1; zw.z = z.z2; zw.w = z.z3;
             T2 zv;
             zv.x = z.z4; zv.y = z.z5;
-            st_stream(zA, zw);
-            st_stream(zB, zv);
+            st_stream(zr->a + lane, zw);
+            st_stream(zr->b + lane, zv);
         }
         R gx, gy, gz, hx, hy, hz;
         pair_fh(ox, oy, oz, ce, ex, ey, ez, gx, gy, gz, hx, hy, hz);
@@ -1275,45 +1266,418 @@ __device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, 
     }
 }
 
-// ONLY: 0 every path; 1 only the particles whose normals are cached (second
-// evaluation); 2 only those whose normals are drawn
-template <class R, int ONLY = 0>
-__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 2 : 1) k_force_fluid(Bufs b, int velver, int groups)
+__global__ void __launch_bounds__(256) k_force_fluid(Bufs b, int velver, int groups)
 {
+    using R = double;
     const CacheUse u(b, velver);
-    if ((ONLY == 1 && !u.maybe) || (ONLY == 2 && u.all)) return;   // uniform over the launch
     const int lane = threadIdx.x & 31, sub = lane % LPP;
     const long long base = pass_base(groups);
-    // the particles of this launch: fluid, their normals cached or not
     SlotHead mine(b, base + lane, lane < groups * GROUP);
-    const bool cached = mine.type == T_FLUID && u.reuse(b, mine.inst);
-    if (mine.type != T_FLUID || (ONLY == 1 && !cached) || (ONLY == 2 && cached)) mine.n = -1;
-    SlotHead h = mine.of_group(0);
-    ListHead hd(b.nbr, base + lane / LPP, b.rows, 0, h.n, sub);
+    if (mine.type != T_FLUID) mine.n = -1;
     ForceSums<R> sums;
     for (int g = 0; g < groups; ++g) {
         const long long s = base + g * GROUP + lane / LPP;
-        SlotHead hn;
-        ListHead hdn;
-        if (g + 1 < groups) {
-            hn = mine.of_group(g + 1);
-            hdn = ListHead(b.nbr, s + GROUP, b.rows, 0, hn.n, sub);
-            prefetch_lists(b, base + (g + 1) * GROUP, hn.n);
-        }
-        if constexpr (ONLY == 0) {
-            if (u.reuse(b, h.inst)) force_fluid_entries<R, true>(b, s, h, hd, sub, u.step, false, sums);
-            else force_fluid_entries<R, false>(b, s, h, hd, sub, u.step, u.fill, sums);
-        } else {
-            force_fluid_entries<R, ONLY == 1>(b, s, h, hd, sub, u.step, ONLY == 1 ? false : u.fill, sums);
-        }
+        const SlotHead h = mine.of_group(g);
+        const ListHead hd(b.nbr, s, b.rows, 0, h.n, sub);
+        if (u.reuse(b, h.inst)) force_fluid_entries<R, true>(b, s, h, hd, sub, u.step, false, sums);
+        else force_fluid_entries<R, false>(b, s, h, hd, sub, u.step, u.fill, sums);
         sums.close_group(g);
-        h = hn;
-        hd = hdn;
     }
     if (mine.n < 0) return;
-    const Inst &I = b.inst[mine.inst];
-    write_fluid_force<R>(b, I, mine.gi, sums.keep[0], sums.keep[1], sums.keep[2], sums.keep[3], sums.keep[4],
-                         sums.keep[5], K<R>::lever(I));
+    write_fluid_force<R>(b, b.inst[mine.inst], mine.gi, sums.keep[0], sums.keep[1], sums.keep[2], sums.keep[3],
+                         sums.keep[4], sums.keep[5], K<R>::lever(b.inst[mine.inst]));
+}
+
+// ------------------------------------------------- direct force pass, FP32
+// The r < h decision of a pair in the guard band, out of line: it is rare,
+// and its FP64 code would cost the pair loop registers.
+__device__ __noinline__ bool within_exactly(const Bufs &b, int inst, int gi, int j)
+{
+    return exact_within(b, b.inst[inst], gi, b.perm[j]);
+}
+
+// One listed pair (i, j) of the FP32 direct pass, added to i's sums where `ok`
+// (within h).  Every lane runs the same straight line: an entry past the end
+// or beyond h is left out of the sums at the end, and a sphere partner
+// (`rig`: Eqs. FijC and FijD only) has zero rotational and random
+// coefficients.  Branches for them cost the pass about a quarter of its
+// instructions (divergence barriers and register moves), though some lane
+// takes the long way almost always.
+__device__ __forceinline__ void pair32(const Bufs &b, const PairK<float> &P, bool ok, bool rig, int j, float rx,
+                                       float ry, float rz, float r2, const float4 &Bi, const float4 &Ci,
+                                       const float4 &Bj, const float4 &Cj, const Z6<float> &z, float (&f)[6])
+{
+    float r, ir;
+    root_and_inverse(r2, r, ir);
+    const float q = r * P.irc, om = one_minus(q);
+    const float om2 = om * om, g = om2 * Cj.w;
+    const float ex = rx * ir, ey = ry * ir, ez = rz * ir;
+    const float vx = Bi.x - Bj.x, vy = Bi.y - Bj.y, vz = Bi.z - Bj.z;
+    const float ev = ex * vx + ey * vy + ez * vz;
+    const float c1 = P.A1 * g, c3 = (rig ? 0.f : P.A3) * g;
+    float ce = P.PC * (Bi.w + Bj.w) * (om2 * r) - P.A2 * g * ev;
+    const float wx = Ci.x + Cj.x, wy = Ci.y + Cj.y, wz = Ci.z + Cj.z;
+    float ox = c1 * vx + c3 * (ry * wz - rz * wy);
+    float oy = c1 * vy + c3 * (rz * wx - rx * wz);
+    float oz = c1 * vz + c3 * (rx * wy - ry * wx);
+    const float rs = om * (Cj.w * rsqrt_ftz(Cj.w));
+    const float sa = (rig ? 0.f : P.T1) * rs, st = (rig ? 0.f : P.T3) * rs;
+    // (explicit roundings from here on: normals drawn and normals read back
+    // give the same bits)
+    ce = fma_rn(st, add_rn(add_rn(z.z0, z.z1), z.z2), ce);
+    ox = fma_rn(sa, fma_rn(z.z4, ez, fma_rn(z.z3, ey, mul_rn(z.z0, ex))), ox);
+    oy = fma_rn(sa, fma_rn(z.z5, ez, fma_rn(z.z1, ey, mul_rn(z.z3, ex))), oy);
+    oz = fma_rn(sa, fma_rn(z.z2, ez, fma_rn(z.z5, ey, mul_rn(z.z4, ex))), oz);
+    float gx, gy, gz, hx, hy, hz;
+    pair_fh(ox, oy, oz, ce, ex, ey, ez, gx, gy, gz, hx, hy, hz);
+    if (ok && rig) {
+        // Eq. F_fpi_DG_reac: -F^DG_s W_sj / S_s
+        const float4 rc = b.rxn32[j];
+        const float W = drag_weight(P, q, om);
+        f[0] = sub_rn(f[0], mul_rn(rc.x, W));
+        f[1] = sub_rn(f[1], mul_rn(rc.y, W));
+        f[2] = sub_rn(f[2], mul_rn(rc.z, W));
+    }
+    if (ok) {
+        f[0] = add_rn(f[0], gx);
+        f[1] = add_rn(f[1], gy);
+        f[2] = add_rn(f[2], gz);
+        f[3] = add_rn(f[3], hx);
+        f[4] = add_rn(f[4], hy);
+        f[5] = add_rn(f[5], hz);
+    }
+}
+
+// The loops below take ZR rows at a time, unrolled, so that a row costs no
+// counters and no moves between registers.  Lists: a lane's ZR entries of the
+// next rows are fetched while the present ones are evaluated (a lane without
+// an entry reads record 0 and adds nothing).
+constexpr int ZR = 4;
+struct ListRows {
+    int e[ZR];
+    // (nb: this lane's entry of the first of the rows, n: entries left from it on)
+    __device__ __forceinline__ void load(const int *nb, int n)
+    {
+#pragma unroll
+        for (int i = 0; i < ZR; ++i) e[i] = i * LPP < n ? ld_stream(nb + i * ROW) : 0;
+    }
+};
+
+// A warp's particles and their totals, in shared memory: registers are what
+// these two kernels are short of.
+struct WarpSlots {
+    int gi[32], inst[32], n[32];   // n < 0: not a particle of this launch
+    float f[32][6];
+    // every lane puts its own slot's in
+    __device__ __forceinline__ void set(const SlotHead &h)
+    {
+        const int lane = threadIdx.x & 31;
+        gi[lane] = h.gi;
+        inst[lane] = h.inst;
+        n[lane] = h.n;
+        __syncwarp();
+    }
+    // the totals of group g's particles: the lanes of a particle all end with them
+    __device__ __forceinline__ void put(int g, float (&v)[6])
+    {
+#pragma unroll
+        for (int c = 0; c < 6; ++c) v[c] = lanes_sum(v[c]);
+        const int lane = threadIdx.x & 31;
+        if (lane % LPP == 0)
+#pragma unroll
+            for (int c = 0; c < 6; ++c) f[g * GROUP + lane / LPP][c] = v[c];
+    }
+    // and written out, each by a lane of its own
+    __device__ __forceinline__ void write(const Bufs &b)
+    {
+        __syncwarp();
+        const int lane = threadIdx.x & 31;
+        if (n[lane] < 0) return;
+        const Inst &I = b.inst[inst[lane]];
+        write_fluid_force<float>(b, I, gi[lane], f[lane][0], f[lane][1], f[lane][2], f[lane][3], f[lane][4], f[lane][5],
+                                 K<float>::lever(I));
+    }
+};
+
+// What a lane holds of its particle.
+struct Own32 {
+    Geo<float> geo;
+    PairK<float> P;
+    int4 A;
+    float4 B, C;
+    __device__ __forceinline__ Own32(const Bufs &b, int inst, uint32_t step, long long s)
+        : Own32(b.inst[inst], step, b.A32[s], b.B32[s], b.C32[s])
+    {}
+    __device__ __forceinline__ Own32(const Inst &I, uint32_t step, const int4 &a, const float4 &bb, const float4 &c)
+        : geo(I), P(I, step, c, c), A(a), B(bb), C(c)   // (FP32 keeps nothing of the pair constants in D)
+    {}
+};
+
+// The displacement of a listed pair and whether it lies within h.
+__device__ __forceinline__ bool near32(const Bufs &b, const Own32 &o, const WarpSlots &w, int slot, bool live, int j,
+                                       const int4 &Aj, float &rx, float &ry, float &rz, float &r2)
+{
+    o.geo.disp(o.A, Aj, rx, ry, rz);
+    r2 = rx * rx + ry * ry + rz * rz;
+    bool ok = live && r2 < o.geo.ghi;
+    if (ok && r2 >= o.geo.glo) ok = within_exactly(b, w.inst[slot], w.gi[slot], j);
+    return ok;
+}
+
+// The drawing pass: the particles whose normals are not cached.  With the
+// cache on, the first evaluation of a step (fill) stores the normals of every
+// entry in its row, a NaN marker for an entry beyond h (those of a sphere
+// partner are stored too and enter with a zero coefficient).  Two rows are
+// drawn together for the packed Box-Muller.
+__global__ void __launch_bounds__(256, 2) k_force_draw(Bufs b, int velver, int groups)
+{
+    __shared__ WarpSlots tables[8];
+    const CacheUse u(b, velver);
+    if (u.all) return;   // uniform over the launch
+    WarpSlots &tab = tables[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31, sub = lane % LPP;
+    const unsigned FULL = 0xffffffffu;
+    const long long base = pass_base(groups);
+    {
+        SlotHead mine(b, base + lane, lane < groups * GROUP);
+        if (mine.type != T_FLUID || u.reuse(b, mine.inst)) mine.n = -1;
+        tab.set(mine);
+    }
+    for (int g = 0; g < groups; ++g) {
+        float f[6] = { 0.f, 0.f, 0.f, 0.f, 0.f, 0.f };
+        const int slot = g * GROUP + lane / LPP, n = tab.n[slot];
+        if (g + 1 < groups) prefetch_lists(b, base + (g + 1) * GROUP, tab.n[slot + GROUP]);
+        const int gr = entry_rows(__reduce_max_sync(FULL, max(n, 0)));
+        if (gr > 0) {
+            const long long s = n > 0 ? base + slot : 0;   // an idle lane reads slot 0 and adds nothing
+            const Own32 o(b, tab.inst[slot], u.step, s);
+            const uint32_t gid = mir_gid(b.D32[s]);
+            const bool fill = u.fill && o.P.noise, draw = __any_sync(FULL, o.P.noise);
+            const int *__restrict__ nb = b.nbr + entry_at(sub, s, b.rows);
+            NormalRow<float> *__restrict__ zr = (NormalRow<float> *)b.zd + (size_t)(s / GROUP) * b.rows;
+            int left = n - sub;   // this lane has an entry in row i of the present ones when i LPP < left
+            ListRows cur, next;
+            cur.load(nb, left);
+            // positions and gids of the next two rows fetched ahead: the
+            // draws start from them, the other records come meanwhile
+            int4 A[2];
+            uint32_t gj[2];
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                A[t] = b.A32[cur.e[t]];
+                gj[t] = mir_gid(b.D32[cur.e[t]]);
+            }
+            for (int r0 = 0; r0 < gr; r0 += ZR) {
+                nb += ZR * ROW;
+                next.load(nb, left - ZR * LPP);
+#pragma unroll
+                for (int i = 0; i < ZR; i += 2) {
+                    if (i && r0 + i >= gr) break;   // uniform
+                    float rx[2], ry[2], rz[2], r2[2];
+                    bool ok[2], live[2], rig[2];
+                    float4 Bj[2], Cj[2];
+                    uint32_t g2[2];
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        const int j = cur.e[i + t];
+                        Bj[t] = b.B32[j];
+                        Cj[t] = b.C32[j];
+                        live[t] = (i + t) * LPP < left;
+                        rig[t] = A[t].w == T_RIGID;
+                        ok[t] = near32(b, o, tab, slot, live[t], j, A[t], rx[t], ry[t], rz[t], r2[t]);
+                        g2[t] = gj[t];
+                    }
+#pragma unroll
+                    for (int t = 0; t < 2; ++t) {
+                        const int jn = i + 2 < ZR ? cur.e[(i + 2 + t) % ZR] : next.e[t];
+                        A[t] = b.A32[jn];
+                        gj[t] = mir_gid(b.D32[jn]);
+                    }
+                    float z[2][6] = { { 0.f, 0.f, 0.f, 0.f, 0.f, 0.f }, { 0.f, 0.f, 0.f, 0.f, 0.f, 0.f } };
+                    if (draw) {
+                        const float is2 = 0.70710678118654752440f;
+                        pair_normals2(gid, g2[0], g2[1], o.P.step, o.P.key0, o.P.key1, z[0], z[1]);
+#pragma unroll
+                        for (int t = 0; t < 2; ++t) {
+                            for (int c = 3; c < 6; ++c) z[t][c] = mul_rn(z[t][c], is2);
+                            if (fill && live[t]) {
+                                st_stream(zr[i + t].a + lane, make_float4(ok[t] ? z[t][0] : NAN, z[t][1], z[t][2], z[t][3]));
+                                st_stream(zr[i + t].b + lane, make_float2(z[t][4], z[t][5]));
+                            }
+                        }
+                    }
+#pragma unroll
+                    for (int t = 0; t < 2; ++t)
+                        pair32(b, o.P, ok[t], rig[t], cur.e[i + t], rx[t], ry[t], rz[t], r2[t], o.B, o.C, Bj[t], Cj[t],
+                               Z6<float>{ z[t][0], z[t][1], z[t][2], z[t][3], z[t][4], z[t][5] }, f);
+                }
+                cur = next;
+                left -= ZR * LPP;
+                zr += ZR;
+            }
+        }
+        tab.put(g, f);
+    }
+    tab.write(b);
+}
+
+// The second evaluation of FP32 pairs, normals from the cache.  24 bytes of
+// normals an entry are most of what the pass reads from HBM, and register
+// loads one row ahead left 1.9 MB in flight on the chip where 6.8 TB/s at a
+// microsecond want 7 MB: the pass ran at 2.2 TB/s and took 1.38 times what it
+// takes without them.  The rows of a block are contiguous, so each warp has
+// them copied into a ring in shared memory by the copy engine (PTX
+// cp.async.bulk on an mbarrier), ZR rows at a time and ZS chunks ahead, across
+// the groups it works through, at no registers or load instructions.
+constexpr int ZS = 2, ZTHREADS = 128;
+struct NormalRing {
+    NormalRow<float> z[ZS][ZR];
+    uint64_t bar[ZS];
+    uint64_t pad[16 - ZS];   // rings start on 128 bytes
+    int zrows[8];            // rows of normals of each group
+    WarpSlots tab;
+    int fill[24];
+};
+static_assert(sizeof(NormalRow<float>) == 768 && sizeof(NormalRing) % 128 == 0, "bulk copies are 16-byte aligned");
+constexpr int RING_WAIT_LIMIT = 1 << 22;
+
+__device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
+
+// Waits (bounded) for the phase of parity `par`; false when it gave up.
+__device__ __forceinline__ bool ring_wait(uint64_t *bar, unsigned par)
+{
+    const unsigned a = smem_addr(bar);
+    for (int it = 0; it < RING_WAIT_LIMIT; ++it) {
+        unsigned done;
+        asm volatile("{\n\t.reg .pred P;\n\tmbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
+                     "selp.u32 %0, 1, 0, P;\n\t}"
+                     : "=r"(done)
+                     : "r"(a), "r"(par)
+                     : "memory");
+        if (done) return true;
+    }
+    return false;
+}
+
+__global__ void __launch_bounds__(ZTHREADS, 4) k_force_cached(Bufs b, int groups)
+{
+    __shared__ __align__(128) NormalRing rings[ZTHREADS / 32];
+    const CacheUse u(b, 2);
+    if (!u.maybe) return;   // uniform over the launch
+    NormalRing &ring = rings[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31, sub = lane % LPP;
+    const unsigned FULL = 0xffffffffu;
+    if (lane == 0) {
+        for (int i = 0; i < ZS; ++i)
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(ring.bar + i)) : "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    }
+    __syncwarp();
+    const long long base = pass_base(groups);
+    WarpSlots &tab = ring.tab;
+    {
+        SlotHead mine(b, base + lane, lane < groups * GROUP);
+        if (mine.type != T_FLUID || !u.reuse(b, mine.inst)) mine.n = -1;
+        tab.set(mine);
+        // rows of each group's lists whose normals are wanted (some particle's
+        // instance has noise)
+        int rows = max(mine.n, 0), noisy = mine.n > 0 && b.inst[mine.inst].noise;
+#pragma unroll
+        for (int o = 1; o < GROUP; o <<= 1) {
+            rows = max(rows, __shfl_xor_sync(FULL, rows, o));
+            noisy |= __shfl_xor_sync(FULL, noisy, o);
+        }
+        if (lane % GROUP == 0) ring.zrows[lane / GROUP] = noisy ? entry_rows(rows) : 0;
+        __syncwarp();
+    }
+    // the copies, chunk by chunk through the groups
+    int pg = 0, pr = 0;   // next row to ask for: of group pg
+    auto request = [&](int st) {
+        while (pg < groups && pr >= ring.zrows[pg]) {
+            ++pg;
+            pr = 0;
+        }
+        if (pg >= groups) return;
+        const int have = ring.zrows[pg];
+        const unsigned bytes = (unsigned)min(ZR, have - pr) * (unsigned)sizeof(NormalRow<float>);
+        if (lane == 0) {
+            const void *src = (const NormalRow<float> *)b.zd + (size_t)(base / GROUP + pg) * b.rows + pr;
+            const unsigned bar = smem_addr(ring.bar + st);
+            asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                             smem_addr(ring.z[st])),
+                         "l"(src), "r"(bytes), "r"(bar)
+                         : "memory");
+        }
+        pr += ZR;
+    };
+    unsigned chunk = 0;   // chunks consumed: in stage chunk % ZS, its phase chunk / ZS
+    for (int i = 0; i < ZS; ++i) request(i);
+    for (int g = 0; g < groups; ++g) {
+        float f[6] = { 0.f, 0.f, 0.f, 0.f, 0.f, 0.f };
+        const int slot = g * GROUP + lane / LPP, n = tab.n[slot];
+        if (g + 1 < groups) prefetch_lists(b, base + (g + 1) * GROUP, tab.n[slot + GROUP]);
+        const int gr = entry_rows(__reduce_max_sync(FULL, max(n, 0)));
+        const bool normals = ring.zrows[g] > 0;
+        if (gr > 0) {
+            const long long s = n > 0 ? base + slot : 0;   // an idle lane reads slot 0 and adds nothing
+            const Own32 o(b, tab.inst[slot], u.step, s);
+            const int *__restrict__ nb = b.nbr + entry_at(sub, s, b.rows);
+            int left = n - sub;   // this lane has an entry in row i of the present ones when i LPP < left
+            ListRows cur, next;
+            cur.load(nb, left);
+            // the records of the next row are fetched ahead
+            int4 A = b.A32[cur.e[0]];
+            float4 B = b.B32[cur.e[0]], C = b.C32[cur.e[0]];
+            for (int r0 = 0; r0 < gr; r0 += ZR) {
+                nb += ZR * ROW;
+                next.load(nb, left - ZR * LPP);
+                const int st = chunk % ZS;
+                if (normals && !ring_wait(ring.bar + st, (chunk / ZS) & 1u)) {
+                    // give the copy one more bounded wait before its buffer is left
+                    atomicOr(b.err, ERR_TIMEOUT);
+                    (void)ring_wait(ring.bar + st, (chunk / ZS) & 1u);
+                }
+                const NormalRow<float> *zrow = ring.z[st];
+#pragma unroll
+                for (int i = 0; i < ZR; ++i) {
+                    if (i && r0 + i >= gr) break;   // uniform
+                    const int j = cur.e[i], jn = i + 1 < ZR ? cur.e[(i + 1) % ZR] : next.e[0];
+                    const int4 Aj = A;
+                    const float4 Bj = B, Cj = C;
+                    A = b.A32[jn];
+                    B = b.B32[jn];
+                    C = b.C32[jn];
+                    float rx, ry, rz, r2;
+                    const bool ok = near32(b, o, tab, slot, i * LPP < left, j, Aj, rx, ry, rz, r2);
+                    Z6<float> z{ 0.f, 0.f, 0.f, 0.f, 0.f, 0.f };
+                    if (normals) {
+                        const float4 za = zrow[i].a[lane];
+                        const float2 zb = zrow[i].b[lane];
+                        z = Z6<float>{ za.x, za.y, za.z, za.w, zb.x, zb.y };
+                        // an instance without noise has no normals, and an entry
+                        // that was beyond h in the first evaluation none yet
+                        if (ok && (!o.P.noise || is_nan(za.x))) {
+                            float t[6] = { 0.f, 0.f, 0.f, 0.f, 0.f, 0.f };
+                            if (o.P.noise)
+                                draw_rare<float>(mir_gid(b.D32[s]), mir_gid(b.D32[j]), o.P.step, o.P.key0, o.P.key1, t);
+                            z = Z6<float>{ t[0], t[1], t[2], t[3], t[4], t[5] };
+                        }
+                    }
+                    pair32(b, o.P, ok, Aj.w == T_RIGID, j, rx, ry, rz, r2, o.B, o.C, Bj, Cj, z, f);
+                }
+                if (normals) {
+                    __syncwarp();   // every lane has read the chunk
+                    request(st);
+                    ++chunk;
+                }
+                cur = next;
+                left -= ZR * LPP;
+            }
+        }
+        tab.put(g, f);
+    }
+    tab.write(b);
 }
 
 // Newton-3 force pass, phase 1: every fluid or wall particle evaluates the
@@ -2005,16 +2369,13 @@ void launch_forces(const Bufs &b, int precision, int velver, int newton3, cudaSt
             k_force_half<double, true><<<nb, bs, 0, st>>>(b, velver, groups);
             k_force_gather<double, true><<<nb, bs, 0, st>>>(b, groups);
         }
-    } else if (precision == SDPD_PREC_SPLIT && velver == 2) {
-        // the pass reading the cached normals compiled alone (no D records,
-        // no drawing code), then the drawing pass for the instances whose
-        // lists were rebuilt since
-        k_force_fluid<float, 1><<<nb, bs, 0, st>>>(b, velver, groups);
-        k_force_fluid<float, 2><<<nb, bs, 0, st>>>(b, velver, groups);
     } else if (precision == SDPD_PREC_SPLIT) {
-        k_force_fluid<float, 2><<<nb, bs, 0, st>>>(b, velver, groups);
+        // second evaluation: the pass that reads the cached normals, then the
+        // drawing pass for the instances whose lists were rebuilt since
+        if (velver == 2) k_force_cached<<<pass_blocks(b.N, ZTHREADS, groups), ZTHREADS, 0, st>>>(b, groups);
+        k_force_draw<<<nb, bs, 0, st>>>(b, velver, groups);
     } else {
-        k_force_fluid<double><<<nb, bs, 0, st>>>(b, velver, groups);
+        k_force_fluid<<<nb, bs, 0, st>>>(b, velver, groups);
     }
     if (b.nrigid) {
         const unsigned g = nblk(b.nrigid, RPB);
