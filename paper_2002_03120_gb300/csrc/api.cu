@@ -545,7 +545,7 @@ sdpd_status sdpd_init(const sdpd_params *params, int n_instances, const long lon
         b.ownA = oa; b.ownB = ob;
     }
     IALLOC(b.dsp, N);
-    IALLOC(b.aclose, N); IALLOC(b.aclose_ok, 1); IALLOC(b.sdr, N); IALLOC(b.xs, 3 * N);
+    IALLOC(b.aclose, N); IALLOC(b.aclose_ok, 1); IALLOC(b.sdr, N); IALLOC(b.side32, N); IALLOC(b.xs, 3 * N);
     const size_t ni = (size_t)n_instances + 1;
     IALLOC(b.need_build, ni); IALLOC(b.fresh, 1);
     IALLOC(b.list_epoch, ni); IALLOC(b.cache_epoch, ni); IALLOC(b.cache_step, 1);

@@ -135,48 +135,28 @@ template <> struct Rel<double> {
     }
 };
 
-// Neumaier-compensated running sum (split precision density and filter).
-struct KSum {
-    float s, c;
-    __device__ __forceinline__ void add(float v)
+// Compensated FP32 sums of two rows at a time (the halves of the packed
+// operations).
+struct Sum2 {
+    F2 s, c;
+    // both halves start from v0; value() takes one of them off again
+    __device__ __forceinline__ explicit Sum2(float v0) : s(v0), c(0.0f) {}
+    // terms v with 0 <= v <= v0, so that |s| >= |v| at every step (Dekker's
+    // fast two-sum error term)
+    __device__ __forceinline__ void add_small(F2 v)
     {
-        const float t = s + v;
-        c += (fabsf(s) >= fabsf(v)) ? ((s - t) + v) : ((v - t) + s);
+        const F2 t = add2(s, v);
+        c = add2(c, add2(fma2(t, F2(-1.0f), s), v));
         s = t;
     }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-template <class R> struct Acc;
-template <> struct Acc<float> {
-    KSum k;
-    __device__ __forceinline__ explicit Acc(double v0) : k{ (float)v0, 0.f } {}
-    __device__ __forceinline__ void add(float v) { k.add(v); }
-    __device__ __forceinline__ double value() const { return k.value(); }
-};
-// The density sum: every term is W(q) <= W(0), and the sum starts at the
-// self term W(0), so |s| >= |v| at every step and the compensation needs no
-// branch (Dekker's fast two-sum error term; the same result as KSum there).
-template <class R> struct PosAcc;
-template <> struct PosAcc<float> {
-    float s, c;
-    __device__ __forceinline__ explicit PosAcc(double v0) : s((float)v0), c(0.f) {}
-    __device__ __forceinline__ void add(float v)
+    // any terms (Knuth's two-sum)
+    __device__ __forceinline__ void add_any(F2 v)
     {
-        const float t = s + v;
-        c += (s - t) + v;
+        const F2 t = add2(s, v), z = fma2(s, F2(-1.0f), t);
+        const F2 es = fma2(fma2(z, F2(-1.0f), t), F2(-1.0f), s), ev = fma2(z, F2(-1.0f), v);
+        c = add2(c, add2(es, ev));
         s = t;
     }
-    __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-template <> struct Acc<double> {
-    double s;
-    __device__ __forceinline__ explicit Acc(double v0) : s(v0) {}
-    // a separate rounding of each term (no multiply-add fused into the sum)
-    __device__ __forceinline__ void add(double v) { s = __dadd_rn(s, v); }
-    __device__ __forceinline__ double value() const { return s; }
-};
-template <> struct PosAcc<double> : Acc<double> {
-    using Acc<double>::Acc;
 };
 
 // Eq. prtcpres: p = p0 (rho / rho0)^alpha - beta; an integer alpha (7 in
@@ -323,17 +303,22 @@ __device__ __forceinline__ bool lanes_any(bool v)
     const unsigned m = __ballot_sync(0xffffffffu, v);
     return (m >> ((threadIdx.x & 31) & ~(LPP - 1))) & ((1u << LPP) - 1u);
 }
-// FP32 compensated sums: s + c over the lanes, error terms kept (Knuth's
-// two-sum, no ordering of the operands assumed)
-__device__ __forceinline__ void lanes_sum(float &s, float &c)
+// FP32 compensated sums: both halves over the lanes of a particle, error terms
+// kept (Knuth's two-sum, no ordering of the operands assumed)
+__device__ __forceinline__ void join(float &s, float &c, float s2, float c2)
 {
+    const float t = __fadd_rn(s, s2), z = __fsub_rn(t, s);
+    c = __fadd_rn(__fadd_rn(c, c2), __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(s2, z)));
+    s = t;
+}
+__device__ __forceinline__ void lanes_sum(const Sum2 &v, float &s, float &c)
+{
+    float s2, c2;
+    v.s.get(s, s2);
+    v.c.get(c, c2);
+    join(s, c, s2, c2);
 #pragma unroll
-    for (int o = 1; o < LPP; o <<= 1) {
-        const float s2 = __shfl_xor_sync(0xffffffffu, s, o), c2 = __shfl_xor_sync(0xffffffffu, c, o);
-        const float t = s + s2, z = t - s;
-        c = (c + c2) + ((s - (t - z)) + (s2 - z));
-        s = t;
-    }
+    for (int o = 1; o < LPP; o <<= 1) join(s, c, __shfl_xor_sync(0xffffffffu, s, o), __shfl_xor_sync(0xffffffffu, c, o));
 }
 
 // ------------------------------------------------------------------ density
@@ -383,44 +368,48 @@ __device__ __forceinline__ void finish_density(const Bufs &b, const Inst &I, int
     b.aclose[s] = close ? 1 : 0;
     b.sd[s] = d;
     b.sp[s] = p;
+    // (defer: bit 0 the pressure filter follows, bit 1 the reinitialisation)
+    if (sizeof(R) == 4 && defer) b.side32[s] = defer & 2 ? (float)d : (float)p;
     if (!defer) {
         b.sp2[s] = p;
         finalize_slot<R>(b, s, d, p);
     }
 }
 
-// The kernel sum of the entries [k0, n) of slot s on this lane; close: a
+// The FP64 kernel sum of the entries [k0, n) of slot s on this lane; close: a
 // mobile neighbour inside the collision radius of the artificial viscosity (a
 // superset: the collision pass decides exactly; CLOSE: some instance of the
 // context has it)
-template <class R, bool CLOSE, class ACC>
-__device__ __forceinline__ void density_entries(const Bufs &b, const Inst &I, long long s, int gi, int ti, int k0,
-                                                int n, int sub, const ListHead &hd, ACC &acc, bool &close)
+template <bool CLOSE>
+__device__ __forceinline__ double density_entries(const Bufs &b, const Inst &I, long long s, int gi, int ti, int k0,
+                                                  int n, int sub, bool &close)
 {
     const bool want_close = CLOSE && I.artvis && (ti == T_FLUID || ti == T_RIGID);
-    const R close_r2 = (R)(I.artvis_r2f_hi * 1.0001f);
-    const auto *A = Mir<R>::A(b);
-    const auto Ai = A[s];
-    const Geo<R> geo(I);
-    const R Wc = K<R>::Wc(I), irc = K<R>::inv_rc(I);
-    for_each_entry(b.nbr, s, b.rows, k0, n, sub, hd, A, nullptr, [&](int, uint32_t e, const decltype(Ai) &Aj, double) {
+    const double close_r2 = (double)(I.artvis_r2f_hi * 1.0001f);
+    const double4_32a *A = b.A64;
+    const double4_32a Ai = A[s];
+    const Geo<double> geo(I);
+    const double Wc = I.Wc, irc = I.inv_rc;
+    double acc = 0.0;
+    for_each_entry(b.nbr, s, b.rows, k0, n, sub, ListHead(b.nbr, s, b.rows, k0, n, sub), A, nullptr,
+                   [&](int, uint32_t e, const double4_32a &Aj, double) {
         if (e & NB_FAR) return;
-        R rx, ry, rz, r2;
-        if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) return;
+        double rx, ry, rz, r2;
+        if (!Rel<double>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) return;
         if (CLOSE && want_close && r2 <= close_r2) {
             const int tj = mir_type(Aj);
             close |= (tj == T_FLUID || tj == T_RIGID);
         }
-        // float: correctly rounded sqrt
-        R r = 0, ir;
-        if constexpr (sizeof(R) == 4) r = sqrtf(r2);
-        else root_and_inverse(r2, r, ir);
-        const R q = r * irc, om = one_minus(q);
-        acc.add(Wc * (R(1) + R(3) * q) * om * om * om);
+        double r, ir;
+        root_and_inverse(r2, r, ir);
+        const double q = r * irc, om = one_minus(q);
+        // a separate rounding of each term (no multiply-add fused into the sum)
+        acc = __dadd_rn(acc, Wc * (1.0 + 3.0 * q) * om * om * om);
     });
+    return acc;
 }
 
-template <class R, bool CLOSE>
+template <bool CLOSE>
 __global__ void __launch_bounds__(256) k_density(Bufs b, int defer, const int *gate, int groups)
 {
     if (gate && *gate == 0) return;
@@ -428,60 +417,28 @@ __global__ void __launch_bounds__(256) k_density(Bufs b, int defer, const int *g
     const long long base = pass_base(groups);
     if (base == 0 && lane == 0) *b.aclose_ok = 1;   // the marks below are for these positions
     const SlotHead mine(b, base + lane, lane < groups * GROUP);
-    SlotHead h = mine.of_group(0);
-    ListHead hd(b.nbr, base + lane / LPP, b.rows, 0, h.type == T_OUTER ? 0 : h.n, sub);
-    R ks = 0, kc = 0;
+    double kown = 0.0, koth = 0.0;
     int kclose = 0;
     for (int g = 0; g < groups; ++g) {
         const long long s = base + g * GROUP + lane / LPP;
-        SlotHead hn;
-        ListHead hdn;
-        if (g + 1 < groups) {
-            hn = mine.of_group(g + 1);
-            hdn = ListHead(b.nbr, s + GROUP, b.rows, 0, hn.type == T_OUTER ? 0 : hn.n, sub);
-            prefetch_lists(b, base + (g + 1) * GROUP, hn.type == T_OUTER ? 0 : hn.n);
-        }
+        const SlotHead h = mine.of_group(g);
         bool close = false;
-        R sum = 0, comp = 0;
+        double own = 0.0, oth = 0.0;
         if (h.type != T_OUTER) {
+            // the owned and the other entries apart, as the half-pair form
+            // sums them (the same additions)
             const Inst &I = b.inst[h.inst];
-            if constexpr (sizeof(R) == 4) {
-                // every lane starts from W(0) (PosAcc wants |sum| >= |term|);
-                // all but one of them are taken off below
-                PosAcc<R> acc(I.W0);
-                density_entries<R, CLOSE>(b, I, s, h.gi, h.type, 0, h.n, sub, hd, acc, close);
-                sum = acc.s;
-                comp = acc.c;
-            } else {
-                // the owned and the other entries apart, as the half-pair
-                // form sums them (the same additions)
-                PosAcc<R> own(0.0), oth(0.0);
-                density_entries<R, CLOSE>(b, I, s, h.gi, h.type, 0, h.nf, sub, hd, own, close);
-                density_entries<R, CLOSE>(b, I, s, h.gi, h.type, h.nf, h.n, sub,
-                                          ListHead(b.nbr, s, b.rows, h.nf, h.n, sub), oth, close);
-                sum = own.s;
-                comp = oth.s;
-            }
+            own = density_entries<CLOSE>(b, I, s, h.gi, h.type, 0, h.nf, sub, close);
+            oth = density_entries<CLOSE>(b, I, s, h.gi, h.type, h.nf, h.n, sub, close);
         }
-        if constexpr (sizeof(R) == 4) {
-            lanes_sum(sum, comp);
-        } else {
-            sum = lanes_sum(sum);
-            comp = lanes_sum(comp);
-        }
-        keep_group(sum, g, ks);
-        keep_group(comp, g, kc);
+        keep_group(lanes_sum(own), g, kown);
+        keep_group(lanes_sum(oth), g, koth);
         if constexpr (CLOSE) keep_group((int)lanes_any(close), g, kclose);
-        h = hn;
-        hd = hdn;
     }
     const long long s = base + lane;
     if (lane >= groups * GROUP || s >= b.N) return;
     const Inst &I = b.inst[mine.inst];
-    double v;
-    if constexpr (sizeof(R) == 4) v = ((double)ks - (double)(LPP - 1) * (double)(float)I.W0) + (double)kc;
-    else v = __dadd_rn(__dadd_rn(I.W0, ks), kc);
-    finish_density<R>(b, I, mine.type, s, v, kclose, defer);
+    finish_density<double>(b, I, mine.type, s, __dadd_rn(__dadd_rn(I.W0, kown), koth), kclose, defer);
 }
 
 // FP64 density with each unordered pair evaluated once (Newton 3): phase 1
@@ -599,163 +556,258 @@ __global__ void __launch_bounds__(256) k_density_gather(Bufs b, int defer, const
 // theirs; the pressure follows from Eq. prtcpres.  The new densities go to
 // sdr (the neighbours' old values are still read) and k_reinit_copy moves
 // them back.
-// A ratio of two kernel sums over the list of slot s: totals on every lane of
-// the particle (FP32: compensated, the FP64 ratio from both parts).
-template <class R> struct TwoSums;
-template <> struct TwoSums<float> {
-    KSum num{ 0.f, 0.f }, den{ 0.f, 0.f };
-    float ks[4] = { 0.f, 0.f, 0.f, 0.f };
-    __device__ __forceinline__ void add(float a, float b) { num.add(a); den.add(b); }
-    __device__ __forceinline__ void close_group(int g)
-    {
-        lanes_sum(num.s, num.c);
-        lanes_sum(den.s, den.c);
-        keep_group(num.s, g, ks[0]);
-        keep_group(num.c, g, ks[1]);
-        keep_group(den.s, g, ks[2]);
-        keep_group(den.c, g, ks[3]);
-        num = KSum{ 0.f, 0.f };
-        den = KSum{ 0.f, 0.f };
-    }
-    __device__ __forceinline__ double ratio(double a0, double b0) const
-    {
-        return (a0 + ((double)ks[0] + (double)ks[1])) / (b0 + ((double)ks[2] + (double)ks[3]));
-    }
-};
-template <> struct TwoSums<double> {
-    double num = 0.0, den = 0.0, ks[2] = { 0.0, 0.0 };
-    // a separate rounding of each term (no multiply-add fused into the sum)
-    __device__ __forceinline__ void add(double a, double b) { num = __dadd_rn(num, a); den = __dadd_rn(den, b); }
-    __device__ __forceinline__ void close_group(int g)
-    {
-        keep_group(lanes_sum(num), g, ks[0]);
-        keep_group(lanes_sum(den), g, ks[1]);
-        num = den = 0.0;
-    }
-    __device__ __forceinline__ double ratio(double a0, double b0) const { return (a0 + ks[0]) / (b0 + ks[1]); }
-};
-
-// The kernel weight of a listed pair within h, for the two Shepard averages.
-template <class R>
-__device__ __forceinline__ R shepard_weight(const Inst &I, R r2)
+// The FP64 ratio of two kernel sums over the list of slot s (on all lanes of
+// the particle): numerator and denominator of the two Shepard averages.
+template <bool REINIT>
+__device__ __forceinline__ void shepard_entries(const Bufs &b, const Inst &I, long long s, const SlotHead &h, int sub,
+                                                double &num, double &den)
 {
-    R r = 0, ir;
-    if constexpr (sizeof(R) == 4) r = sqrtf(r2);
-    else root_and_inverse(r2, r, ir);
-    const R q = r * K<R>::inv_rc(I), om = one_minus(q);
-    return K<R>::Wc(I) * (R(1) + R(3) * q) * om * om * om;
+    const double4_32a *A = b.A64;
+    const double4_32a Ai = A[s];
+    const Geo<double> geo(I);
+    for_each_entry(b.nbr, s, b.rows, 0, h.n, sub, ListHead(b.nbr, s, b.rows, 0, h.n, sub), A, REINIT ? b.sd : b.sp,
+                   [&](int, uint32_t e, const double4_32a &Aj, double v) {
+        if (e & NB_FAR) return;
+        double rx, ry, rz, r2, r, ir;
+        if (!Rel<double>::get(b, I, geo, Ai, Aj, h.gi, (int)e, rx, ry, rz, r2)) return;
+        root_and_inverse(r2, r, ir);
+        const double q = r * I.inv_rc, om = one_minus(q);
+        const double W = I.Wc * (1.0 + 3.0 * q) * om * om * om;
+        // a separate rounding of each term (no multiply-add fused into the sum)
+        num = __dadd_rn(num, REINIT ? W : __dmul_rn(v, W));
+        den = __dadd_rn(den, REINIT ? __ddiv_rn(W, v) : W);
+    });
 }
 
-template <class R>
-__global__ void __launch_bounds__(256) k_reinit(Bufs b, int any_filter, const int *gate, int groups)
+// What the two averages do with their sums: reinitialised density and
+// pressure, or filtered pressure.
+template <class R, bool REINIT>
+__device__ __forceinline__ void finish_shepard(const Bufs &b, const Inst &I, int type, long long s, double num, double den,
+                                               int any_filter)
+{
+    const bool on = (REINIT ? I.reinit : I.filter) && type != T_OUTER;
+    if constexpr (REINIT) {
+        const double di = b.sd[s];
+        const double d = on ? (I.W0 + num) / (I.W0 / di + den) : di;
+        double p = eos_pressure(I, I.mf * d);
+        if (I.clamp && p < 0.0) p = 0.0;
+        b.sdr[s] = d;
+        if (I.reinit) b.sp[s] = p;
+        if (!any_filter) {
+            b.sp2[s] = b.sp[s];
+            finalize_slot<R>(b, s, d, b.sp[s]);
+        }
+    } else {
+        const double pi = b.sp[s];
+        const double pf = on ? (pi * I.W0 + num) / (I.W0 + den) : pi;
+        b.sp2[s] = pf;
+        finalize_slot<R>(b, s, b.sd[s], pf);
+    }
+}
+
+template <bool REINIT>
+__global__ void __launch_bounds__(256) k_shepard(Bufs b, int any_filter, const int *gate, int groups)
 {
     if (gate && *gate == 0) return;
     const int lane = threadIdx.x & 31, sub = lane % LPP;
     const long long base = pass_base(groups);
     const SlotHead mine(b, base + lane, lane < groups * GROUP);
-    SlotHead h = mine.of_group(0);
-    ListHead hd(b.nbr, base + lane / LPP, b.rows, 0, h.type == T_OUTER ? 0 : h.n, sub);
-    TwoSums<R> sums;
+    double knum = 0.0, kden = 0.0;
     for (int g = 0; g < groups; ++g) {
-        const long long s = base + g * GROUP + lane / LPP;
-        SlotHead hn;
-        ListHead hdn;
-        if (g + 1 < groups) {
-            hn = mine.of_group(g + 1);
-            hdn = ListHead(b.nbr, s + GROUP, b.rows, 0, hn.type == T_OUTER ? 0 : hn.n, sub);
-            prefetch_lists(b, base + (g + 1) * GROUP, hn.type == T_OUTER ? 0 : hn.n);
-        }
-        if (h.type != T_OUTER) {
-            const int gi = h.gi;
-            const Inst &I = b.inst[h.inst];
-            if (I.reinit) {
-                const auto *A = Mir<R>::A(b);
-                const auto Ai = A[s];
-                const Geo<R> geo(I);
-                for_each_entry(b.nbr, s, b.rows, 0, h.n, sub, hd, A, b.sd,
-                               [&](int, uint32_t e, const decltype(Ai) &Aj, double dj) {
-                    if (e & NB_FAR) return;
-                    R rx, ry, rz, r2;
-                    if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) return;
-                    const R W = shepard_weight<R>(I, r2);
-                    sums.add(W, W / (R)dj);
-                });
-            }
-        }
-        sums.close_group(g);
-        h = hn;
-        hd = hdn;
+        const SlotHead h = mine.of_group(g);
+        const Inst &I = b.inst[h.inst];
+        double num = 0.0, den = 0.0;
+        if (h.type != T_OUTER && (REINIT ? I.reinit : I.filter))
+            shepard_entries<REINIT>(b, I, base + g * GROUP + lane / LPP, h, sub, num, den);
+        keep_group(lanes_sum(num), g, knum);
+        keep_group(lanes_sum(den), g, kden);
     }
     const long long s = base + lane;
     if (lane >= groups * GROUP || s >= b.N) return;
-    const Inst &I = b.inst[mine.inst];
-    const double di = b.sd[s];
-    const double d = I.reinit && mine.type != T_OUTER ? sums.ratio(I.W0, I.W0 / di) : di;
-    double p = eos_pressure(I, I.mf * d);
-    if (I.clamp && p < 0.0) p = 0.0;
-    b.sdr[s] = d;
-    if (I.reinit) b.sp[s] = p;
-    if (!any_filter) {
-        b.sp2[s] = b.sp[s];
-        finalize_slot<R>(b, s, d, b.sp[s]);
-    }
+    finish_shepard<double, REINIT>(b, b.inst[mine.inst], mine.type, s, knum, kden, any_filter);
 }
+
 
 __global__ void k_reinit_copy(Bufs b, const int *gate)
 {
     if (gate && *gate == 0) return;
     const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (s < b.N) b.sd[s] = b.sdr[s];
+    if (s >= b.N) return;
+    b.sd[s] = b.sdr[s];
+    if (b.side32) b.side32[s] = (float)b.sp[s];   // for the pressure filter
 }
 
-// ------------------------------------------------------------ pressure filter
-template <class R>
-__global__ void __launch_bounds__(256) k_filter(Bufs b, const int *gate, int groups)
+// The r < h decision of a pair in the guard band, out of line: it is rare,
+// and its FP64 code would cost the pair loop registers.
+__device__ __noinline__ bool within_exactly(const Bufs &b, int inst, int gi, int j)
+{
+    return exact_within(b, b.inst[inst], gi, b.perm[j]);
+}
+
+// The loops below take ZR rows at a time, unrolled, so that a row costs no
+// counters and no moves between registers.  Lists: a lane's ZR entries of the
+// next rows are fetched while the present ones are evaluated (a lane without
+// an entry reads record 0 and adds nothing).
+constexpr int ZR = 4;
+struct ListRows {
+    int e[ZR];
+    // (nb: this lane's entry of the first of the rows, n: entries left from it on)
+    __device__ __forceinline__ void load(const int *nb, int n)
+    {
+#pragma unroll
+        for (int i = 0; i < ZR; ++i) e[i] = i * LPP < n ? ld_stream(nb + i * ROW) : 0;
+    }
+};
+
+// ---------------------------------- density and Shepard averages, FP32
+// These passes are a list walk with little arithmetic a pair: bound by issue
+// slots.  The 8 lanes of a particle take ZR rows at a time, unrolled, two rows
+// in the halves of the packed operations: 52 instructions an entry where one
+// entry at a time with branches and a library square root took 80, and 0.40
+// ms where that took 0.65 (662,305 particles).
+//
+// f(W, j0, j1, ok0, ok1, r2_0, r2_1, type0, type1) sees the kernel weights of
+// two entries (0 for an entry past the end, beyond h or of contact range only).
+template <class F>
+__device__ __forceinline__ void weights32(const Bufs &b, const Inst &I, const SlotHead &h, long long s, int n, int gr,
+                                          int sub, F &&f)
+{
+    const Geo<float> geo(I);
+    const F2 u0(geo.u0), u1(geo.u1), u2(geo.u2), irc(I.inv_rcf), Wc(I.Wcf), one(1.0f), minus(-1.0f);
+    const float beyond = 4.0f * geo.ghi;   // stands for r^2 of an entry left out: W = 0
+    const int4 Ai = b.A32[s];
+    const int *__restrict__ nb = b.nbr + entry_at(sub, s, b.rows);
+    int left = n - sub;   // this lane has an entry in row i of the present ones when i LPP < left
+    ListRows cur, next;
+    cur.load(nb, left);
+    int4 A[2] = { b.A32[cur.e[0] & ~NB_FAR], b.A32[cur.e[1] & ~NB_FAR] };   // two rows ahead
+    for (int r0 = 0; r0 < gr; r0 += ZR) {
+        nb += ZR * ROW;
+        next.load(nb, left - ZR * LPP);
+#pragma unroll
+        for (int i = 0; i < ZR; i += 2) {
+            if (i && r0 + i >= gr) break;   // uniform
+            const int e0 = cur.e[i], e1 = cur.e[i + 1];
+            const int4 A0 = A[0], A1 = A[1];
+            A[0] = b.A32[(i + 2 < ZR ? cur.e[(i + 2) % ZR] : next.e[0]) & ~NB_FAR];
+            A[1] = b.A32[(i + 2 < ZR ? cur.e[(i + 3) % ZR] : next.e[1]) & ~NB_FAR];
+            const F2 rx = mul2(F2((float)fixed_diff(Ai.x, A0.x), (float)fixed_diff(Ai.x, A1.x)), u0);
+            const F2 ry = mul2(F2((float)fixed_diff(Ai.y, A0.y), (float)fixed_diff(Ai.y, A1.y)), u1);
+            const F2 rz = mul2(F2((float)fixed_diff(Ai.z, A0.z), (float)fixed_diff(Ai.z, A1.z)), u2);
+            float a0, a1;
+            fma2(rz, rz, fma2(ry, ry, mul2(rx, rx))).get(a0, a1);
+            bool ok0 = i * LPP < left && e0 >= 0 && a0 < geo.ghi, ok1 = (i + 1) * LPP < left && e1 >= 0 && a1 < geo.ghi;
+            if (ok0 && a0 >= geo.glo) ok0 = within_exactly(b, h.inst, h.gi, e0);
+            if (ok1 && a1 >= geo.glo) ok1 = within_exactly(b, h.inst, h.gi, e1);
+            // (coincident particles: r = 0 and W = W(0), not 0 times infinity)
+            const float c0 = ok0 ? fmaxf(a0, 1.2e-38f) : beyond, c1 = ok1 ? fmaxf(a1, 1.2e-38f) : beyond;
+            // sqrt by Newton's iteration from the hardware reciprocal root:
+            // s + (x - s^2) y / 2, within an ulp's half but for rare ties
+            const F2 x(c0, c1), y(rsqrt_ftz(c0), rsqrt_ftz(c1));
+            const F2 t = mul2(x, y), e = fma2(mul2(t, minus), t, x);
+            const F2 q = mul2(fma2(e, mul2(y, F2(0.5f)), t), irc);
+            float m0, m1;
+            fma2(q, minus, one).get(m0, m1);
+            const F2 om(fmaxf(m0, 0.0f), fmaxf(m1, 0.0f));
+            const F2 W = mul2(mul2(mul2(mul2(Wc, fma2(q, F2(3.0f), one)), om), om), om);
+            f(W, e0 & ~NB_FAR, e1 & ~NB_FAR, ok0, ok1, a0, a1, A0.w, A1.w);
+        }
+        cur = next;
+        left -= ZR * LPP;
+    }
+}
+
+template <bool CLOSE>
+__global__ void __launch_bounds__(256) k_density32(Bufs b, int defer, const int *gate, int groups)
 {
     if (gate && *gate == 0) return;
     const int lane = threadIdx.x & 31, sub = lane % LPP;
+    const unsigned FULL = 0xffffffffu;
     const long long base = pass_base(groups);
-    const SlotHead mine(b, base + lane, lane < groups * GROUP);
-    SlotHead h = mine.of_group(0);
-    ListHead hd(b.nbr, base + lane / LPP, b.rows, 0, h.type == T_OUTER ? 0 : h.n, sub);
-    TwoSums<R> sums;
+    if (base == 0 && lane == 0) *b.aclose_ok = 1;   // the marks below are for these positions
+    SlotHead mine(b, base + lane, lane < groups * GROUP);
+    if (mine.type == T_OUTER) mine.n = 0;
+    float ks = 0.f, kc = 0.f;
+    int kclose = 0;
     for (int g = 0; g < groups; ++g) {
-        const long long s = base + g * GROUP + lane / LPP;
-        SlotHead hn;
-        ListHead hdn;
-        if (g + 1 < groups) {
-            hn = mine.of_group(g + 1);
-            hdn = ListHead(b.nbr, s + GROUP, b.rows, 0, hn.type == T_OUTER ? 0 : hn.n, sub);
-            prefetch_lists(b, base + (g + 1) * GROUP, hn.type == T_OUTER ? 0 : hn.n);
+        const SlotHead h = mine.of_group(g);
+        if (g + 1 < groups) prefetch_lists(b, base + (g + 1) * GROUP, mine.of_group(g + 1).n);
+        const int gr = entry_rows(__reduce_max_sync(FULL, max(h.n, 0)));
+        const Inst &I = b.inst[h.inst];
+        const float W0 = (float)I.W0;
+        Sum2 sum(W0);
+        bool close = false;
+        if (gr > 0) {
+            const bool want_close = CLOSE && I.artvis && (h.type == T_FLUID || h.type == T_RIGID);
+            const float close_r2 = want_close ? I.artvis_r2f_hi * 1.0001f : -1.0f;
+            const long long s = h.n > 0 ? base + g * GROUP + lane / LPP : 0;
+            weights32(b, I, h, s, h.n, gr, sub,
+                      [&](F2 W, int, int, bool ok0, bool ok1, float r0, float r1, int t0, int t1) {
+                sum.add_small(W);
+                if (CLOSE) {
+                    close |= ok0 && r0 <= close_r2 && (t0 == T_FLUID || t0 == T_RIGID);
+                    close |= ok1 && r1 <= close_r2 && (t1 == T_FLUID || t1 == T_RIGID);
+                }
+            });
         }
-        if (h.type != T_OUTER) {
-            const int gi = h.gi;
-            const Inst &I = b.inst[h.inst];
-            if (I.filter) {
-                const auto *A = Mir<R>::A(b);
-                const auto Ai = A[s];
-                const Geo<R> geo(I);
-                for_each_entry(b.nbr, s, b.rows, 0, h.n, sub, hd, A, b.sp,
-                               [&](int, uint32_t e, const decltype(Ai) &Aj, double pj) {
-                    if (e & NB_FAR) return;
-                    R rx, ry, rz, r2;
-                    if (!Rel<R>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) return;
-                    const R W = shepard_weight<R>(I, r2);
-                    sums.add((R)pj * W, W);
-                });
-            }
-        }
-        sums.close_group(g);
-        h = hn;
-        hd = hdn;
+        float ss, cc;
+        lanes_sum(sum, ss, cc);
+        keep_group(ss, g, ks);
+        keep_group(cc, g, kc);
+        if constexpr (CLOSE) keep_group((int)lanes_any(close), g, kclose);
     }
     const long long s = base + lane;
     if (lane >= groups * GROUP || s >= b.N) return;
     const Inst &I = b.inst[mine.inst];
-    const double pi = b.sp[s];
-    const double pf = I.filter && mine.type != T_OUTER ? sums.ratio(pi * I.W0, I.W0) : pi;
-    b.sp2[s] = pf;
-    finalize_slot<R>(b, s, b.sd[s], pf);
+    // the sum held W(0) once in each half of each lane
+    const double v = ((double)ks - (double)(2 * LPP - 1) * (double)(float)I.W0) + (double)kc;
+    finish_density<float>(b, I, mine.type, s, v, kclose, defer);
+}
+
+template <bool REINIT>
+__global__ void __launch_bounds__(256) k_shepard32(Bufs b, int any_filter, const int *gate, int groups)
+{
+    if (gate && *gate == 0) return;
+    const int lane = threadIdx.x & 31, sub = lane % LPP;
+    const unsigned FULL = 0xffffffffu;
+    const long long base = pass_base(groups);
+    SlotHead mine(b, base + lane, lane < groups * GROUP);
+    if (mine.type == T_OUTER || !(REINIT ? b.inst[mine.inst].reinit : b.inst[mine.inst].filter)) mine.n = 0;
+    float kn[2] = { 0.f, 0.f }, kd[2] = { 0.f, 0.f };
+    for (int g = 0; g < groups; ++g) {
+        const SlotHead h = mine.of_group(g);
+        if (g + 1 < groups) prefetch_lists(b, base + (g + 1) * GROUP, mine.of_group(g + 1).n);
+        const int gr = entry_rows(__reduce_max_sync(FULL, max(h.n, 0)));
+        Sum2 num(0.0f), den(0.0f);
+        if (gr > 0) {
+            const Inst &I = b.inst[h.inst];
+            const long long s = h.n > 0 ? base + g * GROUP + lane / LPP : 0;
+            weights32(b, I, h, s, h.n, gr, sub,
+                      [&](F2 W, int j0, int j1, bool ok0, bool ok1, float, float, int, int) {
+                float v0 = b.side32[j0], v1 = b.side32[j1];
+                if constexpr (REINIT) {
+                    float w0, w1;
+                    W.get(w0, w1);
+                    num.add_any(W);
+                    den.add_any(F2(ok0 ? w0 / v0 : 0.f, ok1 ? w1 / v1 : 0.f));
+                } else {
+                    num.add_any(mul2(F2(v0, v1), W));
+                    den.add_any(W);
+                }
+            });
+        }
+        float ss, cc;
+        lanes_sum(num, ss, cc);
+        keep_group(ss, g, kn[0]);
+        keep_group(cc, g, kn[1]);
+        lanes_sum(den, ss, cc);
+        keep_group(ss, g, kd[0]);
+        keep_group(cc, g, kd[1]);
+    }
+    const long long s = base + lane;
+    if (lane >= groups * GROUP || s >= b.N) return;
+    finish_shepard<float, REINIT>(b, b.inst[mine.inst], mine.type, s, (double)kn[0] + (double)kn[1],
+                                  (double)kd[0] + (double)kd[1], any_filter);
 }
 
 // ---------------------------------------------------------------- drag (A5)
@@ -1289,13 +1341,6 @@ __global__ void __launch_bounds__(256) k_force_fluid(Bufs b, int velver, int gro
 }
 
 // ------------------------------------------------- direct force pass, FP32
-// The r < h decision of a pair in the guard band, out of line: it is rare,
-// and its FP64 code would cost the pair loop registers.
-__device__ __noinline__ bool within_exactly(const Bufs &b, int inst, int gi, int j)
-{
-    return exact_within(b, b.inst[inst], gi, b.perm[j]);
-}
-
 // One listed pair (i, j) of the FP32 direct pass, added to i's sums where `ok`
 // (within h).  Every lane runs the same straight line: an entry past the end
 // or beyond h is left out of the sums at the end, and a sphere partner
@@ -1347,21 +1392,6 @@ __device__ __forceinline__ void pair32(const Bufs &b, const PairK<float> &P, boo
         f[5] = add_rn(f[5], hz);
     }
 }
-
-// The loops below take ZR rows at a time, unrolled, so that a row costs no
-// counters and no moves between registers.  Lists: a lane's ZR entries of the
-// next rows are fetched while the present ones are evaluated (a lane without
-// an entry reads record 0 and adds nothing).
-constexpr int ZR = 4;
-struct ListRows {
-    int e[ZR];
-    // (nb: this lane's entry of the first of the rows, n: entries left from it on)
-    __device__ __forceinline__ void load(const int *nb, int n)
-    {
-#pragma unroll
-        for (int i = 0; i < ZR; ++i) e[i] = i * LPP < n ? ld_stream(nb + i * ROW) : 0;
-    }
-};
 
 // A warp's particles and their totals, in shared memory: registers are what
 // these two kernels are short of.
@@ -2295,42 +2325,34 @@ static int pass_groups(long long N)
 // Blocks of `block` threads that cover N particles at `groups` groups a warp.
 static unsigned pass_blocks(long long N, int block, int groups) { return nblk(N, block / 32 * GROUP * groups); }
 
-template <class R>
-static void launch_density_tail(const Bufs &b, int any_filter, int any_reinit, const int *gate, int groups,
-                                cudaStream_t st)
-{
-    const int bs = b.pair_block;
-    const unsigned nb = pass_blocks(b.N, bs, groups);
-    if (any_reinit) {
-        k_reinit<R><<<nb, bs, 0, st>>>(b, any_filter, gate, groups);
-        k_reinit_copy<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
-    }
-    if (any_filter) k_filter<R><<<nb, bs, 0, st>>>(b, gate, groups);
-}
-
 void launch_density(const Bufs &b, int precision, int dflags, int newton3, const int *gate, cudaStream_t st)
 {
     if (!b.N) return;
     const int any_filter = dflags & 1, any_reinit = (dflags >> 1) & 1, any_artvis = (dflags >> 2) & 1;
     // the density kernels leave the mirrors to a later pass when one follows
-    const int defer = any_filter | any_reinit;
+    const int defer = any_filter | (any_reinit << 1);
     const int groups = pass_groups(b.N), bs = b.pair_block;
     const unsigned nb = pass_blocks(b.N, bs, groups);
     if (precision == SDPD_PREC_SPLIT) {
-        if (any_artvis) k_density<float, true><<<nb, bs, 0, st>>>(b, defer, gate, groups);
-        else k_density<float, false><<<nb, bs, 0, st>>>(b, defer, gate, groups);
-        launch_density_tail<float>(b, any_filter, any_reinit, gate, groups, st);
-        return;
-    }
-    if (newton3) {
-        k_density_half<<<nb, bs, 0, st>>>(b, gate, groups);
-        k_density_gather<<<nb, bs, 0, st>>>(b, defer, gate, groups);
-    } else if (any_artvis) {
-        k_density<double, true><<<nb, bs, 0, st>>>(b, defer, gate, groups);
+        if (any_artvis) k_density32<true><<<nb, bs, 0, st>>>(b, defer, gate, groups);
+        else k_density32<false><<<nb, bs, 0, st>>>(b, defer, gate, groups);
+        if (any_reinit) k_shepard32<true><<<nb, bs, 0, st>>>(b, any_filter, gate, groups);
     } else {
-        k_density<double, false><<<nb, bs, 0, st>>>(b, defer, gate, groups);
+        if (newton3) {
+            k_density_half<<<nb, bs, 0, st>>>(b, gate, groups);
+            k_density_gather<<<nb, bs, 0, st>>>(b, defer, gate, groups);
+        } else if (any_artvis) {
+            k_density<true><<<nb, bs, 0, st>>>(b, defer, gate, groups);
+        } else {
+            k_density<false><<<nb, bs, 0, st>>>(b, defer, gate, groups);
+        }
+        if (any_reinit) k_shepard<true><<<nb, bs, 0, st>>>(b, any_filter, gate, groups);
     }
-    launch_density_tail<double>(b, any_filter, any_reinit, gate, groups, st);
+    if (any_reinit) k_reinit_copy<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
+    if (any_filter) {
+        if (precision == SDPD_PREC_SPLIT) k_shepard32<false><<<nb, bs, 0, st>>>(b, 0, gate, groups);
+        else k_shepard<false><<<nb, bs, 0, st>>>(b, 0, gate, groups);
+    }
 }
 
 void launch_drag(const Bufs &b, int precision, cudaStream_t st)
