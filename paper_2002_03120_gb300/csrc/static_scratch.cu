@@ -39,7 +39,7 @@ static __device__ __align__(256) int g_scratch[SCRATCH_INTS];
 
 struct Grid {
     double lo[3], cs[3], inv_cs[3], box[3], inv_box[3];
-    unsigned long long hbox[3];   // bits of box / 2
+    int hbox[3];                  // high word of box / 2 on periodic axes, else above every finite number's
     int nc[3], periodic[3];
     // fixed-point coordinates of the candidate test: units of window / 2^32,
     // the window a whole fraction of a periodic box and at least 4 r_c wide
@@ -175,12 +175,14 @@ __device__ __forceinline__ double na_term(const Grid &G, const double xi[3], con
     for (int a = 0; a < 3; ++a) {
         double t = __dsub_rn(xi[a], x[3 * (long long)j + a]);
         // minimum image; in-box coordinates need at most one box length
-        if (G.periodic[a] && abs_bits(t) > G.hbox[a]) t = __dsub_rn(t, __dmul_rn(G.box[a], rint(t * G.inv_box[a])));
+        if (hi_abs(t) >= G.hbox[a]) t = __dsub_rn(t, __dmul_rn(G.box[a], rint(t * G.inv_box[a])));
         r[a] = t;
     }
     const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])), __dmul_rn(r[2], r[2]));
-    if (!(abs_bits(r2) < abs_bits(G.rc2))) return 0.0;   // also a NaN (its bits are above any finite value's)
-    const double q1 = r2 > 0.0 ? r2 * rsqrt(r2) * G.inv_rc : 0.0, om = 1.0 - q1;
+    if (!lt_pos(r2, G.rc2)) return 0.0;   // also a NaN
+    double root, inv;
+    root_and_inverse(r2, root, inv);
+    const double q1 = hi_abs(r2) >= 0x00100000 ? root * G.inv_rc : 0.0, om = 1.0 - q1;   // (r2 zero or subnormal: q is 0)
     return G.Wc * (1.0 + 3.0 * q1) * om * om * om;
 }
 
@@ -375,7 +377,9 @@ extern "C" sdpd_status sdpd_density_noalloc(const sdpd_params *p, long long n, c
         G.unit[a] = (float)(window / 4294967296.0);
         G.inv_box[a] = 1.0 / G.box[a];
         const double hb = 0.5 * G.box[a];
-        std::memcpy(&G.hbox[a], &hb, sizeof hb);
+        unsigned long long bits;
+        std::memcpy(&bits, &hb, sizeof hb);
+        G.hbox[a] = G.periodic[a] ? (int)(bits >> 32) : 0x7FFFFFFF;
     }
     // FP32 products of fixed-point differences: relative error of r^2 below 1e-6
     G.r2_hi = (float)(G.rc2 * (1.0 + 1e-5));
