@@ -69,6 +69,15 @@ struct sdpd_ctx {
 
 namespace {
 
+// the high word of x, ordered like x (hi_key of the update kernel)
+int hi_key_of(double x)
+{
+    int64_t k;
+    std::memcpy(&k, &x, sizeof k);
+    const int h = (int)(k >> 32);
+    return h ^ ((h >> 31) & 0x7FFFFFFF);
+}
+
 template <class T> sdpd_status dalloc(sdpd_ctx *c, T **p, size_t count, bool geo = false)
 {
     if (count == 0) count = 1;
@@ -275,9 +284,15 @@ sdpd_status prepare(sdpd_ctx *c)
         I.half_skin = 0.5 * skin * h;
         for (int a = 0; a < 3; ++a) {
             I.dom_hi[a] = I.origin[a] + I.box[a];
-            const double hb = 0.5 * I.box[a];
-            std::memcpy(&I.hbox_bits[a], &hb, sizeof hb);
+            // (a step inwards keeps -0 and +0, equal but two words apart, on the safe side)
+            I.key_lo[a] = hi_key_of(I.origin[a]) + 1;
+            I.key_hi[a] = hi_key_of(I.dom_hi[a]) - 1;
         }
+        I.drift_hi = std::max(1, hi_key_of(I.half_skin));   // (no skin: any drift)
+        // two coordinates are off by half a unit each and axis, the products in
+        // FP32 by less than 1e-6
+        const double moved = I.half_skin * (1.0 - 1e-5) - 4.0 * std::max({ I.unit[0], I.unit[1], I.unit[2] });
+        I.moved2 = moved > 0.0 ? (float)(moved * moved) : 0.0f;
         I.rb2f = (float)(rb * rb * (1.0 + 1e-5));
         I.guard_lo = (float)(I.rc2 * (1.0 - 1e-5));
         I.guard_hi = (float)(I.rc2 * (1.0 + 1e-5));
@@ -544,7 +559,7 @@ sdpd_status sdpd_init(const sdpd_params *params, int n_instances, const long lon
         b.zd = arena;
         b.ownA = oa; b.ownB = ob;
     }
-    IALLOC(b.dsp, N);
+    IALLOC(b.A32_build, N);
     IALLOC(b.aclose, N); IALLOC(b.aclose_ok, 1); IALLOC(b.sdr, N); IALLOC(b.side32, N); IALLOC(b.xs, 3 * N);
     const size_t ni = (size_t)n_instances + 1;
     IALLOC(b.need_build, ni); IALLOC(b.fresh, 1);

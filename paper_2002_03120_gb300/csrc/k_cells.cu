@@ -156,8 +156,7 @@ __global__ void k_rank(Bufs b, const int *gate)
     b.slot_of[g] = s0 + r;
 }
 
-// Cell-sorted mirrors for the pair kernels; resets the displacement since
-// the build.
+// Cell-sorted mirrors for the pair kernels; displacements count from here.
 __global__ void k_gather(Bufs b, int precision, const int *gate)
 {
     GATE;
@@ -173,8 +172,7 @@ __global__ void k_gather(Bufs b, int precision, const int *gate)
     const uint32_t lg = (uint32_t)(g - I.p_begin);
     // (both precisions: the neighbour search and the split-precision pair
     // kernels work on the fixed-point coordinates)
-    b.A32[s] = make_int4(fixed_coord(x0, I, 0), fixed_coord(x1, I, 1), fixed_coord(x2, I, 2), t);
-    b.dsp[s] = make_double4_32a(0.0, 0.0, 0.0, 0.0);
+    b.A32[s] = b.A32_build[s] = make_int4(fixed_coord(x0, I, 0), fixed_coord(x1, I, 1), fixed_coord(x2, I, 2), t);
     if (precision == SDPD_PREC_SPLIT) {
         b.B32[s] = make_float4((float)b.v[3 * g], (float)b.v[3 * g + 1], (float)b.v[3 * g + 2],
                                (float)b.R[g]);

@@ -165,7 +165,7 @@ __global__ void k_na_scatter(int *scr, Grid G, const double *x)
 //    when the FP64 part runs; it re-decides r < r_c as before.
 // One thread per particle over unsorted candidates, each wrapped by an FP64
 // division per axis, took 13.4 ms for 46,255 particles; the call now takes
-// 0.95 ms (0.5 ms at the measured FP64 rate).
+// 0.82 ms (0.5 ms at the measured FP64 rate).
 constexpr int ND_WARPS = 4;
 
 __device__ __forceinline__ double na_term(const Grid &G, const double xi[3], const double *__restrict__ x, int j)
