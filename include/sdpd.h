@@ -270,7 +270,9 @@ sdpd_status sdpd_set_cell_factor(sdpd_ctx *ctx, int cells);
  * order.  Invalidates the grid and the graph.  Synchronous. */
 sdpd_status sdpd_set_skin(sdpd_ctx *ctx, double skin);
 
-/* Number of kernel nodes in the captured one-step graph of sdpd_step (0 if
+/* Number of kernel nodes every launch of the captured one-step graph of
+ * sdpd_step runs (the list build, taken only where the skin is used up, is
+ * the body of a conditional node and not counted; 0 if
  * sdpd_step has not run yet).  Synchronous. */
 sdpd_status sdpd_graph_kernels(sdpd_ctx *ctx, long long *n_kernels);
 

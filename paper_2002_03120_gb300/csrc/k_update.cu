@@ -60,11 +60,13 @@ __device__ __forceinline__ int hi_key(double x)
 __device__ __forceinline__ bool finite_bits(double x) { return hi_abs(x) < 0x7FF00000; }
 
 // A particle has used up half the skin: its instance's lists are rebuilt
-// before the next pair pass.
-__device__ __forceinline__ void request_build(const Bufs &b, int inst)
+// before the next pair pass.  In the captured step `build` opens the
+// conditional node that holds the build.
+__device__ __forceinline__ void request_build(const Bufs &b, int inst, cudaGraphConditionalHandle build)
 {
     b.need_build[0] = 1;
     b.need_build[1 + inst] = 1;
+    if (build) cudaGraphSetConditional(build, 1);
 }
 // The displacement since the build, from the fixed-point coordinates.  A
 // single move of half the skin or more along an axis is told apart by its
@@ -77,9 +79,17 @@ __device__ __forceinline__ bool moved_far(const int4 &now, const int4 &build, co
     return dx * dx + dy * dy + dz * dz > I.moved2;
 }
 
+__device__ __forceinline__ void step_done(const Bufs &b)
+{
+    *b.step += 1;
+    *b.fresh = 0;
+}
+__global__ void k_step_done(Bufs b) { step_done(b); }   // (a context without particles)
+
 // Velocity Verlet (Eqs. newton1, newton2): v += dt/2 F/m, w += dt/2 N/I;
 // velver 1 also drifts x += dt v, wraps periodic axes and mirrors particles
-// that crossed a wall plane (normal velocity reversed).  The arithmetic is
+// that crossed a wall plane (normal velocity reversed); velver 2 also closes
+// the step (nothing after it reads the step number).  The arithmetic is
 // written without fused multiply-adds so it repeats the oracle bit for bit;
 // the decisions (wrap, reflection, finiteness) are taken on the integer pipe
 // from the bit patterns, with the oracle's outcomes.
@@ -92,10 +102,13 @@ __device__ __forceinline__ bool moved_far(const int4 &now, const int4 &build, co
 // every step.  Dam break of 374,000 particles, 164,000 of them moving: 54 ->
 // 26 us with the drift, 22 -> 20 us without.
 template <class R>
-__global__ void __launch_bounds__(256) k_integrate(Bufs b, int velver)
+__global__ void __launch_bounds__(256) k_integrate(Bufs b, int velver, cudaGraphConditionalHandle gate)
 {
     const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (velver == 1 && s == 0) *b.aclose_ok = 0;   // the drift moves the particles
+    if (s == 0) {
+        if (velver == 1) *b.aclose_ok = 0;   // the drift moves the particles
+        else step_done(b);
+    }
     if (s >= b.N) return;
     const int g = b.perm[s];
     const int t = b.stype[s];
@@ -152,7 +165,7 @@ __global__ void __launch_bounds__(256) k_integrate(Bufs b, int velver)
         // keep the mirrors of the unchanged slot order current; the
         // displacement since the build decides whether the list still holds
         const int4 now = make_int4(fixed_coord(x[0], I, 0), fixed_coord(x[1], I, 1), fixed_coord(x[2], I, 2), t);
-        if (far || moved_far(now, build, I)) request_build(b, inst);
+        if (far || moved_far(now, build, I)) request_build(b, inst, gate);
         b.A32[s] = now;
         if (b.A64) {
             double4_32a a64 = b.A64[s];
@@ -210,7 +223,7 @@ __global__ void k_absorb(Bufs b, const double *__restrict__ xs, int has_x)
             a64.x = x[0]; a64.y = x[1]; a64.z = x[2];
             b.A64[s] = a64;
         }
-        if (far || moved_far(now, b.A32_build[s], I)) request_build(b, b.pinst[g]);
+        if (far || moved_far(now, b.A32_build[s], I)) request_build(b, b.pinst[g], 0);
     }
     const double v[3] = { b.v[3 * g], b.v[3 * g + 1], b.v[3 * g + 2] };
     const double w[3] = { b.w[3 * g], b.w[3 * g + 1], b.w[3 * g + 2] };
@@ -292,12 +305,6 @@ __global__ void k_artvis_apply(Bufs b)
         w[a] = b.w[3 * g + a];
     }
     write_vel_mirror<R>(b, s, v, w);
-}
-
-__global__ void k_step_done(Bufs b)
-{
-    *b.step += 1;
-    *b.fresh = 0;
 }
 
 // ----------------------------------------------------- viscometer read-out
@@ -398,19 +405,21 @@ __global__ void k_mark_pairs(Bufs b, uint8_t *flags)
 // ---------------------------------------------------------------- launchers
 static inline unsigned nblk(long long n, int bs) { return (unsigned)((n + bs - 1) / bs); }
 
-void launch_integrate(const Bufs &b, int precision, int velver, int any_artvis, cudaStream_t st)
+void launch_integrate(const Bufs &b, int precision, int velver, int any_artvis, cudaStream_t st,
+                      cudaGraphConditionalHandle build)
 {
-    if (!b.N) return;
-    if (precision == SDPD_PREC_SPLIT) k_integrate<float><<<nblk(b.N, 256), 256, 0, st>>>(b, velver);
-    else k_integrate<double><<<nblk(b.N, 256), 256, 0, st>>>(b, velver);
+    if (!b.N) {
+        if (velver == 2) k_step_done<<<1, 1, 0, st>>>(b);
+        return;
+    }
+    if (precision == SDPD_PREC_SPLIT) k_integrate<float><<<nblk(b.N, 256), 256, 0, st>>>(b, velver, build);
+    else k_integrate<double><<<nblk(b.N, 256), 256, 0, st>>>(b, velver, build);
     if (velver == 2 && any_artvis) {
         k_artvis<<<nblk(b.N, 128), 128, 0, st>>>(b);
         if (precision == SDPD_PREC_SPLIT) k_artvis_apply<float><<<nblk(b.N, 256), 256, 0, st>>>(b);
         else k_artvis_apply<double><<<nblk(b.N, 256), 256, 0, st>>>(b);
     }
 }
-
-void launch_step_done(const Bufs &b, cudaStream_t st) { k_step_done<<<1, 1, 0, st>>>(b); }
 
 void launch_probe(const Bufs &b, int inst, int nbins, cudaStream_t st, long long n)
 {
