@@ -180,6 +180,27 @@ __device__ __forceinline__ float gelu(float z)
     const float h = (p * t) * ex2_approx(z * z * -0.72134752044448170f);
     return z * (z >= 0.0f ? 1.0f - h : h);
 }
+// The same operations on two values at once (packed FP32 instructions; the
+// special-function unit takes one value each): the same bits.
+__device__ __forceinline__ F2 gelu2(F2 z)
+{
+    F2 a = mul2(z, F2(0.70710678118654752f));
+    a.v &= 0x7FFFFFFF7FFFFFFFull;
+    float z0, z1, d0, d1, e0, e1;
+    fma2(F2(0.3275911f), a, F2(1.0f)).get(d0, d1);
+    mul2(mul2(z, z), F2(-0.72134752044448170f)).get(e0, e1);
+    const F2 t(rcp_approx(d0), rcp_approx(d1));
+    F2 p = fma2(F2(0.5f * 1.061405429f), t, F2(0.5f * -1.453152027f));
+    p = fma2(p, t, F2(0.5f * 1.421413741f));
+    p = fma2(p, t, F2(0.5f * -0.284496736f));
+    p = mul2(fma2(p, t, F2(0.5f * 0.254829592f)), t);
+    const F2 e(ex2_approx(e0), ex2_approx(e1)), h = mul2(p, e);
+    float h0, h1, g0, g1;
+    h.get(h0, h1);
+    fma2(h, F2(-1.0f), F2(1.0f)).get(g0, g1);
+    z.get(z0, z1);
+    return mul2(z, F2(z0 >= 0.0f ? g0 : h0, z1 >= 0.0f ? g1 : h1));
+}
 __device__ __forceinline__ float gelu_prime(float z)
 {
     return 0.5f * (1.0f + erf_as(z * 0.70710678118654752f)) +
@@ -192,6 +213,18 @@ __device__ __forceinline__ void put8(uint8_t *tile, int r, int k0, const float *
     __nv_bfloat162 h[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) h[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+    *reinterpret_cast<uint4 *>(tile + core_off(r, k0)) = *reinterpret_cast<uint4 *>(h);
+}
+
+__device__ __forceinline__ void put8(uint8_t *tile, int r, int k0, const F2 *v)
+{
+    __nv_bfloat162 h[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        float a, b;
+        v[i].get(a, b);
+        h[i] = __floats2bfloat162_rn(a, b);
+    }
     *reinterpret_cast<uint4 *>(tile + core_off(r, k0)) = *reinterpret_cast<uint4 *>(h);
 }
 
@@ -209,16 +242,25 @@ struct Net {
 };
 
 // ------------------------------------------------------------- inference
-// Persistent over 128-row tiles with NWG warpgroups per CTA: each warpgroup
-// owns one tile at a time (its own activation operand in shared memory and
-// its own 128 accumulator columns in tensor memory) and synchronises only
-// with itself (named barrier g + 1), so the MMAs of one warpgroup overlap
-// the GELU epilogues of the others.  The three hidden weight tiles are
-// staged once per CTA and shared.
-constexpr int NWG = 4;
-constexpr size_t FWD_SMEM = (size_t)(3 + NWG) * TILE_BYTES + 128;
+// Persistent over 128-row tiles with NWG groups of two warpgroups per CTA:
+// each group owns one tile at a time (its own activation operand in shared
+// memory and its own 128 accumulator columns in tensor memory) and
+// synchronises only with itself (named barrier g + 1), so the MMAs of one
+// group overlap the GELU epilogues of the others.  Thread (part, row) takes
+// half the columns of its row.  The three hidden weight tiles are staged once
+// per CTA and shared.
+// Bound by the FP32 pipe (12 packed operations for two GELUs, busy 62 % of the
+// time) and by issue slots; the special-function unit is half busy.  10^6 rows:
+// 358 us with scalar GELUs, 326 us with packed ones, 316 us with two threads a
+// row (eight warps a scheduler instead of four).  Tiles go round the CTAs
+// before a CTA gets a second one: 20,000 rows take 31 us, 47 us when a CTA was
+// filled first.
+constexpr int NWG = 4, PARTS = 2, FWD_GROUP = 128 * PARTS;
+// weight and activation tiles; mbarriers, flags, TMEM slot; the input layer's
+// weights and biases of two units each as pairs
+constexpr size_t FWD_BARS = (size_t)(3 + NWG) * TILE_BYTES, FWD_IN = FWD_BARS + 128, FWD_SMEM = FWD_IN + (WID / 2) * 32;
 
-__device__ __forceinline__ void wg_bar(int g) { asm volatile("bar.sync %0, 128;" ::"r"(g + 1) : "memory"); }
+__device__ __forceinline__ void wg_bar(int g) { asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(FWD_GROUP) : "memory"); }
 
 // Row r (output unit) of one hidden weight tile, as the B operand.
 __device__ __forceinline__ void stage_row(uint8_t *tile, const __nv_bfloat16 *W, int r)
@@ -233,12 +275,12 @@ __device__ __forceinline__ void stage_row(uint8_t *tile, const __nv_bfloat16 *W,
 // (flag in shared memory read after the barrier), so the warpgroup leaves
 // its loop together.
 __device__ bool wg_gemm(uint8_t *A, uint8_t *B, uint32_t dtmem, uint64_t *mbar, uint32_t &parity, int g,
-                        int tt, volatile int *flag, int *err)
+                        bool first, volatile int *flag, int *err)
 {
     proxy_fence();
     tc_fence_before();
     wg_bar(g);
-    if (tt == 0) {
+    if (first) {
         tc_fence_after();
         const uint32_t a0 = smem_u32(A), b0 = smem_u32(B);
 #pragma unroll
@@ -256,21 +298,28 @@ __device__ bool wg_gemm(uint8_t *A, uint8_t *B, uint32_t dtmem, uint64_t *mbar, 
     return *flag == 0;
 }
 
-__global__ void __launch_bounds__(128 * NWG, 1) k_mlp_forward(const float *__restrict__ P,
+__global__ void __launch_bounds__(FWD_GROUP *NWG, 1) k_mlp_forward(const float *__restrict__ P,
                                                               const __nv_bfloat16 *__restrict__ Wb,
                                                               const float *__restrict__ X, float *__restrict__ Y,
                                                               long long n, int *err)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t *sB = smem;                                        // 3 weight tiles
-    const int g = threadIdx.x >> 7, tt = threadIdx.x & 127;
+    const int g = threadIdx.x / FWD_GROUP, part = (threadIdx.x >> 7) % PARTS, tt = threadIdx.x & 127;
+    const bool first = threadIdx.x % FWD_GROUP == 0;
     uint8_t *sA = smem + (3 + g) * TILE_BYTES;                 // this warpgroup's activations
     uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + (3 + NWG) * TILE_BYTES) + g;
     volatile int *flag = reinterpret_cast<int *>(smem + (3 + NWG) * TILE_BYTES + 64) + g;
     uint32_t *slot = reinterpret_cast<uint32_t *>(smem + (3 + NWG) * TILE_BYTES + 96);
     for (int r = threadIdx.x; r < 3 * WID; r += blockDim.x)
         stage_row(sB + (r >> 7) * TILE_BYTES, Wb + (r >> 7) * WID * WID, r & 127);
-    if (tt == 0) {
+    float2 *sin = reinterpret_cast<float2 *>(smem + FWD_IN);   // [64][w0, w1, w2, b] of units 2i, 2i + 1
+    if (threadIdx.x < WID / 2 * 4) {
+        const int i = threadIdx.x >> 2, k = threadIdx.x & 3;
+        sin[threadIdx.x] = k < 3 ? make_float2(P[OFF_W0 + 6 * i + k], P[OFF_W0 + 6 * i + 3 + k])
+                                 : make_float2(P[OFF_B0 + 2 * i], P[OFF_B0 + 2 * i + 1]);
+    }
+    if (first) {
         mbar_init(mbar);
         *flag = 0;
     }
@@ -283,60 +332,66 @@ __global__ void __launch_bounds__(128 * NWG, 1) k_mlp_forward(const float *__res
     const float4 *P4 = reinterpret_cast<const float4 *>(P);
     uint32_t parity = 0;
     bool ok = true;
-    for (long long tile = (long long)blockIdx.x * NWG + g; ok && tile * WID < n; tile += (long long)gridDim.x * NWG) {
+    for (long long tile = (long long)g * gridDim.x + blockIdx.x; ok && tile * WID < n; tile += (long long)gridDim.x * NWG) {
         const long long row = tile * WID + tt;
         const bool valid = row < n;
         const float x0 = valid ? X[3 * row] : 0.f, x1 = valid ? X[3 * row + 1] : 0.f,
                     x2 = valid ? X[3 * row + 2] : 0.f;
-        // input layer 3 -> 128 (FP32), W0 rows 8c..8c+7 = 24 floats = 6 float4
+        // input layer 3 -> 128 (FP32)
+        const F2 xx0(x0), xx1(x1), xx2(x2);
 #pragma unroll 2
-        for (int c = 0; c < 16; ++c) {
-            float w[24], bb[8], h[8];
+        for (int c = part * (16 / PARTS); c < (part + 1) * (16 / PARTS); ++c) {
+            F2 h[4];
 #pragma unroll
-            for (int k = 0; k < 6; ++k) {
-                const float4 q = __ldg(P4 + (OFF_W0 / 4) + 6 * c + k);
-                w[4 * k] = q.x; w[4 * k + 1] = q.y; w[4 * k + 2] = q.z; w[4 * k + 3] = q.w;
+            for (int i = 0; i < 4; ++i) {
+                const ulonglong2 *q = reinterpret_cast<const ulonglong2 *>(sin + 4 * (4 * c + i));
+                const ulonglong2 wa = q[0], wb = q[1];
+                F2 w0, w1, w2, bb;
+                w0.v = wa.x; w1.v = wa.y; w2.v = wb.x; bb.v = wb.y;
+                h[i] = gelu2(fma2(w0, xx0, fma2(w1, xx1, fma2(w2, xx2, bb))));
             }
-#pragma unroll
-            for (int k = 0; k < 2; ++k) {
-                const float4 q = __ldg(P4 + (OFF_B0 / 4) + 2 * c + k);
-                bb[4 * k] = q.x; bb[4 * k + 1] = q.y; bb[4 * k + 2] = q.z; bb[4 * k + 3] = q.w;
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) h[i] = gelu(fmaf(w[3 * i], x0, fmaf(w[3 * i + 1], x1, fmaf(w[3 * i + 2], x2, bb[i]))));
             put8(sA, tt, 8 * c, h);
         }
         float y = 0.f;
         for (int l = 1; l <= 3; ++l) {
-            ok = wg_gemm(sA, sB + (l - 1) * TILE_BYTES, tcols, mbar, parity, g, tt, flag, err);
+            ok = wg_gemm(sA, sB + (l - 1) * TILE_BYTES, tcols, mbar, parity, g, first, flag, err);
             if (!ok) break;
-            for (int c = 0; c < 8; ++c) {
+#pragma unroll 2
+            for (int c = part * (8 / PARTS); c < (part + 1) * (8 / PARTS); ++c) {
                 float v[16];
                 tc_ld16(tl + (uint32_t)(c * 16), v);
-                float bb[16];
+                F2 h[8];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     const float4 q = __ldg(P4 + off_b(l) / 4 + 4 * c + k);
-                    bb[4 * k] = q.x; bb[4 * k + 1] = q.y; bb[4 * k + 2] = q.z; bb[4 * k + 3] = q.w;
+                    h[2 * k] = gelu2(add2(F2(v[4 * k], v[4 * k + 1]), F2(q.x, q.y)));
+                    h[2 * k + 1] = gelu2(add2(F2(v[4 * k + 2], v[4 * k + 3]), F2(q.z, q.w)));
                 }
                 if (l < 3) {
-#pragma unroll
-                    for (int i = 0; i < 16; ++i) v[i] = gelu(v[i] + bb[i]);
-                    put8(sA, tt, 16 * c, v);
-                    put8(sA, tt, 16 * c + 8, v + 8);
+                    put8(sA, tt, 16 * c, h);
+                    put8(sA, tt, 16 * c + 8, h + 4);
                 } else {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
                         const float4 q = __ldg(P4 + OFF_W4 / 4 + 4 * c + k);
-                        y = fmaf(gelu(v[4 * k] + bb[4 * k]), q.x, y);
-                        y = fmaf(gelu(v[4 * k + 1] + bb[4 * k + 1]), q.y, y);
-                        y = fmaf(gelu(v[4 * k + 2] + bb[4 * k + 2]), q.z, y);
-                        y = fmaf(gelu(v[4 * k + 3] + bb[4 * k + 3]), q.w, y);
+                        float a0, a1, a2, a3;
+                        h[2 * k].get(a0, a1);
+                        h[2 * k + 1].get(a2, a3);
+                        y = fmaf(a0, q.x, y);
+                        y = fmaf(a1, q.y, y);
+                        y = fmaf(a2, q.z, y);
+                        y = fmaf(a3, q.w, y);
                     }
                 }
             }
         }
-        if (valid && ok) Y[row] = y + P[OFF_B4];
+        // the second half's sum passes through the row's first chunk of the
+        // activation tile, which only the first half's thread writes
+        float *other = reinterpret_cast<float *>(sA + core_off(tt, 0));
+        if (part == 1) *other = y;
+        wg_bar(g);
+        if (part == 0) y += *other;
+        if (valid && ok && part == 0) Y[row] = y + P[OFF_B4];
     }
     tc_fence_before();
     __syncthreads();
@@ -403,8 +458,11 @@ __device__ __forceinline__ void tc_ld_cols(uint32_t taddr, float *v)
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
                      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                      : "r"(taddr));
+    } else if constexpr (N == 16) {
+        tc_ld16(taddr, v);
+        return;
     } else {
-        static_assert(N == 8, "4 or 8 columns");
+        static_assert(N == 8, "4, 8 or 16 columns");
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
                      : "r"(taddr));
@@ -674,6 +732,138 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(Net net, const flo
     if (w == 0) tc_dealloc(tm, 512);
 }
 
+// Inference of few rows: a tile of ROWS (16, 32 or 64) rows per CTA in the
+// gradient kernel's transposed form, so the chain of layers is short and the
+// 16 warps of every SM take part.  Bound by latency: the weights' way into
+// shared memory and four layers in turn.  1,001 rows take 16 us a call (46 us
+// with 128-row tiles packed four to a CTA, 29 us one to a CTA), 5,000 rows 19
+// us.  Same operations per row as above, in the same order.
+template <int ROWS> struct RowsSmem {
+    static constexpr uint32_t A_BYTES = (ROWS / 8) * TG;
+    static constexpr uint32_t OFF_A = 3 * W_BYTES;         // two activation tiles, in turn
+    static constexpr uint32_t OFF_H = OFF_A + 2 * A_BYTES; // FP32 [128][ROWS + 1]: last hidden layer
+    static constexpr uint32_t OFF_X = OFF_H + 128 * (ROWS + 1) * 4;
+    static constexpr uint32_t OFF_BAR = OFF_X + ROWS * 16; // 3 mbarriers, TMEM slot, flag
+    static constexpr uint32_t BYTES = OFF_BAR + 128;
+};
+
+template <int ROWS>
+__global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_rows(const float *__restrict__ P,
+                                                              const __nv_bfloat16 *__restrict__ Wb,
+                                                              const float *__restrict__ X, float *__restrict__ Y,
+                                                              long long n, int *err)
+{
+    using S = RowsSmem<ROWS>;
+    constexpr int RPT = ROWS / 4;             // rows of a thread
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const uint32_t sbase = smem_u32(smem);
+    float *hbuf = reinterpret_cast<float *>(smem + S::OFF_H);
+    float4 *xs = reinterpret_cast<float4 *>(smem + S::OFF_X);
+    uint64_t *mbar = reinterpret_cast<uint64_t *>(smem + S::OFF_BAR);
+    uint32_t *slot = reinterpret_cast<uint32_t *>(smem + S::OFF_BAR + 64);
+    volatile int *flag = reinterpret_cast<int *>(smem + S::OFF_BAR + 72);
+    const int t = threadIdx.x, w = t >> 5, cg = w >> 2;
+    const int o = (w & 3) * 32 + (t & 31);    // this thread's feature
+    const long long r0 = (long long)blockIdx.x * ROWS;
+    // the weight tiles, one copy group per layer
+    for (int l = 0; l < 3; ++l) {
+        for (int q = t; q < WID * 16; q += GRAD_THREADS) {
+            const int r = q >> 4, c = q & 15;
+            cp_async16(sbase + l * W_BYTES + (r >> 3) * TG + c * TC + (r & 7) * 16, Wb + (l * WID + r) * WID + 8 * c);
+        }
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    if (t < 3) mbar_init(mbar + t);
+    if (t == 0) *flag = 0;
+    if (w == 0) tc_alloc(slot, 64);
+    if (t < ROWS) {
+        const long long row = r0 + t;
+        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row < n) { x.x = X[3 * row]; x.y = X[3 * row + 1]; x.z = X[3 * row + 2]; }
+        xs[t] = x;
+    }
+    const float w0 = P[OFF_W0 + 3 * o], w1 = P[OFF_W0 + 3 * o + 1], w2 = P[OFF_W0 + 3 * o + 2];
+    const float b[4] = { P[OFF_B0 + o], P[off_b(1) + o], P[off_b(2) + o], P[off_b(3) + o] };
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tm = *slot;
+    const uint32_t lanes = (uint32_t)((w & 3) * 32) << 16;
+    // this thread's feature of its rows, two at a time, into a tile [row][feature]
+    auto put = [&](uint32_t off, const F2 *v) {
+#pragma unroll
+        for (int i = 0; i < RPT; i += 2) {
+            const int r = cg * RPT + i;
+            float a0, a1;
+            v[i / 2].get(a0, a1);
+            __nv_bfloat16 *q = reinterpret_cast<__nv_bfloat16 *>(smem + off + (r >> 3) * TG + (o >> 3) * TC + (r & 7) * 16 +
+                                                                 (o & 7) * 2);
+            q[0] = __float2bfloat16_rn(a0);
+            q[8] = __float2bfloat16_rn(a1);   // the next row: 16 bytes on
+        }
+    };
+    {
+        F2 h[RPT / 2];
+#pragma unroll
+        for (int i = 0; i < RPT / 2; ++i) {
+            const float4 p = xs[cg * RPT + 2 * i], q = xs[cg * RPT + 2 * i + 1];
+            h[i] = gelu2(fma2(F2(w0), F2(p.x, q.x), fma2(F2(w1), F2(p.y, q.y), fma2(F2(w2), F2(p.z, q.z), F2(b[0])))));
+        }
+        put(S::OFF_A, h);
+    }
+#pragma unroll
+    for (int l = 1; l <= 3; ++l) {
+        if (l == 1) asm volatile("cp.async.wait_group 2;\n" ::: "memory");
+        else if (l == 2) asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        else asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        proxy_fence();
+        __syncthreads();
+        if (t == 0) {
+            tc_fence_after();
+            const uint32_t a0 = sbase + (l - 1) * W_BYTES, b0 = sbase + S::OFF_A + ((l - 1) & 1) * S::A_BYTES;
+#pragma unroll
+            for (int s = 0; s < 8; ++s)
+                mma_any(tm, desc_of(a0 + s * 2 * TC, TC, TG), desc_of(b0 + s * 2 * TC, TC, TG), idesc_n(ROWS, 0, 0), s > 0);
+            mma_commit(mbar + l - 1);
+        }
+        if (!mbar_wait(mbar + l - 1, 0)) {
+            *flag = 1;
+            atomicOr(err, ERR_MMA_TIMEOUT);
+            (void)mbar_wait(mbar + l - 1, 0);
+        }
+        tc_fence_after();
+        float v[RPT];
+        F2 h[RPT / 2];
+        tc_ld_cols<RPT>(tm + lanes + (uint32_t)(cg * RPT), v);
+#pragma unroll
+        for (int i = 0; i < RPT / 2; ++i) h[i] = gelu2(add2(F2(v[2 * i], v[2 * i + 1]), F2(b[l])));
+        if (l < 3) {
+            put(S::OFF_A + (l & 1) * S::A_BYTES, h);
+        } else {
+#pragma unroll
+            for (int i = 0; i < RPT / 2; ++i) {
+                float a0, a1;
+                h[i].get(a0, a1);
+                hbuf[o * (ROWS + 1) + cg * RPT + 2 * i] = a0;
+                hbuf[o * (ROWS + 1) + cg * RPT + 2 * i + 1] = a1;
+            }
+        }
+        tc_fence_before();
+    }
+    __syncthreads();
+    // output layer: the row's sum over the features in order, one thread per row
+    if (t < ROWS && r0 + t < n && *flag == 0) {
+        float y = 0.f, y1 = 0.f;
+#pragma unroll 16
+        for (int k = 0; k < WID / 2; ++k) {
+            y = fmaf(hbuf[k * (ROWS + 1) + t], __ldg(P + OFF_W4 + k), y);
+            y1 = fmaf(hbuf[(k + WID / 2) * (ROWS + 1) + t], __ldg(P + OFF_W4 + WID / 2 + k), y1);
+        }
+        Y[r0 + t] = (y + y1) + P[OFF_B4];
+    }
+    if (w == 0) tc_dealloc(tm, 64);
+}
+
 // Gradient and loss of the batch: the tiles' shares added in tile order.
 __device__ __forceinline__ float tile_sum(const float *__restrict__ q, size_t stride, int ntile)
 {
@@ -817,6 +1007,9 @@ sdpd_status mlp_init(int in, int width, int depth, unsigned long long seed, int 
     n.step = 0;
     k_mlp_refresh<<<(3 * WID * WID + 255) / 256, 256>>>(n);
     cudaFuncSetAttribute(k_mlp_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FWD_SMEM);
+    cudaFuncSetAttribute(k_mlp_rows<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RowsSmem<16>::BYTES);
+    cudaFuncSetAttribute(k_mlp_rows<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RowsSmem<32>::BYTES);
+    cudaFuncSetAttribute(k_mlp_rows<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RowsSmem<64>::BYTES);
     cudaFuncSetAttribute(k_mlp_grad<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GradSmem<16>::BYTES);
     cudaFuncSetAttribute(k_mlp_grad<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GradSmem<32>::BYTES);
     if (cudaDeviceSynchronize() != cudaSuccess) {
@@ -899,10 +1092,24 @@ sdpd_status mlp_infer(sdpd_mlp *h, const float *X, float *Y, long long n, void *
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const long long tiles = (n + WID - 1) / WID;
-    const int grid = (int)std::min<long long>((tiles + NWG - 1) / NWG, (long long)nsm);
+    cudaStream_t st = (cudaStream_t)stream;
     (void)cudaGetLastError();
-    k_mlp_forward<<<grid, 128 * NWG, FWD_SMEM, (cudaStream_t)stream>>>(h->net.P, h->net.Wb, X, Y, n, h->net.err);
+    // The smallest tile that covers the rows with one CTA per SM: a call of a
+    // given size takes the longer the larger its tiles (1,001 rows: 17.7 us in
+    // tiles of 16, 18.3 of 32, 19.4 of 64, 29.5 of 128), and a second round of
+    // small ones costs more than the next size up (2,500 rows: 24.6, 18.5;
+    // 5,000: 27.3 of 32, 20.1 of 64; 10,000: 28.7 of 64, 26.2 of 128).
+    const int rows = n <= 16LL * nsm ? 16 : n <= 32LL * nsm ? 32 : n <= 64LL * nsm ? 64 : WID;
+    const unsigned grid = (unsigned)std::min<long long>((n + rows - 1) / rows, nsm);
+    const Net &N = h->net;
+    if (rows == 16)
+        k_mlp_rows<16><<<grid, GRAD_THREADS, RowsSmem<16>::BYTES, st>>>(N.P, N.Wb, X, Y, n, N.err);
+    else if (rows == 32)
+        k_mlp_rows<32><<<grid, GRAD_THREADS, RowsSmem<32>::BYTES, st>>>(N.P, N.Wb, X, Y, n, N.err);
+    else if (rows == 64)
+        k_mlp_rows<64><<<grid, GRAD_THREADS, RowsSmem<64>::BYTES, st>>>(N.P, N.Wb, X, Y, n, N.err);
+    else
+        k_mlp_forward<<<grid, FWD_GROUP * NWG, FWD_SMEM, st>>>(N.P, N.Wb, X, Y, n, N.err);
     if (cudaGetLastError() != cudaSuccess) return mlp_fail(SDPD_E_CUDA, "mlp_infer: launch");
     return SDPD_OK;
 }
