@@ -2375,9 +2375,18 @@ void init_pair_kernels()
                          (int)rigid_smem_bytes(SDPD_MAX_NEIGHBORS));
 }
 
-void launch_forces(const Bufs &b, int precision, int velver, int newton3, cudaStream_t st)
+void launch_forces(const Bufs &b, int precision, int velver, int newton3, cudaStream_t st, cudaStream_t rigid)
 {
     if (!b.N) return;
+    // the spheres' forces first: few blocks of long chains, which the fluid
+    // pass then fills up around where `rigid` is a stream of its own
+    if (b.nrigid) {
+        const unsigned g = nblk(b.nrigid, RPB);
+        const size_t smem = rigid_smem_bytes(b.cap);
+        if (precision == SDPD_PREC_SPLIT) k_force_rigid<float><<<g, RB, smem, rigid>>>(b, velver);
+        else k_force_rigid<double><<<g, RB, smem, rigid>>>(b, velver);
+        if (velver == 2) k_hist_copy<<<nblk(b.nrigid, 64), 64, 0, rigid>>>(b);
+    }
     const int bs = b.pair_block, groups = pass_groups(b.N);
     const unsigned nb = pass_blocks(b.N, bs, groups);
     if (newton3 == 1 || newton3 == 4) {
@@ -2398,13 +2407,6 @@ void launch_forces(const Bufs &b, int precision, int velver, int newton3, cudaSt
         k_force_draw<<<nb, bs, 0, st>>>(b, velver, groups);
     } else {
         k_force_fluid<<<nb, bs, 0, st>>>(b, velver, groups);
-    }
-    if (b.nrigid) {
-        const unsigned g = nblk(b.nrigid, RPB);
-        const size_t smem = rigid_smem_bytes(b.cap);
-        if (precision == SDPD_PREC_SPLIT) k_force_rigid<float><<<g, RB, smem, st>>>(b, velver);
-        else k_force_rigid<double><<<g, RB, smem, st>>>(b, velver);
-        if (velver == 2) k_hist_copy<<<nblk(b.nrigid, 64), 64, 0, st>>>(b);
     }
 }
 
