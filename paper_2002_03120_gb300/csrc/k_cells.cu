@@ -310,7 +310,12 @@ __device__ void nb_scan_cell(const Bufs &b, int c, int s0, int s1, int4 *stage, 
 }
 
 // The lists: lanes are candidates.  `parts` warps share a cell, each taking
-// every parts-th group of NG_G of its particles.  A warp flattens the
+// every parts-th group of NG_G of its particles.  A warp is a block of its own:
+// latency bounds the scan, shared memory (9 KB a warp) the warps on an SM, and
+// in a block of four the memory of those that are done, or had no group, stayed
+// taken until the last one was (374,000 particles: 811 us a build in blocks of
+// four, 647 in blocks of one with the records of a batch fetched a batch ahead;
+// 662,000: 1.58 -> 1.43 ms).  A warp flattens the
 // candidates of the cell's neighbour cells (ascending key, then slot; cells
 // whose slots follow one another are one run).  For each group:
 // * Every batch of 32 candidates is tested against the group's bounding box,
@@ -334,7 +339,6 @@ __device__ void nb_scan_cell(const Bufs &b, int c, int s0, int s1, int4 *stage, 
 constexpr int NG_G = 8;        // particles per group
 constexpr int NG_TAB = 128;    // runs (>= ADJ)
 constexpr int NG_STAGE = 64;   // staged candidates (one batch on top of a partial stage)
-constexpr int NG_MAX_WARPS = 4;
 
 // 16-bit entries: offset bits, and the largest neighbour cell; a run never
 // exceeds twice that (it is cut where the flattened index passes a multiple).
@@ -365,36 +369,40 @@ __host__ __device__ constexpr size_t ng_warp_bytes(int cap)
 }
 
 template <int SUB, bool SPLIT>
-__global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors(Bufs b, int parts, const int *gate)
+__global__ void __launch_bounds__(32, 24) k_neighbors(Bufs b, int parts, const int *gate)
 {
     GATE;
     constexpr int BITS = NgEntry<SUB>::BITS, CELL = NgEntry<SUB>::CELL;
     constexpr int NADJ = (2 * SUB + 1) * (2 * SUB + 1) * (2 * SUB + 1);
     extern __shared__ __align__(16) unsigned char ng_smem[];
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const long long wg = (long long)blockIdx.x * nw + w;
-    const int c = (int)(wg / parts), part = (int)(wg % parts);
-    if (c >= b.ncell_total || !rebuilds(b, gate, b.cell_inst[c])) return;   // the whole warp
+    const int lane = threadIdx.x;
+    const int c = blockIdx.x / parts, part = blockIdx.x % parts;
+    if (!rebuilds(b, gate, b.cell_inst[c])) return;
     const int s0 = b.cstart[c], s1 = b.cstart[c + 1];
     if (s0 + part * NG_G >= s1) return;
     const int cap = b.cap, stride = ng_stride(cap);
-    unsigned char *mine = ng_smem + (size_t)w * ng_warp_bytes(cap);
-    NgShared &S = *reinterpret_cast<NgShared *>(mine);
-    uint16_t *buf = reinterpret_cast<uint16_t *>(mine + ng_head());
+    NgShared &S = *reinterpret_cast<NgShared *>(ng_smem);
+    uint16_t *buf = reinterpret_cast<uint16_t *>(ng_smem + ng_head());
     const unsigned FULL = 0xffffffffu, lt = (1u << lane) - 1u;
 
     // the runs of the neighbour cells (valid keys are a prefix of the row)
     const int *adj = b.cell_adj + (long long)c * ADJ;
     int total = 0, nq = 0, last_end = -1, last_bucket = 0;
     bool fat = false;
-    for (int q0 = 0; q0 < NADJ; q0 += 32) {
-        const int q = q0 + lane;
-        const int key = q < NADJ ? adj[q] : -1;
-        int cnt = 0, js = 0;
-        if (key >= 0) {
-            js = b.cstart[key];
-            cnt = b.cstart[key + 1] - js;
-        }
+    // (all the loads of the chain key -> start first: one latency, not one
+    // for each 32 cells)
+    constexpr int NQ = (NADJ + 31) / 32;
+    int qkey[NQ], qjs[NQ], qend[NQ];
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) qkey[q] = q * 32 + lane < NADJ ? adj[q * 32 + lane] : -1;
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+        qjs[q] = qkey[q] >= 0 ? b.cstart[qkey[q]] : 0;
+        qend[q] = qkey[q] >= 0 ? b.cstart[qkey[q] + 1] : 0;
+    }
+#pragma unroll
+    for (int q0 = 0; q0 < NQ; ++q0) {
+        const int key = qkey[q0], js = qjs[q0], cnt = qend[q0] - js;
         fat = fat || __any_sync(FULL, cnt > CELL);
         int v = cnt;
 #pragma unroll
@@ -544,22 +552,32 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors(Bufs b, int par
         };
 
         int nst = 0, qc = 0;   // staged candidates; the run of the batch's first candidate
-        for (int f0 = 0; f0 < total; f0 += 32) {
+        // the records of a batch are fetched while the one before it is tested
+        int4 An = make_int4(0, 0, 0, 0);
+        int jn = 0, en = 0;
+        auto fetch = [&](int f0) {
             const int f = f0 + lane;
             // the runs that begin inside this batch, as bits at their first
             // candidate (runs are not empty: at most one begins at a place)
             int nx = qc + 1 + lane < nq ? S.pre[qc + 1 + lane] - f0 : 32;
             const unsigned begin = __reduce_or_sync(FULL, nx < 32 ? 1u << nx : 0u);
             const int q = qc + __popc(begin & (lt | (1u << lane)));
-            bool keep = false;
-            int4 Aj = make_int4(0, 0, 0, 0);
-            int j = 0, eq = 0;
-            float rj = 0.f;
             if (f < total) {
                 const int off = f - S.pre[q];
-                j = S.js[q] + off;
-                eq = (q << BITS) | off;
-                Aj = b.A32[j];
+                jn = S.js[q] + off;
+                en = (q << BITS) | off;
+                An = b.A32[jn];
+            }
+            qc += __popc(begin);
+        };
+        if (total > 0) fetch(0);
+        for (int f0 = 0; f0 < total; f0 += 32) {
+            const int4 Aj = An;
+            const int j = jn, eq = en;
+            if (f0 + 32 < total) fetch(f0 + 32);
+            bool keep = false;
+            float rj = 0.f;
+            if (f0 + lane < total) {
                 float px, py, pz;
                 geo.disp(Aj, mid, px, py, pz);
                 const float ex = fmaxf(fabsf(px) - bx, 0.f), ey = fmaxf(fabsf(py) - by, 0.f),
@@ -573,7 +591,6 @@ __global__ void __launch_bounds__(NG_MAX_WARPS * 32) k_neighbors(Bufs b, int par
                 }
                 keep = d2 < lim2;
             }
-            qc += __popc(begin);
             const unsigned km = __ballot_sync(FULL, keep);
             if (keep) {
                 const int pos = nst + __popc(km & lt);
@@ -742,14 +759,17 @@ void init_cell_kernels()
 template <int SUB>
 static void launch_lists(const Bufs &b, const int *gate, cudaStream_t st)
 {
-    // warps per cell: a full cell holds about eight groups, a half cell one or
-    // two (more than one warp for them only where cells alone leave SMs idle)
-    const int parts = SUB == 1 ? 8 : (b.ncell_total < 4096 ? 2 : 1);
+    // Warps per cell: a full cell holds 8 to 24 groups (cells per axis are
+    // whole numbers), a half cell one or two.  More than one warp for half
+    // cells only where the cells alone leave SMs idle (16,000 particles: 166 us
+    // a build with one, 115 with four; 662,000: 1.53 ms with one, 1.66 with four);
+    // a warp without a group leaves at once.  8,192 particles in full cells: 381
+    // us with 8, 198 with 24.
+    const int parts = SUB == 1 ? 24 : std::min(4, std::max(1, 16384 / b.ncell_total));
     const size_t wb = ng_warp_bytes(b.cap);
-    const int ngw = (int)std::min<size_t>(NG_MAX_WARPS, NG_SMEM_MAX / wb);
-    const unsigned nb = nblk((long long)b.ncell_total * parts, ngw);
-    if (b.split) k_neighbors<SUB, true><<<nb, ngw * 32, ngw * wb, st>>>(b, parts, gate);
-    else k_neighbors<SUB, false><<<nb, ngw * 32, ngw * wb, st>>>(b, parts, gate);
+    const unsigned nb = (unsigned)b.ncell_total * parts;
+    if (b.split) k_neighbors<SUB, true><<<nb, 32, wb, st>>>(b, parts, gate);
+    else k_neighbors<SUB, false><<<nb, 32, wb, st>>>(b, parts, gate);
 }
 
 void launch_build(const Bufs &b, int precision, int need_rev, const int *gate, cudaStream_t st)
