@@ -413,10 +413,8 @@ sdpd_status prepare(sdpd_ctx *c)
     return SDPD_OK;
 }
 
-sdpd_status check_err(sdpd_ctx *c)
+sdpd_status report_err(sdpd_ctx *c, int e)
 {
-    int e = 0;
-    CUDA_TRY(cudaMemcpy(&e, c->b.err, sizeof(int), cudaMemcpyDeviceToHost));
     c->sticky_err |= e;
     e = c->sticky_err;
     if (!e) return SDPD_OK;
@@ -429,6 +427,13 @@ sdpd_status check_err(sdpd_ctx *c)
     if (e & ERR_DOMAIN) return fail(SDPD_E_DOMAIN, "particle outside the grid (crossed a wall axis, or moved more than a box length in one step)");
     if (e & ERR_TIMEOUT) return fail(SDPD_E_TIMEOUT, "a copy into shared memory did not complete");
     return fail(SDPD_E_CUDA, "unknown device error");
+}
+
+sdpd_status check_err(sdpd_ctx *c)
+{
+    int e = 0;
+    CUDA_TRY(cudaMemcpy(&e, c->b.err, sizeof(int), cudaMemcpyDeviceToHost));
+    return report_err(c, e);
 }
 
 sdpd_status ensure_geometry(sdpd_ctx *c)
@@ -1145,7 +1150,7 @@ sdpd_status sdpd_viscosity_probe(sdpd_ctx *c, int inst, int n_bins, double *prof
     if (s != SDPD_OK) return s;
     CUDA_TRY(cudaDeviceSynchronize());
     launch_probe(c->b, inst, n_bins, 0, c->hi[inst].n);
-    std::vector<double> h(3 * n_bins + 4);
+    std::vector<double> h(3 * n_bins + 5);
     CUDA_TRY(cudaMemcpy(h.data(), c->b.probe, sizeof(double) * h.size(), cudaMemcpyDeviceToHost));
     for (int k = 0; k < n_bins; ++k)
         if (profile_out) profile_out[k] = h[n_bins + k] > 0 ? h[k] / h[n_bins + k] : 0.0;
@@ -1158,7 +1163,8 @@ sdpd_status sdpd_viscosity_probe(sdpd_ctx *c, int inst, int n_bins, double *prof
                             h[2 * n_bins + 1] / std::max(h[2 * n_bins + 3], 1.0));
     const double D = 0.5 * p.box[p.split_axis];
     if (mu_app_out) *mu_app_out = p.rho0 * p.body_amp * D * D / (12.0 * V);
-    return check_err(c);
+    // (the probe brought the error word along, where it had a particle to run on)
+    return c->hi[inst].n ? report_err(c, (int)h[3 * n_bins + 4]) : check_err(c);
 }
 
 sdpd_status sdpd_viscosity_fit(sdpd_ctx *c, int inst, int n_bins, double *mu_fit_out)

@@ -775,16 +775,16 @@ static void launch_lists(const Bufs &b, const int *gate, cudaStream_t st)
 void launch_build(const Bufs &b, int precision, int need_rev, const int *gate, cudaStream_t st)
 {
     const int nc = b.ncell_total;
-    const int nbk = (nc + 1023) / 1024;
+    const int nbk = (nc + 1023) / 1024, bs = spread_block(b.N);
     k_cell_clear<<<nblk(nc, 256), 256, 0, st>>>(b, gate);
-    if (b.N) k_cell_keys<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
+    if (b.N) k_cell_keys<<<nblk(b.N, bs), bs, 0, st>>>(b, gate);
     k_scan_local<<<nbk, 1024, 0, st>>>(b, gate);
     k_scan_partials<<<1, 1024, 0, st>>>(b, nbk, gate);
     k_scan_add<<<nbk, 1024, 0, st>>>(b, gate);
     if (b.N) {
-        k_scatter<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
-        k_rank<<<nblk(b.N, 256), 256, 0, st>>>(b, gate);
-        k_gather<<<nblk(b.N, 256), 256, 0, st>>>(b, precision, gate);
+        k_scatter<<<nblk(b.N, bs), bs, 0, st>>>(b, gate);
+        k_rank<<<nblk(b.N, bs), bs, 0, st>>>(b, gate);
+        k_gather<<<nblk(b.N, bs), bs, 0, st>>>(b, precision, gate);
         if (b.cell_sub == 2) launch_lists<2>(b, gate, st);
         else launch_lists<1>(b, gate, st);
         if (need_rev) k_rev<<<nblk(b.N * LPP, 128), 128, 0, st>>>(b, gate);

@@ -309,24 +309,40 @@ __global__ void k_artvis_apply(Bufs b)
 
 // ----------------------------------------------------- viscometer read-out
 // probe layout: [0, nb) velocity sums, [nb, 2nb) counts, [2nb, 2nb+4)
-// signed velocity sums and counts of the two halves.
+// signed velocity sums and counts of the two halves, [2nb+4, 3nb+4) position
+// sums, [3nb+4] the error word.  The halves' sums are formed per warp (an atomic for
+// every particle on two addresses was most of the time).
 __global__ void k_probe(Bufs b, int inst, int nb)
 {
     const Inst &I = b.inst[inst];
     const long long g = I.p_begin + (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= I.p_end) return;
-    if (b.type[g] != T_FLUID) return;
+    if (g == I.p_begin) b.probe[3 * nb + 4] = (double)*b.err;
+    const bool use = g < I.p_end && b.type[g] == T_FLUID;
     const int ax = I.split_axis, fa = I.body_axis;
-    const double rel = b.x[3 * g + ax] - I.origin[ax];
-    int bin = (int)floor(rel / I.box[ax] * nb);
-    bin = bin < 0 ? 0 : (bin >= nb ? nb - 1 : bin);
-    const double u = b.v[3 * g + fa];
-    atomicAdd(&b.probe[bin], u);
-    atomicAdd(&b.probe[nb + bin], 1.0);
-    const int half = (rel < 0.5 * I.box[ax]) ? 0 : 1;
-    atomicAdd(&b.probe[2 * nb + half], half == 0 ? u : -u);
-    atomicAdd(&b.probe[2 * nb + 2 + half], 1.0);
-    atomicAdd(&b.probe[2 * nb + 4 + bin], rel);   // mean position of the slab's particles
+    double u = 0.0;
+    int half = 0;
+    if (use) {
+        const double rel = b.x[3 * g + ax] - I.origin[ax];
+        int bin = (int)floor(rel / I.box[ax] * nb);
+        bin = bin < 0 ? 0 : (bin >= nb ? nb - 1 : bin);
+        u = b.v[3 * g + fa];
+        atomicAdd(&b.probe[bin], u);
+        atomicAdd(&b.probe[nb + bin], 1.0);
+        atomicAdd(&b.probe[2 * nb + 4 + bin], rel);   // mean position of the slab's particles
+        half = (rel < 0.5 * I.box[ax]) ? 0 : 1;
+    }
+    const double u0 = warp_sum(use && half == 0 ? u : 0.0), u1 = warp_sum(use && half == 1 ? -u : 0.0);
+    const int n0 = __popc(__ballot_sync(0xffffffffu, use && half == 0)), n1 = __popc(__ballot_sync(0xffffffffu, use && half == 1));
+    if ((threadIdx.x & 31) == 0) {
+        if (n0) {
+            atomicAdd(&b.probe[2 * nb], u0);
+            atomicAdd(&b.probe[2 * nb + 2], (double)n0);
+        }
+        if (n1) {
+            atomicAdd(&b.probe[2 * nb + 1], u1);
+            atomicAdd(&b.probe[2 * nb + 3], (double)n1);
+        }
+    }
 }
 
 // diagnostics layout in probe: [0..2] momentum, [3] sum m v^2, [4] sum m,
@@ -412,8 +428,9 @@ void launch_integrate(const Bufs &b, int precision, int velver, int any_artvis, 
         if (velver == 2) k_step_done<<<1, 1, 0, st>>>(b);
         return;
     }
-    if (precision == SDPD_PREC_SPLIT) k_integrate<float><<<nblk(b.N, 256), 256, 0, st>>>(b, velver, build);
-    else k_integrate<double><<<nblk(b.N, 256), 256, 0, st>>>(b, velver, build);
+    const int bs = spread_block(b.N);
+    if (precision == SDPD_PREC_SPLIT) k_integrate<float><<<nblk(b.N, bs), bs, 0, st>>>(b, velver, build);
+    else k_integrate<double><<<nblk(b.N, bs), bs, 0, st>>>(b, velver, build);
     if (velver == 2 && any_artvis) {
         k_artvis<<<nblk(b.N, 128), 128, 0, st>>>(b);
         if (precision == SDPD_PREC_SPLIT) k_artvis_apply<float><<<nblk(b.N, 256), 256, 0, st>>>(b);
@@ -424,7 +441,7 @@ void launch_integrate(const Bufs &b, int precision, int velver, int any_artvis, 
 void launch_probe(const Bufs &b, int inst, int nbins, cudaStream_t st, long long n)
 {
     cudaMemsetAsync(b.probe, 0, sizeof(double) * (3 * nbins + 4), st);
-    if (n) k_probe<<<nblk(n, 256), 256, 0, st>>>(b, inst, nbins);
+    if (n) k_probe<<<nblk(n, spread_block(n)), spread_block(n), 0, st>>>(b, inst, nbins);
 }
 
 void launch_diag(const Bufs &b, int inst, cudaStream_t st, long long n)
@@ -488,8 +505,9 @@ void launch_noise_normals(int precision, long long n, const uint32_t *gi, const 
 void launch_absorb(const Bufs &b, int precision, const double *xs, int has_x, cudaStream_t st)
 {
     if (!b.N) return;
-    if (precision == SDPD_PREC_SPLIT) k_absorb<float><<<nblk(b.N, 256), 256, 0, st>>>(b, xs, has_x);
-    else k_absorb<double><<<nblk(b.N, 256), 256, 0, st>>>(b, xs, has_x);
+    const int bs = spread_block(b.N);
+    if (precision == SDPD_PREC_SPLIT) k_absorb<float><<<nblk(b.N, bs), bs, 0, st>>>(b, xs, has_x);
+    else k_absorb<double><<<nblk(b.N, bs), bs, 0, st>>>(b, xs, has_x);
 }
 
 void launch_count_pairs(const Bufs &b, cudaStream_t st)
