@@ -64,8 +64,11 @@ struct sdpd_ctx {
     int sticky_err = 0;
     long long host_step = 0;
     cudaStream_t cap_stream = nullptr;
-    cudaGraphExec_t graph = nullptr;
-    cudaGraph_t graph_def = nullptr;
+    struct StepGraph {                 // `steps` steps captured as one graph
+        cudaGraphExec_t exec = nullptr;
+        cudaGraph_t def = nullptr;
+        long long steps = 1;
+    } graph, run;
 };
 
 namespace {
@@ -105,10 +108,11 @@ void free_geo(sdpd_ctx *c)
 
 void drop_graph(sdpd_ctx *c)
 {
-    if (c->graph) cudaGraphExecDestroy(c->graph);
-    if (c->graph_def) cudaGraphDestroy(c->graph_def);
-    c->graph = nullptr;
-    c->graph_def = nullptr;
+    for (sdpd_ctx::StepGraph *g : { &c->graph, &c->run }) {
+        if (g->exec) cudaGraphExecDestroy(g->exec);
+        if (g->def) cudaGraphDestroy(g->def);
+        *g = sdpd_ctx::StepGraph();
+    }
 }
 
 double lucy_W(double r, double h)
@@ -489,14 +493,19 @@ cudaError_t capture_gated_build(sdpd_ctx *c, cudaStream_t cs, cudaGraphCondition
     return cudaStreamUpdateCaptureDependencies(cs, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
 }
 
-// One full step as a graph.  Positions are unchanged between the velver-2
+// Steps a graph of small systems holds: a launch of a graph leaves the chip
+// idle for 5 us, 6 % of a step of 3,456 particles (83 us a step in graphs of
+// one, 80 of two, 79 of five or ten) and 1 % of one of 64,000.
+constexpr long long RUN_STEPS = 5, RUN_PARTICLES = 65536;
+
+// Full steps as a graph.  Positions are unchanged between the velver-2
 // build and the next step's velver 1, so that sub-step reuses the lists and
 // the density exactly.  With the Verlet skin most drifts need no new lists: the
 // build is one conditional node there, where its ten kernels, each leaving on
 // the gate, and ten more with the density at the head of the step had taken a
 // third of the step (ten steps of 3,456 particles: 1.15 -> 1.04 ms; five of a
 // dam break of 374,000: 10.8 -> 10.1 ms).
-sdpd_status capture_step(sdpd_ctx *c)
+sdpd_status capture_steps(sdpd_ctx *c, sdpd_ctx::StepGraph &g, long long steps)
 {
     cudaStream_t cs = c->cap_stream;
     CUDA_TRY(cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
@@ -504,7 +513,6 @@ sdpd_status capture_step(sdpd_ctx *c)
     cudaGraph_t graph = nullptr;
     cudaGraphConditionalHandle cond = 0;
     cudaError_t e = cudaStreamGetCaptureInfo(cs, &status, nullptr, &graph, nullptr, nullptr, nullptr);
-    if (e == cudaSuccess) e = cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault);
     // A branch of its own for the spheres' kernels, ahead in the queues: few
     // blocks and long FP64 chains, next to which the fluid and density passes
     // fill the chip (five steps of a dam break with 3,000 spheres: 10.1 -> 9.5
@@ -523,34 +531,37 @@ sdpd_status capture_step(sdpd_ctx *c)
         if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&side, cudaStreamNonBlocking, greatest);
         if (e != cudaSuccess) side = cs;
     }
-    if (e == cudaSuccess) {
-        launch_drag(c->b, c->precision, cs);
-        order(cs, side);
-        launch_forces(c->b, c->precision, 1, c->newton3, cs, side);
-        order(side, cs);
-        launch_integrate(c->b, c->precision, 1, c->any_artvis, cs, cond);
+    for (long long k = 0; k < steps && e == cudaSuccess; ++k) {
+        e = cudaGraphConditionalHandleCreate(&cond, graph, 0, cudaGraphCondAssignDefault);
+        if (e == cudaSuccess) {
+            launch_drag(c->b, c->precision, cs);
+            order(cs, side);
+            launch_forces(c->b, c->precision, 1, c->newton3, cs, side);
+            order(side, cs);
+            launch_integrate(c->b, c->precision, 1, c->any_artvis, cs, cond);
+        }
+        if (e == cudaSuccess) e = capture_gated_build(c, cs, cond);
+        if (e == cudaSuccess) {
+            // the drag's sums need positions and velocities only, no density
+            order(cs, side);
+            launch_drag(c->b, c->precision, side);
+            launch_density(c->b, c->precision, density_passes(c), half_pairs(c->newton3), nullptr, cs);
+            order(cs, side);
+            order(side, cs);
+            launch_forces(c->b, c->precision, 2, c->newton3, cs, side);
+            order(side, cs);
+            launch_integrate(c->b, c->precision, 2, c->any_artvis, cs);
+        }
     }
-    if (e == cudaSuccess) e = capture_gated_build(c, cs, cond);
-    if (e == cudaSuccess) {
-        // the drag's sums need positions and velocities only, no density
-        order(cs, side);
-        launch_drag(c->b, c->precision, side);
-        launch_density(c->b, c->precision, density_passes(c), half_pairs(c->newton3), nullptr, cs);
-        order(cs, side);
-        order(side, cs);
-        launch_forces(c->b, c->precision, 2, c->newton3, cs, side);
-        order(side, cs);
-        launch_integrate(c->b, c->precision, 2, c->any_artvis, cs);
-    }
-    const cudaError_t end = cudaStreamEndCapture(cs, &c->graph_def);
+    const cudaError_t end = cudaStreamEndCapture(cs, &g.def);
     if (e == cudaSuccess) e = end;
     if (side != cs) cudaStreamDestroy(side);
     if (ev) cudaEventDestroy(ev);
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph, c->graph_def, 0);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&g.exec, g.def, 0);
+    g.steps = steps;
     if (e == cudaSuccess) return SDPD_OK;
-    if (c->graph_def) cudaGraphDestroy(c->graph_def);
-    c->graph = nullptr;
-    c->graph_def = nullptr;
+    if (g.def) cudaGraphDestroy(g.def);
+    g = sdpd_ctx::StepGraph();
     return fail(SDPD_E_CUDA, std::string("step capture: ") + cudaGetErrorString(e));
 }
 
@@ -1027,12 +1038,17 @@ sdpd_status sdpd_step(sdpd_ctx *c, long long n_steps, void *stream)
         launch_density(c->b, c->precision, passes, half_pairs(c->newton3), c->b.fresh, st);
     }
     c->absorbed = false;
-    if (!c->graph) {
-        CUDA_TRY(cudaStreamSynchronize(st));
-        s = capture_step(c);
-        if (s != SDPD_OK) return s;
+    long long left = n_steps;
+    for (sdpd_ctx::StepGraph *g : { &c->run, &c->graph }) {
+        const long long steps = g == &c->run ? RUN_STEPS : 1;
+        if (left < steps || (steps > 1 && c->N > RUN_PARTICLES)) continue;
+        if (!g->exec) {
+            CUDA_TRY(cudaStreamSynchronize(st));
+            s = capture_steps(c, *g, steps);
+            if (s != SDPD_OK) return s;
+        }
+        for (; left >= steps; left -= steps) CUDA_TRY(cudaGraphLaunch(g->exec, st));
     }
-    for (long long k = 0; k < n_steps; ++k) CUDA_TRY(cudaGraphLaunch(c->graph, st));
     c->host_step += n_steps;
     CUDA_TRY(cudaStreamSynchronize(st));
     c->cells_valid = c->density_valid = true;
@@ -1120,18 +1136,19 @@ sdpd_status sdpd_graph_kernels(sdpd_ctx *c, long long *n_kernels)
 {
     if (!c || !n_kernels) return fail(SDPD_E_INVALID, "bad argument");
     *n_kernels = 0;
-    if (!c->graph_def) return SDPD_OK;
+    const sdpd_ctx::StepGraph &g = c->graph.def ? c->graph : c->run;
+    if (!g.def) return SDPD_OK;
     size_t n = 0;
-    CUDA_TRY(cudaGraphGetNodes(c->graph_def, nullptr, &n));
+    CUDA_TRY(cudaGraphGetNodes(g.def, nullptr, &n));
     std::vector<cudaGraphNode_t> nodes(n);
-    CUDA_TRY(cudaGraphGetNodes(c->graph_def, nodes.data(), &n));
+    CUDA_TRY(cudaGraphGetNodes(g.def, nodes.data(), &n));
     long long k = 0;
     for (auto nd : nodes) {
         cudaGraphNodeType t;
         CUDA_TRY(cudaGraphNodeGetType(nd, &t));
         k += (t == cudaGraphNodeTypeKernel);
     }
-    *n_kernels = k;
+    *n_kernels = k / g.steps;
     return SDPD_OK;
 }
 
