@@ -664,11 +664,16 @@ struct ListRows {
 // slots.  The 8 lanes of a particle take ZR rows at a time, unrolled, two rows
 // in the halves of the packed operations: 52 instructions an entry where one
 // entry at a time with branches and a library square root took 80, and 0.40
-// ms where that took 0.65 (662,305 particles).
+// ms where that took 0.65 (662,305 particles).  The gathers of positions then
+// bound them by latency: 64 registers, with a few of them spilled, and 32 warps
+// an SM beat 80 and none with 24 (0.395 -> 0.342 ms; 48 registers: 0.349), and
+// the Shepard averages fetch the neighbours' values with the positions (density
+// and pressure filter of 374,000 particles 0.377 -> 0.330 ms).
 //
-// f(W, j0, j1, ok0, ok1, r2_0, r2_1, type0, type1) sees the kernel weights of
-// two entries (0 for an entry past the end, beyond h or of contact range only).
-template <class F>
+// f(W, v0, v1, ok0, ok1, r2_0, r2_1, type0, type1) sees the kernel weights of
+// two entries (0 for an entry past the end, beyond h or of contact range only)
+// and, with SIDE, their values in side32, fetched with the positions.
+template <bool SIDE, class F>
 __device__ __forceinline__ void weights32(const Bufs &b, const Inst &I, const SlotHead &h, long long s, int n, int gr,
                                           int sub, F &&f)
 {
@@ -681,6 +686,9 @@ __device__ __forceinline__ void weights32(const Bufs &b, const Inst &I, const Sl
     ListRows cur, next;
     cur.load(nb, left);
     int4 A[2] = { b.A32[cur.e[0] & ~NB_FAR], b.A32[cur.e[1] & ~NB_FAR] };   // two rows ahead
+    float V[2] = { 0.f, 0.f };
+    if (SIDE)
+        for (int t = 0; t < 2; ++t) V[t] = b.side32[cur.e[t] & ~NB_FAR];
     for (int r0 = 0; r0 < gr; r0 += ZR) {
         nb += ZR * ROW;
         next.load(nb, left - ZR * LPP);
@@ -689,8 +697,13 @@ __device__ __forceinline__ void weights32(const Bufs &b, const Inst &I, const Sl
             if (i && r0 + i >= gr) break;   // uniform
             const int e0 = cur.e[i], e1 = cur.e[i + 1];
             const int4 A0 = A[0], A1 = A[1];
-            A[0] = b.A32[(i + 2 < ZR ? cur.e[(i + 2) % ZR] : next.e[0]) & ~NB_FAR];
-            A[1] = b.A32[(i + 2 < ZR ? cur.e[(i + 3) % ZR] : next.e[1]) & ~NB_FAR];
+            const float v0 = V[0], v1 = V[1];
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+                const int jn = (i + 2 < ZR ? cur.e[(i + 2 + t) % ZR] : next.e[t]) & ~NB_FAR;
+                A[t] = b.A32[jn];
+                if (SIDE) V[t] = b.side32[jn];
+            }
             const F2 rx = mul2(F2((float)fixed_diff(Ai.x, A0.x), (float)fixed_diff(Ai.x, A1.x)), u0);
             const F2 ry = mul2(F2((float)fixed_diff(Ai.y, A0.y), (float)fixed_diff(Ai.y, A1.y)), u1);
             const F2 rz = mul2(F2((float)fixed_diff(Ai.z, A0.z), (float)fixed_diff(Ai.z, A1.z)), u2);
@@ -710,7 +723,7 @@ __device__ __forceinline__ void weights32(const Bufs &b, const Inst &I, const Sl
             fma2(q, minus, one).get(m0, m1);
             const F2 om(fmaxf(m0, 0.0f), fmaxf(m1, 0.0f));
             const F2 W = mul2(mul2(mul2(mul2(Wc, fma2(q, F2(3.0f), one)), om), om), om);
-            f(W, e0 & ~NB_FAR, e1 & ~NB_FAR, ok0, ok1, a0, a1, A0.w, A1.w);
+            f(W, v0, v1, ok0, ok1, a0, a1, A0.w, A1.w);
         }
         cur = next;
         left -= ZR * LPP;
@@ -718,7 +731,7 @@ __device__ __forceinline__ void weights32(const Bufs &b, const Inst &I, const Sl
 }
 
 template <bool CLOSE>
-__global__ void __launch_bounds__(256) k_density32(Bufs b, int defer, const int *gate, int groups)
+__global__ void __launch_bounds__(256, 4) k_density32(Bufs b, int defer, const int *gate, int groups)
 {
     if (gate && *gate == 0) return;
     const int lane = threadIdx.x & 31, sub = lane % LPP;
@@ -741,8 +754,8 @@ __global__ void __launch_bounds__(256) k_density32(Bufs b, int defer, const int 
             const bool want_close = CLOSE && I.artvis && (h.type == T_FLUID || h.type == T_RIGID);
             const float close_r2 = want_close ? I.artvis_r2f_hi * 1.0001f : -1.0f;
             const long long s = h.n > 0 ? base + g * GROUP + lane / LPP : 0;
-            weights32(b, I, h, s, h.n, gr, sub,
-                      [&](F2 W, int, int, bool ok0, bool ok1, float r0, float r1, int t0, int t1) {
+            weights32<false>(b, I, h, s, h.n, gr, sub,
+                      [&](F2 W, float, float, bool ok0, bool ok1, float r0, float r1, int t0, int t1) {
                 sum.add_small(W);
                 if (CLOSE) {
                     close |= ok0 && r0 <= close_r2 && (t0 == T_FLUID || t0 == T_RIGID);
@@ -765,7 +778,7 @@ __global__ void __launch_bounds__(256) k_density32(Bufs b, int defer, const int 
 }
 
 template <bool REINIT>
-__global__ void __launch_bounds__(256) k_shepard32(Bufs b, int any_filter, const int *gate, int groups)
+__global__ void __launch_bounds__(256, 4) k_shepard32(Bufs b, int any_filter, const int *gate, int groups)
 {
     if (gate && *gate == 0) return;
     const int lane = threadIdx.x & 31, sub = lane % LPP;
@@ -778,13 +791,12 @@ __global__ void __launch_bounds__(256) k_shepard32(Bufs b, int any_filter, const
         const SlotHead h = mine.of_group(g);
         if (g + 1 < groups) prefetch_lists(b, base + (g + 1) * GROUP, mine.of_group(g + 1).n);
         const int gr = entry_rows(__reduce_max_sync(FULL, max(h.n, 0)));
-        Sum2 num(0.0f), den(0.0f);
+        Sum2 num(0.0f), den(REINIT ? 0.0f : (float)b.inst[h.inst].W0);   // (0 <= W <= W(0), see k_density32)
         if (gr > 0) {
             const Inst &I = b.inst[h.inst];
             const long long s = h.n > 0 ? base + g * GROUP + lane / LPP : 0;
-            weights32(b, I, h, s, h.n, gr, sub,
-                      [&](F2 W, int j0, int j1, bool ok0, bool ok1, float, float, int, int) {
-                float v0 = b.side32[j0], v1 = b.side32[j1];
+            weights32<true>(b, I, h, s, h.n, gr, sub,
+                      [&](F2 W, float v0, float v1, bool ok0, bool ok1, float, float, int, int) {
                 if constexpr (REINIT) {
                     float w0, w1;
                     W.get(w0, w1);
@@ -792,7 +804,7 @@ __global__ void __launch_bounds__(256) k_shepard32(Bufs b, int any_filter, const
                     den.add_any(F2(ok0 ? w0 / v0 : 0.f, ok1 ? w1 / v1 : 0.f));
                 } else {
                     num.add_any(mul2(F2(v0, v1), W));
-                    den.add_any(W);
+                    den.add_small(W);
                 }
             });
         }
@@ -806,8 +818,9 @@ __global__ void __launch_bounds__(256) k_shepard32(Bufs b, int any_filter, const
     }
     const long long s = base + lane;
     if (lane >= groups * GROUP || s >= b.N) return;
+    const double den0 = REINIT ? 0.0 : (double)(2 * LPP) * (double)(float)b.inst[mine.inst].W0;   // once in each half of each lane
     finish_shepard<float, REINIT>(b, b.inst[mine.inst], mine.type, s, (double)kn[0] + (double)kn[1],
-                                  (double)kd[0] + (double)kd[1], any_filter);
+                                  ((double)kd[0] - den0) + (double)kd[1], any_filter);
 }
 
 // ---------------------------------------------------------------- drag (A5)
