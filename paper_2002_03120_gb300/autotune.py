@@ -1,10 +1,9 @@
 """Autotuner of the per-workload launch choices of libsdpd.
 
 For one workload (a list of instances and a precision) it times full steps
-under each candidate setting -- force-pass variant (Newton-3 half pairs,
-direct, or the pair stream through shared memory at two register caps),
-Verlet skin, pair-kernel block size, lanes per particle of the direct pass,
-full- or half-size cells of the neighbour search -- picks the fastest, and keeps
+under each candidate setting -- force-pass variant (Newton-3 half pairs or
+direct), Verlet skin, pair-kernel block size, full- or half-size cells of the
+neighbour search -- picks the fastest, and keeps
 the choice in a JSON file keyed by GPU name, precision and size class (total
 particles rounded to a power of two, number of instances), so later contexts
 of the same class reuse it without measuring again.
@@ -25,17 +24,16 @@ import os
 from . import binding as B
 
 DEFAULT_CACHE = os.path.join(os.path.expanduser("~"), ".cache", "sdpd_gb300", "autotune.json")
-# force-pass variants (sdpd_set_force_mode): 1 Newton 3, 0 direct, 5 direct
-# with fewer registers (FP32 only).  Not sampled by default, because they
-# measured slower on every workload here: 2 and 3 (the pair stream: its
-# shared-memory compaction buys nothing where lanes are already busy, and
-# costs L1 and instructions) and 4 (Newton 3 with pushed results: the
-# scattered stores cost more than the coalesced gather saves)
+# force-pass variants (sdpd_set_force_mode): 1 Newton 3, 0 direct; 5, like 2
+# and 3, names the direct pass too (saved choices of it stay valid).  Not
+# sampled by default, because it measured slower on every workload here: 4
+# (Newton 3 with pushed results: the scattered stores cost more than the
+# coalesced gather saves)
 CANDIDATES = {
     "newton3": (1, 0, 5),
     "skin": (0.0, 0.03, 0.06, 0.12),
     "block": (64, 128, 256),
-    "tpp": (1, 2, 4),   # lanes per particle of the direct pass
+    "tpp": (1, 2, 4),   # accepted, without effect: every pair pass runs 8 lanes a particle
     "cells": (1, 2),    # cells per minimum cell width of the neighbour search
 }
 
@@ -69,21 +67,15 @@ def save_cache(cache: dict, path: str = DEFAULT_CACHE) -> None:
 
 
 def _sampled(setting, candidates, precision):
-    """Settings measured, with full-size cells: the Newton-3 passes over the
-    whole grid (the push variant for FP32 pairs only); the direct pass at the
-    default block (every skin) and without skin (every block), its lean form
-    (FP32 only, 128 threads) at the three smaller skins; the pair stream,
-    when asked for, at the two larger blocks and the two middle skins, the
-    three-block variant for FP32 pairs only.  Half-size cells: the Newton-3,
-    direct and lean direct passes at the default block and the three smaller
-    skins, and the direct pass with several lanes per particle at the default
-    block and skin."""
+    """Settings measured.  Full-size cells: the Newton-3 passes over the whole
+    grid (the push variant for FP32 pairs only); the direct pass at the default
+    block (every skin) and without skin (every block); its other names (2, 3
+    and 5, and several lanes per particle) at a few settings.  Half-size
+    cells: the same passes at the default block and the three smaller skins."""
     mode, skin, block = setting["newton3"], setting["skin"], setting["block"]
     skins = candidates["skin"]
     if setting.get("cells", 1) != 1:
-        # half-size cells: the default block, the three smaller skins; Newton
-        # 3, direct and lean direct (FP32) with one lane per particle, and
-        # the direct pass with several lanes at the default skin
+        # half-size cells: the default block, the three smaller skins
         if block != 128 or skin not in skins[:3]:
             return False
         if setting.get("tpp", 1) != 1:

@@ -13,8 +13,9 @@
 // The list is a superset of the pairs within h; every consumer re-decides
 // r_ij < h exactly, so the evaluated pair set equals the paper's.  The list
 // stays valid while no particle has moved more than skin h / 2 since the
-// build; the drift raises `need_build` when one has, and every kernel here
-// is gated on that flag inside the captured step.  Only the instances whose
+// build; the drift raises `need_build` when one has and opens the conditional
+// node of the captured step that holds these kernels (a build enqueued after
+// an upload has the flag as its gate instead).  Only the instances whose
 // own flag is up are rebuilt: an instance's slots are the range of its gids,
 // so the others keep their cells, slots and lists.
 #include <algorithm>

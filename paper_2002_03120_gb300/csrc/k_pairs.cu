@@ -1,10 +1,13 @@
 // k_pairs.cu -- the pair passes of one velocity-Verlet sub-step.
 //
-//   k_density      compute_particle_dens + compute_particle_pres (Eqs. compdens,
+//   k_density32 (FP32), k_density or k_density_half + k_density_gather (FP64)
+//                  compute_particle_dens + compute_particle_pres (Eqs. compdens,
 //                  prtcpres; kernel normalisation; negative-pressure clamp)
-//   k_filter       smoothe_particle_pres (Shepard-weighted pressure)
-//   k_drag         compute_fpi_action (Eqs. fvfdef, beta, F_fpi_DG)
-//   k_force_half + k_force_gather (Newton-3) or k_force_fluid (direct):
+//   k_shepard32, k_shepard  smoothe_particle_pres (Shepard-weighted pressure),
+//                  density reinitialisation
+//   k_drag, k_drag_law  compute_fpi_action (Eqs. fvfdef, beta, F_fpi_DG)
+//   k_force_half + k_force_gather (Newton-3), k_force_draw and k_force_cached
+//   (direct, FP32) or k_force_fluid (direct, FP64):
 //                  compute_fluid on fluid particles + compute_fpi_reaction
 //                  (Eqs. FijC, FijD, FijR, FijT, F_fpi_DG_reac) + torque
 //   k_force_rigid  compute_fluid on rigid particles (Eq. F_fpi_PG) +
