@@ -379,7 +379,7 @@ __device__ __forceinline__ void finish_density(const Bufs &b, const Inst &I, int
     }
 }
 
-// The FP64 kernel sum of the entries [k0, n) of slot s on this lane; close: a
+// The FP64 sum of W / W(0) over the entries [k0, n) of slot s on this lane; close: a
 // mobile neighbour inside the collision radius of the artificial viscosity (a
 // superset: the collision pass decides exactly; CLOSE: some instance of the
 // context has it)
@@ -392,7 +392,7 @@ __device__ __forceinline__ double density_entries(const Bufs &b, const Inst &I, 
     const double4_32a *A = b.A64;
     const double4_32a Ai = A[s];
     const Geo<double> geo(I);
-    const double Wc = I.Wc, irc = I.inv_rc;
+    const double irc = I.inv_rc;
     double acc = 0.0;
     for_each_entry(b.nbr, s, b.rows, k0, n, sub, ListHead(b.nbr, s, b.rows, k0, n, sub), A, nullptr,
                    [&](int, uint32_t e, const double4_32a &Aj, double) {
@@ -407,7 +407,7 @@ __device__ __forceinline__ double density_entries(const Bufs &b, const Inst &I, 
         root_and_inverse(r2, r, ir);
         const double q = r * irc, om = one_minus(q);
         // a separate rounding of each term (no multiply-add fused into the sum)
-        acc = __dadd_rn(acc, Wc * (1.0 + 3.0 * q) * om * om * om);
+        acc = __dadd_rn(acc, (1.0 + 3.0 * q) * om * om * om);
     });
     return acc;
 }
@@ -441,11 +441,11 @@ __global__ void __launch_bounds__(256) k_density(Bufs b, int defer, const int *g
     const long long s = base + lane;
     if (lane >= groups * GROUP || s >= b.N) return;
     const Inst &I = b.inst[mine.inst];
-    finish_density<double>(b, I, mine.type, s, __dadd_rn(__dadd_rn(I.W0, kown), koth), kclose, defer);
+    finish_density<double>(b, I, mine.type, s, I.W0 * __dadd_rn(__dadd_rn(1.0, kown), koth), kclose, defer);
 }
 
 // FP64 density with each unordered pair evaluated once (Newton 3): phase 1
-// sums W over the owned prefix of the list and stores each W for the partner
+// sums W / W(0) over the owned prefix of the list and stores each for the partner
 // (negated when the pair lies inside the collision radius of the artificial
 // viscosity; 0 for pairs beyond h) in the partner's column of the pair
 // buffer, which is free between force passes (a scattered store, which does
@@ -477,7 +477,7 @@ __global__ void __launch_bounds__(256) k_density_half(Bufs b, const int *gate, i
             const Geo<double> geo(I);
             const double close_r2 = (double)(I.artvis_r2f_hi * 1.0001f);
             const bool want_close = I.artvis != 0;
-            const double irc = K<double>::inv_rc(I), Wc = K<double>::Wc(I);
+            const double irc = K<double>::inv_rc(I);
             for_each_entry(b.nbr, s, b.rows, 0, h.nf, sub, ListHead(b.nbr, s, b.rows, 0, h.nf, sub), A, nullptr,
                            [&](int k, uint32_t e, const double4_32a &Aj, double) {
                 double W = 0.0;
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(256) k_density_half(Bufs b, const int *gate, i
                         double r, ir;
                         root_and_inverse(r2, r, ir);
                         const double q = r * irc, om = one_minus(q);
-                        W = Wc * (1.0 + 3.0 * q) * om * om * om;
+                        W = (1.0 + 3.0 * q) * om * om * om;
                         acc = __dadd_rn(acc, W);
                         if (want_close && r2 <= close_r2) {
                             const int tj = mir_type(Aj);
@@ -549,7 +549,7 @@ __global__ void __launch_bounds__(256) k_density_gather(Bufs b, int defer, const
     const int ti = mine.type;
     const Inst &I = b.inst[mine.inst];
     const bool close = (b.aclose[s] != 0 || kclose) && (ti == T_FLUID || ti == T_RIGID);
-    finish_density<double>(b, I, ti, s, __dadd_rn(__dadd_rn(I.W0, b.sd[s]), keep), close, defer);
+    finish_density<double>(b, I, ti, s, I.W0 * __dadd_rn(__dadd_rn(1.0, b.sd[s]), keep), close, defer);
 }
 
 // ------------------------------------------------------ density reinitialisation
