@@ -765,8 +765,10 @@ static void launch_lists(const Bufs &b, const int *gate, cudaStream_t st)
     // cells only where the cells alone leave SMs idle (16,000 particles: 166 us
     // a build with one, 115 with four; 662,000: 1.53 ms with one, 1.66 with four);
     // a warp without a group leaves at once.  8,192 particles in full cells: 381
-    // us with 8, 198 with 24.
-    const int parts = SUB == 1 ? 24 : std::min(4, std::max(1, 16384 / b.ncell_total));
+    // us with 8, 198 with 24; fewer where most cells are empty, so that
+    // a large domain is not a launch of idle blocks.
+    const int parts = SUB == 1 ? (int)std::min<long long>(24, std::max<long long>(1, 4 * b.N / b.ncell_total))
+                               : std::min(4, std::max(1, 16384 / b.ncell_total));
     const size_t wb = ng_warp_bytes(b.cap);
     const unsigned nb = (unsigned)b.ncell_total * parts;
     if (b.split) k_neighbors<SUB, true><<<nb, 32, wb, st>>>(b, parts, gate);
