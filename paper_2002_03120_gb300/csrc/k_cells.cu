@@ -436,8 +436,10 @@ __global__ void __launch_bounds__(32, 24) k_neighbors(Bufs b, int parts, const i
         if (__ballot_sync(FULL, key >= 0) != FULL) break;
     }
     if (fat) {
-        // the list buffer serves as the routine's stage (512 bytes)
-        if (part == 0) nb_scan_cell(b, c, s0, s1, reinterpret_cast<int4 *>(buf), lane);
+        // the staging records, idle here, serve as the routine's stage (the list
+        // buffer is smaller than 32 records for capacities up to 8)
+        static_assert(NG_STAGE >= 32, "the routine stages 32 records");
+        if (part == 0) nb_scan_cell(b, c, s0, s1, S.sa, lane);
         return;
     }
     if (lane == 0) S.pre[nq] = total;
