@@ -1603,15 +1603,20 @@ struct NormalRing {
     int fill[24];
 };
 static_assert(sizeof(NormalRow<float>) == 768 && sizeof(NormalRing) % 128 == 0, "bulk copies are 16-byte aligned");
-constexpr int RING_WAIT_LIMIT = 1 << 22;
+// tries of a wait: for the chunk that is next, and for what is still on its
+// way when one of those gave up (a test builds the pass with no tries)
+#ifndef RING_TRIES
+#define RING_TRIES (1 << 22)
+#endif
+constexpr int RING_DRAIN_TRIES = 1 << 22;
 
 __device__ __forceinline__ unsigned smem_addr(const void *p) { return (unsigned)__cvta_generic_to_shared(p); }
 
-// Waits (bounded) for the phase of parity `par`; false when it gave up.
-__device__ __forceinline__ bool ring_wait(uint64_t *bar, unsigned par)
+// Waits (at most `tries` times) for the phase of parity `par`; false when it gave up.
+__device__ __forceinline__ bool ring_wait(uint64_t *bar, unsigned par, int tries)
 {
     const unsigned a = smem_addr(bar);
-    for (int it = 0; it < RING_WAIT_LIMIT; ++it) {
+    for (int it = 0; it < tries; ++it) {
         unsigned done;
         asm volatile("{\n\t.reg .pred P;\n\tmbarrier.try_wait.parity.shared::cta.b64 P, [%1], %2;\n\t"
                      "selp.u32 %0, 1, 0, P;\n\t}"
@@ -1656,6 +1661,7 @@ __global__ void __launch_bounds__(ZTHREADS, 4) k_force_cached(Bufs b, int groups
     }
     // the copies, chunk by chunk through the groups
     int pg = 0, pr = 0;   // next row to ask for: of group pg
+    unsigned asked = 0;   // chunks asked for
     auto request = [&](int st) {
         while (pg < groups && pr >= ring.zrows[pg]) {
             ++pg;
@@ -1674,6 +1680,7 @@ __global__ void __launch_bounds__(ZTHREADS, 4) k_force_cached(Bufs b, int groups
                          : "memory");
         }
         pr += ZR;
+        ++asked;
     };
     unsigned chunk = 0;   // chunks consumed: in stage chunk % ZS, its phase chunk / ZS
     for (int i = 0; i < ZS; ++i) request(i);
@@ -1697,10 +1704,13 @@ __global__ void __launch_bounds__(ZTHREADS, 4) k_force_cached(Bufs b, int groups
                 nb += ZR * ROW;
                 next.load(nb, left - ZR * LPP);
                 const int st = chunk % ZS;
-                if (normals && !ring_wait(ring.bar + st, (chunk / ZS) & 1u)) {
-                    // give the copy one more bounded wait before its buffer is left
-                    atomicOr(b.err, ERR_TIMEOUT);
-                    (void)ring_wait(ring.bar + st, (chunk / ZS) & 1u);
+                if (normals && !__all_sync(FULL, ring_wait(ring.bar + st, (chunk / ZS) & 1u, RING_TRIES))) {
+                    // the warp leaves: no barrier is armed again within its
+                    // phase, and every copy still on its way gets one more
+                    // bounded wait before its buffer is left
+                    if (lane == 0) atomicOr(b.err, ERR_TIMEOUT);
+                    for (unsigned c = chunk; c < asked; ++c) (void)ring_wait(ring.bar + c % ZS, (c / ZS) & 1u, RING_DRAIN_TRIES);
+                    return;
                 }
                 const NormalRow<float> *zrow = ring.z[st];
 #pragma unroll
