@@ -403,9 +403,7 @@ __device__ __forceinline__ double density_entries(const Bufs &b, const Inst &I, 
             const int tj = mir_type(Aj);
             close |= (tj == T_FLUID || tj == T_RIGID);
         }
-        double r, ir;
-        root_and_inverse(r2, r, ir);
-        const double q = r * irc, om = one_minus(q);
+        const double q = root(r2) * irc, om = one_minus(q);
         // a separate rounding of each term (no multiply-add fused into the sum)
         acc = __dadd_rn(acc, (1.0 + 3.0 * q) * om * om * om);
     });
@@ -484,9 +482,7 @@ __global__ void __launch_bounds__(256) k_density_half(Bufs b, const int *gate, i
                 if (!(e & NB_FAR)) {
                     double rx, ry, rz, r2;
                     if (Rel<double>::get(b, I, geo, Ai, Aj, gi, (int)e, rx, ry, rz, r2)) {
-                        double r, ir;
-                        root_and_inverse(r2, r, ir);
-                        const double q = r * irc, om = one_minus(q);
+                        const double q = root(r2) * irc, om = one_minus(q);
                         W = (1.0 + 3.0 * q) * om * om * om;
                         acc = __dadd_rn(acc, W);
                         if (want_close && r2 <= close_r2) {
@@ -571,10 +567,9 @@ __device__ __forceinline__ void shepard_entries(const Bufs &b, const Inst &I, lo
     for_each_entry(b.nbr, s, b.rows, 0, h.n, sub, ListHead(b.nbr, s, b.rows, 0, h.n, sub), A, REINIT ? b.sd : b.sp,
                    [&](int, uint32_t e, const double4_32a &Aj, double v) {
         if (e & NB_FAR) return;
-        double rx, ry, rz, r2, r, ir;
+        double rx, ry, rz, r2;
         if (!Rel<double>::get(b, I, geo, Ai, Aj, h.gi, (int)e, rx, ry, rz, r2)) return;
-        root_and_inverse(r2, r, ir);
-        const double q = r * I.inv_rc, om = one_minus(q);
+        const double q = root(r2) * I.inv_rc, om = one_minus(q);
         const double W = I.Wc * (1.0 + 3.0 * q) * om * om * om;
         // a separate rounding of each term (no multiply-add fused into the sum)
         num = __dadd_rn(num, REINIT ? W : __dmul_rn(v, W));
@@ -910,9 +905,7 @@ __global__ void __launch_bounds__(RB) k_drag(Bufs b)
                 const double Rj = b.R[b.perm[j]];
                 Vsum += 4.0 / 3.0 * PI * Rj * Rj * Rj;
             } else {
-                R r, ir;
-                root_and_inverse(r2, r, ir);
-                const R q = r * irc, om = R(1) - q;
+                const R q = root(r2) * irc, om = R(1) - q;
                 const R W = Wc * (R(1) + R(3) * q) * om * om * om;
                 Sr += W;
                 u0 += W * Bu[u].x;

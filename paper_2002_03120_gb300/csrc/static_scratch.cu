@@ -47,7 +47,7 @@ struct Grid {
     double fix[3];                // 2^32 / window
     float unit[3];                // window / 2^32
     float r2_hi;                  // r_c^2 widened past the error of the test
-    double inv_rc, rc2, Wc, Cn, mf, inv_dx3, rho0, p0, alpha, beta_p;
+    double inv_rc, inv_rc_lo, rc2, Wc, Cn, mf, inv_dx3, rho0, p0, alpha, beta_p;
     int clamp;
     long long n;
 };
@@ -166,8 +166,10 @@ __global__ void k_na_scatter(int *scr, Grid G, const double *x)
 //    when the FP64 part runs; it re-decides r < r_c as before.
 // One thread per particle over unsorted candidates, each wrapped by an FP64
 // division per axis, took 13.4 ms for 46,255 particles; the call now takes
-// 0.56 ms (0.82 with the image by a rounded quotient wherever a lane of a warp
-// wraps).
+// 0.58 ms (0.82 with the image by a rounded quotient wherever a lane of a warp
+// wraps; 0.56 with r / r_c to 1.75 ulp, whose densities were 6 % further off
+// than those of a rounded root and quotient: rms 1.96e-15 against 1.85e-15 of
+// the value, now 1.81e-15).
 constexpr int ND_WARPS = 4;
 
 __device__ __forceinline__ double na_term(const Grid &G, const double xi[3], const double *__restrict__ x, int j)
@@ -190,9 +192,9 @@ __device__ __forceinline__ double na_term(const Grid &G, const double xi[3], con
     }
     const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])), __dmul_rn(r[2], r[2]));
     if (!lt_pos(r2, G.rc2)) return 0.0;   // also a NaN
-    double root, inv;
-    root_and_inverse(r2, root, inv);
-    const double q1 = hi_abs(r2) >= 0x00100000 ? root * G.inv_rc : 0.0, om = 1.0 - q1;   // (r2 zero or subnormal: q is 0)
+    // r / r_c by the reciprocal of r_c in two parts: the rounding of the quotient
+    const double r1 = root(r2), q = fma(r1, G.inv_rc, r1 * G.inv_rc_lo);
+    const double q1 = hi_abs(r2) >= 0x00100000 ? q : 0.0, om = 1.0 - q1;   // (r2 zero or subnormal: q is 0)
     return (1.0 + 3.0 * q1) * om * om * om;   // W / W(0)
 }
 
@@ -377,6 +379,7 @@ extern "C" sdpd_status sdpd_density_noalloc(const sdpd_params *p, long long n, c
     }
     const double h = p->r_c;
     G.inv_rc = 1.0 / h;
+    G.inv_rc_lo = std::fma(-G.inv_rc, h, 1.0) * G.inv_rc;
     G.rc2 = h * h;
     for (int a = 0; a < 3; ++a) {
         // a periodic box is a whole number of windows (the fixed-point
