@@ -193,9 +193,8 @@ __device__ __forceinline__ double na_term(const Grid &G, const double xi[3], con
     const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])), __dmul_rn(r[2], r[2]));
     if (!lt_pos(r2, G.rc2)) return 0.0;   // also a NaN
     // r / r_c by the reciprocal of r_c in two parts: the rounding of the quotient
-    const double r1 = root(r2), q = fma(r1, G.inv_rc, r1 * G.inv_rc_lo);
-    const double q1 = hi_abs(r2) >= 0x00100000 ? q : 0.0, om = 1.0 - q1;   // (r2 zero or subnormal: q is 0)
-    return (1.0 + 3.0 * q1) * om * om * om;   // W / W(0)
+    const double r1 = root(r2), q = fma(r1, G.inv_rc, r1 * G.inv_rc_lo), om = 1.0 - q;
+    return (1.0 + 3.0 * q) * om * om * om;   // W / W(0)
 }
 
 __global__ void __launch_bounds__(ND_WARPS * 32) k_na_density(const int *scr, Grid G, const double *x, const int *type,
