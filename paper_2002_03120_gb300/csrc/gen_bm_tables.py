@@ -2,7 +2,8 @@
 Box-Muller transform of the GPU pair kernels (correctly rounded doubles,
 computed with mpmath at 60 digits).
 
-  LOG_TAB[j]  = { -2 ln(1 + j/2048), 1 / (1 + j/2048) }           j = 0..2047
+  LOG_TAB[j]  = { -2 ln c_j, 1 / (1 + j/2048) }                   j = 0..2047
+                c_j = 1 + j/2048 in the lower half, (1 + j/2048) / 2 in the upper
   LOG_E[e]    = -2 (e - 24) ln 2                                  e = 0..31
   SC_HI[h]    = { sin(pi/2 h/1024), cos(pi/2 h/1024) }             h = 0..1023
   SC_LO[l]    = { sin, cos of pi/2 (2 l + 1) / 2^22 }              l = 0..2047
@@ -31,7 +32,7 @@ def main():
         lines.append("};")
 
     c = [1 + mpmath.mpf(j) / 2048 for j in range(2048)]
-    table("static __device__ const double2 BM_LOG_TAB[2048]", [f"{{{d(-2 * mpmath.log(x))}, {d(1 / x)}}}" for x in c])
+    table("static __device__ const double2 BM_LOG_TAB[2048]", [f"{{{d(-2 * mpmath.log(x if j < 1024 else x / 2))}, {d(1 / x)}}}" for j, x in enumerate(c)])
     table("static __device__ const double BM_LOG_E[32]", [d(-2 * (e - 24) * mpmath.log(2)) for e in range(32)])
     hi = [mpmath.pi / 2 * h / 1024 for h in range(1024)]
     lo = [mpmath.pi / 2 * (2 * k + 1) / 2 ** 22 for k in range(2048)]
