@@ -43,10 +43,12 @@ struct Grid {
     int fbox[3];                  // high word of 1.49 box
     int nc[3], periodic[3];
     // fixed-point coordinates of the candidate test: units of window / 2^32,
-    // the window a whole fraction of a periodic box and at least 4 r_c wide
+    // the window a whole fraction of a periodic box and at least 4 r_c wide.
+    // The test's lengths are in r_c, so that its FP32 squares suit any r_c
+    // (in the caller's units they left FP32's range beyond 1e19 and 1e-19).
     double fix[3];                // 2^32 / window
-    float unit[3];                // window / 2^32
-    float r2_hi;                  // r_c^2 widened past the error of the test
+    float unit[3];                // window / (2^32 r_c)
+    float r2_hi;                  // 1, widened past the error of the test
     double inv_rc, inv_rc_lo, rc2, Wc, Cn, mf, inv_dx3, rho0, p0, alpha, beta_p;
     int clamp;
     long long n;
@@ -122,11 +124,13 @@ __global__ void k_na_scan(int *scr, int ncell, long long n)
 // Records in cell order: the coordinates in fixed point, modulo a window of at
 // least 4 r_c, and the particle's index.  The difference of two such
 // coordinates wraps like the minimum image, so the candidate test needs no
-// branch on periodic axes, and is off by about 2^-28 r_c, far inside the
-// margin of r2_hi.  That holds for positions in the grid and on periodic axes
-// within 2^16 boxes of it (w below has an error of 2^-53 of its size); a
-// particle further out passes every candidate test (REC_FAR) and the FP64
-// part decides.  A non-finite position is nobody's neighbour: index -1.
+// branch on periodic axes, and is off by about 2^-28 r_c for positions in the
+// box and by up to 2^-22 r_c for positions on periodic axes within 2^16 boxes
+// of it (w below has an error of 2^-52 of its size; the cells' limit leaves an
+// axis fewer than 2^11 windows), inside the margin of r2_hi.  A particle
+// further out, or outside the grid on a wall axis, passes every candidate test
+// (REC_FAR) and the FP64 part decides.  A non-finite position is nobody's
+// neighbour: index -1.
 constexpr int REC_FAR = 1 << 30;
 static_assert(NMAX <= REC_FAR, "the flag bit is above every index");
 
@@ -386,7 +390,7 @@ extern "C" sdpd_status sdpd_density_noalloc(const sdpd_params *p, long long n, c
         const double k = std::max(1.0, std::floor(G.box[a] / (4.0 * h)));
         const double window = G.periodic[a] ? G.box[a] / k : 4.0 * h;
         G.fix[a] = 4294967296.0 / window;
-        G.unit[a] = (float)(window / 4294967296.0);
+        G.unit[a] = (float)(window / h / 4294967296.0);
         G.inv_box[a] = 1.0 / G.box[a];
         const double hb = 0.5 * G.box[a];
         unsigned long long bits;
@@ -397,7 +401,7 @@ extern "C" sdpd_status sdpd_density_noalloc(const sdpd_params *p, long long n, c
         G.fbox[a] = (int)(bits >> 32);
     }
     // FP32 products of fixed-point differences: relative error of r^2 below 1e-6
-    G.r2_hi = (float)(G.rc2 * (1.0 + 1e-5));
+    G.r2_hi = 1.0f + 1e-5f;
     G.Wc = 105.0 / (16.0 * sdpd::PI * h * h * h);
     const int m = (int)std::ceil(h / p->dx) + 1;
     double lat = 0.0;
