@@ -284,6 +284,9 @@ sdpd_status prepare(sdpd_ctx *c)
         I.coeff_cf = (float)p.coeff_c; I.coeff_df = (float)p.coeff_d;
         I.coeff_rf = (float)p.coeff_r; I.coeff_tf = (float)p.coeff_t;
         I.lever_fluidf = (float)I.lever_fluid;
+        const int m4 = (int)std::floor(-0.75 * std::log2(p.dx * p.dx));   // log4(1 / dx^3)
+        I.d_scale = (float)std::ldexp(1.0, 2 * m4);
+        I.d_unscale = (float)std::ldexp(1.0, -m4);
         I.rb = rb;
         I.rb2 = rb * rb;
         I.half_skin = 0.5 * skin * h;
