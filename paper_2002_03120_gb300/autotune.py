@@ -70,7 +70,8 @@ def _sampled(setting, candidates, precision):
     """Settings measured.  Full-size cells: the Newton-3 passes over the whole
     grid (the push variant for FP32 pairs only); the direct pass at the default
     block (every skin) and without skin (every block); its other names (2, 3
-    and 5, and several lanes per particle) at a few settings.  Half-size
+    and 5, and several lanes per particle) at a few settings, which take its
+    time without a run of their own (once_per_kernel).  Half-size
     cells: the same passes at the default block and the three smaller skins."""
     mode, skin, block = setting["newton3"], setting["skin"], setting["block"]
     skins = candidates["skin"]
@@ -114,6 +115,22 @@ def search(measure, candidates=CANDIDATES, precision=None):
         if t is not None and t < best_t:
             best, best_t = setting, t
     return best, table
+
+
+def once_per_kernel(measure):
+    """`measure` called once for all settings that run the same kernels: the
+    force modes 0, 2, 3 and 5 are one pass, whatever the lanes per particle.
+    The first name met keeps the time (0 and one lane in the candidates' order),
+    so an alias never wins by noise."""
+    seen = {}
+
+    def timed(setting):
+        key = tuple(sorted((k, 0 if k == "newton3" and v in (2, 3, 5) else v) for k, v in setting.items() if k != "tpp"))
+        if key not in seen:
+            seen[key] = measure(setting)
+        return seen[key]
+
+    return timed
 
 
 def apply(sim: "B.Sim", setting: dict) -> None:
@@ -160,7 +177,7 @@ def tune(cases, precision=B.SDPD_PREC_SPLIT, steps=10, warmup=3, cache_path=DEFA
             return None
 
     try:
-        best, table = search(measure, candidates, precision)
+        best, table = search(once_per_kernel(measure), candidates, precision)
     finally:
         sim.close()
     cache[key] = {"best": best, "table": table, "particles": n, "instances": len(cases)}
