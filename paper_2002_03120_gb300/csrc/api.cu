@@ -60,6 +60,7 @@ struct sdpd_ctx {
     double skin = 0.03;                // Verlet skin as a fraction of h
     int cell_sub = 1;                  // cells per minimum cell width: 1 (27-cell stencil) or 2 (125)
     bool geometry_ready = false, cells_valid = false, density_valid = false, drag_valid = false;
+    bool built = false;                // some build has put every particle in a slot
     bool absorbed = false;             // positions uploaded since the last step, lists kept
     int sticky_err = 0;
     long long host_step = 0;
@@ -459,6 +460,7 @@ void enqueue_build(sdpd_ctx *c, cudaStream_t st, const int *gate = nullptr)
     // the FP64 density of the direct pass sums in the half-pair pass's order
     c->b.split = c->precision == SDPD_PREC_FP64 || half_pairs(c->newton3);
     launch_build(c->b, c->precision, half_pairs(c->newton3), gate, st);
+    c->built = true;
 }
 
 int density_passes(const sdpd_ctx *c) { return c->any_filter | (c->any_reinit << 1) | (c->any_artvis << 2); }
@@ -694,6 +696,9 @@ sdpd_status sdpd_init(const sdpd_params *params, int n_instances, const long lon
         cudaMemset(b.list_epoch, 0, sizeof(unsigned) * ni) != cudaSuccess ||
         cudaMemset(b.cache_epoch, 0xFF, sizeof(unsigned) * ni) != cudaSuccess ||
         cudaMemset(b.cache_step, 0xFF, sizeof(long long)) != cudaSuccess)
+        return cleanup(fail(SDPD_E_CUDA, "cudaMemset failed"));
+    // slots in range and no density before the first build (the diagnostics read them)
+    if (N && (cudaMemset(b.slot_of, 0, sizeof(int) * N) != cudaSuccess || cudaMemset(b.sd, 0, sizeof(double) * N) != cudaSuccess))
         return cleanup(fail(SDPD_E_CUDA, "cudaMemset failed"));
     if (cudaMemset(b.err, 0, sizeof(int)) != cudaSuccess || cudaMemset(b.step, 0, sizeof(long long)) != cudaSuccess ||
         cudaMemset(b.F, 0, sizeof(double) * (n3 ? n3 : 1)) != cudaSuccess ||
@@ -1006,7 +1011,7 @@ sdpd_status sdpd_integrate(sdpd_ctx *c, int velver, void *stream)
     if (!c) return fail(SDPD_E_INVALID, "NULL context");
     (void)cudaGetLastError();  // launch errors below are this call's own
     if (velver != 1 && velver != 2) return fail(SDPD_E_INVALID, "velver must be 1 or 2");
-    if (!c->geometry_ready || !c->b.inst) return fail(SDPD_E_STATE, "no forces computed yet");
+    if (!c->geometry_ready || !c->b.inst || (c->N && !c->built)) return fail(SDPD_E_STATE, "no forces computed yet");
     cudaStream_t st = (cudaStream_t)stream;
     launch_integrate(c->b, c->precision, velver, c->any_artvis, st);
     if (velver == 2) c->host_step += 1;
