@@ -278,8 +278,8 @@ sdpd_status prepare(sdpd_ctx *c)
         I.lever_fluid = 0.5 * p.dx;
         I.key0 = (uint32_t)(p.seed & 0xFFFFFFFFull);
         I.key1 = (uint32_t)(p.seed >> 32) ^ (uint32_t)k;
-        I.rcf = (float)h; I.inv_rcf = (float)(1.0 / h);
-        I.Wcf = (float)I.Wc; I.Fcf = (float)I.Fc; I.W0f = (float)I.W0;
+        I.inv_rcf = (float)(1.0 / h);
+        I.Wcf = (float)I.Wc; I.Fcf = (float)I.Fc;
         I.Caf = (float)I.Ca; I.Cbf = (float)I.Cb; I.Kaf = (float)I.Ka; I.Kbf = (float)I.Kb;
         I.isqrt_dtf = (float)I.isqrt_dt;
         I.coeff_cf = (float)p.coeff_c; I.coeff_df = (float)p.coeff_d;
@@ -644,7 +644,7 @@ sdpd_status sdpd_init(const sdpd_params *params, int n_instances, const long lon
     IALLOC(b.rxn, N); IALLOC(b.rxn32, N);
     IALLOC(b.A32, N);
     if (precision == SDPD_PREC_SPLIT) {
-        IALLOC(b.B32, N); IALLOC(b.C32, N); IALLOC(b.D32, N);
+        IALLOC(b.B32, N); IALLOC(b.C32, N); IALLOC(b.D32, N); IALLOC(b.side32, N);
     } else {
         IALLOC(b.A64, N); IALLOC(b.B64, N); IALLOC(b.C64, N); IALLOC(b.D64, N);
     }
@@ -682,7 +682,7 @@ sdpd_status sdpd_init(const sdpd_params *params, int n_instances, const long lon
         b.ownA = oa; b.ownB = ob;
     }
     IALLOC(b.A32_build, N);
-    IALLOC(b.aclose, N); IALLOC(b.aclose_ok, 1); IALLOC(b.sdr, N); IALLOC(b.side32, N); IALLOC(b.xs, 3 * N);
+    IALLOC(b.aclose, N); IALLOC(b.aclose_ok, 1); IALLOC(b.sdr, N); IALLOC(b.xs, 3 * N);
     const size_t ni = (size_t)n_instances + 1;
     IALLOC(b.need_build, ni); IALLOC(b.fresh, 1);
     IALLOC(b.list_epoch, ni); IALLOC(b.cache_epoch, ni); IALLOC(b.cache_step, 1);

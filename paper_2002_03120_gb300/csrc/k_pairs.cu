@@ -78,7 +78,6 @@ template <> struct K<float> {
     __device__ __forceinline__ static float inv_rc(const Inst &I) { return I.inv_rcf; }
     __device__ __forceinline__ static float Wc(const Inst &I) { return I.Wcf; }
     __device__ __forceinline__ static float Fc(const Inst &I) { return I.Fcf; }
-    __device__ __forceinline__ static float W0(const Inst &I) { return I.W0f; }
     __device__ __forceinline__ static float Ca(const Inst &I) { return I.Caf; }
     __device__ __forceinline__ static float Cb(const Inst &I) { return I.Cbf; }
     __device__ __forceinline__ static float Ka(const Inst &I) { return I.Kaf; }
@@ -94,7 +93,6 @@ template <> struct K<double> {
     __device__ __forceinline__ static double inv_rc(const Inst &I) { return I.inv_rc; }
     __device__ __forceinline__ static double Wc(const Inst &I) { return I.Wc; }
     __device__ __forceinline__ static double Fc(const Inst &I) { return I.Fc; }
-    __device__ __forceinline__ static double W0(const Inst &I) { return I.W0; }
     __device__ __forceinline__ static double Ca(const Inst &I) { return I.Ca; }
     __device__ __forceinline__ static double Cb(const Inst &I) { return I.Cb; }
     __device__ __forceinline__ static double Ka(const Inst &I) { return I.Ka; }
@@ -200,8 +198,6 @@ __device__ __forceinline__ void finalize_slot(const Bufs &b, long long s, double
 // cache are each read or written once per pass and would otherwise push the
 // particle records, which every list revisits, out of L2.
 __device__ __forceinline__ int ld_stream(const int *p) { return __ldcs(p); }
-__device__ __forceinline__ float4 ld_stream(const float4 *p) { return __ldcs(p); }
-__device__ __forceinline__ float2 ld_stream(const float2 *p) { return __ldcs(p); }
 __device__ __forceinline__ double2 ld_stream(const double2 *p) { return __ldcs(p); }
 __device__ __forceinline__ double4_32a ld_stream(const double4_32a *p)
 {
@@ -1273,13 +1269,14 @@ template <class R> struct NormalRow {   // a row of 32 entries of the cache
     T2 b[ROW];
 };
 
-template <class R, bool REUSE>
+template <bool REUSE>
 __device__ __forceinline__ void force_fluid_entries(const Bufs &b, long long s, const SlotHead &h, const ListHead &hd,
-                                                    int sub, uint32_t step, bool fill, ForceSums<R> &sums)
+                                                    int sub, uint32_t step, bool fill, ForceSums<double> &sums)
 {
-    using T4 = typename Vec<R>::T4;
-    using TA = typename Mir<R>::TA;
-    using T2 = typename Vec2<R>::T2;
+    using R = double;
+    using T4 = double4_32a;
+    using TA = double4_32a;
+    using T2 = double2;
     const int gi = h.gi;
     const Inst &I = b.inst[h.inst];
     const Geo<R> geo(I);
@@ -1374,8 +1371,8 @@ __global__ void __launch_bounds__(256) k_force_fluid(Bufs b, int velver, int gro
         const long long s = base + g * GROUP + lane / LPP;
         const SlotHead h = mine.of_group(g);
         const ListHead hd(b.nbr, s, b.rows, 0, h.n, sub);
-        if (u.reuse(b, h.inst)) force_fluid_entries<R, true>(b, s, h, hd, sub, u.step, false, sums);
-        else force_fluid_entries<R, false>(b, s, h, hd, sub, u.step, u.fill, sums);
+        if (u.reuse(b, h.inst)) force_fluid_entries<true>(b, s, h, hd, sub, u.step, false, sums);
+        else force_fluid_entries<false>(b, s, h, hd, sub, u.step, u.fill, sums);
         sums.close_group(g);
     }
     if (mine.n < 0) return;

@@ -210,14 +210,6 @@ __device__ __forceinline__ float gelu_prime(float z)
 }
 
 // Eight values of one row, written as one 16-byte core-matrix row.
-__device__ __forceinline__ void put8(uint8_t *tile, int r, int k0, const float *v)
-{
-    __nv_bfloat162 h[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) h[i] = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
-    *reinterpret_cast<uint4 *>(tile + core_off(r, k0)) = *reinterpret_cast<uint4 *>(h);
-}
-
 __device__ __forceinline__ void put8(uint8_t *tile, int r, int k0, const F2 *v)
 {
     __nv_bfloat162 h[4];
