@@ -167,7 +167,8 @@ sdpd_status sdpd_compute_forces(sdpd_ctx *ctx, int velver, void *stream);
 /* update(velver) (Algorithm 1; Eqs. newton1, newton2): velocity-Verlet half
  * kick of v and w; velver 1 also drifts x and applies the periodic wrap / wall
  * reflection; velver 2 applies the artificial viscosity (collision method) if
- * enabled and advances the step counter. */
+ * enabled and advances the step counter.  SDPD_E_STATE before the first list
+ * build. */
 sdpd_status sdpd_integrate(sdpd_ctx *ctx, int velver, void *stream);
 
 /* Algorithm 1 for n_steps full steps (both sub-steps, all stages), replayed

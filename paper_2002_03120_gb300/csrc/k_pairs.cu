@@ -981,8 +981,9 @@ __device__ __forceinline__ void ext_accel(const Inst &I, const double *x, double
 //   T1 = ct Ka/sqrt(dt d_i), T3 = ct (Kb - Ka)/(3 sqrt(dt d_i)) (sigma = K
 //   sqrt(F)/sqrt(d_i d_j)).  FP32 takes one root of the product instead, X = S/d_i
 //   times 1/d_j with S = 4^m, and T1, T3 hold 2^-m in the place of 1/sqrt(d_i):
-//   one hardware root a pair (two, one each, made the factor's rms error 1.3
-//   times as large), the same bits seen from i and from j.
+//   one hardware root a pair, the same bits seen from i and from j.  (Two, one of
+//   each density, save a product: 0.7 % of a step of 1.6M particles, at 1.3 times
+//   the factor's rms error.)
 template <class R> struct PairK {
     R irc, Wc, PC, A1, A2, A3, T1, T3, X;
     bool noise;

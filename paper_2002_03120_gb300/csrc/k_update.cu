@@ -99,7 +99,7 @@ __global__ void k_step_done(Bufs b) { step_done(b); }   // (a context without pa
 // gathers by gid, so every load stands before the first store (a store to one
 // axis once held back the loads of the next).  Displacements come from the
 // fixed-point coordinates instead of an FP64 sum that was read and written
-// every step.  Dam break of 374,000 particles, 151,000 of them moving: 54 ->
+// every step.  Dam break of 374,000 particles, 148,000 of them moving: 54 ->
 // 26 us with the drift, 22 -> 20 us without.
 template <class R>
 __global__ void __launch_bounds__(256) k_integrate(Bufs b, int velver, cudaGraphConditionalHandle gate)

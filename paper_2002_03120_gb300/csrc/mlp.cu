@@ -188,7 +188,7 @@ __device__ __forceinline__ F2 gelu2(F2 z)
     float z0, z1, d0, d1, e0, e1;
     z.get(z0, z1);
     // (a scalar product takes the absolute value with it; the packed one would
-    // cost two masks more: 10^6 rows 320 -> 310 us)
+    // cost two masks more: 10^6 rows 312 -> 303 us)
     const F2 a(fabsf(z0) * 0.70710678118654752f, fabsf(z1) * 0.70710678118654752f);
     fma2(F2(0.3275911f), a, F2(1.0f)).get(d0, d1);
     mul2(mul2(z, z), F2(-0.72134752044448170f)).get(e0, e1);
@@ -243,13 +243,13 @@ struct Net {
 // group overlap the GELU epilogues of the others.  Thread (part, row) takes
 // half the columns of its row.  The three hidden weight tiles are staged once
 // per CTA and shared.
-// Bound by the FP32 pipe (12 packed operations for two GELUs, busy 62 % of the
-// time) and by issue slots; the special-function unit is half busy.  10^6 rows:
-// 358 us with scalar GELUs, 326 us with packed ones, 316 us with two threads a
-// row (eight warps a scheduler instead of four), 308 us with the scalar
-// absolute value.  Tiles go round the CTAs
-// before a CTA gets a second one: 20,000 rows take 31 us, 47 us when a CTA was
-// filled first.
+// Bound by the FP32 pipe (12 packed operations for two GELUs, busy 65 % of the
+// time) and by issue slots (66 %); the special-function unit is a third busy.
+// 10^6 rows, calls back to back: 358 us with scalar GELUs and one thread a row,
+// 303 us with packed ones, two threads a row (eight warps a scheduler instead of
+// four) and the scalar absolute value.  Tiles go round the CTAs before a CTA
+// gets a second one: 20,000 rows take 25 us, and took half as long again when a
+// CTA was filled first.
 constexpr int NWG = 4, PARTS = 2, FWD_GROUP = 128 * PARTS;
 // weight and activation tiles; mbarriers, flags, TMEM slot; the input layer's
 // weights and biases of two units each as pairs
@@ -730,9 +730,9 @@ __global__ void __launch_bounds__(GRAD_THREADS, 1) k_mlp_grad(Net net, const flo
 // Inference of few rows: a tile of ROWS (16, 32 or 64) rows per CTA in the
 // gradient kernel's transposed form, so the chain of layers is short and the
 // 16 warps of every SM take part.  Bound by latency: the weights' way into
-// shared memory and four layers in turn.  1,001 rows take 16 us a call (46 us
-// with 128-row tiles packed four to a CTA, 29 us one to a CTA), 5,000 rows 19
-// us.  Same operations per row as above, in the same order.
+// shared memory and four layers in turn.  Calls back to back: 1,001 rows take
+// 10.3 us (18.5 us in 128-row tiles), 5,000 rows 13.2 us (20.0 us).  Same
+// operations per row as above, in the same order.
 template <int ROWS> struct RowsSmem {
     static constexpr uint32_t A_BYTES = (ROWS / 8) * TG;
     static constexpr uint32_t OFF_A = 3 * W_BYTES;         // two activation tiles, in turn
@@ -1101,10 +1101,11 @@ sdpd_status mlp_infer(sdpd_mlp *h, const float *X, float *Y, long long n, void *
     cudaStream_t st = (cudaStream_t)stream;
     (void)cudaGetLastError();
     // The smallest tile that covers the rows with one CTA per SM: a call of a
-    // given size takes the longer the larger its tiles (1,001 rows: 17.7 us in
-    // tiles of 16, 18.3 of 32, 19.4 of 64, 29.5 of 128), and a second round of
-    // small ones costs more than the next size up (2,500 rows: 24.6, 18.5;
-    // 5,000: 27.3 of 32, 20.1 of 64; 10,000: 28.7 of 64, 26.2 of 128).
+    // given size takes the longer the larger its tiles (calls of 1,001 rows back
+    // to back: 10.3 us in tiles of 16 or 32, 12.3 of 64, 18.5 of 128), and a second
+    // round of small ones costs more than the next size up (2,500 rows: 18.4 of
+    // 16, 12.3 of 32; 5,000: 18.5 of 32, 13.2 of 64; 10,000: 22.5 of 64, 20.5 of
+    // 128).
     const int rows = n <= 16LL * nsm ? 16 : n <= 32LL * nsm ? 32 : n <= 64LL * nsm ? 64 : WID;
     const unsigned grid = (unsigned)std::min<long long>((n + rows - 1) / rows, nsm);
     const Net &N = h->net;

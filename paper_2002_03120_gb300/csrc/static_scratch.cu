@@ -6,7 +6,7 @@
 // whole device and forbids foreign cudaMalloc calls, and control loops that
 // cannot afford the implicit device-wide synchronisation cudaMalloc and
 // cudaFree may cause.  This entry point serves them: its scratch (cell keys,
-// slots, counts, starts and the particle permutation) lives in one file-scope
+// slots, counts, starts and cell-ordered records) lives in one file-scope
 // __device__ array of fixed size that every GPU loading the library keeps
 // until process exit; the caller passes only inputs and outputs.
 //
