@@ -49,7 +49,9 @@ struct Grid {
     double fix[3];                // 2^32 / window
     float unit[3];                // window / (2^32 r_c)
     float r2_hi;                  // 1, widened past the error of the test
-    double inv_rc, inv_rc_lo, rc2, Wc, Cn, mf, inv_dx3, rho0, p0, alpha, beta_p;
+    double two_k, R, R4;          // 2^k, 2^k r_c in [1, 2) and four times it
+    double self, norm;            // the weight of r = 0; d = norm x the sum of the weights
+    double rc2, mf, inv_dx3, rho0, p0, alpha, beta_p;
     int clamp;
     long long n;
 };
@@ -170,13 +172,18 @@ __global__ void k_na_scatter(int *scr, Grid G, const double *x)
 //    when the FP64 part runs; it re-decides r < r_c as before.
 // One thread per particle over unsorted candidates, each wrapped by an FP64
 // division per axis, took 13.4 ms for 46,255 particles; the call now takes
-// 0.58 ms (0.82 with the image by a rounded quotient wherever a lane of a warp
-// wraps; 0.56 with r / r_c to 1.75 ulp, whose densities were 6 % further off
-// than those of a rounded root and quotient: rms 1.96e-15 against 1.85e-15 of
-// the value, now 1.81e-15).
+// 0.53 ms (0.82 with the image by a rounded quotient wherever a lane of a warp
+// wraps; 0.56 with r / r_c by a reciprocal, whose rounding moved all densities
+// one way, 0.58 by a reciprocal in two parts).  Densities are off by 1.4e-16 to
+// 2.8e-16 of their value, rms against 113-bit sums at six spacings (5e-16 to
+// 1.8e-15 with one thread a particle, the normalisation summed site by site).
 constexpr int ND_WARPS = 4;
 
-__device__ __forceinline__ double na_term(const Grid &G, const double xi[3], const double *__restrict__ x, int j)
+// `sum` plus the weight of the pair (i, j) where r < r_c.  With t = 2^k (r_c - r),
+// one rounding, W is (4 R - 3 t) t^3 of R = 2^k r_c in [1, 2), but for a factor
+// that the normalisation divides out: five operations from the root, the last
+// of them the addition, and no quotient or reciprocal of r_c to be rounded.
+__device__ __forceinline__ double na_add(const Grid &G, const double xi[3], const double *__restrict__ x, int j, double sum)
 {
     double r[3];
 #pragma unroll
@@ -195,10 +202,9 @@ __device__ __forceinline__ double na_term(const Grid &G, const double xi[3], con
         r[a] = t;
     }
     const double r2 = __dadd_rn(__dadd_rn(__dmul_rn(r[0], r[0]), __dmul_rn(r[1], r[1])), __dmul_rn(r[2], r[2]));
-    if (!lt_pos(r2, G.rc2)) return 0.0;   // also a NaN
-    // r / r_c by the reciprocal of r_c in two parts: the rounding of the quotient
-    const double r1 = root(r2), q = fma(r1, G.inv_rc, r1 * G.inv_rc_lo), om = 1.0 - q;
-    return (1.0 + 3.0 * q) * om * om * om;   // W / W(0)
+    if (!lt_pos(r2, G.rc2)) return sum;   // also a NaN
+    const double t = fma(-root(r2), G.two_k, G.R);
+    return fma(fma(-3.0, t, G.R4), t * t * t, sum);
 }
 
 __global__ void __launch_bounds__(ND_WARPS * 32) k_na_density(const int *scr, Grid G, const double *x, const int *type,
@@ -241,7 +247,7 @@ __global__ void __launch_bounds__(ND_WARPS * 32) k_na_density(const int *scr, Gr
             nq += __popc(m);
             __syncwarp();
             if (nq >= 32) {
-                sum += na_term(G, xi, x, q[lane]);
+                sum = na_add(G, xi, x, q[lane], sum);
                 const int rest = lane < nq - 32 ? q[32 + lane] : 0;
                 __syncwarp();
                 if (lane < nq - 32) q[lane] = rest;
@@ -267,9 +273,9 @@ __global__ void __launch_bounds__(ND_WARPS * 32) k_na_density(const int *scr, Gr
             if (G.periodic[0] && c0 == G.nc[0] - 1) run(start[row], start[row + 1]);
         }
     }
-    if (lane < nq) sum += na_term(G, xi, x, q[lane]);
+    if (lane < nq) sum = na_add(G, xi, x, q[lane], sum);
     sum = warp_sum(sum);
-    if (lane == 0) d_out[i] = G.Cn * (G.Wc * (1.0 + sum));   // the self term W(0)
+    if (lane == 0) d_out[i] = G.norm * (G.self + sum);
 }
 
 // The equation of state, one thread per particle (a general power: on one
@@ -306,12 +312,6 @@ struct NaErr {
     void operator=(const std::string &m) { sdpd::set_last_error(m.c_str()); }
 } g_na_err;
 
-double na_W(double r, double h)
-{
-    if (r >= h) return 0.0;
-    const double q = r / h, om = 1.0 - q;
-    return 105.0 / (16.0 * sdpd::PI * h * h * h) * (1.0 + 3.0 * q) * om * om * om;
-}
 }  // namespace
 
 extern "C" sdpd_status sdpd_density_noalloc(const sdpd_params *p, long long n, const double *x,
@@ -381,9 +381,11 @@ extern "C" sdpd_status sdpd_density_noalloc(const sdpd_params *p, long long n, c
         return SDPD_E_INVALID;
     }
     const double h = p->r_c;
-    G.inv_rc = 1.0 / h;
-    G.inv_rc_lo = std::fma(-G.inv_rc, h, 1.0) * G.inv_rc;
     G.rc2 = h * h;
+    int ex = 0;
+    G.R = 2.0 * std::frexp(h, &ex);
+    G.two_k = std::ldexp(1.0, 1 - ex);
+    G.R4 = 4.0 * G.R;
     for (int a = 0; a < 3; ++a) {
         // a periodic box is a whole number of windows (the fixed-point
         // coordinates wrap with it); a box below 8 r_c is one window
@@ -402,13 +404,27 @@ extern "C" sdpd_status sdpd_density_noalloc(const sdpd_params *p, long long n, c
     }
     // FP32 products of fixed-point differences: relative error of r^2 below 1e-6
     G.r2_hi = 1.0f + 1e-5f;
-    G.Wc = 105.0 / (16.0 * sdpd::PI * h * h * h);
+    // the normalisation: the weights of a perfect lattice, self included, sum to
+    // 1 / (norm dx^3).  Sums of rows of planes: rounded a dozen times on the way,
+    // not once a site.
+    auto weight = [&](double r) {
+        if (r >= h) return 0.0;
+        const double t = std::fma(-r, G.two_k, G.R);
+        return std::fma(-3.0, t, G.R4) * (t * t * t);
+    };
     const int m = (int)std::ceil(h / p->dx) + 1;
     double lat = 0.0;
-    for (int k = -m; k <= m; ++k)
-        for (int j = -m; j <= m; ++j)
-            for (int i = -m; i <= m; ++i) lat += na_W(std::sqrt((double)(i * i + j * j + k * k)) * p->dx, h);
-    G.Cn = 1.0 / (p->dx * p->dx * p->dx * lat);
+    for (int k = -m; k <= m; ++k) {
+        double plane = 0.0;
+        for (int j = -m; j <= m; ++j) {
+            double row = 0.0;
+            for (int i = -m; i <= m; ++i) row += weight(std::sqrt((double)(i * i + j * j + k * k)) * p->dx);
+            plane += row;
+        }
+        lat += plane;
+    }
+    G.norm = 1.0 / (p->dx * p->dx * p->dx * lat);
+    G.self = weight(0.0);
     G.mf = p->rho0 * p->dx * p->dx * p->dx;
     G.inv_dx3 = 1.0 / (p->dx * p->dx * p->dx);
     G.rho0 = p->rho0;
